@@ -127,7 +127,11 @@ typedef struct {
  *           of the kept indices only (inverse iteration, back-transformation);
  *           (8/3) n^3 + O(n^2) flops whatever the rank.
  *   AUTO    BIDIAG where the matrices can have full rank (n >= 64 and the
- *           plaquette's inner dimension d^2 >= n / 2), JACOBI elsewhere.
+ *           plaquette's inner dimension d^2 >= n / 2), JACOBI elsewhere; a
+ *           level with d^2 < n (the first one that trajectories split on
+ *           their own) through the d^2 x d^2 core of the QR factors of the
+ *           plaquette's two operands, whose singular values are the nonzero
+ *           ones of its matrices, by the same rule at side d^2.
  *   BAND    AUTO's choice, with the two-stage route in place of BIDIAG where
  *           n is a multiple of 8 from 64 to 256 (chi <= 16): the reduction's
  *           (8/3) n^3 flops as exact integer products of 8-bit digit slices

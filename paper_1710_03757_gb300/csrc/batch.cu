@@ -38,6 +38,7 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "kernels_bd.h"
+#include "kernels_lr.h"
 #include "kernels_tc.h"
 #include "mctrg_internal.h"
 
@@ -128,15 +129,22 @@ __global__ void k_fill_random(double* x, int64_t n, uint64_t seed) {
 
 // Workspace bytes of one item of level k of a job (packed per segment).
 struct ItemLayout {
-  size_t x, m, w, bd, sig, perm, nnz, kept, sigt, nk, vrows, oz, ozexp, total;
+  size_t x, m, w, bd, sig, perm, nnz, kept, sigt, nk, vrows, oz, ozexp, lr_vt, lr_tau, lr_h;
 };
 
 ItemLayout layout(const mctrg_ctx* c, int k, int prec) {
   const LevelInfo& a = c->lv[k];
   const LevelInfo& p = c->lv[k - 1];
-  const size_t n = a.n, np = a.n_pad, d2 = (size_t)p.D * p.D;
+  const size_t d2 = (size_t)p.D * p.D;
+  const SvdDims v = svd_dims(c->opt, a, (int)d2);
+  const size_t n = v.n, np = v.n_pad;              // the split's matrices
   ItemLayout L{};
-  L.x = n * d2 * sizeof(double);
+  L.x = (size_t)a.n * d2 * sizeof(double);
+  if (v.lowrank) {
+    L.lr_vt = lowrank_vt_doubles(a.n, v.n) * sizeof(double);
+    L.lr_tau = lowrank_tau_doubles(v.n) * sizeof(double);
+    L.lr_h = lowrank_halves_doubles(v.n, a.kc) * sizeof(double);
+  }
   L.m = n * n * sizeof(double);
   L.w = np * n * sizeof(double);
   L.bd = 3 * n * sizeof(double);
@@ -148,17 +156,15 @@ ItemLayout layout(const mctrg_ctx* c, int k, int prec) {
   L.sigt = ks * sizeof(double);
   L.nk = sizeof(int);
   L.vrows = ks * n * sizeof(double);
-  L.oz = (prec == MCTRG_FP64TC && gemm_ozaki_supported((int)n, (int)d2)) ? 8 * n * d2 * 2 : 0;
+  L.oz = (prec == MCTRG_FP64TC && !v.lowrank && gemm_ozaki_supported((int)n, (int)d2)) ? 8 * n * d2 * 2 : 0;
   L.ozexp = L.oz ? n * sizeof(int) : 0;
-  L.total = 2 * L.x + L.m + L.w + L.bd + L.sig + L.perm + L.nnz + L.kept + L.sigt + L.nk + L.vrows + 2 * L.oz +
-            2 * L.ozexp;
   return L;
 }
 
 // Pointers of a segment's arrays inside the workspace (each array covers the
 // segment's cnt items contiguously).
 struct SegPtrs {
-  double *X, *Y, *M, *W, *bd, *sig, *sigt, *vrows;
+  double *X, *Y, *M, *W, *bd, *sig, *sigt, *vrows, *lr_vt, *lr_tau, *lr_h;
   int *perm, *nnz, *kept, *nk, *ezX, *ezY;
   void *ozX, *ozY;
 };
@@ -185,12 +191,18 @@ SegPtrs carve(char* base, size_t off, const ItemLayout& L, int64_t cnt) {
     p.ezX = (int*)take(L.ozexp);
     p.ezY = (int*)take(L.ozexp);
   }
+  if (L.lr_vt) {
+    p.lr_vt = (double*)take(L.lr_vt);
+    p.lr_tau = (double*)take(L.lr_tau);
+    p.lr_h = (double*)take(L.lr_h);
+  }
   return p;
 }
 
 size_t segment_bytes(const ItemLayout& L, int64_t cnt) {
   size_t b = 0;
-  const size_t per[] = {L.x, L.x, L.m, L.w, L.bd, L.sig, L.perm, L.nnz, L.kept, L.sigt, L.nk, L.vrows};
+  const size_t per[] = {L.x,    L.x,    L.m,     L.w,      L.bd,    L.sig, L.perm, L.nnz,
+                        L.kept, L.sigt, L.nk, L.vrows, L.lr_vt, L.lr_tau, L.lr_h};
   for (size_t s : per) b += align_up(s * (size_t)cnt);
   if (L.oz) b += 2 * align_up(L.oz * (size_t)cnt) + 2 * align_up(L.ozexp * (size_t)cnt);
   return b;
@@ -344,7 +356,6 @@ struct BatchRunner {
     const int used = (int)std::min<size_t>(segs.size(), kStreams);
     std::vector<SegPtrs> ptr(segs.size());
     std::vector<SvdItem> items;
-    std::vector<int> item_n;          // side of each item (for chunking by shape)
     int n_max = 0, kmax = 0;
     size_t smem = 0;
     BCK(fork(used) == MCTRG_OK ? cudaSuccess : cudaErrorUnknown);
@@ -362,10 +373,21 @@ struct BatchRunner {
       xa.H = c->Hbuf[r.prev].as<double>(); xa.h_item0 = 0; xa.d = p.D; xa.D = p.kc; xa.c0 = g.i0;
       xa.n_items = g.cnt; xa.Nnew = a.N; xa.Nold = p.N; xa.L = c->L; xa.level_old = g.k - 1;
       xa.fixed_parents = 0; xa.X = q.X; xa.Yt = q.Y;
-      BCK(launch_form_xy(xa, ss));
       const int Kd = p.D * p.D;
+      const SvdDims v = svd_dims(c->opt, a, Kd);
+      xa.by_parity = v.lowrank;
+      BCK(launch_form_xy(xa, ss));
       const int tc_kind = (prec == MCTRG_TF32 || prec == MCTRG_TF32X3) ? 0 : 1;
-      if (oz_mode && gemm_ozaki_supported(a.n, Kd)) {
+      if (v.lowrank) {               // QR of both factors, then the K x K core in the place of M
+        LowRankQrArgs qa{};
+        qa.X = q.X; qa.Yt = q.Y; qa.Vt = q.lr_vt; qa.taus = q.lr_tau; qa.n = a.n; qa.K = Kd; qa.S = (int)g.cnt;
+        BCK(launch_lowrank_qr(qa, ss));
+        GemmArgs gm{};
+        gm.X = q.X; gm.Yt = q.Y; gm.M = q.M; gm.D = p.D; gm.K = Kd; gm.c0 = 0; gm.n_items = g.cnt; gm.Nnew = 1;
+        gm.L = c->L; gm.level_new = g.k; gm.fixed_parity = 0; gm.in_stride = (int64_t)a.n * Kd; gm.upper = 1;
+        BCK(launch_gemm_f64(gm, ss));
+        launches += 2;
+      } else if (oz_mode && gemm_ozaki_supported(a.n, Kd)) {
         int bits, slices;
         ozaki_params(Kd, &bits, &slices);
         BCK(launch_ozaki_split(q.X, g.cnt * a.n, Kd, q.ozX, q.ezX, ss));
@@ -389,25 +411,25 @@ struct BatchRunner {
       if (g.bidiag) {
         for (int64_t i = 0; i < g.cnt; ++i) {
           SvdItem t{};
-          t.M = q.M + (size_t)i * a.n * a.n; t.W = q.W + (size_t)i * a.n_pad * a.n; t.bd = q.bd + (size_t)i * 3 * a.n;
-          t.sig = q.sig + (size_t)i * a.n_pad; t.perm = q.perm + (size_t)i * a.n_pad; t.nnz = q.nnz + i;
+          t.M = q.M + (size_t)i * v.n * v.n; t.W = q.W + (size_t)i * v.n_pad * v.n; t.bd = q.bd + (size_t)i * 3 * v.n;
+          t.sig = q.sig + (size_t)i * v.n_pad; t.perm = q.perm + (size_t)i * v.n_pad; t.nnz = q.nnz + i;
           const size_t ks = kept_stride(c->chi);
           t.lns1 = c->ilns1.as<double>() + g.i0 + i; t.kept = q.kept + (size_t)i * ks; t.nk = q.nk + i;
-          t.vrows = q.vrows + (size_t)i * ks * a.n; t.zero_rel = zero_fp64(a.n); t.n = a.n; t.n_pad = a.n_pad;
+          t.vrows = q.vrows + (size_t)i * ks * v.n; t.zero_rel = zero_fp64(a.n); t.n = v.n; t.n_pad = v.n_pad;
           items.push_back(t);
-          item_n.push_back(a.n);
         }
-        n_max = std::max(n_max, a.n);
+        n_max = std::max(n_max, v.n);
         kmax = std::max(kmax, a.kc);
-        smem = std::max(smem, bidiag_smem_bytes(a.n));
+        smem = std::max(smem, bidiag_smem_bytes(v.n));
       } else {
         // the Jacobi route (low-rank levels): per segment, as mctrg_run does
         JacobiArgs ja{};
         ja.M = q.M; ja.W = q.W; ja.sig = q.sig; ja.perm = q.perm; ja.lns1 = c->ilns1.as<double>() + g.i0;
-        ja.nnz = q.nnz; ja.mflags = c->iflags.as<uint32_t>() + g.i0; ja.n = a.n; ja.n_pad = a.n_pad;
+        ja.nnz = q.nnz; ja.mflags = c->iflags.as<uint32_t>() + g.i0; ja.n = v.n; ja.n_pad = v.n_pad;
         ja.S = (int)g.cnt; ja.max_sweeps = c->opt.max_sweeps; ja.zero_rel = zero_fp64(a.n);
         BCK(launch_jacobi(ja, ss));
         BCK(launch_sample_split(sample_args(r, g, q, 0, s), ss, tuned(a.n, a.kc).sample_grid));
+        BCK(expand_lowrank(r, g, q, ss));
         launches += 2;
       }
     }
@@ -453,6 +475,7 @@ struct BatchRunner {
           const LevelInfo& a = r.ctx->lv[segs[s].k];
           BCK(launch_sample_split(sample_args(r, segs[s], ptr[s], 2, s), pool[s % kStreams],
                                   tuned(a.n, a.kc).sample_grid));
+          BCK(expand_lowrank(r, segs[s], ptr[s], pool[s % kStreams]));
           ++launches;
         }
       BCK(join(used) == MCTRG_OK ? cudaSuccess : cudaErrorUnknown);
@@ -463,17 +486,33 @@ struct BatchRunner {
   SampleArgs sample_args(JobRun& r, const Segment& g, const SegPtrs& q, int mode, size_t s) {
     mctrg_ctx* c = r.ctx;
     const LevelInfo& a = c->lv[g.k];
+    const SvdDims v = svd_dims(c->opt, a, c->lv[g.k - 1].D * c->lv[g.k - 1].D);
     SampleArgs sa{};
     sa.M = q.M; sa.sig = q.sig; sa.nnz = q.nnz; sa.Urows = nullptr; sa.perm = q.perm;
-    sa.n = a.n; sa.n_pad = a.n_pad; sa.chi = c->chi; sa.kc = a.kc; sa.stochastic = 1; sa.shared_svd = 0;
+    sa.n = v.n; sa.n_pad = v.n_pad; sa.chi = c->chi; sa.kc = a.kc; sa.stochastic = 1; sa.shared_svd = 0;
     sa.item0 = g.i0; sa.n_items = g.cnt; sa.N = a.N; sa.L = c->L; sa.level = g.k; sa.seed = r.job.seed;
-    sa.traj0 = r.job.first_traj; sa.H = c->Hbuf[r.cur].as<double>(); sa.h_item0 = 0;
-    sa.iflags = c->iflags.as<uint32_t>(); sa.scratch = smp_scr.as<double>() + (s % kStreams) * smp_region;
+    sa.traj0 = r.job.first_traj;
+    sa.H = v.lowrank ? q.lr_h : c->Hbuf[r.cur].as<double>();   // the level's halves, or those of its cores
+    sa.h_item0 = v.lowrank ? g.i0 : 0;
+    sa.iflags = c->iflags.as<uint32_t>() + sa.h_item0; sa.scratch = smp_scr.as<double>() + (s % kStreams) * smp_region;
     sa.mode = mode;
     sa.kstride = kept_stride(c->chi);
     if (mode == 0) { sa.W = q.W; }
     else { sa.W = nullptr; sa.kept = q.kept; sa.sigt = q.sigt; sa.nk = q.nk; sa.vrows = q.vrows; }
     return sa;
+  }
+
+  // the level's halves from those of a low-rank segment's cores
+  cudaError_t expand_lowrank(JobRun& r, const Segment& g, const SegPtrs& q, cudaStream_t ss) {
+    if (!q.lr_vt) return cudaSuccess;
+    mctrg_ctx* c = r.ctx;
+    const LevelInfo& a = c->lv[g.k];
+    LowRankExpandArgs ea{};
+    ea.Vt = q.lr_vt; ea.taus = q.lr_tau; ea.Hc = q.lr_h;
+    ea.H = c->Hbuf[r.cur].as<double>() + (size_t)g.i0 * 2 * a.n * a.kc;
+    ea.n = a.n; ea.K = c->lv[g.k - 1].D * c->lv[g.k - 1].D; ea.S = (int)g.cnt; ea.kc = a.kc;
+    ++launches;
+    return launch_lowrank_expand(ea, ss);
   }
 
   // ---- the autotuner ---------------------------------------------------------
@@ -604,9 +643,10 @@ extern "C" int mctrg_batch_run(const mctrg_options* opt, const mctrg_job* jobs, 
     if (c->all_exact) continue;
     for (int k = c->s0 + 1; k < c->nlev && status == MCTRG_OK; ++k) {
       const int Kd = c->lv[k - 1].D * c->lv[k - 1].D;
-      if (!c->use_bidiag(c->lv[k].n, Kd)) continue;
-      if (R.tune.count(TuneKey{c->lv[k].n, c->lv[k].kc})) continue;
-      status = R.tune_shape(c->lv[k].n, c->lv[k].kc);
+      const int n = svd_dims(c->opt, c->lv[k], Kd).n;
+      if (!c->use_bidiag(n, Kd)) continue;
+      if (R.tune.count(TuneKey{n, c->lv[k].kc})) continue;
+      status = R.tune_shape(n, c->lv[k].kc);
     }
   }
   if (status == MCTRG_OK && R.tune_dirty) {
@@ -652,7 +692,7 @@ extern "C" int mctrg_batch_run(const mctrg_options* opt, const mctrg_job* jobs, 
           mctrg_ctx* c = r.ctx;
           const ItemLayout L = layout(c, r.k, R.opt.precision);
           const int Kd = c->lv[r.k - 1].D * c->lv[r.k - 1].D;
-          const bool bd = c->use_bidiag(c->lv[r.k].n, Kd);
+          const bool bd = c->use_bidiag(svd_dims(c->opt, c->lv[r.k], Kd).n, Kd);
           int64_t cap = std::min<int64_t>(r.items - r.next, 1 << 16);
           // every job still at work gets an equal share of the workspace
           int active = 0;

@@ -113,6 +113,22 @@ constexpr uint32_t FLAG_SPLIT_CLUSTER = 1u, FLAG_DRAW_TIE = 2u, FLAG_TINY_KEPT =
                    FLAG_NOCONV = 16u;
 constexpr double GAP_TOL = 1e-8, TIE_TOL = 1e-9, TINY_TOL = 1e-7;
 
+// 4-value warp sum: on return lanes 0, 8, 16, 24 hold the sums of p0, p1, p2, p3.
+__device__ __forceinline__ double reduce4(double p0, double p1, double p2, double p3, int lane) {
+  const bool hi16 = lane & 16, hi8 = lane & 8;
+  double q0 = hi16 ? p2 : p0, q1 = hi16 ? p3 : p1;
+  const double r0 = hi16 ? p0 : p2, r1 = hi16 ? p1 : p3;
+  q0 += __shfl_xor_sync(0xffffffffu, r0, 16);
+  q1 += __shfl_xor_sync(0xffffffffu, r1, 16);
+  double t = hi8 ? q1 : q0;
+  const double tr = hi8 ? q0 : q1;
+  t += __shfl_xor_sync(0xffffffffu, tr, 8);
+  t += __shfl_xor_sync(0xffffffffu, t, 4);
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  return t;
+}
+
 // Raise a kernel's dynamic shared-memory limit on the current device, once
 // per (kernel, device); safe to call from several host threads at once (a
 // race only repeats the call).  `done` holds one bit per device ordinal

@@ -1108,7 +1108,7 @@ __global__ void __launch_bounds__(kChaseWarps * 32) k_band_chase(BandArgs a, int
 }
 
 // ---------------------------------------------------------------------------
-// v = P1 P2 v_B for up to 16 kept vectors of one matrix, one CTA of 128
+// v = P1 P2 v_B for a group of up to 16 kept vectors of one matrix, one CTA of 128
 // threads; the vectors in shared memory (row stride n + 1: the 16 vectors in
 // different banks).  P2: the chase's sweeps in reverse order; the right
 // reflectors of one sweep act on disjoint column blocks c0 = i + 1 + 8q, so
@@ -1124,8 +1124,10 @@ __global__ void __launch_bounds__(kBtThreads) k_band_backtr(BandArgs a, BandVecA
   const int s = blockIdx.x, n = a.n, t = threadIdx.x;
   const int ld = n + 1;
   double* Us = Vs + (size_t)16 * ld;
-  const int nk = min(va.nk[s], 16);
-  double* vrow = va.vrows + (size_t)s * va.kstride * n;
+  const int g0 = 16 * blockIdx.y;                     // first kept vector of this group
+  const int nk = min(va.nk[s] - g0, 16);
+  if (nk <= 0) return;
+  double* vrow = va.vrows + ((size_t)s * va.kstride + g0) * n;
   for (int e = t; e < nk * n; e += kBtThreads) Vs[(e / n) * ld + e % n] = vrow[e];
   __syncthreads();
   const double* refl = a.refl + (size_t)s * nref * B;
@@ -1193,7 +1195,7 @@ __global__ void __launch_bounds__(kBtThreads) k_band_backtr(BandArgs a, BandVecA
     __syncthreads();
   }
   const double* sg = va.sig + (size_t)s * va.n_pad;
-  const int* kept = va.kept + (size_t)s * va.kstride;
+  const int* kept = va.kept + (size_t)s * va.kstride + g0;
   for (int e = t; e < nk * n; e += kBtThreads) {
     const double x = Vs[(e / n) * ld + e % n];
     vrow[e] = va.unit_rows ? x : sg[kept[e / n]] * x;
@@ -1256,7 +1258,8 @@ cudaError_t launch_band_backtr(const BandVecArgs& va, cudaStream_t st) {
   const size_t smem = bytes(a.n);
   cudaError_t e = raise_smem_limit(k_band_backtr, (int)bytes(256), at);
   if (e != cudaSuccess) return e;
-  k_band_backtr<<<a.S, kBtThreads, smem, st>>>(a, va, band_nref(a.n));
+  const dim3 grid((unsigned)a.S, (unsigned)((std::max(1, va.kmax) + 15) / 16));
+  k_band_backtr<<<grid, kBtThreads, smem, st>>>(a, va, band_nref(a.n));
   return cudaGetLastError();
 }
 

@@ -89,22 +89,6 @@ __device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >
 //    warp takes up to four rows at a time and reduces their dots together;
 //    the right reflector enters as us = sqrt(tauR) u (G = I - us us^T).
 
-// 4-value warp sum: on return lanes 0, 8, 16, 24 hold the sums of p0, p1, p2, p3.
-__device__ __forceinline__ double reduce4(double p0, double p1, double p2, double p3, int lane) {
-  const bool hi16 = lane & 16, hi8 = lane & 8;
-  double q0 = hi16 ? p2 : p0, q1 = hi16 ? p3 : p1;
-  const double r0 = hi16 ? p0 : p2, r1 = hi16 ? p1 : p3;
-  q0 += __shfl_xor_sync(0xffffffffu, r0, 16);
-  q1 += __shfl_xor_sync(0xffffffffu, r1, 16);
-  double t = hi8 ? q1 : q0;
-  const double tr = hi8 ? q0 : q1;
-  t += __shfl_xor_sync(0xffffffffu, tr, 8);
-  t += __shfl_xor_sync(0xffffffffu, t, 4);
-  t += __shfl_xor_sync(0xffffffffu, t, 2);
-  t += __shfl_xor_sync(0xffffffffu, t, 1);
-  return t;
-}
-
 struct BdStep {
   double* A;
   const double* vcol;

@@ -36,6 +36,30 @@ __global__ void k_form_xy(XYArgs a) {
   auto half_left = [&](int q) { return a.H + (b * a.Nold + par[q] - a.h_item0) * stride; };
   auto half_right = [&](int q) { return half_left(q) + (int64_t)d2 * D; };
   const int sel = blockIdx.y;
+  if (a.by_parity && tensor_parity(a.L, a.level_old + 1, c) == 1) {
+    // sublattice B in its own matricization: rows (be,de) and (ga,al), inner (i,m)
+    const double* F1 = half_left(3);
+    const double* F2 = half_left(2);
+    const double* F3 = half_right(0);
+    const double* F4 = half_right(1);
+    const bool x = blockIdx.z == 0;          // X': sel = be, inner rows de; Yt': sel = ga, inner rows al
+    for (int e = threadIdx.x; e < d2; e += blockDim.x) s_a[e] = x ? F4[(int64_t)sel * d2 + e] : F2[(int64_t)e * D + sel];
+    double* Oo = (x ? a.X : a.Yt) + ((int64_t)it * D * D + (int64_t)sel * D) * d2;
+    for (int in = 0; in < D; ++in) {
+      __syncthreads();
+      for (int e = threadIdx.x; e < d2; e += blockDim.x) s_b[e] = x ? F1[(int64_t)e * D + in] : F3[(int64_t)in * d2 + e];
+      __syncthreads();
+      for (int e = threadIdx.x; e < d2; e += blockDim.x) {
+        const int i = e / d, m = e - i * d;
+        double acc = 0.0;
+        // X': sum_k F4[be][k,i] F1[m,k][de];  Yt': sum_j F2[j,m][ga] F3[al][i,j]
+        if (x) for (int k = 0; k < d; ++k) acc = fma(s_a[k * d + i], s_b[m * d + k], acc);
+        else for (int j = 0; j < d; ++j) acc = fma(s_a[j * d + m], s_b[i * d + j], acc);
+        Oo[(int64_t)in * d2 + e] = acc;
+      }
+    }
+    return;
+  }
   if (blockIdx.z == 0) {
     // X[(al,be)][(j,k)] = sum_i F3[al][i*d+j] * F4[be][k*d+i]
     const double* F3 = half_right(0) + (int64_t)sel * d2;
@@ -95,12 +119,13 @@ __global__ void __launch_bounds__(256) k_gemm_f64(GemmArgs a) {
   const int tiles_c = (n + TM - 1) / TM;
   const int tr = blockIdx.y / tiles_c, tcol = blockIdx.y % tiles_c;
   const int64_t it = blockIdx.x;
-  const double* X = a.X + (int64_t)it * n * K;
-  const double* Y = a.Yt + (int64_t)it * n * K;
+  const int64_t stride = a.in_stride > 0 ? a.in_stride : (int64_t)n * K;
+  const double* X = a.X + it * stride;
+  const double* Y = a.Yt + it * stride;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int r0 = tr * TM, c0 = tcol * TM;
   double acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += TK) {
+  for (int k0 = a.upper ? max(r0, c0) : 0; k0 < K; k0 += TK) {
     for (int e = threadIdx.x; e < TM * TK; e += 256) {
       const int rr = e / TK, kk = e - rr * TK;
       const int gr = r0 + rr, gc = c0 + rr, gk = k0 + kk;

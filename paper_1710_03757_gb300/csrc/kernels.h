@@ -78,7 +78,10 @@ cudaError_t launch_u_rows(const double* M, const double* W, const double* sig, c
 // ---- K5: plaquette contraction ----------------------------------------------
 // New tensor T'[al,be,de,ga] = sum_{i,j,k,m} F3[al,i,j] F4[be,k,i] F2[j,m,ga] F1[m,k,de]
 // from the four parent halves, as X[(al,be)][(j,k)] = sum_i F3 F4 and
-// Yt[(de,ga)][(j,k)] = sum_m F2 F1, then T' = X Yt^T.
+// Yt[(de,ga)][(j,k)] = sum_m F2 F1, then T' = X Yt^T.  With by_parity a tensor
+// of sublattice B gets the factors of its own matricization instead, cut
+// through the other pair of bonds: M[(be,de)][(ga,al)] = X' Yt'^T with
+// X'[(be,de)][(i,m)] = sum_k F4 F1 and Yt'[(ga,al)][(i,m)] = sum_j F2 F3.
 struct XYArgs {
   const double* H;       // parent halves (level k-1), stride 2 d^2 D per item
   int64_t h_item0;       // item index of H[0]
@@ -87,6 +90,7 @@ struct XYArgs {
   int64_t Nnew, Nold;    // tensors per trajectory at the new / parent level
   int L, level_old;      // geometry of the parent level
   int fixed_parents;     // 1: parents are items (0,1,1,0) (shared plaquette)
+  int by_parity;         // 1: the factors of the new tensor's own matricization (below)
   double* X;             // [n_items][D*D][d*d]
   double* Yt;            // [n_items][D*D][d*d]
 };
@@ -101,6 +105,8 @@ struct GemmArgs {
   int64_t c0, n_items, Nnew;
   int L, level_new;      // geometry for the parity of the new tensors
   int fixed_parity;      // >= 0 overrides the geometry (0 = A / raw)
+  int64_t in_stride;     // doubles between items of X (and of Yt); 0 = D*D*K
+  int upper;             // 1: X and Yt are upper triangular (K = D*D): products start at max(row, column)
 };
 cudaError_t launch_gemm_f64(const GemmArgs& a, cudaStream_t st);
 

@@ -49,14 +49,14 @@ cudaError_t launch_band_chase(const BandArgs& a, cudaStream_t st);
 
 // v = P1 P2 v_B for the kept vectors: vrows[s][a][:] holds v_B on entry
 // (unit vectors of the bidiagonal, from the inverse iteration) and s_r v_r on
-// return (v_r with unit_rows).  kmax <= 16.
+// return (v_r with unit_rows).  kmax: the largest nk of the batch.
 struct BandVecArgs {
   const BandArgs* band;   // the reduction's buffers (host copy of the struct)
   const double* sig;      // [S][n_pad]
   const int* kept;        // [S][kstride]
   const int* nk;          // [S]
   double* vrows;          // [S][kstride][n]
-  int n_pad, kstride, unit_rows;
+  int n_pad, kstride, unit_rows, kmax;
 };
 cudaError_t launch_band_backtr(const BandVecArgs& a, cudaStream_t st);
 

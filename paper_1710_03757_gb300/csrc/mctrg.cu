@@ -6,7 +6,9 @@
 // the translation-invariant network are still identical), so only the
 // sampling and the split run per (trajectory, tensor).  Every later level
 // runs, per sub-batch of (trajectory, tensor) items:
-//   form X, Yt -> GEMM (+ matricization) -> Jacobi SVD -> sample + split,
+//   form X, Yt -> GEMM (+ matricization) -> SVD -> sample + split
+// (a level of inner dimension below the matrix side: form X, Yt -> QR of both
+// -> core -> SVD of the core -> sample + split -> expand the halves),
 // then adds each tensor's ln s_1 to its trajectory.  The last level's halves
 // are contracted and traced directly.
 #include <algorithm>
@@ -20,6 +22,7 @@
 #include "kernels.h"
 #include "kernels_band.h"
 #include "kernels_bd.h"
+#include "kernels_lr.h"
 #include "kernels_tc.h"
 #include "mctrg_internal.h"
 
@@ -167,7 +170,7 @@ size_t mctrg_ctx::held_bytes() const {
                          &Mb, &Wb, &Xb, &Yb, &sigb, &permb, &nnzb, &ilns1, &iflags, &lnacc, &tflags,
                          &scratch, &o_lnabs, &o_sign, &o_flags, &o_tflags, &stats, &tcXh, &tcYh, &tcXl,
                          &tcYl, &tcScale, &tcErr, &ozExp, &Timp, &bdb, &keptb, &sigtb, &nkb, &vrowsb, &bdscr,
-                         &bandb};
+                         &bandb, &lrb};
   size_t b = 0;
   for (const DevBuf* d : all) b += d->bytes;
   return b;
@@ -181,7 +184,7 @@ void mctrg_ctx::release_all() {
                    &Mb, &Wb, &Xb, &Yb, &sigb, &permb, &nnzb, &ilns1, &iflags, &lnacc, &tflags,
                    &scratch, &o_lnabs, &o_sign, &o_flags, &o_tflags, &stats, &tcXh, &tcYh, &tcXl,
                    &tcYl, &tcScale, &tcErr, &ozExp, &Timp, &bdb, &keptb, &sigtb, &nkb, &vrowsb, &bdscr,
-                   &bandb};
+                   &bandb, &lrb};
   for (DevBuf* b : all) b->release();
 }
 
@@ -314,6 +317,15 @@ bool route_bidiag(const mctrg_options& o, int n, int K) {
 bool route_band(const mctrg_options& o, int n, int K) {
   return o.svd == MCTRG_SVD_BAND && band_supported(n) && route_bidiag(o, n, K);
 }
+// A level of inner dimension K < n goes through the K x K core of its factors
+// (kernels_lr.h), unless the caller named a route for the matrices themselves
+// or the contraction's rounding (the mixed modes, where their GEMM covers the
+// level) is part of the result.
+bool route_lowrank(const mctrg_options& o, int n, int K) {
+  if (o.svd == MCTRG_SVD_JACOBI || o.svd == MCTRG_SVD_BIDIAG || !lowrank_supported(n, K)) return false;
+  if (o.precision == MCTRG_FP64 || o.precision == MCTRG_FP64TC) return true;
+  return !gemm_tc_supported(n, K, (o.precision == MCTRG_TF32 || o.precision == MCTRG_TF32X3) ? 0 : 1);
+}
 }  // namespace mctrg
 
 bool mctrg_ctx::use_bidiag(int n, int K) const { return route_bidiag(opt, n, K); }
@@ -422,6 +434,11 @@ static size_t tc_operand_bytes(int prec, int n, int d2) {
 }
 
 namespace mctrg {
+SvdDims svd_dims(const mctrg_options& o, const LevelInfo& a, int K) {
+  if (route_lowrank(o, a.n, K)) return SvdDims{true, K, K + (K & 1)};
+  return SvdDims{false, a.n, a.n_pad};
+}
+
 // The sampler's CTA count for a run over levels s0 .. nlev-1 (from the largest
 // side), and the table scratch it needs.
 int run_sample_grid(const std::vector<LevelInfo>& lv, int s0, int nlev, int chi) {
@@ -456,15 +473,17 @@ void plan_run(const std::vector<LevelInfo>& lv, int s0, int nlev, int chi, const
     if (k > s0) {
       maxN = std::max<int64_t>(maxN, a.N);
       const size_t d2 = (size_t)lv[k - 1].D * lv[k - 1].D;
-      size_t pi = (2 * (size_t)a.n * d2 + (size_t)a.n * a.n + (size_t)a.n_pad * a.n + a.n_pad) * sizeof(double) +
-                  (a.n_pad + 1) * sizeof(int) + sizeof(double) + sizeof(uint32_t);
-      pi += tc_operand_bytes(opt.precision, a.n, (int)d2);
-      if (route_bidiag(opt, a.n, (int)d2)) {   // d, e, tau; kept values and vectors
+      const SvdDims v = svd_dims(opt, a, (int)d2);      // the split's matrices: the level's, or its cores
+      size_t pi = (2 * (size_t)a.n * d2 + (size_t)v.n * v.n + (size_t)v.n_pad * v.n + v.n_pad) * sizeof(double) +
+                  (v.n_pad + 1) * sizeof(int) + sizeof(double) + sizeof(uint32_t);
+      if (v.lowrank) pi += lowrank_item_doubles(a.n, v.n, a.kc) * sizeof(double);
+      else pi += tc_operand_bytes(opt.precision, a.n, (int)d2);
+      if (route_bidiag(opt, v.n, (int)d2)) {   // d, e, tau; kept values and vectors
         const size_t ks = kept_stride(chi);
-        pi += (3 * (size_t)a.n + ks + ks * (size_t)a.n) * sizeof(double) + (ks + 1) * sizeof(int);
-        bd_scr = std::max(bd_scr, bd_vectors_scratch_doubles(a.n, 1 << 16, a.kc) * sizeof(double));
+        pi += (3 * (size_t)v.n + ks + ks * (size_t)v.n) * sizeof(double) + (ks + 1) * sizeof(int);
+        bd_scr = std::max(bd_scr, bd_vectors_scratch_doubles(v.n, 1 << 16, a.kc) * sizeof(double));
         // the band route: band, panel scratch, chase reflectors, exponent
-        if (route_band(opt, a.n, (int)d2)) pi += band_item_bytes(a.n);
+        if (route_band(opt, v.n, (int)d2)) pi += band_item_bytes(v.n);
       }
       per_item = std::max(per_item, pi);
     }
@@ -592,7 +611,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
     CK(lnacc.ensure(sizeof(double) * (size_t)B));
     const int grid_s = run_sample_grid(lv, s0, nlev, chi);
     const int ks = kept_stride(chi);
-    size_t max_h = 0, max_items = 0, max_xy = 0, max_m = 0, max_w = 0, max_np = 0, max_scr = 0;
+    size_t max_h = 0, max_items = 0, max_xy = 0, max_m = 0, max_w = 0, max_np = 0, max_scr = 0, max_lr = 0;
     for (int k = s0; k < nlev; ++k) {
       const LevelInfo& a = lv[k];
       max_h = std::max(max_h, (size_t)B * a.N * 2 * a.n * a.kc);
@@ -600,10 +619,12 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
       max_scr = std::max(max_scr, sample_scratch_doubles(a.n, chi, grid_s));
       if (k > s0) {
         const size_t d2 = (size_t)lv[k - 1].D * lv[k - 1].D;
+        const SvdDims v = svd_dims(opt, a, (int)d2);
         max_xy = std::max(max_xy, (size_t)S * a.n * d2);
-        max_m = std::max(max_m, (size_t)S * a.n * a.n);
-        max_w = std::max(max_w, (size_t)S * a.n_pad * a.n);
-        max_np = std::max(max_np, (size_t)S * a.n_pad);
+        max_m = std::max(max_m, (size_t)S * v.n * v.n);
+        max_w = std::max(max_w, (size_t)S * v.n_pad * v.n);
+        max_np = std::max(max_np, (size_t)S * v.n_pad);
+        if (v.lowrank) max_lr = std::max(max_lr, (size_t)S * lowrank_item_doubles(a.n, v.n, a.kc));
       }
     }
     {
@@ -629,17 +650,23 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
     CK(permb.ensure(sizeof(int) * std::max<size_t>(max_np, 1)));
     CK(nnzb.ensure(sizeof(int) * std::max<int64_t>(S, 1)));
     CK(scratch.ensure(sizeof(double) * max_scr));
+    CK(lrb.ensure(sizeof(double) * max_lr));
     {  // bidiagonalization route buffers (levels that take it)
       size_t bd_n = 0, bd_scr = 0;
       for (int k = s0 + 1; k < nlev; ++k) {
         const LevelInfo& a = lv[k];
-        if (!use_bidiag(a.n, lv[k - 1].D * lv[k - 1].D)) continue;
-        bd_n = std::max(bd_n, (size_t)a.n);
-        bd_scr = std::max(bd_scr, bd_vectors_scratch_doubles(a.n, (int)std::min<int64_t>(S, 1 << 16), a.kc));
+        const int Kd = lv[k - 1].D * lv[k - 1].D;
+        const SvdDims v = svd_dims(opt, a, Kd);
+        if (!use_bidiag(v.n, Kd)) continue;
+        bd_n = std::max(bd_n, (size_t)v.n);
+        bd_scr = std::max(bd_scr, bd_vectors_scratch_doubles(v.n, (int)std::min<int64_t>(S, 1 << 16), a.kc));
       }
       size_t band_n = 0;
-      for (int k = s0 + 1; k < nlev; ++k)
-        if (use_band(lv[k].n, lv[k - 1].D * lv[k - 1].D)) band_n = std::max(band_n, (size_t)lv[k].n);
+      for (int k = s0 + 1; k < nlev; ++k) {
+        const int Kd = lv[k - 1].D * lv[k - 1].D;
+        const SvdDims v = svd_dims(opt, lv[k], Kd);
+        if (use_band(v.n, Kd)) band_n = std::max(band_n, (size_t)v.n);
+      }
       if (band_n) {
         CK(bandb.ensure((size_t)std::max<int64_t>(S, 1) * band_item_bytes((int)band_n) + 256));
         CK(cudaMemsetAsync(bandb.p, 0, bandb.bytes, st));
@@ -675,7 +702,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
       size_t oz_elems = 0, oz_rows = 0;
       for (int k = s0 + 1; k < nlev; ++k) {
         const int Kd = lv[k - 1].D * lv[k - 1].D;
-        if (!gemm_ozaki_supported(lv[k].n, Kd)) continue;
+        if (route_lowrank(opt, lv[k].n, Kd) || !gemm_ozaki_supported(lv[k].n, Kd)) continue;
         oz_elems = std::max(oz_elems, (size_t)S * lv[k].n * Kd);
         oz_rows = std::max(oz_rows, (size_t)S * lv[k].n);
       }
@@ -756,13 +783,32 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
           xa.H = Hbuf[prev].as<double>(); xa.h_item0 = 0; xa.d = p.D; xa.D = p.kc; xa.c0 = i0;
           xa.n_items = Si; xa.Nnew = a.N; xa.Nold = p.N; xa.L = L; xa.level_old = k - 1;
           xa.fixed_parents = 0; xa.X = Xb.as<double>(); xa.Yt = Yb.as<double>();
+          const int Kd = p.D * p.D;
+          const SvdDims v = svd_dims(opt, a, Kd);
+          xa.by_parity = v.lowrank;
           const double D2 = (double)p.kc * p.kc, dd = p.D;
           CK(timed(MCTRG_K_FORM_XY, Si, Si * 4.0 * D2 * dd * dd * dd,
                    8.0 * Si * (4.0 * p.kc * dd * dd + 2.0 * D2 * dd * dd), [&] { return launch_form_xy(xa, st); }));
-          const int Kd = p.D * p.D;
-          const bool used_tc = tc_mode && gemm_tc_supported(a.n, Kd, tc_kind);
-          const bool used_oz = oz_mode && gemm_ozaki_supported(a.n, Kd);
-          if (used_oz) {
+          const bool used_tc = !v.lowrank && tc_mode && gemm_tc_supported(a.n, Kd, tc_kind);
+          const bool used_oz = !v.lowrank && oz_mode && gemm_ozaki_supported(a.n, Kd);
+          double* const lr_vt = lrb.as<double>();       // low-rank levels: reflectors, taus, the cores' halves
+          double* const lr_tau = lr_vt + Si * lowrank_vt_doubles(a.n, Kd);
+          double* const lr_h = lr_tau + Si * lowrank_tau_doubles(Kd);
+          if (v.lowrank) {
+            // QR of both factors, then the K x K core in the place of M
+            LowRankQrArgs qa{};
+            qa.X = Xb.as<double>(); qa.Yt = Yb.as<double>(); qa.Vt = lr_vt; qa.taus = lr_tau;
+            qa.n = a.n; qa.K = Kd; qa.S = (int)Si;
+            const double nd = a.n, kd = Kd;
+            CK(timed(MCTRG_K_OTHER, Si, Si * 2.0 * (2.0 * nd * kd * kd - 2.0 / 3.0 * kd * kd * kd),
+                     8.0 * Si * 2.0 * (2.0 * nd * kd + kd * kd), [&] { return launch_lowrank_qr(qa, st); }));
+            GemmArgs gm{};
+            gm.X = Xb.as<double>(); gm.Yt = Yb.as<double>(); gm.M = Mb.as<double>(); gm.D = p.D; gm.K = Kd;
+            gm.c0 = 0; gm.n_items = Si; gm.Nnew = 1; gm.L = L; gm.level_new = k; gm.fixed_parity = 0;
+            gm.in_stride = (int64_t)a.n * Kd; gm.upper = 1;
+            CK(timed(MCTRG_K_GEMM, Si, Si * 2.0 / 3.0 * kd * kd * kd, 8.0 * Si * 2.0 * kd * kd,
+                     [&] { return launch_gemm_f64(gm, st); }));
+          } else if (used_oz) {
             // FP64-accurate on the tensor cores: BF16 slices of X and Yt, exact slice products
             int oz_bits, oz_slices;
             ozaki_params(Kd, &oz_bits, &oz_slices);
@@ -806,22 +852,26 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
             CK(timed(MCTRG_K_GEMM, Si, Si * 2.0 * a.n * a.n * gm.K, 8.0 * Si * (2.0 * a.n * gm.K + (double)a.n * a.n),
                      [&] { return launch_gemm_f64(gm, st); }));
           }
-          const double nn = a.n;
           const double zero_rel = opt.zero_tol_scale *
-              (used_tc ? std::min(std::sqrt(nn) * tc_unit_roundoff(prec), 1.0 / 64.0) : nn * 0x1.0p-52);
+              (used_tc ? std::min(std::sqrt((double)a.n) * tc_unit_roundoff(prec), 1.0 / 64.0)
+                       : (double)a.n * 0x1.0p-52);
+          const double nn = v.n;
           SampleArgs sa{};
           sa.M = Mb.as<double>(); sa.sig = sigb.as<double>(); sa.nnz = nnzb.as<int>(); sa.Urows = nullptr;
-          sa.n = a.n; sa.n_pad = a.n_pad; sa.chi = chi; sa.kc = a.kc; sa.stochastic = 1; sa.shared_svd = 0;
+          sa.n = v.n; sa.n_pad = v.n_pad; sa.chi = chi; sa.kc = a.kc; sa.stochastic = 1; sa.shared_svd = 0;
           sa.item0 = i0; sa.n_items = Si; sa.N = a.N; sa.L = L; sa.level = k; sa.seed = seed;
-          sa.traj0 = traj0; sa.H = Hbuf[cur].as<double>(); sa.h_item0 = 0;
-          sa.iflags = iflags.as<uint32_t>(); sa.scratch = scratch.as<double>();
-          if (use_bidiag(a.n, Kd)) {
+          sa.traj0 = traj0; sa.scratch = scratch.as<double>();
+          // the halves of the level, or those of its cores (expanded below)
+          sa.H = v.lowrank ? lr_h : Hbuf[cur].as<double>();
+          sa.h_item0 = v.lowrank ? i0 : 0;
+          sa.iflags = iflags.as<uint32_t>() + sa.h_item0;
+          if (use_bidiag(v.n, Kd)) {
             // bidiagonalization (one stage, or dense -> band -> bidiagonal), bisection,
             // choice of the kept indices, their vectors, halves
-            const bool band = use_band(a.n, Kd);
+            const bool band = use_band(v.n, Kd);
             BandArgs bda{};
             if (band) {
-              band_carve(bandb.p, a.n, Si, bda);
+              band_carve(bandb.p, v.n, Si, bda);
               bda.M = Mb.as<double>(); bda.Wk = (int64_t*)Wb.p; bda.bd = bdb.as<double>(); bda.S = (int)Si;
               bda.err = band_err;
               CK(timed(MCTRG_K_BAND, Si, Si * (8.0 / 3.0) * nn * nn * nn, 8.0 * Si * (nn * nn + 9.0 * nn),
@@ -830,22 +880,22 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
                        [&] { return launch_band_chase(bda, st); }));
             } else {
               BidiagArgs ba{};
-              ba.M = Mb.as<double>(); ba.W = Wb.as<double>(); ba.bd = bdb.as<double>(); ba.n = a.n; ba.S = (int)Si;
+              ba.M = Mb.as<double>(); ba.W = Wb.as<double>(); ba.bd = bdb.as<double>(); ba.n = v.n; ba.S = (int)Si;
               CK(timed(MCTRG_K_BIDIAG, Si, Si * (8.0 / 3.0) * nn * nn * nn, 8.0 * Si * (2.0 * nn * nn + 3.0 * nn),
                        [&] { return launch_bidiag(ba, st); }));
             }
-            CK(timed(MCTRG_K_BISECT, Si, 0.0, 8.0 * Si * (3.0 * nn + a.n_pad) + 4.0 * Si * (a.n_pad + 1), [&] {
-              return launch_bd_bisect(bdb.as<double>(), a.n, a.n_pad, (int)Si, sigb.as<double>(), permb.as<int>(),
+            CK(timed(MCTRG_K_BISECT, Si, 0.0, 8.0 * Si * (3.0 * nn + v.n_pad) + 4.0 * Si * (v.n_pad + 1), [&] {
+              return launch_bd_bisect(bdb.as<double>(), v.n, v.n_pad, (int)Si, sigb.as<double>(), permb.as<int>(),
                                       nnzb.as<int>(), ilns1.as<double>() + i0, zero_rel, st); }));
             sa.mode = 1; sa.kept = keptb.as<int>(); sa.sigt = sigtb.as<double>(); sa.nk = nkb.as<int>();
             sa.kstride = ks;
             sa.W = nullptr; sa.perm = permb.as<int>();
-            CK(timed(MCTRG_K_SAMPLE, Si, Si * 4.0 * nn * a.kc, 8.0 * Si * (a.n_pad + 2.0 * ks),
+            CK(timed(MCTRG_K_SAMPLE, Si, Si * 4.0 * nn * a.kc, 8.0 * Si * (v.n_pad + 2.0 * ks),
                      [&] { return launch_sample_split(sa, st, grid_s); }));
             BdVecArgs va{};
             va.bd = bdb.as<double>(); va.R = Wb.as<double>(); va.sig = sigb.as<double>(); va.kept = keptb.as<int>();
             va.nk = nkb.as<int>(); va.vrows = vrowsb.as<double>(); va.scratch = bdscr.as<double>();
-            va.n = a.n; va.n_pad = a.n_pad; va.S = (int)Si; va.kmax = a.kc; va.kstride = ks;
+            va.n = v.n; va.n_pad = v.n_pad; va.S = (int)Si; va.kmax = a.kc; va.kstride = ks;
             va.skip_backtr = band ? 1 : 0;
             CK(timed(MCTRG_K_VECTORS, Si, Si * ((band ? 4.0 : 2.0) * nn * nn * a.kc + 40.0 * nn * a.kc),
                      8.0 * Si * (nn * nn / 2.0 + 3.0 * nn + 2.0 * a.kc * nn), [&] {
@@ -853,7 +903,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
               if (e != cudaSuccess || !band) return e;
               BandVecArgs bv{};
               bv.band = &bda; bv.sig = sigb.as<double>(); bv.kept = keptb.as<int>(); bv.nk = nkb.as<int>();
-              bv.vrows = vrowsb.as<double>(); bv.n_pad = a.n_pad; bv.kstride = ks; bv.unit_rows = 0;
+              bv.vrows = vrowsb.as<double>(); bv.n_pad = v.n_pad; bv.kstride = ks; bv.unit_rows = 0; bv.kmax = a.kc;
               return launch_band_backtr(bv, st); }));
             sa.mode = 2; sa.vrows = vrowsb.as<double>();
             CK(timed(MCTRG_K_SAMPLE, Si, Si * 2.0 * nn * nn * a.kc, 8.0 * Si * (2.0 * nn * nn + 2.0 * nn * a.kc),
@@ -862,16 +912,22 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
             JacobiArgs ja{};
             ja.M = Mb.as<double>(); ja.W = Wb.as<double>(); ja.sig = sigb.as<double>();
             ja.perm = permb.as<int>(); ja.lns1 = ilns1.as<double>() + i0; ja.nnz = nnzb.as<int>();
-            ja.mflags = iflags.as<uint32_t>() + i0; ja.n = a.n; ja.n_pad = a.n_pad; ja.S = (int)Si;
+            ja.mflags = iflags.as<uint32_t>() + i0; ja.n = v.n; ja.n_pad = v.n_pad; ja.S = (int)Si;
             ja.max_sweeps = opt.max_sweeps;
             ja.zero_rel = zero_rel;
             if (used_tc) ja.noise_u = tc_unit_roundoff(prec);
             CK(timed(MCTRG_K_JACOBI, Si, Si * ((8.0 / 3.0) * nn * nn * nn + 4.0 * nn * nn * a.kc),
-                     8.0 * Si * (nn * nn + (double)a.n_pad * nn + 1.5 * a.n_pad), [&] { return launch_jacobi(ja, st); }));
+                     8.0 * Si * (nn * nn + (double)v.n_pad * nn + 1.5 * v.n_pad), [&] { return launch_jacobi(ja, st); }));
             sa.mode = 0; sa.W = Wb.as<double>(); sa.perm = permb.as<int>();
             CK(timed(MCTRG_K_SAMPLE, Si, Si * (4.0 * nn * a.kc + 2.0 * nn * nn * a.kc),
                      8.0 * Si * (2.0 * nn * nn + 2.0 * nn * a.kc), [&] { return launch_sample_split(sa, st, grid_s); }));
-        
+          }
+          if (v.lowrank) {
+            LowRankExpandArgs ea{};
+            ea.Vt = lr_vt; ea.taus = lr_tau; ea.Hc = lr_h; ea.H = Hbuf[cur].as<double>() + (size_t)i0 * 2 * a.n * a.kc;
+            ea.n = a.n; ea.K = Kd; ea.S = (int)Si; ea.kc = a.kc;
+            CK(timed(MCTRG_K_VECTORS, Si, Si * 8.0 * a.n * Kd * a.kc, 8.0 * Si * 2.0 * (Kd + 2.0 * a.kc) * a.n,
+                     [&] { return launch_lowrank_expand(ea, st); }));
           }
         }
         CK(timed(MCTRG_K_OTHER, Bc, 0.0, 12.0 * items, [&] {

@@ -31,8 +31,17 @@ struct LevelInfo {
   int D, n, n_pad, kc;
 };
 
+// The matrices of a level's split: the level's own, or the K x K cores of its
+// factors (low-rank levels).
+struct SvdDims {
+  bool lowrank;
+  int n, n_pad;
+};
+SvdDims svd_dims(const mctrg_options& o, const LevelInfo& a, int K);
+
 bool route_bidiag(const mctrg_options& o, int n, int K);
 bool route_band(const mctrg_options& o, int n, int K);
+bool route_lowrank(const mctrg_options& o, int n, int K);
 void plan_run(const std::vector<LevelInfo>& lv, int s0, int nlev, int chi, const mctrg_options& opt,
               size_t budget, int64_t n_samples, int64_t& B, int64_t& S, size_t& total);
 void plan_run_bound(int L, int chi, int D0, const mctrg_options& opt, size_t budget, int64_t n_samples,
@@ -68,6 +77,7 @@ struct mctrg_ctx {
   mctrg::DevBuf Timp;                                      // impurity tensor (level0_distinct)
   mctrg::DevBuf bdb, keptb, sigtb, nkb, vrowsb, bdscr;    // bidiagonalization route
   mctrg::DevBuf bandb;                                     // band route: band, scratch, reflectors
+  mctrg::DevBuf lrb;                                       // low-rank levels: reflectors, taus, core halves
 
   // per-kernel-class statistics (MCTRG_K_*)
   mctrg_kernel_stat kstat[MCTRG_K_COUNT]{};

@@ -194,7 +194,7 @@ extern "C" int mctrg_svd_band_batched(const double* M, int n, int64_t batch, dou
       if (e == cudaSuccess) {
         BandVecArgs bv{};
         bv.band = &a; bv.sig = sig; bv.kept = kept; bv.nk = nk; bv.vrows = vrows; bv.n_pad = np; bv.kstride = ks;
-        bv.unit_rows = 1;
+        bv.unit_rows = 1; bv.kmax = n_vec;
         e = launch_band_backtr(bv, st);
       }
     }
