@@ -16,8 +16,9 @@
 //                     against underflow; it is the exact count of a matrix
 //                     within a few ulps of T entrywise, so each value carries
 //                     an absolute error of a few eps |B|, the accuracy class
-//                     of LAPACK's SVD.  FP32 counts narrow each bracket (their
-//                     rounding is relative too), FP64 counts verify it, and
+//                     of LAPACK's SVD.  FP32 and then two-FP32 counts narrow
+//                     each bracket (their rounding is relative too), FP64
+//                     counts verify it where that is not yet the tolerance, and
 //                     Illinois steps on det(T - x I) finish isolated values.
 //  (the sampler then chooses the kept indices)
 //  3. k_bd_invit      right singular vectors of B for the kept indices: inverse
@@ -476,12 +477,12 @@ __device__ __forceinline__ int sturm_eval(const double* __restrict__ oo, int n, 
 // matrix whose singular values are within a relative 2n 2^-23 of B's; it
 // serves to narrow a bracket that FP64 counts then verify.  The pair is
 // rescaled every step (x >= 2^-53 shrinks it by at most 2^-77 a step).
-__device__ __forceinline__ int sturm_count_f32(const float* __restrict__ oo, int n, float x) {
+__device__ __forceinline__ int sturm_count_f32(const float2* __restrict__ oo, int n, float x) {
   float pp = 1.0f, p = -x;
   int neg = 1;
   const int m = 2 * n;
   for (int k = 2; k <= m; ++k) {
-    float q = fmaf(-x, p, -oo[k - 2] * pp);
+    float q = fmaf(-x, p, -oo[k - 2].x * pp);
     int qb = __float_as_int(q);
     if ((qb << 1) == 0) {
       q = -p * 0x1.0p-30f;
@@ -506,15 +507,60 @@ __device__ __forceinline__ double pow2i(int d) {
   return __hiloint2double((1023 + d) << 20, 0);
 }
 
-// Each thread finds the values of its ranks: the bracket from a coarse grid of
-// FP32 counts (the lowest bin starting at the zero bound), narrowed with FP32
-// counts and verified with FP64 ones, then bisection while the bracket holds
-// more than one value (geometric while it spans more than a factor 2), and
-// Illinois steps (regula falsi on det(T - x I), halving the retained end's
-// value when the same end moves twice) once it holds exactly one; three moves
-// of one end in a row force a bisection step.  The bracket always satisfies
-// count(lo) <= j < count(hi), so the result is within the final width of the
-// count's crossing, whatever the interpolation does.
+// The same count and determinant with every number an unevaluated sum of two
+// FP32 (Dekker 1971): a step costs about 28 FP32 and integer instructions
+// instead of two FP64 ones, a quarter of the pipe time (an FP64 warp
+// instruction holds its pipe 16 cycles).  Each product and sum is rounded to
+// a relative 2^-45 at most, so the count is exact for a matrix whose singular
+// values are within a relative n 2^-44 of B's (terms that leave FP32's range
+// move them by less than 2^-62 |T|).  f and fe only steer the interpolation.
+__device__ __forceinline__ int sturm_eval_ff(const float2* __restrict__ oo, int n, double x, float& f, int& fe) {
+  const float xh = (float)x, xl = (float)(x - (double)xh);
+  float ph = -xh, pl = -xl, gh = 1.0f, gl = 0.0f;    // P_{k-1}, P_{k-2}
+  int neg = 1, E = 0;
+  const int m = 2 * n;
+  for (int k = 2; k <= m; ++k) {
+    const float2 o = oo[k - 2];
+    const float h1 = __fmul_rn(xh, ph), h2 = __fmul_rn(o.x, gh);
+    const float e1 = fmaf(xl, ph, fmaf(xh, pl, fmaf(xh, ph, -h1)));
+    const float e2 = fmaf(o.y, gh, fmaf(o.x, gl, fmaf(o.x, gh, -h2)));
+    const float s = __fadd_rn(h1, h2), b = __fsub_rn(s, h1);
+    const float l = __fadd_rn(__fadd_rn(__fsub_rn(h1, __fsub_rn(s, b)), __fsub_rn(h2, b)), __fadd_rn(e1, e2));
+    float qh = -__fadd_rn(s, l), ql = -__fsub_rn(l, __fsub_rn(-qh, s));
+    if (qh == 0.0f) { qh = -ph * 0x1.0p-30f; ql = 0.0f; }
+    neg += (int)((unsigned)(__float_as_int(qh) ^ __float_as_int(ph)) >> 31);
+    gh = ph; gl = pl;
+    ph = qh; pl = ql;
+    const int em = max((__float_as_int(ph) >> 23) & 0xff, (__float_as_int(gh) >> 23) & 0xff);
+    if (em < 127 - 40) {                  // rescale the pair by 2^(127 - em), exactly
+      const float sc = __int_as_float((254 - em) << 23);
+      ph *= sc; pl *= sc; gh *= sc; gl *= sc;
+      E -= 127 - em;
+    }
+  }
+  f = ph;
+  fe = E;
+  return neg - n;
+}
+
+// Each thread finds the values of its ranks in three precisions, each
+// narrowing what the next verifies: the bracket from a coarse grid of FP32
+// counts (the lowest bin starting at the zero bound), narrowed by FP32
+// bisection (geometric while it spans more than a factor 2); then two-FP32
+// counts verify it and narrow it to their own error n 2^-43; a bracket that is
+// then within the tolerance (every value below about 2^-16 |T| at n = 256, the
+// greater part of a spectrum that decays over 16 decades) is done, the others
+// are verified and finished by FP64 counts.  Both finishing loops bisect while
+// the bracket holds more than one value and take Illinois steps (regula falsi
+// on det(T - x I), halving the retained end's value when the same end moves
+// twice) once it holds exactly one; three moves of one end in a row force a
+// bisection step.  The bracket always satisfies count(lo) <= j < count(hi), so
+// the result is within the final width of the count's crossing, whatever the
+// interpolation does.  FP64 counts bound the kernel: about 18 a warp without
+// the two-FP32 stage, 4 for the largest values and none for the rest with it
+// (1920 level matrices of n = 256 32.4 -> 9.7 ms, 3584 of n = 64 8.7 -> 1.9,
+// where one thread per value in place of 256 adds CTAs an SM).
+constexpr int kBisGrid = 256;
 __global__ void __launch_bounds__(kBisThreads) k_bd_bisect(const double* bd, int n, int n_pad, double* sig,
                                                             int* perm, int* nnz, double* lns1, double zero_rel,
                                                             const SvdItem* items) {
@@ -526,19 +572,19 @@ __global__ void __launch_bounds__(kBisThreads) k_bd_bisect(const double* bd, int
     zero_rel = t.zero_rel;
     mat = 0;
   }
+  const int nt = blockDim.x;
   double* oo = sm;                                   // [2n]
-  int* cnt = (int*)(oo + 2 * n);                     // [kBisThreads] FP32 grid counts
-  float* oof = (float*)(cnt + kBisThreads);          // [2n] oo in FP32
+  float2* oof = (float2*)(oo + 2 * n);               // [2n] oo as two FP32
+  int* cnt = (int*)(oof + 2 * n);                    // [kBisGrid] FP32 grid counts
   __shared__ double red[32];
-  __shared__ double s_f0;
-  __shared__ int s_zlo, s_nnz, s_e0;
+  __shared__ int s_zlo, s_nnz;
   const int tid = threadIdx.x;
   const double* d = bd + (size_t)mat * 3 * n;
   const double* e = d + n;
   double* sg = sig + (size_t)mat * n_pad;
   // G = max_k (|o_{k-1}| + |o_k|) >= |T| >= s_1 (Gershgorin), omax = max |o_k| <= s_1
   double g = 0.0, om = 0.0;
-  for (int k = tid; k < 2 * n - 1; k += kBisThreads) {
+  for (int k = tid; k < 2 * n - 1; k += nt) {
     const double ok = fabs((k & 1) ? e[k >> 1] : d[k >> 1]);
     const double on = (k + 1 < 2 * n - 1) ? fabs(((k + 1) & 1) ? e[(k + 1) >> 1] : d[(k + 1) >> 1]) : 0.0;
     g = fmax(g, ok + on);
@@ -547,64 +593,112 @@ __global__ void __launch_bounds__(kBisThreads) k_bd_bisect(const double* bd, int
   const double G = block_max(g, red);
   const double omax = block_max(om, red);
   if (!(G > 0.0)) {                                  // the zero matrix
-    for (int r = tid; r < n_pad; r += kBisThreads) { sg[r] = 0.0; perm[(size_t)mat * n_pad + r] = r; }
+    for (int r = tid; r < n_pad; r += nt) { sg[r] = 0.0; perm[(size_t)mat * n_pad + r] = r; }
     if (tid == 0) { nnz[mat] = 0; if (lns1) lns1[mat] = -INFINITY; }
     return;
   }
   const double invG = 1.0 / G;
-  for (int k = tid; k < 2 * n - 1; k += kBisThreads) {
+  for (int k = tid; k < 2 * n - 1; k += nt) {
     const double ok = ((k & 1) ? e[k >> 1] : d[k >> 1]) * invG;
-    oo[k] = ok * ok;
-    oof[k] = (float)(ok * ok);
+    const double o2 = ok * ok;
+    const float h = (float)o2;
+    oo[k] = o2;
+    oof[k] = make_float2(h, (float)(o2 - (double)h));
   }
   const double zr = zero_rel > 0.0 ? zero_rel : (double)n * kEps;
   const double tlo = zr * omax * invG;               // <= the zero threshold zr s_1 / G
   __syncthreads();
   // coarse grid of FP32 counts: x_t = (t + 1) / T, the last point above |T|
   const double top = 1.0 + 0x1.0p-20;
-  {
-    const double xt = (tid == kBisThreads - 1) ? top : (double)(tid + 1) / kBisThreads;
-    cnt[tid] = sturm_count_f32(oof, n, (float)xt);
-    if (tid == 0) {
-      double f0;
-      int e0;
-      s_zlo = sturm_eval(oo, n, tlo, f0, e0);
-      s_f0 = f0;
-      s_e0 = e0;
-    }
+  for (int t = tid; t < kBisGrid; t += nt) {
+    const double xt = (t == kBisGrid - 1) ? top : (double)(t + 1) / kBisGrid;
+    cnt[t] = sturm_count_f32(oof, n, (float)xt);
+  }
+  if (tid == 0) {
+    double f0;
+    int e0;
+    s_zlo = sturm_eval(oo, n, tlo, f0, e0);
   }
   __syncthreads();
   const int zlo = s_zlo;
   const double tol = 0x1.0p-51;
-  for (int r = tid; r < n; r += kBisThreads) {
+  const double mff = (double)n * 0x1.0p-43;          // relative error allowed to a two-FP32 count
+  for (int r = tid; r < n; r += nt) {
     const int j = n - 1 - r;                         // ascending index of the r-th largest
     if (j < zlo) { sg[r] = 0.0; continue; }          // below tlo: a zero
     // FP32: the grid bin, then bisection (geometric across decades) to a
-    // relative width of 2^-16
+    // relative width of 2^-12
     int t = 0;
-    while (t < kBisThreads - 1 && cnt[t] < j + 1) ++t;
-    float lo32 = t > 0 ? (float)t / kBisThreads : (float)tlo;
-    float hi32 = (t == kBisThreads - 1) ? (float)top : (float)(t + 1) / kBisThreads;
-    for (int it = 0; it < 48 && hi32 > lo32 * (1.0f + 0x1.0p-16f); ++it) {
+    while (t < kBisGrid - 1 && cnt[t] < j + 1) ++t;
+    float lo32 = t > 0 ? (float)t / kBisGrid : (float)tlo;
+    float hi32 = (t == kBisGrid - 1) ? (float)top : (float)(t + 1) / kBisGrid;
+    for (int it = 0; it < 48 && hi32 > lo32 * (1.0f + 0x1.0p-12f); ++it) {
       const float x = (hi32 > 2.0f * lo32) ? sqrtf(lo32 * hi32) : 0.5f * (lo32 + hi32);
       if (!(x > lo32 && x < hi32)) break;
       if (sturm_count_f32(oof, n, x) >= j + 1) hi32 = x; else lo32 = x;
     }
-    // FP64: verify the bracket widened by 2^-12 on each side (the FP32 count's
-    // error is a relative 2n 2^-23 at most); if it does not hold, start from
-    // the whole range [zero bound, |T|]
-    double lo = fmax(tlo, (double)lo32 * (1.0 - 0x1.0p-12));
-    double hi = fmin(top, (double)hi32 * (1.0 + 0x1.0p-12));
-    // a bracket already within the tolerance (the small values: their FP32
-    // bracket, a relative 2^-11 wide, is below 2^-51 |T| in absolute terms)
-    // needs no FP64 count: the refinement below would not move it
+    // the FP32 count's error is a relative 2n 2^-23 at most
+    double lo = fmax(tlo, (double)lo32 * (1.0 - 0x1.0p-11));
+    double hi = fmin(top, (double)hi32 * (1.0 + 0x1.0p-11));
+    // a bracket already within the tolerance needs no further count
     if (hi - lo <= tol) { sg[r] = G * (0.5 * (lo + hi)); continue; }
+    // two FP32: verify (else start from the whole range), then narrow
+    {
+      float f_lo, f_hi;
+      int e_lo, e_hi;
+      int c_lo = sturm_eval_ff(oof, n, lo, f_lo, e_lo);
+      int c_hi = sturm_eval_ff(oof, n, hi, f_hi, e_hi);
+      if (!(c_lo <= j && c_hi >= j + 1)) {
+        lo = tlo; c_lo = sturm_eval_ff(oof, n, lo, f_lo, e_lo);
+        hi = top; c_hi = sturm_eval_ff(oof, n, hi, f_hi, e_hi);
+      }
+      int last = 0, run = 0;
+      for (int it = 0; it < 80 && hi - lo > fmax(0.25 * tol, mff * hi); ++it) {
+        const bool interp = c_lo == j && c_hi == j + 1 && run < 3;
+        double x = (lo > 0.0 && hi > 2.0 * lo) ? (double)sqrtf((float)lo * (float)hi) : 0.5 * (lo + hi);
+        if (interp) {
+          const int dd = e_lo - e_hi;
+          const float al = fabsf(f_lo) * (dd < 0 ? exp2f((float)max(dd, -120)) : 1.0f);
+          const float ah = fabsf(f_hi) * (dd > 0 ? exp2f((float)max(-dd, -120)) : 1.0f);
+          const float den = al + ah;
+          // aimed a quarter of the final width past the crossing, towards the
+          // farther end, so that the next step's end closes the bracket
+          if (den > 0.0f) {
+            const float w = al / den;
+            const double del = 0.25 * fmax(0.25 * tol, mff * hi);
+            const double xi = lo + (double)w * (hi - lo) + (w < 0.5f ? del : -del);
+            if (xi > lo && xi < hi) x = xi;
+          }
+        } else if (!(x > lo && x < hi)) {
+          x = 0.5 * (lo + hi);
+        }
+        float f;
+        int fe;
+        const int c = sturm_eval_ff(oof, n, x, f, fe);
+        if (c >= j + 1) {
+          hi = x; c_hi = c; f_hi = f; e_hi = fe;
+          if (interp && last == 1) e_lo -= 1;        // Illinois: halve the retained end
+          run = (last == 1) ? run + 1 : 1;
+          last = 1;
+        } else {
+          lo = x; c_lo = c; f_lo = f; e_lo = fe;
+          if (interp && last == -1) e_hi -= 1;
+          run = (last == -1) ? run + 1 : 1;
+          last = -1;
+        }
+        if (!interp) run = 0;
+      }
+      lo = fmax(tlo, lo * (1.0 - mff));
+      hi = fmin(top, hi * (1.0 + mff));
+    }
+    if (hi - lo <= tol) { sg[r] = G * (0.5 * (lo + hi)); continue; }
+    // FP64: verify; if it does not hold, start from the whole range [zero bound, |T|]
     double f_lo, f_hi;
     int e_lo, e_hi;
     int c_lo = sturm_eval(oo, n, lo, f_lo, e_lo);
     int c_hi = sturm_eval(oo, n, hi, f_hi, e_hi);
     if (!(c_lo <= j && c_hi >= j + 1)) {
-      lo = tlo; c_lo = zlo; f_lo = s_f0; e_lo = s_e0;
+      lo = tlo; c_lo = sturm_eval(oo, n, lo, f_lo, e_lo);
       hi = top; c_hi = sturm_eval(oo, n, hi, f_hi, e_hi);
     }
     // FP64 refinement to 2^-51 |T|: Illinois steps while the bracket holds one
@@ -621,7 +715,10 @@ __global__ void __launch_bounds__(kBisThreads) k_bd_bisect(const double* bd, int
         const double ah = fabs(f_hi) * (dd > 0 ? pow2i(-dd) : 1.0);
         const double den = al + ah;
         if (den > 0.0) {
-          const double xi = lo + (al / den) * (hi - lo);
+          // aimed just past the crossing, towards the farther end: the two last
+          // steps then straddle it within the tolerance
+          const double w = al / den;
+          const double xi = lo + w * (hi - lo) + (w < 0.5 ? 0.45 * tol : -0.45 * tol);
           if (xi > lo && xi < hi) x = xi;
         }
       }
@@ -643,14 +740,14 @@ __global__ void __launch_bounds__(kBisThreads) k_bd_bisect(const double* bd, int
     }
     sg[r] = G * (0.5 * (lo + hi));
   }
-  for (int r = n + tid; r < n_pad; r += kBisThreads) sg[r] = 0.0;
-  for (int r = tid; r < n_pad; r += kBisThreads) perm[(size_t)mat * n_pad + r] = r;
+  for (int r = n + tid; r < n_pad; r += nt) sg[r] = 0.0;
+  for (int r = tid; r < n_pad; r += nt) perm[(size_t)mat * n_pad + r] = r;
   if (tid == 0) s_nnz = 0;
   __syncthreads();
   const double s1 = sg[0];
   const double tau = zr * s1;
   int c = 0;
-  for (int r = tid; r < n; r += kBisThreads) c += sg[r] > tau;
+  for (int r = tid; r < n; r += nt) c += sg[r] > tau;
   if (c) atomicAdd(&s_nnz, c);
   __syncthreads();
   if (tid == 0) {
@@ -1000,26 +1097,30 @@ cudaError_t launch_bidiag(const BidiagArgs& a, cudaStream_t st) {
   return cudaErrorInvalidValue;
 }
 
+// One thread per value up to 256 (results do not depend on the count).
+static int bisect_threads(int n) { return std::max(64, std::min(kBisThreads, (n + 31) / 32 * 32)); }
+static size_t bisect_smem(int n) { return (size_t)2 * n * (sizeof(double) + sizeof(float2)) + kBisGrid * sizeof(int); }
+
 cudaError_t launch_bd_bisect(const double* bd, int n, int n_pad, int S, double* sig, int* perm, int* nnz,
                              double* lns1, double zero_rel, cudaStream_t st) {
   if (S <= 0) return cudaSuccess;
-  const size_t smem = (size_t)2 * n * (sizeof(double) + sizeof(float)) + kBisThreads * sizeof(int);
+  const size_t smem = bisect_smem(n);
   if (smem > 200 * 1024) return cudaErrorInvalidValue;
   static std::atomic<uint64_t> attr{0};
   cudaError_t e = raise_smem_limit(k_bd_bisect, 200 * 1024, attr);
   if (e != cudaSuccess) return e;
-  k_bd_bisect<<<S, kBisThreads, smem, st>>>(bd, n, n_pad, sig, perm, nnz, lns1, zero_rel, nullptr);
+  k_bd_bisect<<<S, bisect_threads(n), smem, st>>>(bd, n, n_pad, sig, perm, nnz, lns1, zero_rel, nullptr);
   return cudaGetLastError();
 }
 
 cudaError_t launch_bd_bisect_items(const SvdItem* items, int S, int n_max, cudaStream_t st) {
   if (S <= 0) return cudaSuccess;
-  const size_t smem = (size_t)2 * n_max * (sizeof(double) + sizeof(float)) + kBisThreads * sizeof(int);
+  const size_t smem = bisect_smem(n_max);
   if (smem > 200 * 1024) return cudaErrorInvalidValue;
   static std::atomic<uint64_t> attr{0};
   cudaError_t e = raise_smem_limit(k_bd_bisect, 200 * 1024, attr);
   if (e != cudaSuccess) return e;
-  k_bd_bisect<<<S, kBisThreads, smem, st>>>(nullptr, 0, 0, nullptr, nullptr, nullptr, nullptr, 0.0, items);
+  k_bd_bisect<<<S, bisect_threads(n_max), smem, st>>>(nullptr, 0, 0, nullptr, nullptr, nullptr, nullptr, 0.0, items);
   return cudaGetLastError();
 }
 

@@ -94,6 +94,23 @@ def test_values_and_kept_vectors_against_lapack(torch, n, kind):
                 assert abs(np.linalg.norm(proj) - 1.0) <= 1e-10
 
 
+@pytest.mark.parametrize("n", [2, 5, 33, 64, 96, 257, 300])
+def test_values_across_the_precisions_of_the_counts(torch, n):
+    """Close pairs at every scale: splits of 2^-6 (FP32 counts tell them apart), 2^-18 and 2^-30 (two-FP32 counts),
+    2^-44 (FP64 counts) and none, from s_1 down to 2^-40 s_1, where the two-FP32 bracket is the last one.  The counts
+    leave 2^-51 |T| <= 2^-50 s_1; the reduction adds a few eps s_1 sqrt(n): 64 eps s_1 in all up to n = 300."""
+    rng = np.random.default_rng(n)
+    scale = 2.0 ** np.linspace(0.0, -40.0, (n + 1) // 2)
+    split = np.resize([2.0 ** -6, 2.0 ** -18, 2.0 ** -30, 2.0 ** -44, 0.0], (n + 1) // 2)
+    s = np.stack([scale, scale * (1 - split)], 1).ravel()[:n]
+    U, _ = np.linalg.qr(rng.standard_normal((n, n)))
+    V, _ = np.linalg.qr(rng.standard_normal((n, n)))
+    A = (U * s) @ V.T
+    sg, _ = _run(torch, A[None], 0)
+    ref = np.linalg.svd(A, compute_uv=False)
+    assert np.abs(sg[0] - ref).max() <= 64 * np.finfo(float).eps * ref[0]
+
+
 @pytest.mark.parametrize("n,kind,nv", [(1040, "lowrank", 48), (1600, "gauss", 40), (1600, "graded", 40),
                                        (1600, "pairs", 40), (2304, "gauss", 64)])
 def test_wide_values_and_vectors_against_lapack(torch, n, kind, nv):
