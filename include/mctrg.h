@@ -414,7 +414,7 @@ int mctrg_svd_bidiag_batched(const double* M, int n, int64_t batch, double* sigm
  * panels of 8 columns (QR of each column panel and LQ of its row panel in
  * FP64; the products with the trailing matrix, and its two-sided update, as
  * exact integer products of 8-bit digit slices on the tensor cores, the
- * trailing matrix held in 59-bit fixed point relative to |M|_F), the band is
+ * trailing matrix held in 62-bit fixed point relative to |M|_F), the band is
  * reduced to bidiagonal form by bulge chasing (FP64), and the singular values
  * and right vectors follow as in mctrg_svd_bidiag_batched (bisection,
  * inverse iteration, and the two stages' right reflectors applied back).

@@ -13,10 +13,10 @@
 //     A <- A - [V | Y] [Z ; U], Z = T^T W, Y = (X - V Z U^T) T_U (k_band_update).
 //     The three products carry the (8/3) n^3 flops.  They run as exact
 //     integer products on the tensor cores: the trailing matrix is held in
-//     59-bit fixed point (int64 relative to 2^e > |A|_F; orthogonal updates
+//     62-bit fixed point (int64 relative to 2^e > 2 |A|_F; orthogonal updates
 //     keep every entry below |A|_F), the FP64 operands (V, U, Y, Z) in 62-bit
 //     fixed point relative to their own row or column exponent, each operand
-//     split into eight signed 8-bit digits stored as BF16 (exact), and the
+//     split into eight signed 8-bit digits stored as FP16 (exact), and the
 //     digit products with i + j <= 7 accumulated by tcgen05.mma in tensor
 //     memory, one FP32 accumulator per digit group g = i + j (Ozaki, Ogita,
 //     Oishi and Rump 2012; sums of up to 256 products of 8-bit digits are
@@ -37,7 +37,7 @@
 //
 // Every mbarrier wait is bounded; on expiry a kernel records an error word
 // and skips its output, and frees its tensor memory.
-#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include <cstdint>
 
@@ -51,8 +51,8 @@ using namespace tcptx;
 
 namespace {
 constexpr int B = kBandW;        // band width / panel width
-constexpr int kSl = 8;           // digit slices per operand
-constexpr int kFixBits = 59;     // fixed-point fraction bits of the trailing matrix
+constexpr int kSl = 8;           // digit slices per operand (8 bits each)
+constexpr int kFixBits = 62;     // fixed-point fraction bits of the trailing matrix (|A|_F below 2^61)
 constexpr int kFloatP = 62;      // fixed-point bits of an FP64 operand below 2^e
 constexpr int kZeroExp = -1100;  // exponent of an all-zero row or column
 constexpr int kWin = 24;         // chase window: offsets c - r in [-7, 15] (+1 pad)
@@ -114,83 +114,82 @@ __device__ __forceinline__ int exp_above(double amax) {
   return be ? be - 1022 : -1022;
 }
 
-// The eight balanced 8-bit digits of each of eight integers (|x| < 2^63 -
-// 2^62), as BF16 (exact), packed per slice: out[s] holds slice s (s = 0 the
-// top digit) of x[0..7].  Adding 0x80 to every byte turns the balanced digits
-// into the plain bytes of one 64-bit sum, so each digit costs a byte permute
-// and an FP32 subtraction.
+// The eight balanced 8-bit digits of two integers (|x| < 2^63 - 2^62), as FP16
+// (exact), packed per slice: out[s] holds digit s (0 the top one) of x0 in the
+// low half and of x1 in the high half.  Adding 0x80 to every byte turns the
+// balanced digits into the plain bytes of one 64-bit sum; a byte b placed
+// under the exponent of 1024 reads as 1024 + b, so one permute and one packed
+// subtraction make two digits.
+__device__ __forceinline__ void digits2(long long x0, long long x1, uint32_t (&out)[kSl]) {
+  const unsigned long long y0 = (unsigned long long)x0 + 0x8080808080808080ull;
+  const unsigned long long y1 = (unsigned long long)x1 + 0x8080808080808080ull;
+  const __half2 off = __halves2half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480));   // 1024 + 128
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {                  // the 32-bit halves, high first
+    const uint32_t w0 = (uint32_t)(h ? y0 : y0 >> 32), w1 = (uint32_t)(h ? y1 : y1 >> 32);
+    const uint32_t top = __byte_perm(w0, w1, 0x7632), low = __byte_perm(w0, w1, 0x5410);
+    const uint32_t d[4] = {__byte_perm(top, 0x64646464u, 0x4341), __byte_perm(top, 0x64646464u, 0x4240),
+                           __byte_perm(low, 0x64646464u, 0x4341), __byte_perm(low, 0x64646464u, 0x4240)};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const __half2 v = __hsub2(*reinterpret_cast<const __half2*>(&d[i]), off);
+      out[h * 4 + i] = *reinterpret_cast<const uint32_t*>(&v);
+    }
+  }
+}
+// The digits of eight consecutive K values, one 16-byte piece per slice.
 __device__ __forceinline__ void digits8(const long long (&x)[8], uint4 (&out)[kSl]) {
-  uint32_t lo[8], hi[8];
+  uint32_t d[4][kSl];
 #pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    const unsigned long long y = (unsigned long long)x[e] + 0x8080808080808080ull;
-    lo[e] = (uint32_t)y;
-    hi[e] = (uint32_t)(y >> 32);
-  }
+  for (int p = 0; p < 4; ++p) digits2(x[2 * p], x[2 * p + 1], d[p]);
 #pragma unroll
-  for (int s = 0; s < kSl; ++s) {
-    const int bi = 7 - s;                       // byte of the digit, 7 = top
-    uint32_t f[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const uint32_t w = bi >= 4 ? hi[e] : lo[e];
-      const float v = __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u | (uint32_t)(bi & 3))) - 8388736.0f;
-      f[e] = __float_as_uint(v);
-    }
-    out[s].x = __byte_perm(f[0], f[1], 0x7632);
-    out[s].y = __byte_perm(f[2], f[3], 0x7632);
-    out[s].z = __byte_perm(f[4], f[5], 0x7632);
-    out[s].w = __byte_perm(f[6], f[7], 0x7632);
-  }
+  for (int s = 0; s < kSl; ++s) out[s] = make_uint4(d[0][s], d[1][s], d[2][s], d[3][s]);
 }
 
-// Store the slices of eight consecutive K values (k-step q, half kh = K/8 & 1)
-// of row rho into the slice tiles at `tiles` (per k-step two 16 KB tiles of
-// 128 rows x 128 bytes, 4 slices side by side in the 128-byte swizzle).
-__device__ __forceinline__ void store_slices(uint8_t* tiles, uint32_t tile_bytes, int q, int kh, int rho,
-                                             const uint4 (&d)[kSl]) {
+// Operand A of a k-step (128 rows x 16 K values): two 16 KB tiles of 128 rows x
+// 128 bytes, four slices side by side in the 128-byte swizzle.  Byte offset of
+// the 16-byte piece of slice s, row rho, half kh of the K values.
+__device__ __forceinline__ uint32_t a_piece(int s, int rho, int kh) {
+  return (uint32_t)((s >> 2) * kTileBytes + rho * 128 + (((((s & 3) << 1) | kh) ^ (rho & 7)) << 4));
+}
+// Operand B: 128 rows (slice s, column j: row 16 s + j) x 128 bytes, four
+// k-steps (or four column tiles) side by side in slots of 32 bytes.
+__device__ __forceinline__ uint32_t b_piece(int s, int j, int slot, int kh) {
+  return (uint32_t)((s * 16 + j) * 128 + ((((slot << 1) | kh) ^ (j & 7)) << 4));
+}
+
+// The 36 digit products of a k-step as eight MMAs: slice i of A times the
+// slices 0 .. 7-i of B side by side (N = 16 (8 - i)) adds to the accumulators of
+// the digit groups i .. 7, 16 columns each.  One MMA per product read the A
+// slice from shared memory 36 times, eight of them read it 8 times.
+__device__ __forceinline__ void issue_products(uint32_t tmem, const uint8_t* A, const uint8_t* Bt, int slot, bool first) {
+  const uint64_t a0 = umma_desc(smem_u32(A)), b0 = umma_desc(smem_u32(Bt)) + (uint64_t)(slot * 2);
 #pragma unroll
-  for (int s = 0; s < kSl; ++s) {
-    uint8_t* t = tiles + (size_t)(q * 2 + (s >> 2)) * tile_bytes;
-    const int chunk = (((s & 3) << 1) | kh) ^ (rho & 7);
-    *(uint4*)(t + rho * 128 + chunk * 16) = d[s];
+  for (int i = 0; i < kSl; ++i) {
+    const uint64_t ad = a0 + (uint64_t)((((uint32_t)(i >> 2) * kTileBytes) + (i & 3) * 32) >> 4);
+    umma<1>(tmem + (uint32_t)(i * 16), ad, b0, umma_idesc_f16(kTileM, 16 * (kSl - i)), (first && i == 0) ? 0u : 1u);
   }
 }
 
-// The 36 products of a k-step: accumulator g = i + j at columns g * N.  Two
-// descriptors are formed per call; each product's start addresses differ from
-// them by compile-time offsets (the 14-bit start field holds address / 16).
-__device__ __forceinline__ void issue_products(uint32_t tmem, const uint8_t* A, uint32_t abytes, const uint8_t* Bt,
-                                               uint32_t bbytes, int q, int N, uint32_t idesc, bool first) {
-  const uint64_t a0 = umma_desc(smem_u32(A + (size_t)q * 2 * abytes));
-  const uint64_t b0 = umma_desc(smem_u32(Bt + (size_t)q * 2 * bbytes));
-#pragma unroll
-  for (int g = 0; g < kSl; ++g)
-#pragma unroll
-    for (int i = 0; i <= g; ++i) {
-      const int j = g - i;
-      const uint64_t ad = a0 + (uint64_t)((((i >> 2) * abytes) + (i & 3) * 32) >> 4);
-      const uint64_t bd = b0 + (uint64_t)((((j >> 2) * bbytes) + (j & 3) * 32) >> 4);
-      umma<1>(tmem + (uint32_t)(g * N), ad, bd, idesc, (first && i == 0) ? 0u : 1u);
-    }
-}
-
-static __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-static __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
+// Tensor-memory loads without the wait: 32 lanes x 8 or 4 columns (lane = row),
+// and 16 rows x 8 columns as four registers (rows lane / 4 and lane / 4 + 8,
+// columns 2 (lane % 4) and the next).
+static __device__ __forceinline__ void tmem_ld_x8(uint32_t taddr, uint32_t (&v)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
                : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
+static __device__ __forceinline__ void tmem_ld_x4(uint32_t taddr, uint32_t (&v)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(taddr));
+}
+static __device__ __forceinline__ void tmem_ld_16x8(uint32_t taddr, uint32_t (&v)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(taddr));
+}
+static __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
@@ -380,131 +379,170 @@ __global__ void __launch_bounds__(256) k_band_qr(BandArgs a, int k) {
 }
 
 // ---------------------------------------------------------------------------
-// Tensor-core products.  One CTA of 128 threads per (matrix, 128-row tile):
-// the threads split the operands into digit slices in shared memory, thread 0
-// issues the 36 products per k-step and commits them to an mbarrier that the
-// next chunk's split waits on.  Operand A is 128 rows x K; operand B is N
-// rows x K; K runs in chunks of 32 (two k-steps of 16).
+// Tensor-core products W = V^T A and X = A U^T: one CTA of 256 threads per
+// (matrix, 128 columns or rows of the trailing matrix, the MMA's M side); N is
+// the reflectors' side (8 columns, padded to 16, for each of 8 slices) and K
+// runs in stages of 16.  The threads split a stage of A into digit slices in
+// one of two shared-memory buffers while the MMAs of the other run, thread 0
+// issues the eight MMAs and commits them to the buffer's mbarrier; the
+// reflectors are split four stages at a time.
+//
+// What bounds them: reading the trailing matrix (8 bytes an element; W at 2.8
+// TB/s of DRAM) and splitting it (about 14 instructions an element), and X's
+// FP64 epilogue; two CTAs an SM.  Third panel of 304 matrices of n = 256: W 141
+// -> 54 us, X 129 -> 82 us, against one buffer, stages of 32 and one MMA per
+// digit product.
 namespace {
-constexpr int kChunkK = 32;
-constexpr uint32_t kABytes = 4 * kTileBytes;   // 2 k-steps x 2 slice halves
-}
+constexpr uint32_t kStageBytes = 2 * kTileBytes;   // one k-step of A
+constexpr uint32_t kBBytes = 128 * 128;            // B: 128 rows x 4 k-steps
 
-// W^T = A^T V over the rows k..n-1 (K) for the trailing columns k+b.. of one
-// 128-column tile (the MMA's rows), N = 16 (V's b columns, zero padded).
-__global__ void __launch_bounds__(256) k_band_gemm_w(BandArgs a, int k) {
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* As = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  constexpr int N = 16;
-  constexpr uint32_t bt = N * 128;                 // one B tile
-  uint8_t* Bs = As + kABytes;
-  __shared__ __align__(8) uint64_t bar;
-  __shared__ uint32_t tmem_slot;
-  __shared__ int s_fail;
-  const int s = blockIdx.x, n = a.n, t = threadIdx.x, warp = t >> 5;
-  const int rho = t & 127, hk = t >> 7;             // MMA row, and which 16 of a chunk's 32 K values
-  const int c = k + B + blockIdx.y * kTileM + rho;  // this thread's column (MMA row)
-  const int m = n - k;
-  const long long* A = (const long long*)a.Wk + (size_t)s * n * n;
-  Work w = work_of(a.work + (size_t)s * work_stride(n), n);
-  if (t == 0) {
-    s_fail = 0;
-    mbar_init(&bar, 1);
+// Shared state of a product kernel.
+struct ProdShared {
+  uint64_t bar[2];
+  uint32_t tmem_slot;
+  int fail;
+};
+__device__ __forceinline__ uint8_t* align1k(uint8_t* p) { return (uint8_t*)(((uintptr_t)p + 1023) & ~(uintptr_t)1023); }
+
+__device__ __forceinline__ uint32_t prod_begin(ProdShared& ps, uint8_t* Bs, uint32_t bbytes) {
+  if (threadIdx.x == 0) {
+    ps.fail = 0;
+    mbar_init(&ps.bar[0], 1);
+    mbar_init(&ps.bar[1], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // B rows b..15 stay zero
-  for (int i = t; i < (int)(4 * bt / 16); i += blockDim.x) ((uint4*)Bs)[i] = make_uint4(0, 0, 0, 0);
-  if (warp == 0) tmem_alloc(&tmem_slot, 128);
+  // the rows 8 .. 15 of each slice of B stay zero
+  for (int i = threadIdx.x; i < (int)(bbytes / 16); i += blockDim.x) ((uint4*)Bs)[i] = make_uint4(0, 0, 0, 0);
+  if (threadIdx.x < 32) tmem_alloc(&ps.tmem_slot, 128);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = tmem_slot;
-  const uint32_t idesc = umma_idesc(1, kTileM, N);
-  const int nchunk = (m + kChunkK - 1) / kChunkK;
-  // the next chunk's 16 values of this thread, loaded while the products of
-  // the current chunk run
-  long long x[16];
-  auto load = [&](int ch) {
-    const int rb = k + ch * kChunkK + hk * 16;
+  return ps.tmem_slot;
+}
+
+// The stage loop: split(st, dst) writes stage st of A (and fetches the next
+// one's data), refl(r, j) is the FP64 value of reflector j at K index r.
+// Returns false when a wait expired.
+template <class Split, class Refl>
+__device__ __forceinline__ bool prod_stages(ProdShared& ps, uint32_t tmem, uint8_t* As, uint8_t* Bs, int klen,
+                                            Split split, Refl refl) {
+  const int t = threadIdx.x, nst = (klen + 15) >> 4;
+  int committed = 0;
+  for (int st = 0; st < nst; ++st) {
+    const int buf = st & 1;
+    // the MMAs of stage st - 2 (and all before them) are done with this buffer
+    if (st >= 2 && !mbar_wait(&ps.bar[buf], ((st >> 1) - 1) & 1)) atomicOr(&ps.fail, 1);
+    split(st, As + (size_t)buf * kStageBytes);
+    uint8_t* Bb = Bs + (size_t)((st >> 2) & 1) * kBBytes;
+    if ((st & 3) == 0) {                             // the reflectors of the next four stages
+      const int j = t & 7, kk = 2 * (t >> 3), r = st * 16 + kk;
+      uint32_t d[kSl];
+      digits2(r < klen ? fix_of(refl(r, j), kFloatP - 1) : 0ll,
+              r + 1 < klen ? fix_of(refl(r + 1, j), kFloatP - 1) : 0ll, d);
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
-      const int r = rb + e;
-      x[e] = (c < n && r < n) ? A[(size_t)r * n + c] : 0ll;
-    }
-  };
-  load(0);
-  int committed = 0;                                 // commits thread 0 issued (the same count in every thread)
-  for (int ch = 0; ch < nchunk; ++ch) {
-    if (ch > 0 && !mbar_wait(&bar, (ch - 1) & 1)) atomicOr(&s_fail, 1);
-    __syncthreads();
-    if (s_fail) break;
-    const int r0 = k + ch * kChunkK;
-#pragma unroll
-    for (int g = 0; g < 2; ++g) {
-      long long y[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) y[e] = x[g * 8 + e];
-      uint4 d[kSl];
-      digits8(y, d);
-      store_slices(As, kTileBytes, hk, g, rho, d);
-    }
-    if (t < 32) {                                    // V: row j = t & 7 of B, 8 K values per thread
-      const int j = t & 7, g8 = t >> 3;
-      long long y[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int r = r0 + g8 * 8 + e;
-        y[e] = r < n ? fix_of(w.V[(size_t)(r - k) * 8 + j], kFloatP - 1) : 0ll;
-      }
-      uint4 d[kSl];
-      digits8(y, d);
-      store_slices(Bs, bt, g8 >> 1, g8 & 1, j, d);
+      for (int s = 0; s < kSl; ++s)
+        *(uint32_t*)(Bb + b_piece(s, j, kk >> 4, (kk >> 3) & 1) + (kk & 7) * 2) = d[s];
     }
     fence_async_smem();
     __syncthreads();
+    if (ps.fail) break;
     if (t == 0) {
       tc_fence_after();
-      issue_products(tmem, As, kTileBytes, Bs, bt, 0, N, idesc, ch == 0);
-      issue_products(tmem, As, kTileBytes, Bs, bt, 1, N, idesc, false);
-      umma_commit(&bar);
+      issue_products(tmem, As + (size_t)buf * kStageBytes, Bb, st & 3, st == 0);
+      umma_commit(&ps.bar[buf]);
     }
     ++committed;
-    if (ch + 1 < nchunk) load(ch + 1);
   }
-  if (!s_fail && !mbar_wait(&bar, (nchunk - 1) & 1)) atomicOr(&s_fail, 1);
+  const int last = committed - 1;
+  if (last >= 0 && !mbar_wait(&ps.bar[last & 1], (last >> 1) & 1)) atomicOr(&ps.fail, 1);
   tc_fence_after();
   __syncthreads();
-  if (!s_fail && warp < 4) {
-    // row c of W^T: value = (hi 2^32 + lo) 2^(eA - 64)
-    long long hi[8], lo[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) { hi[j] = 0; lo[j] = 0; }
-#pragma unroll
-    for (int g = 0; g < kSl; ++g) {
-      uint32_t v[16];
-      tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(g * N), v);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const long long G = __float2ll_rn(__uint_as_float(v[j]));
-        if (g < 4) hi[j] = (hi[j] << 8) + G;
-        else lo[j] = (lo[j] << 8) + G;
-      }
-    }
-    if (c < n) {
-      const double sc = p2(a.eA[s] - 64);
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        w.Z[(size_t)j * n + (c - k - B)] = fma((double)hi[j], 4294967296.0 * sc, (double)lo[j] * sc);
-    }
-  } else if (s_fail && t == 0) {
-    atomicOr(a.err, 1u);
+  return ps.fail == 0;
+}
+
+__device__ __forceinline__ void prod_end(ProdShared& ps, uint32_t tmem, bool ok, uint32_t* err) {
+  if (!ok && threadIdx.x == 0) {
+    atomicOr(err, 1u);
+    // give products still in flight another bounded wait before their memory is freed
+    for (uint32_t i = 0; i < kSpinLimit; ++i) __nanosleep(20);
   }
-  // after an expired wait, give the products in flight another bounded wait
-  // before their tensor memory is freed
-  if (s_fail && committed > 0) mbar_wait(&bar, (committed - 1) & 1);
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) tmem_free(tmem, 128);
+  if (threadIdx.x < 32) tmem_free(tmem, 128);
+}
+
+// Columns 0 .. NJ-1 from `col` of this thread's row: the group sums g back as
+// hi 2^32 + lo.
+template <int NJ>
+__device__ __forceinline__ void prod_read(uint32_t taddr, long long (&hi)[NJ], long long (&lo)[NJ]) {
+  uint32_t v[kSl][NJ];
+#pragma unroll
+  for (int g = 0; g < kSl; ++g) {
+    if constexpr (NJ == 8) tmem_ld_x8(taddr + (uint32_t)(g * 16), v[g]);
+    else tmem_ld_x4(taddr + (uint32_t)(g * 16), v[g]);
+  }
+  tmem_wait_ld();
+#pragma unroll
+  for (int j = 0; j < NJ; ++j) {
+    hi[j] = __float2int_rn(__uint_as_float(v[0][j]));
+    lo[j] = __float2int_rn(__uint_as_float(v[4][j]));
+#pragma unroll
+    for (int g = 1; g < 4; ++g) {
+      hi[j] = (hi[j] << 8) + __float2int_rn(__uint_as_float(v[g][j]));
+      lo[j] = (lo[j] << 8) + __float2int_rn(__uint_as_float(v[4 + g][j]));
+    }
+  }
+}
+constexpr size_t kProdSmem = 2 * kStageBytes + 2 * kBBytes + 1024;
+}  // namespace
+
+// W^T = A^T V over the rows k..n-1 (K) for the trailing columns k+b.. of one
+// 128-column tile; a thread splits 8 rows of its column per stage (the warps
+// read whole rows of the tile).
+__global__ void __launch_bounds__(256, 2) k_band_gemm_w(BandArgs a, int k) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ ProdShared ps;
+  uint8_t* As = align1k(smem_raw);
+  uint8_t* Bs = As + 2 * kStageBytes;
+  const int s = blockIdx.x, n = a.n, t = threadIdx.x, warp = t >> 5;
+  const int rho = t & 127, kh = t >> 7;             // MMA row (column of A), and which 8 of a stage's 16 rows
+  const int c = k + B + blockIdx.y * kTileM + rho;
+  const int m = n - k;
+  const long long* A = (const long long*)a.Wk + (size_t)s * n * n;
+  Work w = work_of(a.work + (size_t)s * work_stride(n), n);
+  const uint32_t tmem = prod_begin(ps, Bs, 2 * kBBytes);
+  long long x[8];
+  auto load = [&](int st) {
+    const int rb = st * 16 + kh * 8;                 // relative to k; m is a multiple of 8
+    const long long* p = A + (size_t)(k + rb) * n + c;
+    const bool in = c < n && rb < m;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) x[e] = in ? p[(size_t)e * n] : 0ll;
+  };
+  load(0);
+  const bool ok = prod_stages(
+      ps, tmem, As, Bs, m,
+      [&](int st, uint8_t* dst) {
+        uint4 d[kSl];
+        digits8(x, d);
+#pragma unroll
+        for (int sl = 0; sl < kSl; ++sl) *(uint4*)(dst + a_piece(sl, rho, kh)) = d[sl];
+        load(st + 1);                                // past the end: zeros
+      },
+      [&](int r, int j) { return w.V[(size_t)r * 8 + j]; });
+  if (ok) {
+    // row c of W^T: value = (hi 2^32 + lo) 2^(eA - 67); the two warp groups take four columns each
+    const int jh = kh * 4;
+    long long hi[4], lo[4];
+    prod_read<4>(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)jh, hi, lo);
+    if (c < n) {
+      const double sc = p2(a.eA[s] - kFixBits - 5);
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        w.Z[(size_t)(jh + j) * n + (c - k - B)] = fma((double)hi[j], 4294967296.0 * sc, (double)lo[j] * sc);
+    }
+  }
+  prod_end(ps, tmem, ok, a.err);
 }
 
 // ---------------------------------------------------------------------------
@@ -609,113 +647,56 @@ __global__ void __launch_bounds__(256) k_band_lq(BandArgs a, int k) {
 // ---------------------------------------------------------------------------
 // X = A U^T over the trailing rows (one 128-row tile, the MMA's rows) and
 // columns k+b.. (K); then per row Y = (X - V Z U^T) T_U and the row exponent
-// of [V | Y].
-__global__ void __launch_bounds__(256) k_band_gemm_x(BandArgs a, int k) {
+// of [V | Y].  Eight lanes read the 128 bytes of a row's 16 columns (two each),
+// so a warp's load covers whole sectors of four rows; the rows of one load are
+// two apart, which keeps their pieces in different banks.
+__global__ void __launch_bounds__(256, 2) k_band_gemm_x(BandArgs a, int k) {
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* As = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  constexpr int N = 16;
-  constexpr uint32_t bt = N * 128;
-  uint8_t* Bs = As + kABytes;
-  __shared__ __align__(8) uint64_t bar;
-  __shared__ uint32_t tmem_slot;
-  __shared__ int s_fail;
+  __shared__ ProdShared ps;
   __shared__ double ZUs[64], TUs[64];
-  const int s = blockIdx.x, n = a.n, t = threadIdx.x, warp = t >> 5;
-  const int rho = t & 127, hk = t >> 7;
-  const int r = k + B + blockIdx.y * kTileM + rho;  // this thread's row
+  uint8_t* As = align1k(smem_raw);
+  uint8_t* Bs = As + 2 * kStageBytes;
+  const int s = blockIdx.x, n = a.n, t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int r0 = k + B + blockIdx.y * kTileM;
   const int mp = n - k - B;                          // K = columns k+b .. n-1
   const long long* A = (const long long*)a.Wk + (size_t)s * n * n;
   const double* Ad = (const double*)A;
   Work w = work_of(a.work + (size_t)s * work_stride(n), n);
-  if (t == 0) {
-    s_fail = 0;
-    mbar_init(&bar, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
   if (t < 64) { ZUs[t] = w.ZU[t]; TUs[t] = Ad[(size_t)(k + t / B) * n + k + (t % B)]; }
-  for (int i = t; i < (int)(4 * bt / 16); i += blockDim.x) ((uint4*)Bs)[i] = make_uint4(0, 0, 0, 0);
-  if (warp == 0) tmem_alloc(&tmem_slot, 128);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = tmem_slot;
-  const uint32_t idesc = umma_idesc(1, kTileM, N);
-  const int nchunk = (mp + kChunkK - 1) / kChunkK;
-  long long x[16];
-  auto load = [&](int ch) {
-    const int cb = k + B + ch * kChunkK + hk * 16;  // n and cb are multiples of 8
+  const uint32_t tmem = prod_begin(ps, Bs, 2 * kBBytes);
+  const int l8 = lane & 7;
+  // row (within the tile) of load q
+  auto row_of = [&](int q) { return warp * 16 + (q >> 1) * 8 + (q & 1) + 2 * (lane >> 3); };
+  longlong2 x[4];
+  auto load = [&](int st) {
+    const int cb = st * 16 + 2 * l8;                 // relative to k + b
 #pragma unroll
-    for (int g = 0; g < 2; ++g) {
-      if (r < n && cb + 8 * g < n) {
-        const longlong2* p = (const longlong2*)(A + (size_t)r * n + cb + 8 * g);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) { const longlong2 q = p[e]; x[8 * g + 2 * e] = q.x; x[8 * g + 2 * e + 1] = q.y; }
-      } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) x[8 * g + e] = 0ll;
-      }
+    for (int q = 0; q < 4; ++q) {
+      const int r = r0 + row_of(q);
+      x[q] = (r < n && cb < mp) ? *(const longlong2*)(A + (size_t)r * n + k + B + cb) : make_longlong2(0, 0);
     }
   };
   load(0);
-  int committed = 0;                                 // commits thread 0 issued (the same count in every thread)
-  for (int ch = 0; ch < nchunk; ++ch) {
-    if (ch > 0 && !mbar_wait(&bar, (ch - 1) & 1)) atomicOr(&s_fail, 1);
-    __syncthreads();
-    if (s_fail) break;
-    const int c0 = k + B + ch * kChunkK;
+  const bool ok = prod_stages(
+      ps, tmem, As, Bs, mp,
+      [&](int st, uint8_t* dst) {
 #pragma unroll
-    for (int g = 0; g < 2; ++g) {
-      long long y[8];
+        for (int q = 0; q < 4; ++q) {
+          uint32_t d[kSl];
+          digits2(x[q].x, x[q].y, d);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) y[e] = x[g * 8 + e];
-      uint4 d[kSl];
-      digits8(y, d);
-      store_slices(As, kTileBytes, hk, g, rho, d);
-    }
-    if (t < 32) {                                    // U: row j of B, 8 K values per thread
-      const int j = t & 7, g8 = t >> 3;
-      long long y[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int cc = c0 + g8 * 8 + e;
-        y[e] = cc < n ? fix_of(Ad[(size_t)(k + j) * n + cc], kFloatP - 1) : 0ll;
-      }
-      uint4 d[kSl];
-      digits8(y, d);
-      store_slices(Bs, bt, g8 >> 1, g8 & 1, j, d);
-    }
-    fence_async_smem();
-    __syncthreads();
-    if (t == 0) {
-      tc_fence_after();
-      issue_products(tmem, As, kTileBytes, Bs, bt, 0, N, idesc, ch == 0);
-      issue_products(tmem, As, kTileBytes, Bs, bt, 1, N, idesc, false);
-      umma_commit(&bar);
-    }
-    ++committed;
-    if (ch + 1 < nchunk) load(ch + 1);
-  }
-  if (!s_fail && !mbar_wait(&bar, (nchunk - 1) & 1)) atomicOr(&s_fail, 1);
-  tc_fence_after();
-  __syncthreads();
-  if (!s_fail && warp < 4) {
+          for (int sl = 0; sl < kSl; ++sl) *(uint32_t*)(dst + a_piece(sl, row_of(q), l8 >> 2) + (l8 & 3) * 4) = d[sl];
+        }
+        load(st + 1);
+      },
+      [&](int r, int j) { return Ad[(size_t)(k + j) * n + k + B + r]; });
+  if (ok && warp < 4) {
+    const int r = r0 + t;
     long long hi[8], lo[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) { hi[j] = 0; lo[j] = 0; }
-#pragma unroll
-    for (int g = 0; g < kSl; ++g) {
-      uint32_t v[16];
-      tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(g * N), v);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const long long G = __float2ll_rn(__uint_as_float(v[j]));
-        if (g < 4) hi[j] = (hi[j] << 8) + G;
-        else lo[j] = (lo[j] << 8) + G;
-      }
-    }
+    prod_read<8>(tmem + ((uint32_t)(warp * 32) << 16), hi, lo);
     if (r < n) {
-      const double sc = p2(a.eA[s] - 64);
-      double vr[B], x[B], y[B];
+      const double sc = p2(a.eA[s] - kFixBits - 5);
+      double vr[B], xv[B], y[B];
 #pragma unroll
       for (int i = 0; i < B; ++i) vr[i] = w.V[(size_t)(r - k) * 8 + i];
 #pragma unroll
@@ -723,7 +704,7 @@ __global__ void __launch_bounds__(256) k_band_gemm_x(BandArgs a, int k) {
         double acc = fma((double)hi[j], 4294967296.0 * sc, (double)lo[j] * sc);
 #pragma unroll
         for (int i = 0; i < B; ++i) acc = fma(-vr[i], ZUs[i * B + j], acc);
-        x[j] = acc;
+        xv[j] = acc;
       }
       // exponent of the update's left operand row [V 2^eA | Y] (both parts of
       // the order of |A|; the right operand carries Z 2^-eA)
@@ -733,7 +714,7 @@ __global__ void __launch_bounds__(256) k_band_gemm_x(BandArgs a, int k) {
       for (int j = 0; j < B; ++j) {
         double acc = 0.0;
 #pragma unroll
-        for (int i = 0; i <= j; ++i) acc = fma(x[i], TUs[i * B + j], acc);
+        for (int i = 0; i <= j; ++i) acc = fma(xv[i], TUs[i * B + j], acc);
         y[j] = acc;
         mx = fmax(mx, fmax(fabs(acc), fabs(vr[j]) * up));
       }
@@ -742,202 +723,198 @@ __global__ void __launch_bounds__(256) k_band_gemm_x(BandArgs a, int k) {
       for (int j = 0; j < B; ++j) w.Y[(size_t)ro * 8 + j] = y[j];
       w.el[ro] = exp_above(mx);
     }
-  } else if (s_fail && t == 0) {
-    atomicOr(a.err, 1u);
   }
-  // after an expired wait, give the products in flight another bounded wait
-  // before their tensor memory is freed
-  if (s_fail && committed > 0) mbar_wait(&bar, (committed - 1) & 1);
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 0) tmem_free(tmem, 128);
+  prod_end(ps, tmem, ok, a.err);
 }
 
 // ---------------------------------------------------------------------------
 // Trailing update A[k+b:][k+b:] -= [V | Y] [Z ; U] for one 128-row tile, its
-// 32-column tiles in turn: K = 2b = 16 (one k-step), applied in fixed point.
+// 16-column tiles in turn: K = 2b = 16 (one k-step), applied in fixed point.
 // The operands are [V 2^eA | Y] and [Z 2^-eA ; U] (the same product): V and U
 // are of order 1, Y and Z of order |A|.  The row operand shares one exponent
-// over the tile's rows, the column operand one over each 32-column tile (both
-// the largest of the per-row / per-column exponents: digits keep 62 bits of
-// the largest entry), so every element of a tile takes the same shifts.  256
-// threads: the row operand is split once (V halves by threads 0-127, Y halves
-// by 128-255); per column tile two warps split the column operand, thread 0
-// issues the 36 products, and warp w applies the results of rows 32 (w % 4)
-// .. +31 (its tensor-memory lanes) and columns 16 (w / 4) .. +15 of the tile,
-// the row segment loaded before the products run.
+// over the tile's rows, the column operand one over each block of 64 columns
+// (the largest of the per-row / per-column exponents: digits keep 62 bits of
+// the largest entry), so every element of a tile takes the same shifts.
+//
+// Both operands are split once, before the loop over the column tiles; its two
+// accumulators (128 columns of tensor memory each) let the MMAs of the next
+// tile run while the warps apply this one, with no block barrier: a full
+// mbarrier per accumulator is completed by the MMAs, an empty one by the eight
+// warps.  A warp takes 16 rows; the 16 x 8 form of the tensor-memory load gives
+// four lanes the eight columns of a row, so the reads and writes of the
+// trailing matrix cover whole sectors (one row per lane, the first form of
+// this kernel, touched 32 lines with every instruction and wrote half sectors:
+// 186 us for the third panel of 304 matrices of n = 256, 88 us so).  What bounds
+// it: the 16 bytes an element read and written (2.7 TB/s of DRAM at that size).
+struct UpdShared {
+  uint64_t full[2], empty[2];
+  uint32_t tmem_slot;
+  int fail, el, er[4];
+};
 __global__ void __launch_bounds__(256, 2) k_band_update(BandArgs a, int k) {
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* As = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  constexpr int N = 32, NH = 16;
-  constexpr uint32_t bt = N * 128;
-  uint8_t* Bs = As + 2 * kTileBytes;
-  __shared__ __align__(8) uint64_t bar;
-  __shared__ uint32_t tmem_slot;
-  __shared__ int s_fail, s_el, s_er;
+  __shared__ UpdShared us;
+  uint8_t* As = align1k(smem_raw);
+  uint8_t* Bs = As + kStageBytes;                    // blocks of 64 columns: 128 rows x 128 bytes
   const int s = blockIdx.x, n = a.n, t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int r0 = k + B + blockIdx.y * kTileM;       // first row of the tile
+  const int mp = n - k - B;
   long long* A = (long long*)a.Wk + (size_t)s * n * n;
   const double* Ad = (const double*)A;
   Work w = work_of(a.work + (size_t)s * work_stride(n), n);
   const int eA = a.eA[s];
   if (t == 0) {
-    s_fail = 0;
-    s_el = kZeroExp;
-    mbar_init(&bar, 1);
+    us.fail = 0;
+    us.el = kZeroExp;
+    for (int q = 0; q < 4; ++q) us.er[q] = kZeroExp;
+    for (int q = 0; q < 2; ++q) { mbar_init(&us.full[q], 1); mbar_init(&us.empty[q], 8); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) tmem_alloc(&tmem_slot, 256);
+  if (warp == 0) tmem_alloc(&us.tmem_slot, 256);
   __syncthreads();
   {
-    // the tile's row exponent: the largest el of its rows
-    const int r = r0 + (t & 127);
-    int e = (t < 128 && r < n) ? w.el[r - k - B] : kZeroExp;
+    // the largest row exponent of the tile and the column exponents of the blocks
+    int e = (t < 128 && r0 + t < n) ? w.el[r0 + t - k - B] : kZeroExp, f = t < mp ? w.er[t] : kZeroExp;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-    if (lane == 0 && t < 128) atomicMax(&s_el, e);
+    for (int o = 16; o > 0; o >>= 1) {
+      e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+      f = max(f, __shfl_xor_sync(0xffffffffu, f, o));
+    }
+    if (lane == 0) {
+      if (t < 128) atomicMax(&us.el, e);
+      atomicMax(&us.er[t >> 6], f);
+    }
   }
   __syncthreads();
-  const int el = s_el;
+  const int el = us.el;
   {
     // A operand: row rho = [V[r] 2^eA | Y[r]]
     const int rho = t & 127, part = t >> 7, r = r0 + rho;
     long long x[8];
-    if (r < n && el != kZeroExp) {
+    const bool in = r < n && el != kZeroExp;
 #pragma unroll
-      for (int e = 0; e < 8; ++e)
-        x[e] = part == 0 ? fix_of(w.V[(size_t)(r - k) * 8 + e], kFloatP - el + eA)
-                         : fix_of(w.Y[(size_t)(r - k - B) * 8 + e], kFloatP - el);
-    } else {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) x[e] = 0;
-    }
+    for (int e = 0; e < 8; ++e)
+      x[e] = !in ? 0ll
+                 : part == 0 ? fix_of(w.V[(size_t)(r - k) * 8 + e], kFloatP - el + eA)
+                             : fix_of(w.Y[(size_t)(r - k - B) * 8 + e], kFloatP - el);
     uint4 d[kSl];
     digits8(x, d);
-    store_slices(As, kTileBytes, 0, part, rho, d);
+#pragma unroll
+    for (int sl = 0; sl < kSl; ++sl) *(uint4*)(As + a_piece(sl, rho, part)) = d[sl];
   }
+  for (int p = t; p < 2 * ((mp + 15) & ~15); p += 256) {
+    // B operand: column c = [Z[:, c] 2^-eA ; U[:, c]]
+    const int half = (mp + 15) & ~15, part = p >= half, c = p - part * half;
+    const int er = us.er[c >> 6];
+    const bool in = c < mp && er != kZeroExp;
+    long long x[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      x[e] = !in ? 0ll
+                 : part == 0 ? fix_of(w.Z[(size_t)e * n + c], kFloatP - er - eA)
+                             : fix_of(Ad[(size_t)(k + e) * n + k + B + c], kFloatP - er);
+    uint4 d[kSl];
+    digits8(x, d);
+    uint8_t* Bb = Bs + (size_t)(c >> 6) * kBBytes;
+#pragma unroll
+    for (int sl = 0; sl < kSl; ++sl) *(uint4*)(Bb + b_piece(sl, c & 15, (c >> 4) & 3, part)) = d[sl];
+  }
+  fence_async_smem();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = tmem_slot;
-  const uint32_t idesc = umma_idesc(1, kTileM, N);
-  const int quad = warp & 3, hc = warp >> 2;
-  const int rho = quad * 32 + lane, r = r0 + rho;
-  const int ntile = (n - k - B + N - 1) / N;
-  int committed = 0;                                 // commits thread 0 issued (the same count in every thread)
+  const uint32_t tmem = us.tmem_slot;
+  const int ntile = (mp + 15) >> 4;
+  // MMAs of tile ct into accumulator ct & 1 (thread 0)
+  auto issue = [&](int ct) {
+    issue_products(tmem + (uint32_t)((ct & 1) * 128), As, Bs + (size_t)(ct >> 2) * kBBytes, ct & 3, true);
+    umma_commit(&us.full[ct & 1]);
+  };
+  // this thread's rows (two) and column pair within a tile
+  const int rw = (warp & 3) * 32 + (warp >> 2) * 16 + (lane >> 2), cl = 2 * (lane & 3);
+  const uint32_t tlane = (uint32_t)((warp & 3) * 32 + (warp >> 2) * 16) << 16;
+  const int ra = r0 + rw, rb = ra + 8;
+  long long* pa = A + (size_t)ra * n + k + B + cl;
+  long long* pb = pa + (size_t)8 * n;
+  const bool oka = ra < n && el != kZeroExp, okb = rb < n && el != kZeroExp;
+  longlong2 nx[4];                                   // the next tile's elements: (row a, row b) x (columns, columns + 8)
+  auto load = [&](int ct) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int c = ct * 16 + 8 * h;                 // mp is a multiple of 8
+      nx[2 * h] = (oka && c < mp) ? *(const longlong2*)(pa + c) : make_longlong2(0, 0);
+      nx[2 * h + 1] = (okb && c < mp) ? *(const longlong2*)(pb + c) : make_longlong2(0, 0);
+    }
+  };
+  if (t == 0) issue(0);
+  __syncwarp();
+  load(0);
   for (int ct = 0; ct < ntile; ++ct) {
-    const int cb = k + B + ct * N;                  // first column of the tile
-    // this warp's 16 columns of the row, loaded before the products run; n and
-    // cw are multiples of 8, so the first 8 exist when cw < n and the second 8
-    // when cw + 8 < n
-    const int cw = cb + hc * NH;
-    const bool rowok = r < n && el != kZeroExp && cw < n;
-    const bool half2 = cw + 8 < n;
-    longlong2* rowp = (longlong2*)(A + (size_t)r * n + cw);
-    longlong2 q[NH / 2];
-#pragma unroll
-    for (int i = 0; i < NH / 2; ++i) q[i] = make_longlong2(0, 0);
-    if (rowok) {
-#pragma unroll
-      for (int i = 0; i < NH / 4; ++i) q[i] = rowp[i];
-      if (half2) {
-#pragma unroll
-        for (int i = NH / 4; i < NH / 2; ++i) q[i] = rowp[i];
-      }
-    }
-    if (t < 2 * N) {                                 // B operand: column c = [Z[:, c] 2^-eA ; U[:, c]]
-      const int cc = t & (N - 1), part = t >> 5, c = cb + cc;
-      int er = c < n ? w.er[c - k - B] : kZeroExp;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) er = max(er, __shfl_xor_sync(0xffffffffu, er, o));
-      if (t == 0) s_er = er;                         // the tile's column exponent
-      long long x[8];
-      if (c < n && er != kZeroExp) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-          x[e] = part == 0 ? fix_of(w.Z[(size_t)e * n + (c - k - B)], kFloatP - er - eA)
-                           : fix_of(Ad[(size_t)(k + e) * n + c], kFloatP - er);
-      } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) x[e] = 0;
-      }
-      uint4 d[kSl];
-      digits8(x, d);
-      store_slices(Bs, bt, 0, part, cc, d);
-    }
-    fence_async_smem();
-    tc_fence_before();
-    __syncthreads();
-    if (t == 0) {
+    bool ok = true;
+    if (t == 0 && ct + 1 < ntile) {
+      // the warps have read tile ct - 1 out of the accumulator that tile ct + 1 takes
+      if (ct >= 1) ok = mbar_wait(&us.empty[(ct + 1) & 1], ((ct - 1) >> 1) & 1);
       tc_fence_after();
-      issue_products(tmem, As, kTileBytes, Bs, bt, 0, N, idesc, true);
-      umma_commit(&bar);
+      if (ok) issue(ct + 1);
     }
-    ++committed;
-    if (!mbar_wait(&bar, ct & 1)) atomicOr(&s_fail, 1);
+    __syncwarp();
+    longlong2 q[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) q[i] = nx[i];
+    if (ct + 1 < ntile) load(ct + 1);
+    ok = mbar_wait(&us.full[ct & 1], (ct >> 1) & 1) && ok;
+    if (__any_sync(0xffffffffu, !ok)) {              // expired: the other warps' waits expire too
+      if (lane == 0) atomicOr(&us.fail, 1);
+      break;
+    }
     tc_fence_after();
-    __syncthreads();
-    if (s_fail) break;
-    const int er = s_er;
-    // value of an element: (hi 2^32 + lo) 2^(el + er - 68), in fixed-point
-    // units 2^(eA - 59): shifted by sh = el + er - eA - 9, the same for the
-    // whole tile.  The tensor-memory loads are warp-collective: every lane
-    // issues them; only the arithmetic and the stores depend on the row.
-    const bool apply = rowok && er != kZeroExp;
-    const int sh = el + er - eA - 9;
+    const int er = us.er[ct >> 2];
+    // value of an element: (hi 2^32 + lo) 2^(el + er - 68), in fixed-point units 2^(eA - kFixBits)
+    const int sh = el + er - eA - 68 + kFixBits;
 #pragma unroll
-    for (int part = 0; part < 2; ++part) {           // this warp's 16 columns, 8 at a time
-      const int jc = hc * NH + part * 8;
-      // group sums here are integers of at most 8 x 16 x 2^14 = 2^21 in
-      // magnitude, read back exactly by adding 1.5 2^23 (an FP32 add; the
-      // bias 0x4B400000 of each is taken out of the pair sums below) and
-      // paired in 32 bits: G0 2^8 + G1 and so on stay below 2^30
-      int gb[kSl][8];
+    for (int h = 0; h < 2; ++h) {
+      // group sums are integers of at most 8 x 16 x 2^14 = 2^21 in magnitude,
+      // read back exactly by adding 1.5 2^23 (an FP32 add; the bias 0x4B400000
+      // of each is taken out of the pair sums) and paired in 32 bits
+      uint32_t v[kSl][4];
 #pragma unroll
-      for (int g = 0; g < kSl; ++g) {
-        uint32_t v[8];
-        tmem_ld8(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(g * N + jc), v);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) gb[g][j] = __float_as_int(__uint_as_float(v[j]) + 12582912.0f);
+      for (int g = 0; g < kSl; ++g)
+        tmem_ld_16x8(tmem + tlane + (uint32_t)((ct & 1) * 128 + g * 16 + h * 8), v[g]);
+      tmem_wait_ld();
+      if (h == 1) {                                  // the last read of this accumulator
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&us.empty[ct & 1]);
       }
-      if (apply) {
-        // (b 2^8 + b) of two biased sums, modulo 2^32 (the pairs are exact in
-        // 32-bit two's complement)
-        constexpr uint32_t kBias = 0x4B400000u * 257u;
-        auto pair = [&](int g, int j) {
-          return (int)((uint32_t)gb[g][j] * 256u + (uint32_t)gb[g + 1][j] - kBias);
-        };
+      constexpr uint32_t kBias = 0x4B400000u * 257u;
+      auto pair = [&](int g, int e) {
+        const uint32_t b0 = __float_as_uint(__uint_as_float(v[g][e]) + 12582912.0f);
+        const uint32_t b1 = __float_as_uint(__uint_as_float(v[g + 1][e]) + 12582912.0f);
+        return (int)(b0 * 256u + b1 - kBias);
+      };
+      long long del[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          long long del[2];
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int j = 2 * i + h;
-            const int h01 = pair(0, j), h23 = pair(2, j), l45 = pair(4, j), l67 = pair(6, j);
-            const long long hi = (long long)h01 * 65536 + h23, lo = (long long)l45 * 65536 + l67;
-            del[h] = shift_round(hi, 32 + sh) + shift_round(lo, sh);
-          }
-          longlong2& qq = q[part * 4 + i];
-          qq.x -= del[0];
-          qq.y -= del[1];
-        }
+      for (int e = 0; e < 4; ++e) {
+        const long long hi = (long long)pair(0, e) * 65536 + pair(2, e);
+        const long long lo = (long long)pair(4, e) * 65536 + pair(6, e);
+        if (sh < 0 && sh > -32) del[e] = (hi << (32 + sh)) + ((lo + (1ll << (-sh - 1))) >> (-sh));
+        else del[e] = shift_round(hi, 32 + sh) + shift_round(lo, sh);
+      }
+      q[2 * h].x -= del[0]; q[2 * h].y -= del[1];
+      q[2 * h + 1].x -= del[2]; q[2 * h + 1].y -= del[3];
+      const int c = ct * 16 + 8 * h;
+      if (c < mp && er != kZeroExp) {
+        if (oka) *(longlong2*)(pa + c) = q[2 * h];
+        if (okb) *(longlong2*)(pb + c) = q[2 * h + 1];
       }
     }
-    if (apply) {
-#pragma unroll
-      for (int i = 0; i < NH / 4; ++i) rowp[i] = q[i];
-      if (half2) {
-#pragma unroll
-        for (int i = NH / 4; i < NH / 2; ++i) rowp[i] = q[i];
-      }
-    }
-    tc_fence_before();
-    __syncthreads();                                 // s_er and the B tiles are rewritten next
   }
-  if (s_fail && t == 0) atomicOr(a.err, 1u);
-  // after an expired wait, give the products in flight another bounded wait
-  // before their tensor memory is freed
-  if (s_fail && committed > 0) mbar_wait(&bar, (committed - 1) & 1);
+  __syncthreads();
+  if (us.fail && t == 0) {
+    atomicOr(a.err, 1u);
+    // give products still in flight another bounded wait before their memory is freed
+    for (uint32_t i = 0; i < kSpinLimit; ++i) __nanosleep(20);
+  }
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_free(tmem, 256);
@@ -1204,19 +1181,15 @@ __global__ void __launch_bounds__(kBtThreads) k_band_backtr(BandArgs a, BandVecA
 
 // ---------------------------------------------------------------------------
 namespace {
-constexpr size_t kGemmSmem = kABytes + 4 * 16 * 128 + 1024;      // A tiles, B tiles (N = 16), alignment
-constexpr size_t kUpdSmemNeed = 2 * kTileBytes + 2 * 32 * 128 + 1024;
-// requested so that at most two update CTAs share an SM (2 x 256 columns of tensor memory)
-constexpr size_t kUpdSmem = 80 * 1024;
+constexpr size_t kUpdSmem = kStageBytes + 4 * kBBytes + 1024;
 }  // namespace
 
 cudaError_t launch_band_reduce(const BandArgs& a, bool chase, cudaStream_t st) {
   if (a.S <= 0) return cudaSuccess;
   if (!band_supported(a.n)) return cudaErrorInvalidValue;
-  static_assert(kUpdSmemNeed <= kUpdSmem, "update tiles exceed the requested shared memory");
   static std::atomic<uint64_t> at_w{0}, at_x{0}, at_u{0};
-  cudaError_t e = raise_smem_limit(k_band_gemm_w, (int)kGemmSmem, at_w);
-  if (e == cudaSuccess) e = raise_smem_limit(k_band_gemm_x, (int)kGemmSmem, at_x);
+  cudaError_t e = raise_smem_limit(k_band_gemm_w, (int)kProdSmem, at_w);
+  if (e == cudaSuccess) e = raise_smem_limit(k_band_gemm_x, (int)kProdSmem, at_x);
   if (e == cudaSuccess) e = raise_smem_limit(k_band_update, (int)kUpdSmem, at_u);
   if (e != cudaSuccess) return e;
   const int n = a.n, S = a.S;
@@ -1228,11 +1201,11 @@ cudaError_t launch_band_reduce(const BandArgs& a, bool chase, cudaStream_t st) {
     if (k + B >= n) break;
     const int mp = n - k - B;
     const int tiles = (mp + kTileM - 1) / kTileM;
-    k_band_gemm_w<<<dim3(S, tiles), 256, kGemmSmem, st>>>(a, k);
+    k_band_gemm_w<<<dim3(S, tiles), 256, kProdSmem, st>>>(a, k);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_band_lq<<<S, 256, 0, st>>>(a, k);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_band_gemm_x<<<dim3(S, tiles), 256, kGemmSmem, st>>>(a, k);
+    k_band_gemm_x<<<dim3(S, tiles), 256, kProdSmem, st>>>(a, k);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_band_update<<<dim3(S, tiles), 256, kUpdSmem, st>>>(a, k);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -27,6 +27,10 @@ static __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t by
                : "memory");
 }
 
+static __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
 static __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -70,6 +74,11 @@ static __host__ __device__ constexpr uint32_t umma_idesc(int kind, int M, int N)
   // kind 0: tf32 (format 2 under kind::tf32); kind 1: bf16 (format 1 under kind::f16)
   return (1u << 4) | ((kind == 0 ? 2u : 1u) << 7) | ((kind == 0 ? 2u : 1u) << 10) |
          ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// The same for FP16 operands (format 0 under kind::f16; issued as umma<1>).
+static __host__ __device__ constexpr uint32_t umma_idesc_f16(int M, int N) {
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 template <int KIND>

@@ -52,6 +52,19 @@ def test_group_sums_stay_exact_in_fp32():
         assert int(f.view(np.int32)) - 0x4B400000 == G
 
 
+def test_group_sums_of_the_62_bit_trailing_matrix():
+    # W and X with entries below 2^61 (top digit <= 32, as V's and U's): the groups of the 62 leading
+    # bits, 0..4, are exact; the update's operands are those above
+    assert max(_group_bound(256, 32, 32, g) for g in range(5)) <= 1 << 24
+
+
+def test_fp16_digits_from_byte_permutes():
+    """A byte b under FP16's exponent of 1024 reads 1024 + b, and 1024 + b - 1152 = b - 128 is exact in FP16."""
+    for b in range(256):
+        v = np.array([0x6400 | b], np.uint16).view(np.float16)[0] - np.array([0x6480], np.uint16).view(np.float16)[0]
+        assert float(v) == b - 128
+
+
 def test_biased_readbacks_pair_in_32_bits():
     rng = np.random.default_rng(2)
     B = 0x4B400000
