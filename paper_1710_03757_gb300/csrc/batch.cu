@@ -37,6 +37,7 @@
 #include "../../include/mctrg.h"
 #include "common.cuh"
 #include "kernels.h"
+#include "kernels_band.h"
 #include "kernels_bd.h"
 #include "kernels_lr.h"
 #include "kernels_tc.h"
@@ -355,8 +356,10 @@ struct BatchRunner {
     const bool tc_mode = prec != MCTRG_FP64 && !oz_mode;
     const int used = (int)std::min<size_t>(segs.size(), kStreams);
     std::vector<SegPtrs> ptr(segs.size());
-    std::vector<SvdItem> items;
-    int n_max = 0, kmax = 0;
+    // matrices of the one-stage reduction (ragged launches) and of the two-stage one
+    // (reduced per segment below); bisection and inverse iteration take both
+    std::vector<SvdItem> items, band_items;
+    int n_max = 0, n_one = 0, kmax = 0;
     size_t smem = 0;
     BCK(fork(used) == MCTRG_OK ? cudaSuccess : cudaErrorUnknown);
     for (size_t s = 0; s < segs.size(); ++s) {
@@ -409,6 +412,15 @@ struct BatchRunner {
       }
       launches += 1;
       if (g.bidiag) {
+        const bool band = c->use_band(v.n, Kd);
+        if (band) {
+          BandArgs ba = band_args(g, q, v.n);
+          BCK(launch_band_reduce(ba, true, ss));
+          launches += 2 + 5 * (v.n / kBandW - 1);
+        } else {
+          n_one = std::max(n_one, v.n);
+          smem = std::max(smem, bidiag_smem_bytes(v.n));
+        }
         for (int64_t i = 0; i < g.cnt; ++i) {
           SvdItem t{};
           t.M = q.M + (size_t)i * v.n * v.n; t.W = q.W + (size_t)i * v.n_pad * v.n; t.bd = q.bd + (size_t)i * 3 * v.n;
@@ -416,11 +428,10 @@ struct BatchRunner {
           const size_t ks = kept_stride(c->chi);
           t.lns1 = c->ilns1.as<double>() + g.i0 + i; t.kept = q.kept + (size_t)i * ks; t.nk = q.nk + i;
           t.vrows = q.vrows + (size_t)i * ks * v.n; t.zero_rel = zero_fp64(a.n); t.n = v.n; t.n_pad = v.n_pad;
-          items.push_back(t);
+          (band ? band_items : items).push_back(t);
         }
         n_max = std::max(n_max, v.n);
         kmax = std::max(kmax, a.kc);
-        smem = std::max(smem, bidiag_smem_bytes(v.n));
       } else {
         // the Jacobi route (low-rank levels): per segment, as mctrg_run does
         JacobiArgs ja{};
@@ -434,19 +445,23 @@ struct BatchRunner {
       }
     }
     BCK(join(used) == MCTRG_OK ? cudaSuccess : cudaErrorUnknown);
+    const int S1 = (int)items.size();        // the table's first S1 items are the one-stage reduction's
+    items.insert(items.end(), band_items.begin(), band_items.end());
     if (!items.empty()) {
       // the ragged SVD launches over every bidiagonalization segment, in chunks of
-      // the tuned size of the largest shape present
+      // the tuned size of the largest one-stage shape present
       if (sizeof(SvdItem) * items.size() > table.bytes) BCK(cudaStreamSynchronize(st));
       BCK(table.ensure(sizeof(SvdItem) * items.size()));
       BCK(cudaMemcpyAsync(table.p, items.data(), sizeof(SvdItem) * items.size(), cudaMemcpyHostToDevice, st));
       const int S = (int)items.size();
-      const int chunk = std::max(1, tuned(n_max, kmax).svd_items);
+      const int chunk = S1 > 0 ? std::max(1, tuned(n_one, kmax).svd_items) : 1 << 16;
+      for (int i0 = 0; i0 < S1; i0 += chunk) {
+        BCK(launch_bidiag_items(table.as<SvdItem>() + i0, std::min(chunk, S1 - i0), n_one, smem, st));
+        ++launches;
+      }
       for (int i0 = 0; i0 < S; i0 += chunk) {
-        const int cnt = std::min(chunk, S - i0);
-        BCK(launch_bidiag_items(table.as<SvdItem>() + i0, cnt, n_max, smem, st));
-        BCK(launch_bd_bisect_items(table.as<SvdItem>() + i0, cnt, n_max, st));
-        launches += 2;
+        BCK(launch_bd_bisect_items(table.as<SvdItem>() + i0, std::min(chunk, S - i0), n_max, st));
+        ++launches;
       }
       BCK(fork(used) == MCTRG_OK ? cudaSuccess : cudaErrorUnknown);
       for (size_t s = 0; s < segs.size(); ++s)
@@ -464,15 +479,22 @@ struct BatchRunner {
       for (int i0 = 0; i0 < S; i0 += chunk) {
         BdVecArgs va{};
         va.n = n_max; va.S = std::min(chunk, S - i0); va.kmax = kmax; va.items = table.as<SvdItem>() + i0;
-        va.scratch = vec_scr.as<double>();
+        va.scratch = vec_scr.as<double>(); va.skip_backtr = 1;
         BCK(launch_bd_vectors(va, st));
-        launches += 2;
+        ++launches;
+      }
+      for (int i0 = 0; i0 < S1; i0 += chunk) {
+        BdVecArgs va{};
+        va.n = n_one; va.S = std::min(chunk, S1 - i0); va.kmax = kmax; va.items = table.as<SvdItem>() + i0;
+        BCK(launch_bd_backtr(va, st));
+        ++launches;
       }
       BCK(fork(used) == MCTRG_OK ? cudaSuccess : cudaErrorUnknown);
       for (size_t s = 0; s < segs.size(); ++s)
         if (segs[s].bidiag) {
           JobRun& r = jr[segs[s].j];
           const LevelInfo& a = r.ctx->lv[segs[s].k];
+          BCK(band_backtr(r, segs[s], ptr[s], pool[s % kStreams]));
           BCK(launch_sample_split(sample_args(r, segs[s], ptr[s], 2, s), pool[s % kStreams],
                                   tuned(a.n, a.kc).sample_grid));
           BCK(expand_lowrank(r, segs[s], ptr[s], pool[s % kStreams]));
@@ -500,6 +522,27 @@ struct BatchRunner {
     if (mode == 0) { sa.W = q.W; }
     else { sa.W = nullptr; sa.kept = q.kept; sa.sigt = q.sigt; sa.nk = q.nk; sa.vrows = q.vrows; }
     return sa;
+  }
+
+  // the two-stage route's buffers of a segment (in the place of its X and Yt)
+  BandArgs band_args(const Segment& g, const SegPtrs& q, int n) {
+    BandArgs ba{};
+    band_carve(q.X, q.Y, n, g.cnt, ba);
+    ba.M = q.M; ba.Wk = (int64_t*)q.W; ba.bd = q.bd; ba.S = (int)g.cnt; ba.err = err.as<uint32_t>();
+    return ba;
+  }
+  cudaError_t band_backtr(JobRun& r, const Segment& g, const SegPtrs& q, cudaStream_t ss) {
+    mctrg_ctx* c = r.ctx;
+    const LevelInfo& a = c->lv[g.k];
+    const int Kd = c->lv[g.k - 1].D * c->lv[g.k - 1].D;
+    const SvdDims v = svd_dims(c->opt, a, Kd);
+    if (!c->use_band(v.n, Kd)) return cudaSuccess;
+    const BandArgs ba = band_args(g, q, v.n);
+    BandVecArgs bv{};
+    bv.band = &ba; bv.sig = q.sig; bv.kept = q.kept; bv.nk = q.nk; bv.vrows = q.vrows; bv.n_pad = v.n_pad;
+    bv.kstride = kept_stride(c->chi); bv.unit_rows = 0; bv.kmax = a.kc;
+    ++launches;
+    return launch_band_backtr(bv, ss);
   }
 
   // the level's halves from those of a low-rank segment's cores
@@ -610,7 +653,7 @@ extern "C" int mctrg_batch_run(const mctrg_options* opt, const mctrg_job* jobs, 
                                double* lnabsZ, int8_t* sign, uint8_t* flags) {
   if (!opt || !jobs || !est || n_jobs < 1) return MCTRG_EINVAL;
   if (opt->precision != MCTRG_FP64 && opt->precision != MCTRG_FP64TC) return MCTRG_EINVAL;
-  if (opt->svd == MCTRG_SVD_BAND) return MCTRG_EINVAL;   // ragged launches take the one-stage route
+  if (opt->svd == MCTRG_SVD_BAND) return MCTRG_EINVAL;   // not offered by name (AUTO takes it where mctrg_run does)
   for (int j = 0; j < n_jobs; ++j) {
     const mctrg_job& b = jobs[j];
     if (b.n_samples < 1 || b.first_traj + (uint64_t)b.n_samples > (1ull << 32)) return MCTRG_EINVAL;
@@ -646,6 +689,11 @@ extern "C" int mctrg_batch_run(const mctrg_options* opt, const mctrg_job* jobs, 
       const int n = svd_dims(c->opt, c->lv[k], Kd).n;
       if (!c->use_bidiag(n, Kd)) continue;
       if (R.tune.count(TuneKey{n, c->lv[k].kc})) continue;
+      if (c->use_band(n, Kd)) {     // reduced per segment: no chunk of a merged launch to time
+        R.tune[TuneKey{n, c->lv[k].kc}] = TuneVal{1 << 16, sample_grid(n, c->lv[k].kc)};
+        R.tune_dirty = true;
+        continue;
+      }
       status = R.tune_shape(n, c->lv[k].kc);
     }
   }

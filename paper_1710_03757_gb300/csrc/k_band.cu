@@ -286,18 +286,15 @@ int band_nref(int n) {
 
 size_t band_work_doubles(int n) { return work_stride(n); }
 
-size_t band_item_bytes(int n) {
-  return sizeof(double) * ((size_t)n * (B + 1) + band_work_doubles(n) + (size_t)band_nref(n) * B) + sizeof(int);
-}
+size_t band_panel_doubles(int n) { return (size_t)n * (B + 1) + band_work_doubles(n) + 1; }
+size_t band_refl_doubles(int n) { return (size_t)band_nref(n) * B; }
 
-void band_carve(void* base, int n, int64_t S, BandArgs& a) {
-  double* p = (double*)base;
-  const size_t nref = (size_t)band_nref(n);
+void band_carve(void* panels, void* refl, int n, int64_t S, BandArgs& a) {
+  double* p = (double*)panels;
   a.band = p; p += (size_t)S * n * (B + 1);
   a.work = p; p += (size_t)S * band_work_doubles(n);
-  a.refl = p; p += (size_t)S * nref * B;
   a.eA = (int*)p;
-  a.err = (uint32_t*)(a.eA + S);
+  a.refl = (double*)refl;
   a.n = n;
 }
 

@@ -1145,16 +1145,21 @@ size_t bd_vectors_scratch_doubles(int n, int S, int kmax) {
 cudaError_t launch_bd_vectors(const BdVecArgs& a, cudaStream_t st) {
   if (a.S <= 0) return cudaSuccess;
   if (a.kmax > kKeptMax || (!a.items && a.kstride < a.kmax)) return cudaErrorInvalidValue;
-  constexpr size_t kSmemCap = 227 * 1024;
-  const int gs = (size_t)16 * a.n * sizeof(double) <= kSmemCap ? 16 : 8;
-  const size_t smem = (size_t)gs * a.n * sizeof(double);
-  if (smem > kSmemCap) return cudaErrorInvalidValue;
   const int ls = invit_stride(a.kmax);
   k_bd_invit<<<invit_slots(a.n, a.S, a.kmax), ls > 32 ? 64 : 32, 0, st>>>(a, ls);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || a.skip_backtr) return e;
+  return launch_bd_backtr(a, st);
+}
+
+cudaError_t launch_bd_backtr(const BdVecArgs& a, cudaStream_t st) {
+  if (a.S <= 0) return cudaSuccess;
+  constexpr size_t kSmemCap = 227 * 1024;
+  const int gs = (size_t)16 * a.n * sizeof(double) <= kSmemCap ? 16 : 8;
+  const size_t smem = (size_t)gs * a.n * sizeof(double);
+  if (smem > kSmemCap) return cudaErrorInvalidValue;
   static std::atomic<uint64_t> attr{0};
-  e = raise_smem_limit(k_bd_backtr, kSmemCap, attr);
+  cudaError_t e = raise_smem_limit(k_bd_backtr, kSmemCap, attr);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)a.S, (unsigned)((std::max(1, a.kmax) + gs - 1) / gs));
   k_bd_backtr<<<grid, 32 * (gs / 4), smem, st>>>(a, gs);

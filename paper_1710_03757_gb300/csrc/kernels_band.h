@@ -35,11 +35,17 @@ struct BandArgs {
   int n, S;
 };
 size_t band_work_doubles(int n);
-// Bytes per matrix of band, work, refl and eA (Wk and bd are the
-// caller's); band_carve lays them out for S matrices from `base` (which must
-// hold S * band_item_bytes(n) + 256 bytes) and puts err after them.
-size_t band_item_bytes(int n);
-void band_carve(void* base, int n, int64_t S, BandArgs& a);
+// Doubles per matrix of the panel buffers (band, work, eA) and of the
+// reflectors (Wk, bd and err are the caller's); band_carve points `a` at those
+// of S matrices, each block laid out from its own base.
+size_t band_panel_doubles(int n);
+size_t band_refl_doubles(int n);
+void band_carve(void* panels, void* refl, int n, int64_t S, BandArgs& a);
+// The operands X and Yt of a level (n K doubles each) are dead once its
+// matrices exist: a context lets the route's buffers take their place.
+inline bool band_fits_operands(int n, int64_t K) {
+  return (int64_t)band_panel_doubles(n) <= n * K && (int64_t)band_refl_doubles(n) <= n * K;
+}
 
 // Stage 1 and 2: M -> band (Wk, band) -> bidiagonal (bd).  Stage 1 alone when
 // chase == false (band filled, bd untouched).

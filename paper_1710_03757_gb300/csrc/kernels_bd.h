@@ -78,6 +78,9 @@ struct BdVecArgs {
   int skip_backtr = 0;  // 1: leave the unit vectors of the bidiagonal in vrows
 };
 cudaError_t launch_bd_vectors(const BdVecArgs& a, cudaStream_t st);
+// Its second half alone: the right reflectors of the one-stage reduction
+// applied to the unit vectors of the bidiagonal in vrows.
+cudaError_t launch_bd_backtr(const BdVecArgs& a, cudaStream_t st);
 size_t bd_vectors_scratch_doubles(int n, int S, int kmax);
 
 }  // namespace mctrg

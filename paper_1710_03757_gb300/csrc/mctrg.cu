@@ -170,7 +170,7 @@ size_t mctrg_ctx::held_bytes() const {
                          &Mb, &Wb, &Xb, &Yb, &sigb, &permb, &nnzb, &ilns1, &iflags, &lnacc, &tflags,
                          &scratch, &o_lnabs, &o_sign, &o_flags, &o_tflags, &stats, &tcXh, &tcYh, &tcXl,
                          &tcYl, &tcScale, &tcErr, &ozExp, &Timp, &bdb, &keptb, &sigtb, &nkb, &vrowsb, &bdscr,
-                         &bandb, &lrb};
+                         &lrb};
   size_t b = 0;
   for (const DevBuf* d : all) b += d->bytes;
   return b;
@@ -184,7 +184,7 @@ void mctrg_ctx::release_all() {
                    &Mb, &Wb, &Xb, &Yb, &sigb, &permb, &nnzb, &ilns1, &iflags, &lnacc, &tflags,
                    &scratch, &o_lnabs, &o_sign, &o_flags, &o_tflags, &stats, &tcXh, &tcYh, &tcXl,
                    &tcYl, &tcScale, &tcErr, &ozExp, &Timp, &bdb, &keptb, &sigtb, &nkb, &vrowsb, &bdscr,
-                   &bandb, &lrb};
+                   &lrb};
   for (DevBuf* b : all) b->release();
 }
 
@@ -313,9 +313,21 @@ bool route_bidiag(const mctrg_options& o, int n, int K) {
   if (o.svd == MCTRG_SVD_BIDIAG) return n >= 2;
   return n >= 64 && 2 * K >= n;
 }
-// The two-stage route replaces the one-stage one on the sizes it takes.
+// The two-stage route replaces the one-stage one on the sizes it takes, unless
+// the caller named that; AUTO takes it above n = 192, where it is the faster one
+// at every batch (values and 16 vectors, two-stage against one-stage: one matrix
+// of n = 256 12.0 ms against 12.8, 256 of them 16.1 against 23.5, 1920 84
+// against 139; below, its panels' launches cost small batches more than large
+// ones gain: n = 144, 64 matrices 6.0 against 4.7, 256 7.0 against 7.8; n = 192,
+// one 8.2 against 7.4).  The choice looks at the side alone, so a trajectory's
+// result does not depend on the batch.  Both are as accurate: singular values
+// against a quadruple-precision Jacobi, rms error over s_1 at n = 64, 1.5e-16 on
+// a flat spectrum and 4e-17 over 14 decades (the one-stage route 1.4e-16 and
+// 8.6e-17 before its bisection was refined, 7e-17 and 2e-17 since).
+constexpr int kAutoBandMin = 200;
 bool route_band(const mctrg_options& o, int n, int K) {
-  return o.svd == MCTRG_SVD_BAND && band_supported(n) && route_bidiag(o, n, K);
+  const bool named = o.svd == MCTRG_SVD_BAND, chosen = o.svd == MCTRG_SVD_AUTO && n >= kAutoBandMin;
+  return (named || chosen) && band_supported(n) && route_bidiag(o, n, K) && band_fits_operands(n, K);
 }
 // A level of inner dimension K < n goes through the K x K core of its factors
 // (kernels_lr.h), unless the caller named a route for the matrices themselves
@@ -482,8 +494,7 @@ void plan_run(const std::vector<LevelInfo>& lv, int s0, int nlev, int chi, const
         const size_t ks = kept_stride(chi);
         pi += (3 * (size_t)v.n + ks + ks * (size_t)v.n) * sizeof(double) + (ks + 1) * sizeof(int);
         bd_scr = std::max(bd_scr, bd_vectors_scratch_doubles(v.n, 1 << 16, a.kc) * sizeof(double));
-        // the band route: band, panel scratch, chase reflectors, exponent
-        if (route_band(opt, v.n, (int)d2)) pi += band_item_bytes(v.n);
+        // (the band route's own buffers take the place of X and Yt)
       }
       per_item = std::max(per_item, pi);
     }
@@ -651,6 +662,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
     CK(nnzb.ensure(sizeof(int) * std::max<int64_t>(S, 1)));
     CK(scratch.ensure(sizeof(double) * max_scr));
     CK(lrb.ensure(sizeof(double) * max_lr));
+    bool any_band = false;
     {  // bidiagonalization route buffers (levels that take it)
       size_t bd_n = 0, bd_scr = 0;
       for (int k = s0 + 1; k < nlev; ++k) {
@@ -658,18 +670,9 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
         const int Kd = lv[k - 1].D * lv[k - 1].D;
         const SvdDims v = svd_dims(opt, a, Kd);
         if (!use_bidiag(v.n, Kd)) continue;
+        any_band = any_band || use_band(v.n, Kd);
         bd_n = std::max(bd_n, (size_t)v.n);
         bd_scr = std::max(bd_scr, bd_vectors_scratch_doubles(v.n, (int)std::min<int64_t>(S, 1 << 16), a.kc));
-      }
-      size_t band_n = 0;
-      for (int k = s0 + 1; k < nlev; ++k) {
-        const int Kd = lv[k - 1].D * lv[k - 1].D;
-        const SvdDims v = svd_dims(opt, lv[k], Kd);
-        if (use_band(v.n, Kd)) band_n = std::max(band_n, (size_t)v.n);
-      }
-      if (band_n) {
-        CK(bandb.ensure((size_t)std::max<int64_t>(S, 1) * band_item_bytes((int)band_n) + 256));
-        CK(cudaMemsetAsync(bandb.p, 0, bandb.bytes, st));
       }
       if (bd_n) {
         const size_t Ss = (size_t)std::max<int64_t>(S, 1);
@@ -712,7 +715,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
         CK(ozExp.ensure(sizeof(int) * 2 * oz_rows));
       }
     }
-    if (prec != MCTRG_FP64 || bandb.p) {
+    if (prec != MCTRG_FP64 || any_band) {
       CK(tcErr.ensure(sizeof(uint32_t)));
       CK(cudaMemsetAsync(tcErr.p, 0, sizeof(uint32_t), st));
     }
@@ -871,7 +874,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
             const bool band = use_band(v.n, Kd);
             BandArgs bda{};
             if (band) {
-              band_carve(bandb.p, v.n, Si, bda);
+              band_carve(Xb.p, Yb.p, v.n, Si, bda);
               bda.M = Mb.as<double>(); bda.Wk = (int64_t*)Wb.p; bda.bd = bdb.as<double>(); bda.S = (int)Si;
               bda.err = band_err;
               CK(timed(MCTRG_K_BAND, Si, Si * (8.0 / 3.0) * nn * nn * nn, 8.0 * Si * (nn * nn + 9.0 * nn),
@@ -960,7 +963,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
   if (sign_out) CK(cudaMemcpyAsync(sign_out, o_sign.p, (size_t)n, cudaMemcpyDefault, st));
   if (flags_out) CK(cudaMemcpyAsync(flags_out, o_flags.p, (size_t)n, cudaMemcpyDefault, st));
   uint32_t tc_err = 0;
-  if ((opt.precision != MCTRG_FP64 || opt.svd == MCTRG_SVD_BAND) && tcErr.p)
+  if (tcErr.p && !all_exact)   // zeroed by every run that has such kernels
     CK(cudaMemcpyAsync(&tc_err, tcErr.p, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   resolve_events();

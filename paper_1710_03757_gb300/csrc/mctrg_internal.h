@@ -76,7 +76,6 @@ struct mctrg_ctx {
   mctrg::DevBuf ozExp;                                     // FP64TC: row exponents of X and Yt
   mctrg::DevBuf Timp;                                      // impurity tensor (level0_distinct)
   mctrg::DevBuf bdb, keptb, sigtb, nkb, vrowsb, bdscr;    // bidiagonalization route
-  mctrg::DevBuf bandb;                                     // band route: band, scratch, reflectors
   mctrg::DevBuf lrb;                                       // low-rank levels: reflectors, taus, core halves
 
   // per-kernel-class statistics (MCTRG_K_*)

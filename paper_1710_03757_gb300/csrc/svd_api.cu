@@ -110,17 +110,20 @@ extern "C" int mctrg_svd_bidiag_batched(const double* M, int n, int64_t batch, d
 }
 
 // Device buffers of the band route for `chunk` matrices of side n, carved
-// from one allocation: Wk (n x n), bd (3n), then band_carve's.
+// from one allocation: Wk (n x n), bd (3n), band_carve's, the error word.
 static size_t band_bytes(int n, int64_t chunk) {
   // rounded up to 256 bytes: the buffers that follow hold doubles
-  const size_t b = (size_t)chunk * (sizeof(double) * ((size_t)n * n + 3 * (size_t)n) + band_item_bytes(n)) + 256;
+  const size_t b = (size_t)chunk * sizeof(double) *
+                       ((size_t)n * n + 3 * (size_t)n + band_panel_doubles(n) + band_refl_doubles(n)) + 256;
   return (b + 255) & ~(size_t)255;
 }
 static void band_all(void* buf, int n, int64_t chunk, BandArgs& a) {
   double* p = (double*)buf;
   a.Wk = (int64_t*)p; p += (size_t)chunk * n * n;
   a.bd = p; p += (size_t)chunk * 3 * n;
-  band_carve(p, n, chunk, a);
+  double* refl = p + (size_t)chunk * band_panel_doubles(n);
+  band_carve(p, refl, n, chunk, a);
+  a.err = (uint32_t*)(refl + (size_t)chunk * band_refl_doubles(n));
 }
 
 extern "C" int mctrg_band_reduce_batched(const double* M, int n, int64_t batch, double* band, double* bd,
