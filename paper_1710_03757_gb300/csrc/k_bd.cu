@@ -96,13 +96,13 @@ struct BdStep {
   const double* wv;
   const double* uv;
   double* wpart;
-  int n, k, lane, warp;
+  int n, k, lane, warp, nw;
 };
 
 // w pass: per-warp partial sums sum_{i>k} v_i A[i][c] over the warp's rows.
 template <int QL>
 __device__ __forceinline__ void bd_w_pass(const BdStep& s) {
-  constexpr int NW = kBdThreads / 32;
+  const int NW = s.nw;
   const int n = s.n, c0 = s.k + 1 + s.lane;
   double acc[QL];
 #pragma unroll
@@ -175,7 +175,7 @@ __device__ __forceinline__ double bd_rows(const BdStep& s, int i0, const double 
 // the diagonal (valid in lane 0).
 template <int QL>
 __device__ __forceinline__ double bd_fused_pass(const BdStep& s, double* vcol_out) {
-  constexpr int NW = kBdThreads / 32;
+  const int NW = s.nw;
   constexpr int RPW = QL <= 8 ? 4 : (QL <= 16 ? 2 : 1);   // rows per warp and pass (register budget)
   const int n = s.n, k = s.k, c0 = k + 1 + s.lane;
   double wr[QL], ur[QL];
@@ -224,7 +224,7 @@ struct BdDispatch<NQ + 1, NQ> {
 // element more than the register form; the same operations in the same order
 // otherwise.
 __device__ __forceinline__ void bdw_w_pass(const BdStep& s) {
-  constexpr int NW = kBdThreads / 32;
+  const int NW = s.nw;
   const int n = s.n, k = s.k;
   double* wp = s.wpart + (size_t)s.warp * n;
   for (int c = k + 1 + s.lane; c < n; c += 32) wp[c] = 0.0;
@@ -287,7 +287,7 @@ __device__ __forceinline__ double bdw_rows(const BdStep& s, int i0, double* vcol
 }
 
 __device__ __forceinline__ double bdw_fused_pass(const BdStep& s, double* vcol_out) {
-  constexpr int NW = kBdThreads / 32;
+  const int NW = s.nw;
   constexpr int RPW = 4;
   const int n = s.n, k = s.k;
   double* wp = s.wpart + (size_t)s.warp * n;
@@ -299,47 +299,89 @@ __device__ __forceinline__ double bdw_fused_pass(const BdStep& s, double* vcol_o
   return nsq;
 }
 
+// Sum of the NW (at most 16) partials, in every lane.
+__device__ __forceinline__ double bd_sum_warps(const double* red, int nw, int lane) {
+  double t = lane < nw ? red[lane] : 0.0;
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return __shfl_sync(0xffffffffu, t, 0);
+}
+
+// Householder reflector of (alpha, x) with sq = |x|^2: H = I - tau v v^T, v =
+// (1, scl x), H (alpha, x) = (beta, 0).  |alpha - beta| = |alpha| + |(alpha, x)|
+// (no cancellation), tau that over the norm.
+struct BdReflector {
+  double beta, tau, scl;
+};
+__device__ __forceinline__ BdReflector bd_reflector(double alpha, double sq) {
+  BdReflector h{alpha, 0.0, 0.0};
+  if (sq > 0.0) {
+    const double t = fma(alpha, alpha, sq), rn = rsqrt(t), nrm = t * rn;
+    h.beta = -copysign(nrm, alpha);
+    const double d = alpha - h.beta;
+    h.tau = fabs(d) * rn;
+    h.scl = 1.0 / d;
+  }
+  return h;
+}
+
+// Threads of a reduction: more than 128 would only add partial sums at the
+// small sides, whose CTAs share an SM.  With this and the reflectors' scalars in
+// one warp (in all eight they were 1,100 of the 1,300 FP64 warp instructions of
+// an average step at n = 64, 28% at n = 256): 3584 matrices of n = 64 13.4 ->
+// 6.0 ms, 672 of n = 144 15.6 -> 12.4, 304 of n = 256 18.4 -> 15.4.
+__host__ __device__ __forceinline__ int bidiag_threads(int n) { return n <= 128 ? 128 : kBdThreads; }
+__host__ __device__ __forceinline__ size_t bidiag_aux_doubles(int n, int nw) { return (size_t)(3 + nw) * n + 32; }
+// Whether the working copy fits in shared memory beside the per-step vectors.
+__host__ __device__ __forceinline__ bool bidiag_in_smem(int n, int nw) {
+  return ((size_t)n * n + bidiag_aux_doubles(n, nw)) * sizeof(double) <= 200 * 1024;
+}
+
 // NQ > 0: the register form for sides up to 32 NQ; NQ = 0: the wide form.
 template <int NQ>
 __global__ void __launch_bounds__(kBdThreads) k_bidiag(BidiagArgs a, int use_smem) {
   extern __shared__ double sm[];
   int n = a.n;
   const int mat = blockIdx.x;
-  constexpr int NW = kBdThreads / 32;
   const double* Mm;
   double* Wm;
   double* bd;
   if (a.items) {                     // ragged: this matrix's size and buffers
     const SvdItem& t = a.items[mat];
     n = t.n; Mm = t.M; Wm = t.W; bd = t.bd;
-    use_smem = NQ > 0 && ((size_t)n * n + (size_t)(3 + NW) * n + 32) * sizeof(double) <= 200 * 1024;
+    use_smem = NQ > 0 && bidiag_in_smem(n, bidiag_threads(n) / 32);
   } else {
     Mm = a.M + (size_t)mat * n * n; Wm = a.W + (size_t)mat * n * n; bd = a.bd + (size_t)mat * 3 * n;
   }
+  // the thread count follows the matrix's own side, so that its sums do not
+  // depend on what else is in the launch; spare threads of a ragged one leave
+  const int nt = bidiag_threads(n), NW = nt >> 5;
+  if ((int)threadIdx.x >= nt) return;
   double* A = use_smem ? sm : Wm;
   double* base = use_smem ? sm + (size_t)n * n : sm;
   double* vcol = base;               // [n] column k (then v), below and on the diagonal
   double* wv = vcol + n;             // [n] w
   double* uv = wv + n;               // [n] u
   double* wpart = uv + n;            // [NW][n] per-warp partial column dots
-  double* red = wpart + (size_t)NW * n;   // [32]
+  double* red = wpart + (size_t)NW * n;   // [NW] partial squares, then the reflector's scalars
+  double* sc = red + 16;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  __shared__ double s_xn2;
-  for (int e = tid; e < n * n; e += kBdThreads) A[e] = Mm[e];
-  for (int e = tid; e < 3 * n; e += kBdThreads) bd[e] = 0.0;
+  for (int e = tid; e < n * n; e += nt) A[e] = Mm[e];
+  for (int e = tid; e < 3 * n; e += nt) bd[e] = 0.0;
   __syncthreads();
   {
     double sq = 0.0;
-    for (int i = tid; i < n; i += kBdThreads) {
+    for (int i = tid; i < n; i += nt) {
       const double x = A[(size_t)i * n];
       vcol[i] = x;
       if (i > 0) sq = fma(x, x, sq);
     }
-    const double t = block_sum(sq, red);
-    if (tid == 0) s_xn2 = t;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if (lane == 0) red[warp] = sq;
   }
   __syncthreads();
-  BdStep st{A, vcol, wv, uv, wpart, n, 0, lane, warp};
+  BdStep st{A, vcol, wv, uv, wpart, n, 0, lane, warp, NW};
   // the column dots of step 0 with the unnormalized column 0: later steps get
   // theirs from the previous fused pass (w is linear in the column)
   if (n > 1) {
@@ -350,73 +392,58 @@ __global__ void __launch_bounds__(kBdThreads) k_bidiag(BidiagArgs a, int use_sme
   for (int k = 0; k < n; ++k) {
     st.k = k;
     const int ql = (n - k - 1 + 31) >> 5;     // live 32-column chunks right of column k
-    // ---- left reflector from column k
-    const double xn2 = s_xn2;
-    const double alpha = vcol[k];
-    double tau = 0.0, beta = alpha, scal = 0.0;
-    if (xn2 > 0.0) {
-      beta = -copysign(sqrt(fma(alpha, alpha, xn2)), alpha);
-      tau = (beta - alpha) / beta;
-      scal = 1.0 / (alpha - beta);
-      for (int i = k + 1 + tid; i < n; i += kBdThreads) vcol[i] *= scal;
+    // ---- left reflector from column k: its scalars by one warp (the square
+    //      root and the reciprocal are some twenty FP64 instructions, and each
+    //      holds the SM's FP64 pipe 16 cycles per warp that issues it)
+    if (warp == 0) {
+      const BdReflector h = bd_reflector(vcol[k], bd_sum_warps(red, NW, lane));
+      if (lane == 0) { sc[0] = h.tau; sc[1] = h.scl; bd[k] = h.beta; }
     }
-    if (tid == 0) bd[k] = beta;
     if (k == n - 1) break;
     __syncthreads();
-    // ---- w = tau (A[k][:] + v^T A[k+1:, :]) on columns > k; wpart holds
-    //      sum_{i>k} x_i A[i][:] for the unnormalized column x (v = scal x)
-    if (tau != 0.0) {
-      for (int jj = k + 1 + tid; jj < n; jj += kBdThreads) {
-        double sum = 0.0;
-        for (int w = 0; w < NW; ++w) sum += wpart[w * n + jj];
-        wv[jj] = tau * fma(scal, sum, A[(size_t)k * n + jj]);
-      }
-    } else {
-      for (int jj = k + 1 + tid; jj < n; jj += kBdThreads) wv[jj] = 0.0;
+    const double tau = sc[0], scl = sc[1];
+    // ---- v; w = tau (A[k][:] + v^T A[k+1:, :]) on columns > k (wpart holds
+    //      sum_{i>k} x_i A[i][:] for the unnormalized column x, v = scl x); row k
+    //      after the left reflector, and its square beyond k+1
+    for (int i = k + 1 + tid; i < n; i += nt) vcol[i] *= scl;
+    double sq = 0.0;
+    for (int jj = k + 1 + tid; jj < n; jj += nt) {
+      double sum = 0.0;
+      for (int w = 0; w < NW; ++w) sum += wpart[w * n + jj];
+      const double akj = A[(size_t)k * n + jj];
+      const double wj = tau * fma(scl, sum, akj), r = akj - wj;
+      wv[jj] = wj;
+      uv[jj] = r;
+      if (jj > k + 1) sq = fma(r, r, sq);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if (lane == 0) red[warp] = sq;
+    __syncthreads();
+    // ---- right reflector from row k: G = I - us us^T with us = sqrt(tauR) u
+    if (warp == 0) {
+      const BdReflector h = bd_reflector(uv[k + 1], bd_sum_warps(red, NW, lane));
+      const double rt = sqrt(h.tau);
+      if (lane == 0) { sc[2] = h.scl; sc[3] = rt; bd[n + k] = h.beta; bd[2 * n + k] = h.tau; }
     }
     __syncthreads();
-    // ---- row k after the left reflector, and the right reflector from it
-    double sq = 0.0;
-    for (int jj = k + 2 + tid; jj < n; jj += kBdThreads) {
-      const double r = A[(size_t)k * n + jj] - wv[jj];
-      uv[jj] = r;
-      sq = fma(r, r, sq);
+    const double scr = sc[2], rt = sc[3];
+    for (int jj = k + 1 + tid; jj < n; jj += nt) {
+      const double u = jj == k + 1 ? 1.0 : uv[jj] * scr;
+      uv[jj] = rt * u;
+      if (jj > k + 1) A[(size_t)k * n + jj] = u;        // kept for the back-transformation
     }
-    const double yn2 = block_sum(sq, red);
-    const double ar = A[(size_t)k * n + k + 1] - wv[k + 1];
-    double taur = 0.0, betar = ar;
-    if (yn2 > 0.0) {
-      betar = -copysign(sqrt(fma(ar, ar, yn2)), ar);
-      taur = (betar - ar) / betar;
-      const double scal = 1.0 / (ar - betar);
-      const double rt = sqrt(taur);               // G = I - us us^T with us = sqrt(tauR) u
-      for (int jj = k + 2 + tid; jj < n; jj += kBdThreads) {
-        const double u = uv[jj] * scal;
-        uv[jj] = rt * u;
-        A[(size_t)k * n + jj] = u;              // kept for the back-transformation
-      }
-    } else {
-      for (int jj = k + 2 + tid; jj < n; jj += kBdThreads) uv[jj] = 0.0;
-    }
-    if (tid == 0) { uv[k + 1] = sqrt(taur); bd[n + k] = betar; bd[2 * n + k] = taur; }
     __syncthreads();
     // ---- fused pass over rows i > k
     double nsq;
     if constexpr (NQ == 0) nsq = bdw_fused_pass(st, vcol);
     else nsq = BdDispatch<1, NQ>::fused(ql, st, vcol);
-    __syncthreads();                            // everyone done with red / vcol reads
-    if (lane == 0) red[warp] = nsq;
-    __syncthreads();
-    if (tid == 0) {
-      double t = 0.0;
-      for (int w = 0; w < NW; ++w) t += red[w];
-      s_xn2 = t;
-    }
+    if (lane == 0) red[warp] = nsq;             // last read before the barrier above
     __syncthreads();
   }
   if (use_smem) {
     __syncthreads();
-    for (int e = tid; e < n * n; e += kBdThreads) Wm[e] = A[e];
+    for (int e = tid; e < n * n; e += nt) Wm[e] = A[e];
   }
 }
 
@@ -1043,21 +1070,20 @@ constexpr size_t kBdSmemCap = 227 * 1024;
 // memory requested that one CTA runs per SM and the matrices stay in L2).
 size_t bidiag_smem_bytes(int n) {
   const size_t rows = (size_t)n * n * sizeof(double);
-  const size_t aux = ((size_t)(3 + kBdThreads / 32) * n + 32) * sizeof(double);
-  return rows + aux <= 200 * 1024 ? rows + aux : std::max<size_t>(aux, 120 * 1024);
+  const size_t aux = bidiag_aux_doubles(n, bidiag_threads(n) / 32) * sizeof(double);
+  return bidiag_in_smem(n, bidiag_threads(n) / 32) ? rows + aux : std::max<size_t>(aux, 120 * 1024);
 }
 
 template <int NQ>
 static cudaError_t launch_bidiag_nq(const BidiagArgs& a, cudaStream_t st) {
   const int n = a.n;
-  const int use_smem = NQ > 0 && (size_t)n * n * sizeof(double) +
-                                         ((size_t)(3 + kBdThreads / 32) * n + 32) * sizeof(double) <=
-                                     200 * 1024;
+  const int threads = bidiag_threads(n);
+  const int use_smem = NQ > 0 && bidiag_in_smem(n, threads / 32);
   const size_t smem = bidiag_smem_bytes(n);
   static std::atomic<uint64_t> attr{0};
   cudaError_t e = raise_smem_limit(k_bidiag<NQ>, kBdSmemCap, attr);
   if (e != cudaSuccess) return e;
-  k_bidiag<NQ><<<a.S, kBdThreads, smem, st>>>(a, use_smem);
+  k_bidiag<NQ><<<a.S, threads, smem, st>>>(a, use_smem);
   return cudaGetLastError();
 }
 
