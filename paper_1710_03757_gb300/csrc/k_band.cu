@@ -215,61 +215,122 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Sums of nd dots over the first m entries of smem vectors: dot d pairs
-// vectors xa[d] and xb[d]; warp w takes dots w, w + nw, ...  Every thread
-// reads the results from out[] after the call's final barrier.
-template <class FA, class FB>
-__device__ __forceinline__ void block_dots(int nd, int m, FA xa, FB xb, double* out) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int d = warp; d < nd; d += nw) {
-    double p = 0.0;
-    for (int t = lane; t < m; t += 32) p = fma(xa(d, t), xb(d, t), p);
-    p = warp_sum(p);
-    if (lane == 0) out[d] = p;
-  }
-  __syncthreads();
+// Householder reflector (dlarfg) of a vector with first entry alpha and
+// squared norm sq of the rest: H = I - tau v v^T, v_0 = 1, v_i = x_i scl,
+// H x = beta e_1.  |alpha - beta| = |alpha| + |x| (no cancellation).
+__device__ __forceinline__ void reflector(double alpha, double sq, double& beta, double& tau, double& scl) {
+  if (sq == 0.0) { beta = alpha; tau = 0.0; scl = 0.0; return; }
+  const double t = fma(alpha, alpha, sq), rn = rsqrt(t), nrm = t * rn;
+  beta = -copysign(nrm, alpha);
+  const double d = alpha - beta;
+  tau = fabs(d) * rn;
+  scl = 1.0 / d;
 }
 
-// Gram values G[a][c] = x_a . x_c for a < c (the 28 that T needs) of b
-// shared-memory vectors of length m, into G[a * b + c].
-template <class FX>
-__device__ __forceinline__ void gram_upper(int m, FX x, double* G) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int d = warp; d < B * (B - 1) / 2; d += nw) {
-    int a = 0, rem = d;
-    while (rem >= B - 1 - a) { rem -= B - 1 - a; ++a; }
-    const int c = a + 1 + rem;
-    double p = 0.0;
-    for (int t = lane; t < m; t += 32) p = fma(x(a, t), x(c, t), p);
-    p = warp_sum(p);
-    if (lane == 0) G[a * B + c] = p;
+// Scalars shared by the phases of a panel factorization.
+struct PanelShared {
+  double p[B], c[B], cs[B], tau[B], scl, G[B * B], T[B * B];
+};
+
+// Householder factorization of eight vectors x_0 .. x_7 of length m in shared
+// memory (x_i at X + i ld): reflector j annihilates x_j beyond entry j and is
+// applied to the later ones.  Per reflector one dot phase (a warp takes one
+// dot over the whole vectors: x_j . x_i over the entries beyond j, j's square
+// among them, with x_j not yet scaled), the scalars in one warp, one update
+// phase.  out(i, j, x) receives the final entry j <= i of x_i; on return X holds
+// the reflectors (unit entry at j, zeros before it).  Bound by the FP64 pipe
+// (a warp-wide FP64 instruction holds it 16 cycles), so the layout counts
+// those: whole-vector dots share one five-step reduction, and the reflector's
+// root and reciprocal are formed once.
+template <class Out>
+__device__ __forceinline__ void panel_factor(double* X, int ld, int m, PanelShared& sh, Out out) {
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nt = blockDim.x;
+  for (int j = 0; j < B; ++j) {
+    const double* xj = X + (size_t)j * ld;
+    if (warp < B - j) {
+      const double* xi = xj + (size_t)warp * ld;
+      double p = 0.0;
+      for (int r = j + 1 + lane; r < m; r += 32) p = fma(xj[r], xi[r], p);
+      p = warp_sum(p);
+      if (lane == 0) sh.p[j + warp] = p;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      double beta, tau, scl;
+      reflector(xj[j], sh.p[j], beta, tau, scl);
+      if (lane > j && lane < B) {
+        const double xl = X[(size_t)lane * ld + j];
+        const double c = tau * fma(scl, sh.p[lane], xl);
+        sh.cs[lane] = c * scl;
+        out(lane, j, xl - c);                        // final: no later reflector touches entry j
+      }
+      if (lane == 0) { sh.tau[j] = tau; sh.scl = scl; out(j, j, beta); }
+      __syncwarp();
+      if (lane >= j && lane < B) X[(size_t)lane * ld + j] = lane == j ? 1.0 : 0.0;
+    }
+    __syncthreads();
+    const double scl = sh.scl;
+    double cs[B];
+#pragma unroll
+    for (int i = 1; i < B; ++i) cs[i] = i > j ? sh.cs[i] : 0.0;
+    for (int r = j + 1 + t; r < m; r += nt) {
+      const double x = xj[r];
+#pragma unroll
+      for (int i = 1; i < B; ++i)
+        if (i > j) X[(size_t)i * ld + r] = fma(-cs[i], x, X[(size_t)i * ld + r]);
+      X[(size_t)j * ld + r] = x * scl;
+    }
+    __syncthreads();
   }
-  __syncthreads();
+}
+
+// Up to four dots a . x_c, c = c0 .. c0 + nd - 1, over m entries by one warp,
+// reduced together; out[0 .. nd-1].
+__device__ __forceinline__ void warp_dots4(const double* a, const double* X, int ld, int c0, int nd, int m, double* out) {
+  const int lane = threadIdx.x & 31;
+  const double* x = X + (size_t)c0 * ld;
+  double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0;
+  for (int r = lane; r < m; r += 32) {
+    const double ar = a[r];
+    p0 = fma(ar, x[r], p0);
+    if (nd > 1) p1 = fma(ar, x[ld + r], p1);
+    if (nd > 2) p2 = fma(ar, x[2 * ld + r], p2);
+    if (nd > 3) p3 = fma(ar, x[3 * ld + r], p3);
+  }
+  const double v = reduce4(p0, p1, p2, p3, lane);
+  if ((lane & 7) == 0 && (lane >> 3) < nd) out[lane >> 3] = v;
 }
 
 // T of Q = H_0 ... H_{b-1} = I - Y T Y^T (forward, columnwise, as LAPACK's
-// dlarft) from the Gram values G[a][c] = y_a . y_c (a < c) and the taus; by
-// one thread.
-__device__ void form_t(const double* G, const double* tau, double* T) {
-  for (int j = 0; j < B; ++j) {
-    for (int i = 0; i < B; ++i) T[i * B + j] = 0.0;
-    T[j * B + j] = tau[j];
-    for (int i = 0; i < j; ++i) {
+// dlarft) for the reflectors X of panel_factor: the 28 products y_a . y_c in
+// groups of up to four that share y_a, then the recurrence by one warp, lane i
+// holding row i of T.
+__device__ __forceinline__ void panel_t(const double* X, int ld, int m, PanelShared& sh) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  // the groups (a, first c): 0:1 0:5 1:2 1:6 2:3 2:7 3:4 4:5 5:6 6:7
+  for (int g = warp; g < 10; g += nw) {
+    const int a = g < 6 ? g >> 1 : g - 3, c0 = a + 1 + (g < 6 ? (g & 1) * 4 : 0);
+    warp_dots4(X + (size_t)a * ld, X, ld, c0, min(4, B - c0), m, sh.G + a * B + c0);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    double row[B];
+#pragma unroll
+    for (int j = 0; j < B; ++j) {
       double s = 0.0;
-      for (int l = i; l < j; ++l) s = fma(T[i * B + l], G[l * B + j], s);
-      T[i * B + j] = -tau[j] * s;
+#pragma unroll
+      for (int l = 0; l < j; ++l) s = fma(row[l], sh.G[l * B + j], s);   // row[l] = 0 for l < i
+      row[j] = lane == j ? sh.tau[j] : (lane < j ? -sh.tau[j] * s : 0.0);
+      if (lane < B) sh.T[lane * B + j] = row[j];
     }
   }
+  __syncthreads();
 }
 
-// Householder reflector (dlarfg) of a vector with first entry alpha and
-// squared norm sq of the rest: H = I - tau v v^T, v_0 = 1, v_i = x_i scl,
-// H x = beta e_1.
-__device__ __forceinline__ void reflector(double alpha, double sq, double& beta, double& tau, double& scl) {
-  if (sq == 0.0) { beta = alpha; tau = 0.0; scl = 0.0; return; }
-  beta = -copysign(sqrt(fma(alpha, alpha, sq)), alpha);
-  tau = (beta - alpha) / beta;
-  scl = 1.0 / (alpha - beta);
+// Exponent e with |x| < 2^e (kZeroExp for 0), from the bits of x: no FP64 instruction.
+__device__ __forceinline__ int exp_of(double x) {
+  const int hi = __double2hiint(x) & 0x7fffffff, be = hi >> 20;
+  return be ? be - 1022 : ((hi | __double2loint(x)) ? -1022 : kZeroExp);
 }
 }  // namespace
 
@@ -318,61 +379,29 @@ __global__ void __launch_bounds__(256) k_band_init(BandArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// Panel k, QR of the column panel A[k:n][k:k+b] (m = n - k rows, one thread
-// per row, the panel in shared memory column by column).  Writes R into the
-// band, V (unit lower trapezoidal) and T into the scratch.
+// Panel k, QR of the column panel A[k:n][k:k+b] (m = n - k rows, the panel in
+// shared memory column by column).  Writes R into the band, V (unit lower
+// trapezoidal) and T into the scratch.
 __global__ void __launch_bounds__(256) k_band_qr(BandArgs a, int k) {
-  __shared__ double P[B][256];
-  __shared__ double red[64], s_tau[B], s_sc[3];
+  extern __shared__ double P[];                      // [b][m]
+  __shared__ PanelShared sh;
   const int s = blockIdx.x, n = a.n, m = n - k, t = threadIdx.x;
   const long long* A = (const long long*)a.Wk + (size_t)s * n * n;
   const double unit = p2(a.eA[s] - kFixBits);
   Work w = work_of(a.work + (size_t)s * work_stride(n), n);
-  if (t < m) {
+  for (int r = t; r < m; r += blockDim.x) {
 #pragma unroll
-    for (int j = 0; j < B; ++j) P[j][t] = (double)A[(size_t)(k + t) * n + k + j] * unit;
-  } else if (t < 256) {
-#pragma unroll
-    for (int j = 0; j < B; ++j) P[j][t] = 0.0;
+    for (int j = 0; j < B; ++j) P[j * m + r] = (double)A[(size_t)(k + r) * n + k + j] * unit;
   }
   __syncthreads();
-  double v[B];
-  for (int j = 0; j < B; ++j) {
-    // squared norm of column j below row j, and alpha = P[j][j]
-    block_dots(1, m, [&](int, int r) { return r > j ? P[j][r] : 0.0; },
-               [&](int, int r) { return P[j][r]; }, red);
-    // the reflector's scalars once (sqrt and divisions cost tens of FP64
-    // instructions), read by every thread
-    if (t == 0) reflector(P[j][j], red[0], s_sc[0], s_sc[1], s_sc[2]);
-    __syncthreads();
-    const double beta = s_sc[0], tau = s_sc[1], scl = s_sc[2];
-    const double vt = t == j ? 1.0 : ((t > j && t < m) ? P[j][t] * scl : 0.0);
-    v[j] = vt;
-    // R[t][j] (t < j) is final: column j is not touched by later reflectors
-    if (t < j) a.band[((size_t)s * n + k + t) * (B + 1) + (j - t)] = P[j][t];
-    if (t == j) a.band[((size_t)s * n + k + j) * (B + 1)] = beta;
-    __syncthreads();                                   // every thread read P[j][*] before it changes
-    P[j][t] = vt;                                      // column j now holds v
-    __syncthreads();
-    // w_c = sum_r v_r P[c][r] for c > j
-    block_dots(B - 1 - j, m, [&](int d, int r) { return P[j][r]; },
-               [&](int d, int r) { return P[j + 1 + d][r]; }, red);
-    if (t >= j && t < m) {
-      for (int c = j + 1; c < B; ++c) P[c][t] = fma(-tau * red[c - j - 1], vt, P[c][t]);
-    }
-    if (t == 0) s_tau[j] = tau;
-    __syncthreads();
-  }
-  if (t < m) {
+  double* band = a.band + ((size_t)s * n + k) * (B + 1);
+  panel_factor(P, m, m, sh, [&](int c, int j, double x) { band[j * (B + 1) + (c - j)] = x; });
+  for (int r = t; r < m; r += blockDim.x) {
 #pragma unroll
-    for (int j = 0; j < B; ++j) w.V[(size_t)t * 8 + j] = v[j];
+    for (int j = 0; j < B; ++j) w.V[(size_t)r * 8 + j] = P[j * m + r];
   }
-  // Gram of the reflectors for T, then T
-  __syncthreads();
-  for (int j = 0; j < B; ++j) P[j][t] = (t < m) ? v[j] : 0.0;
-  __syncthreads();
-  gram_upper(m, [&](int i, int r) { return P[i][r]; }, red);
-  if (t == 0) form_t(red, s_tau, w.T);
+  panel_t(P, m, m, sh);
+  if (t < 64) w.T[t] = sh.T[t];
 }
 
 // ---------------------------------------------------------------------------
@@ -543,27 +572,29 @@ __global__ void __launch_bounds__(256, 2) k_band_gemm_w(BandArgs a, int k) {
 }
 
 // ---------------------------------------------------------------------------
-// Panel k, row panel: Z = T^T W, RP = A[k:k+b][k+b:] - V[0:b] Z, LQ of RP (one
-// thread per column), T_U, Z U^T, the column exponents of [Z ; U].  U and T_U
-// go into the working matrix (rows k..k+b-1), L into the band.
-__global__ void __launch_bounds__(256) k_band_lq(BandArgs a, int k) {
-  __shared__ double R[B][256];
-  __shared__ double red[64], s_tau[B], Ts[64], Vt[64], s_sc[3];
-  const int s = blockIdx.x, n = a.n, t = threadIdx.x;
+// Panel k, row panel: Z = T^T W, RP = A[k:k+b][k+b:] - V[0:b] Z, LQ of RP, T_U,
+// Z U^T, the column exponents of [Z ; U].  U and T_U go into the working matrix
+// (rows k..k+b-1), L into the band.
+__global__ void __launch_bounds__(256, 4) k_band_lq(BandArgs a, int k) {
+  extern __shared__ double R[];                      // [b][mp] the row panel, then Z
+  __shared__ PanelShared sh;
+  __shared__ double Ts[64], Vt[64], zu[64];
+  const int s = blockIdx.x, n = a.n, t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int mp = n - k - B;                          // columns k+b .. n-1
+  double* Zs = R + (size_t)B * mp;
   long long* A = (long long*)a.Wk + (size_t)s * n * n;
   double* Ad = (double*)A;
-  const double unit = p2(a.eA[s] - kFixBits);
+  const int eA = a.eA[s];
+  const double unit = p2(eA - kFixBits);
   Work w = work_of(a.work + (size_t)s * work_stride(n), n);
   if (t < 64) { Ts[t] = w.T[t]; Vt[t] = w.V[t]; }    // T and the top b x b block of V
   __syncthreads();
-  const bool act = t < mp;
-  const int c = k + B + t;
-  double z[B], rp[B];
-  if (act) {
-    double wv[B];
+  for (int q = t; q < mp; q += blockDim.x) {
+    const int c = k + B + q;
+    asm volatile("" ::: "memory");                   // T and V stay in shared memory: in registers they would spill
+    double wv[B], z[B];
 #pragma unroll
-    for (int i = 0; i < B; ++i) wv[i] = w.Z[(size_t)i * n + t];
+    for (int i = 0; i < B; ++i) wv[i] = w.Z[(size_t)i * n + q];
 #pragma unroll
     for (int j = 0; j < B; ++j) {
       double acc = 0.0;
@@ -577,68 +608,35 @@ __global__ void __launch_bounds__(256) k_band_lq(BandArgs a, int k) {
       double acc = fma((double)A[(size_t)(k + i) * n + c], unit, -z[i]);
 #pragma unroll
       for (int j = 0; j < i; ++j) acc = fma(-Vt[i * B + j], z[j], acc);
-      rp[i] = acc;
+      R[i * mp + q] = acc;
+      Zs[i * mp + q] = z[i];
+      w.Z[(size_t)i * n + q] = z[i];
     }
-#pragma unroll
-    for (int j = 0; j < B; ++j) w.Z[(size_t)j * n + t] = z[j];
-  } else {
-#pragma unroll
-    for (int j = 0; j < B; ++j) { z[j] = 0.0; rp[j] = 0.0; }
   }
-#pragma unroll
-  for (int i = 0; i < B; ++i) R[i][t] = rp[i];
   __syncthreads();
-  double u[B];
-  for (int j = 0; j < B; ++j) {
-    block_dots(1, mp, [&](int, int q) { return q > j ? R[j][q] : 0.0; },
-               [&](int, int q) { return R[j][q]; }, red);
-    if (t == 0) reflector(R[j][j], red[0], s_sc[0], s_sc[1], s_sc[2]);
-    __syncthreads();
-    const double beta = s_sc[0], tau = s_sc[1], scl = s_sc[2];
-    const double ut = t == j ? 1.0 : ((t > j && act) ? R[j][t] * scl : 0.0);
-    u[j] = ut;
-    // L[j][t] (t < j) is final: column t is not touched by later reflectors;
-    // L[j][j] = beta.  Row k+j, column k+b+t: band offset b + t - j
-    if (t < j) a.band[((size_t)s * n + k + j) * (B + 1) + (B + t - j)] = R[j][t];
-    if (t == j) a.band[((size_t)s * n + k + j) * (B + 1) + B] = beta;
-    __syncthreads();
-    R[j][t] = ut;                                    // row j now holds u
-    __syncthreads();
-    block_dots(B - 1 - j, mp, [&](int d, int q) { return R[j][q]; },
-               [&](int d, int q) { return R[j + 1 + d][q]; }, red);
-    if (t >= j && act) {
-      for (int i = j + 1; i < B; ++i) R[i][t] = fma(-tau * red[i - j - 1], ut, R[i][t]);
-    }
-    if (t == 0) s_tau[j] = tau;
-    __syncthreads();
+  double* band = a.band + ((size_t)s * n + k) * (B + 1) + B;
+  panel_factor(R, mp, mp, sh, [&](int i, int j, double x) { band[i * (B + 1) + (j - i)] = x; });
+  // Z U^T: warp i takes z_i against u_0..3 and u_4..7
+  for (int g = warp; g < 2 * B; g += blockDim.x >> 5)
+    warp_dots4(Zs + (size_t)(g >> 1) * mp, R, mp, (g & 1) * 4, 4, mp, zu + (g >> 1) * B + (g & 1) * 4);
+  panel_t(R, mp, mp, sh);                            // T_U (its barriers cover zu)
+  if (t < 64) {
+    w.ZU[t] = zu[t];
+    Ad[(size_t)(k + t / B) * n + k + (t % B)] = sh.T[t];
   }
-  // rows of U (u[j] for this column) and the Gram for T_U
-#pragma unroll
-  for (int j = 0; j < B; ++j) R[j][t] = act ? u[j] : 0.0;
-  __syncthreads();
-  gram_upper(mp, [&](int i, int q) { return R[i][q]; }, red);
-  if (t == 0) form_t(red, s_tau, Ts);                // T_U (Ts no longer needed as T)
-  __syncthreads();
-  // Z U^T (64 dots), z in smem for the reductions
-  __shared__ double Zs[B][256];
-#pragma unroll
-  for (int j = 0; j < B; ++j) Zs[j][t] = z[j];
-  __syncthreads();
-  block_dots(B * B, mp, [&](int d, int q) { return Zs[d / B][q]; }, [&](int d, int q) { return R[d % B][q]; }, red);
-  if (t < 64) w.ZU[t] = red[t];
-  // U rows and T_U into the working matrix; the exponent of [Z ; U] per column
-  if (act) {
-    // exponent of the update's right operand column [Z 2^-eA ; U]
-    const double dn = p2(-a.eA[s]);
-    double mx = 0.0;
+  // U rows into the working matrix; the exponent of the update's right operand
+  // column [Z 2^-eA ; U]
+  for (int q = t; q < mp; q += blockDim.x) {
+    int e = kZeroExp;
 #pragma unroll
     for (int j = 0; j < B; ++j) {
-      Ad[(size_t)(k + j) * n + c] = u[j];
-      mx = fmax(mx, fmax(fabs(z[j]) * dn, fabs(u[j])));
+      const double u = R[j * mp + q], z = Zs[j * mp + q];
+      Ad[(size_t)(k + j) * n + k + B + q] = u;
+      const int ez = exp_of(z);
+      e = max(e, max(exp_of(u), ez == kZeroExp ? kZeroExp : ez - eA));
     }
-    w.er[t] = exp_above(mx);
+    w.er[q] = e;
   }
-  if (t < 64) Ad[(size_t)(k + t / B) * n + k + (t % B)] = Ts[t];
 }
 
 // ---------------------------------------------------------------------------
@@ -692,7 +690,8 @@ __global__ void __launch_bounds__(256, 2) k_band_gemm_x(BandArgs a, int k) {
     long long hi[8], lo[8];
     prod_read<8>(tmem + ((uint32_t)(warp * 32) << 16), hi, lo);
     if (r < n) {
-      const double sc = p2(a.eA[s] - kFixBits - 5);
+      const int eA = a.eA[s];
+      const double sc = p2(eA - kFixBits - 5);
       double vr[B], xv[B], y[B];
 #pragma unroll
       for (int i = 0; i < B; ++i) vr[i] = w.V[(size_t)(r - k) * 8 + i];
@@ -705,20 +704,20 @@ __global__ void __launch_bounds__(256, 2) k_band_gemm_x(BandArgs a, int k) {
       }
       // exponent of the update's left operand row [V 2^eA | Y] (both parts of
       // the order of |A|; the right operand carries Z 2^-eA)
-      const double up = p2(a.eA[s]);
-      double mx = 0.0;
+      int e = kZeroExp;
 #pragma unroll
       for (int j = 0; j < B; ++j) {
         double acc = 0.0;
 #pragma unroll
         for (int i = 0; i <= j; ++i) acc = fma(xv[i], TUs[i * B + j], acc);
         y[j] = acc;
-        mx = fmax(mx, fmax(fabs(acc), fabs(vr[j]) * up));
+        const int ev = exp_of(vr[j]);
+        e = max(e, max(exp_of(acc), ev == kZeroExp ? kZeroExp : ev + eA));
       }
       const int ro = r - k - B;
 #pragma unroll
       for (int j = 0; j < B; ++j) w.Y[(size_t)ro * 8 + j] = y[j];
-      w.el[ro] = exp_above(mx);
+      w.el[ro] = e;
     }
   }
   prod_end(ps, tmem, ok, a.err);
@@ -1193,14 +1192,14 @@ cudaError_t launch_band_reduce(const BandArgs& a, bool chase, cudaStream_t st) {
   k_band_init<<<S, 256, 0, st>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   for (int k = 0; k < n; k += B) {
-    k_band_qr<<<S, 256, 0, st>>>(a, k);
+    k_band_qr<<<S, 256, (size_t)B * (n - k) * sizeof(double), st>>>(a, k);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (k + B >= n) break;
     const int mp = n - k - B;
     const int tiles = (mp + kTileM - 1) / kTileM;
     k_band_gemm_w<<<dim3(S, tiles), 256, kProdSmem, st>>>(a, k);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_band_lq<<<S, 256, 0, st>>>(a, k);
+    k_band_lq<<<S, 256, (size_t)2 * B * mp * sizeof(double), st>>>(a, k);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_band_gemm_x<<<dim3(S, tiles), 256, kProdSmem, st>>>(a, k);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
