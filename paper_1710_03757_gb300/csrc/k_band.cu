@@ -220,11 +220,11 @@ __device__ __forceinline__ double warp_sum(double v) {
 // H x = beta e_1.  |alpha - beta| = |alpha| + |x| (no cancellation).
 __device__ __forceinline__ void reflector(double alpha, double sq, double& beta, double& tau, double& scl) {
   if (sq == 0.0) { beta = alpha; tau = 0.0; scl = 0.0; return; }
-  const double t = fma(alpha, alpha, sq), rn = rsqrt(t), nrm = t * rn;
+  const double t = fma(alpha, alpha, sq), rn = inv_sqrt(t), nrm = t * rn;
   beta = -copysign(nrm, alpha);
   const double d = alpha - beta;
   tau = fabs(d) * rn;
-  scl = 1.0 / d;
+  scl = inv(d);
 }
 
 // Scalars shared by the phases of a panel factorization.
@@ -237,7 +237,9 @@ struct PanelShared {
 // applied to the later ones.  Per reflector one dot phase (a warp takes one
 // dot over the whole vectors: x_j . x_i over the entries beyond j, j's square
 // among them, with x_j not yet scaled), the scalars in one warp, one update
-// phase.  out(i, j, x) receives the final entry j <= i of x_i; on return X holds
+// phase (three barriers a reflector; six, a dot phase for the norm alone and
+// the T recurrence in one thread before: QR 6.2 -> 4.6 ms and LQ 10.0 -> 6.8 for
+// 1920 matrices of n = 256).  out(i, j, x) receives the final entry j <= i of x_i; on return X holds
 // the reflectors (unit entry at j, zeros before it).  Bound by the FP64 pipe
 // (a warp-wide FP64 instruction holds it 16 cycles), so the layout counts
 // those: whole-vector dots share one five-step reduction, and the reflector's
@@ -917,29 +919,33 @@ __global__ void __launch_bounds__(256, 2) k_band_update(BandArgs a, int k) {
 }
 
 // ---------------------------------------------------------------------------
-// Stage 2: bulge chasing, two matrices per warp (a half-warp each: every FP64
-// instruction serves both, the reflector's formation included); each band and
-// its bulges in shared memory, entry (r, c) at W[r * kWin + (c - r + 7)]
+// Stage 2: bulge chasing, several matrices per warp (LPM lanes each: every FP64
+// instruction serves all of them, the reflector's formation included); each
+// band and its bulges in shared memory, entry (r, c) at W[r * kWin + (c - r + 7)]
 // (c - r in -7..15).  Per step a right reflector of length L <= b clears a row
-// beyond its superdiagonal over rows row .. row+15 (lane = row), then a left
-// reflector clears the bulge below the diagonal over columns c0 .. c0+15
-// (lane = column).
-__device__ __forceinline__ void chase_reflector(double x, int l16, int L, int hb, double& v, double& tau,
-                                                double& beta) {
-  double p = (l16 >= 1 && l16 < L) ? x * x : 0.0;
+// beyond its superdiagonal over rows row .. row+15 (one or two rows per lane),
+// then a left reflector clears the bulge below the diagonal over columns c0 ..
+// c0+15.
+//
+// Bound by the FP64 pipe: forming a reflector costs about as many warp
+// instructions (18: the norm's reduction, a reciprocal square root, a
+// reciprocal) as applying it with 16 lanes per matrix (17), so eight lanes per
+// matrix, four matrices per warp, take 26 instead of 35 instructions per
+// matrix and step.  Both forms do the same arithmetic in the same order.
+__device__ __forceinline__ void chase_reflector(double x, int l, int L, int hb, double& v, double& tau, double& beta) {
+  double p = (l >= 1 && l < L) ? x * x : 0.0;
   p += __shfl_xor_sync(0xffffffffu, p, 1);
   p += __shfl_xor_sync(0xffffffffu, p, 2);
   p += __shfl_xor_sync(0xffffffffu, p, 4);
   const double sq = __shfl_sync(0xffffffffu, p, hb), alpha = __shfl_sync(0xffffffffu, x, hb);
-  if (sq == 0.0) { v = l16 == 0 ? 1.0 : 0.0; tau = 0.0; beta = alpha; return; }
+  if (sq == 0.0) { v = l == 0 ? 1.0 : 0.0; tau = 0.0; beta = alpha; return; }
   // |beta| = sqrt(alpha^2 + sq); d = alpha - beta (no cancellation);
   // tau = (beta - alpha) / beta = |d| / |beta|, v = x / d
-  const double rn = rsqrt(fma(alpha, alpha, sq));
-  const double nrm = fma(alpha, alpha, sq) * rn;
+  const double t = fma(alpha, alpha, sq), rn = inv_sqrt(t), nrm = t * rn;
   beta = -copysign(nrm, alpha);
   const double d = alpha - beta;
   tau = fabs(d) * rn;
-  v = l16 == 0 ? 1.0 : (l16 < L ? x * (1.0 / d) : 0.0);
+  v = l == 0 ? 1.0 : (l < L ? x * inv(d) : 0.0);
 }
 
 // Steps of sweep i of the chase on an n x n band (right reflectors it stores).
@@ -954,24 +960,28 @@ __host__ __device__ __forceinline__ int sweep_steps(int i, int n) {
 // of its steps), which keeps the regions of concurrent steps apart (a step of
 // sweep i touches rows [c0-8, c0+8) and columns [c0, c0+16) with
 // c0 = i + 1 + 8t).  Progress words in shared memory, a ring of kRing slots
-// holding i * 64 + steps done; waits are bounded (error word on expiry).
+// holding i * 256 + steps done; waits are bounded (error word on expiry).
 constexpr int kChaseWarps = 8, kRing = 16, kLag = 3;
 
-__global__ void __launch_bounds__(kChaseWarps * 32) k_band_chase(BandArgs a, int nref) {
+// mats: matrices per CTA (at most 32 / LPM; fewer where shared memory holds fewer).
+template <int LPM>
+__global__ void __launch_bounds__(kChaseWarps * 32) k_band_chase(BandArgs a, int nref, int mats) {
+  constexpr int RPL = 16 / LPM;                       // rows (or columns) of a 16-block per lane
   extern __shared__ double Bw[];
   __shared__ int prog[kRing];
   __shared__ int s_fail;
   const int n = a.n, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int l16 = lane & 15, half = lane >> 4, hb = lane & 16;
-  const int s = 2 * blockIdx.x + half;
-  const bool live = s < a.S;                          // an odd batch leaves the last half idle
-  double* W = Bw + (size_t)half * n * kWin;
-  for (int i = threadIdx.x; i < 2 * n * kWin; i += blockDim.x) Bw[i] = 0.0;
+  const int l = lane & (LPM - 1), q4 = lane / LPM, hb = lane & ~(LPM - 1);
+  const int s = mats * blockIdx.x + q4;
+  const bool live = q4 < mats && s < a.S;             // lanes of absent matrices touch nothing
+  const int nn = live ? n : 0;
+  double* W = Bw + (size_t)(live ? q4 : 0) * n * kWin;
+  for (int i = threadIdx.x; i < mats * n * kWin; i += blockDim.x) Bw[i] = 0.0;
   if (threadIdx.x < kRing) prog[threadIdx.x] = -1;
   if (threadIdx.x == 0) s_fail = 0;
   __syncthreads();
-  for (int hh = 0; hh < 2; ++hh) {
-    const int sm = 2 * blockIdx.x + hh;
+  for (int hh = 0; hh < mats; ++hh) {
+    const int sm = mats * blockIdx.x + hh;
     if (sm >= a.S) break;
     const double* band = a.band + (size_t)sm * n * (B + 1);
     double* Wm = Bw + (size_t)hh * n * kWin;
@@ -990,7 +1000,7 @@ __global__ void __launch_bounds__(kChaseWarps * 32) k_band_chase(BandArgs a, int
   bool fail = false;
   for (int i = warp; i + 1 < n && !fail; i += kChaseWarps) {
     const int T = sweep_steps(i, n), Tp = i > 0 ? sweep_steps(i - 1, n) : 0;
-    if (lane == 0) vprog[i % kRing] = i * 64;
+    if (lane == 0) vprog[i % kRing] = i * 256;
     int c0 = i + 1, c1 = min(i + B, n - 1), row = i;
     for (int t = 0; t < T; ++t) {
       if (i > 0) {                                    // wait for sweep i-1 to be kLag steps ahead
@@ -999,7 +1009,7 @@ __global__ void __launch_bounds__(kChaseWarps * 32) k_band_chase(BandArgs a, int
           uint32_t it = 0;
           for (;; ++it) {
             const int v = vprog[(i - 1) % kRing];
-            if ((v >> 6) > i - 1 || ((v >> 6) == i - 1 && (v & 63) >= need)) break;
+            if ((v >> 8) > i - 1 || ((v >> 8) == i - 1 && (v & 255) >= need)) break;
             if (it > tcptx::kSpinLimit || *(volatile int*)&s_fail) { atomicOr(&s_fail, 1); break; }
             __nanosleep(20);
           }
@@ -1008,55 +1018,61 @@ __global__ void __launch_bounds__(kChaseWarps * 32) k_band_chase(BandArgs a, int
         __syncwarp();
         if (*(volatile int*)&s_fail) { fail = true; break; }
       }
-      const int L = c1 - c0 + 1;
+      const int L = c1 - c0 + 1, Ll = live ? L : 0;
       const int idx = base + t;
-      double v, tau, beta, vv[B];
+      double v, tau, beta, vv[B], x[RPL][B];
       // right reflector: clear row `row` at columns c0+1 .. c1; rows row .. row+15
-      chase_reflector(l16 < L ? AT(row, c0 + l16) : 0.0, l16, L, hb, v, tau, beta);
-      if (live && l16 < B) refl[(size_t)idx * B + l16] = l16 == 0 ? tau : v;
+      chase_reflector(l < Ll ? AT(row, c0 + l) : 0.0, l, L, hb, v, tau, beta);
+      if (live && l < B) refl[(size_t)idx * B + l] = l == 0 ? tau : v;
 #pragma unroll
       for (int q = 0; q < B; ++q) vv[q] = __shfl_sync(0xffffffffu, v, hb + q);
-      {
-        const int r = row + l16;
+#pragma unroll
+      for (int h = 0; h < RPL; ++h) {
+        const int r = row + l + LPM * h;
         double acc = 0.0;
 #pragma unroll
         for (int q = 0; q < B; ++q) {
           const int cc = c0 + q;
-          if (r < n && cc <= c1 && cc - r >= -7) acc = fma(AT(r, cc), vv[q], acc);
+          x[h][q] = (r < nn && cc <= c1 && cc - r >= -7) ? AT(r, cc) : 0.0;
+          acc = fma(x[h][q], vv[q], acc);
         }
-        acc *= tau;
-        __syncwarp();
+        acc *= -tau;
 #pragma unroll
         for (int q = 0; q < B; ++q) {
           const int cc = c0 + q;
-          if (r < n && cc <= c1 && cc - r >= -7) AT(r, cc) = fma(-acc, vv[q], AT(r, cc));
+          const double y = fma(acc, vv[q], x[h][q]);
+          if (r < nn && cc <= c1 && cc - r >= -7) AT(r, cc) = y;
         }
-        __syncwarp();
-        if (l16 < L) AT(row, c0 + l16) = l16 == 0 ? beta : 0.0;
-        __syncwarp();
       }
+      __syncwarp();
+      if (l < Ll) AT(row, c0 + l) = l == 0 ? beta : 0.0;
+      __syncwarp();
       // left reflector: clear column c0 at rows c0+1 .. c1; columns c0 .. c0+15
-      chase_reflector(l16 < L ? AT(c0 + l16, c0) : 0.0, l16, L, hb, v, tau, beta);
+      chase_reflector(l < Ll ? AT(c0 + l, c0) : 0.0, l, L, hb, v, tau, beta);
 #pragma unroll
       for (int q = 0; q < B; ++q) vv[q] = __shfl_sync(0xffffffffu, v, hb + q);
-      {
-        const int cc = c0 + l16;
+#pragma unroll
+      for (int h = 0; h < RPL; ++h) {
+        const int cc = c0 + l + LPM * h;
         double acc = 0.0;
 #pragma unroll
-        for (int q = 0; q < B; ++q)
-          if (cc < n && q < L) acc = fma(AT(c0 + q, cc), vv[q], acc);
-        acc *= tau;
-        __syncwarp();
+        for (int q = 0; q < B; ++q) {
+          x[h][q] = (cc < nn && q < L) ? AT(c0 + q, cc) : 0.0;
+          acc = fma(x[h][q], vv[q], acc);
+        }
+        acc *= -tau;
 #pragma unroll
-        for (int q = 0; q < B; ++q)
-          if (cc < n && q < L) AT(c0 + q, cc) = fma(-acc, vv[q], AT(c0 + q, cc));
-        __syncwarp();
-        if (l16 < L) AT(c0 + l16, c0) = l16 == 0 ? beta : 0.0;
-        __syncwarp();
+        for (int q = 0; q < B; ++q) {
+          const double y = fma(acc, vv[q], x[h][q]);
+          if (cc < nn && q < L) AT(c0 + q, cc) = y;
+        }
       }
+      __syncwarp();
+      if (l < Ll) AT(c0 + l, c0) = l == 0 ? beta : 0.0;
+      __syncwarp();
       if (lane == 0) {                                // publish: step t of sweep i done
         __threadfence_block();
-        vprog[i % kRing] = i * 64 + t + 1;
+        vprog[i % kRing] = i * 256 + t + 1;
       }
       row = c0;
       c0 += B;
@@ -1071,7 +1087,7 @@ __global__ void __launch_bounds__(kChaseWarps * 32) k_band_chase(BandArgs a, int
   }
   if (live && warp == 0) {
     double* bd = a.bd + (size_t)s * 3 * n;
-    for (int r = l16; r < n; r += 16) {
+    for (int r = l; r < n; r += LPM) {
       bd[r] = AT(r, r);
       bd[n + r] = r + 1 < n ? AT(r, r + 1) : 0.0;
       bd[2 * n + r] = 0.0;
@@ -1209,14 +1225,26 @@ cudaError_t launch_band_reduce(const BandArgs& a, bool chase, cudaStream_t st) {
   return chase ? launch_band_chase(a, st) : cudaSuccess;
 }
 
+template <int LPM>
+static cudaError_t launch_chase(const BandArgs& a, int mats, cudaStream_t st) {
+  static std::atomic<uint64_t> at{0};
+  cudaError_t e = raise_smem_limit(k_band_chase<LPM>, 227 * 1024, at);
+  if (e != cudaSuccess) return e;
+  k_band_chase<LPM><<<(a.S + mats - 1) / mats, kChaseWarps * 32, (size_t)mats * a.n * kWin * sizeof(double), st>>>(
+      a, band_nref(a.n), mats);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_band_chase(const BandArgs& a, cudaStream_t st) {
   if (a.S <= 0) return cudaSuccess;
   if (!band_supported(a.n)) return cudaErrorInvalidValue;
-  static std::atomic<uint64_t> at{0};
-  cudaError_t e = raise_smem_limit(k_band_chase, (int)(2 * 256 * kWin * sizeof(double)), at);
-  if (e != cudaSuccess) return e;
-  k_band_chase<<<(a.S + 1) / 2, kChaseWarps * 32, 2 * a.n * kWin * sizeof(double), st>>>(a, band_nref(a.n));
-  return cudaGetLastError();
+  // four matrices per CTA (of n <= 288: 4 x 48 KB) once two per SM do not hold
+  // the batch: 1920 of n = 256 23.8 -> 19.6 ms; below that two, whose shorter
+  // step is the shorter chain (304: 3.6 ms in 152 CTAs, 4.9 in 76)
+  constexpr size_t kCap = 226 * 1024;
+  const size_t per = (size_t)a.n * kWin * sizeof(double);
+  if (a.S > 2 * 152 && 4 * per <= kCap) return launch_chase<8>(a, 4, st);
+  return launch_chase<16>(a, 2 * per <= kCap ? 2 : 1, st);
 }
 
 cudaError_t launch_band_backtr(const BandVecArgs& va, cudaStream_t st) {

@@ -316,11 +316,11 @@ struct BdReflector {
 __device__ __forceinline__ BdReflector bd_reflector(double alpha, double sq) {
   BdReflector h{alpha, 0.0, 0.0};
   if (sq > 0.0) {
-    const double t = fma(alpha, alpha, sq), rn = rsqrt(t), nrm = t * rn;
+    const double t = fma(alpha, alpha, sq), rn = inv_sqrt(t), nrm = t * rn;
     h.beta = -copysign(nrm, alpha);
     const double d = alpha - h.beta;
     h.tau = fabs(d) * rn;
-    h.scl = 1.0 / d;
+    h.scl = inv(d);
   }
   return h;
 }
@@ -829,8 +829,8 @@ __device__ void block_cgs2(At at, int p0, int c, int len, double* s_dot, double*
 // 3. Inverse iteration, one CTA of one or two warps per matrix (persistent
 //    over matrices), thread a for the a-th kept index.  Scratch per CTA slot,
 //    interleaved by thread with stride ls (16, 32 or 64): DG, DU, DU2 (the LU
-//    factors of T - s I with partial pivoting, in the layout of LAPACK's dgtsv)
-//    and X (the iterate), each 2n entries.  The factorization streams the
+//    factors of T - s I with partial pivoting, in the layout of LAPACK's dgtsv,
+//    the pivots as reciprocals) and X (the iterate), each 2n entries.  The factorization streams the
 //    current row in registers and applies L^-1 P^T to the right-hand side as
 //    it goes; the scale of the previous iterate is folded into the next
 //    right-hand side.
@@ -904,25 +904,23 @@ __global__ void __launch_bounds__(64) k_bd_invit(BdVecArgs a, int ls) {
             const double dun = (i + 1 < m - 1) ? odb[c + 1] : 0.0;
             const double xn = xnb[c] * rs;
             if (fabs(dg) >= fabs(dli)) {
-              const double g = (dg == 0.0) ? kEps : dg;
-              const double f = dli / g;
+              const double g = inv((dg == 0.0) ? kEps : dg);
+              const double f = dli * g;
               DG(i) = g; DU(i) = du; DU2(i) = 0.0; XB(i) = xi;
               dg = -sgm - f * du;
               du = dun;
               xi = xn - f * xi;
             } else {
-              const double f = dg / dli;
-              DG(i) = dli; DU(i) = -sgm; DU2(i) = dun; XB(i) = xn;
+              const double g = inv(dli), f = dg * g;
+              DG(i) = g; DU(i) = -sgm; DU2(i) = dun; XB(i) = xn;
               dg = du + f * sgm;
               du = -f * dun;
               xi = xi - f * xn;
             }
           }
         }
-        const double glast = (dg == 0.0) ? kEps : dg;
-        DG(m - 1) = glast;
         // back substitution U x = y, carrying x_{i+1}, x_{i+2}, in blocks of kCh
-        double x1 = xi / glast;
+        double x1 = xi * inv((dg == 0.0) ? kEps : dg);
         XB(m - 1) = x1;
         double s2 = x1 * x1;
         double x2 = 0.0;
@@ -940,7 +938,7 @@ __global__ void __launch_bounds__(64) k_bd_invit(BdVecArgs a, int ls) {
           for (int c = 0; c < kCh; ++c) {
             const int i = top - c;
             if (i < 0) break;
-            double x = (yb[c] - ub[c] * x1 - u2b[c] * x2) / gb[c];
+            double x = (yb[c] - ub[c] * x1 - u2b[c] * x2) * gb[c];
             if (exp_field(x) > 1023 + 600) {         // growth through tiny pivots: rescale x[i..]
               for (int q = i + 1; q < m; ++q) XB(q) *= 0x1.0p-600;
               x *= 0x1.0p-600; x1 *= 0x1.0p-600; x2 *= 0x1.0p-600; s2 *= 0x1.0p-1200;
