@@ -34,6 +34,28 @@ static __device__ __forceinline__ double group_sum(double v, int G) {
   return v;
 }
 
+// Whether rows of squared norms al, be and product g are to be rotated, |g| >
+// tol sqrt(al be), and the tangent t and cosine of the rotation that makes them
+// orthogonal: with h = be - al and q = 2 g, t = sign(h) q / (|h| + sqrt(h^2 +
+// q^2)) (Rutishauser's formula multiplied through by |q|).  Products leave the
+// exponent range only for rows of extreme scale, which take the ratio form.
+__device__ __forceinline__ bool rotate_pair(double al, double be, double g, double tol) {
+  const double ab = al * be;
+  if (mid_range(ab)) return g * g > tol * tol * ab;
+  return al > 0.0 && be > 0.0 && fabs(g) > tol * sqrt(al) * sqrt(be);
+}
+__device__ __forceinline__ void rotation(double al, double be, double g, double& t, double& cs) {
+  const double h = be - al, q = 2.0 * g, s2 = fma(h, h, q * q);
+  if (mid_range(s2)) {
+    t = copysign(1.0, h) * q * inv(fabs(h) + s2 * inv_sqrt(s2));
+  } else {
+    const double zeta = h / q;
+    if (fabs(zeta) > 1e150) t = 0.5 / zeta;
+    else t = copysign(1.0, zeta) / (fabs(zeta) + sqrt(fma(zeta, zeta, 1.0)));
+  }
+  cs = inv_sqrt(fma(t, t, 1.0));
+}
+
 __global__ void k_jacobi(JacobiArgs a, int use_smem, int G) {
   extern __shared__ double smem[];
   const double nu = a.noise_u > 0.0 ? a.noise_u : 0x1.0p-52;
@@ -66,18 +88,22 @@ __global__ void k_jacobi(JacobiArgs a, int use_smem, int G) {
       if (r < np && gl == 0) nrm[r] = s;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {                   // np <= 32: lane r holds row r
+      const int r = threadIdx.x;
+      const double v = r < np ? nrm[r] : 0.0;
+      double thr2 = s_thr2;
       if (sweep == 0) {                       // |M|_F^2 is invariant under the rotations
-        double f = 0.0;
-        for (int r = 0; r < np; ++r) f += nrm[r];
-        s_thr2 = f * (0.25 * nu * nu);
+        thr2 = group_sum(v, 32) * (0.25 * nu * nu);
+        if (r == 0) s_thr2 = thr2;
       }
-      int na = 0;
-      for (int r = 0; r < np; ++r)
-        if (nrm[r] > s_thr2) act[na++] = r;
-      if (na & 1) act[na] = -1;
-      s_na = na;
-      s_rot = 0;
+      const unsigned m = __ballot_sync(0xffffffffu, v > thr2);
+      const int na = __popc(m);
+      if (v > thr2) act[__popc(m & ((1u << r) - 1u))] = r;
+      if (r == 0) {
+        if (na & 1) act[na] = -1;
+        s_na = na;
+        s_rot = 0;
+      }
     }
     __syncthreads();
     const int na = s_na, nap = na + (na & 1), npairs = nap >> 1;
@@ -99,14 +125,11 @@ __global__ void k_jacobi(JacobiArgs a, int use_smem, int G) {
           for (int c = gl; c < n; c += G) g = fma(ap[c], aq[c], g);
         g = group_sum(g, G);                       // every lane of the warp takes part
         const double al = act_pair ? nrm[P] : 0.0, be = act_pair ? nrm[Q] : 0.0;
-        const bool rot = act_pair && al > 0.0 && be > 0.0 && fabs(g) > tol * sqrt(al) * sqrt(be);
+        const bool rot = act_pair && rotate_pair(al, be, g, tol);
         double nal = al, nbe = be;
         if (rot) {                                 // uniform within the lane group
-          const double zeta = (be - al) / (2.0 * g);
-          double t;
-          if (fabs(zeta) > 1e150) t = 0.5 / zeta;
-          else t = copysign(1.0, zeta) / (fabs(zeta) + sqrt(fma(zeta, zeta, 1.0)));
-          const double cs = 1.0 / sqrt(fma(t, t, 1.0));
+          double t, cs;
+          rotation(al, be, g, t, cs);
           const double sn = cs * t;
           for (int c = gl; c < n; c += G) {
             const double x = ap[c], y = aq[c];
@@ -119,13 +142,15 @@ __global__ void k_jacobi(JacobiArgs a, int use_smem, int G) {
         }
         // heavy cancellation in the norm update: recompute from the rotated rows
         const bool fixP = rot && nal < 0.01 * al, fixQ = rot && nbe < 0.01 * be;
-        double sp = 0.0, sq = 0.0;
-        if (fixP) for (int c = gl; c < n; c += G) sp = fma(ap[c], ap[c], sp);
-        if (fixQ) for (int c = gl; c < n; c += G) sq = fma(aq[c], aq[c], sq);
-        sp = group_sum(sp, G);
-        sq = group_sum(sq, G);
-        if (fixP) nal = sp;
-        if (fixQ) nbe = sq;
+        if (__any_sync(0xffffffffu, fixP || fixQ)) {
+          double sp = 0.0, sq = 0.0;
+          if (fixP) for (int c = gl; c < n; c += G) sp = fma(ap[c], ap[c], sp);
+          if (fixQ) for (int c = gl; c < n; c += G) sq = fma(aq[c], aq[c], sq);
+          sp = group_sum(sp, G);
+          sq = group_sum(sq, G);
+          if (fixP) nal = sp;
+          if (fixQ) nbe = sq;
+        }
         if (rot && gl == 0) { nrm[P] = nal; nrm[Q] = nbe; }
       }
       if (myrot && gl == 0) atomicAdd(&s_rot, myrot);
@@ -417,15 +442,12 @@ __global__ void __launch_bounds__(512) k_jacobi_warp(JacobiArgs a, int use_smem)
           al = nrm[P]; be = nrm[Q];
           const double dp = dsc[P], dq = dsc[Q];
           const double gam = dp * dq * gs;
-          rot = al > 0.0 && be > 0.0 && fabs(gam) > tol * sqrt(al) * sqrt(be);
+          rot = rotate_pair(al, be, gam, tol);
           if (rot) {
-            const double zeta = (be - al) / (2.0 * gam);
             double t;
-            if (fabs(zeta) > 1e150) t = 0.5 / zeta;
-            else t = copysign(1.0, zeta) / (fabs(zeta) + sqrt(fma(zeta, zeta, 1.0)));
-            cs = 1.0 / sqrt(fma(t, t, 1.0));
-            mu1 = t * (dq / dp);
-            mu2 = t * (dp / dq);
+            rotation(al, be, gam, t, cs);
+            mu1 = t * (dq * inv(dp));
+            mu2 = t * (dp * inv(dq));
             nal = fma(-t, gam, al);
             nbe = fma(t, gam, be);
           }
@@ -574,8 +596,6 @@ cudaError_t launch_jacobi(const JacobiArgs& a, cudaStream_t st) {
   }
 
   // n <= 32: lane groups of G < 32 lanes per pair
-
-  if (a.S <= 0) return cudaSuccess;
   const int n = a.n, np = a.n_pad;
   const size_t rows_bytes = (size_t)np * n * sizeof(double);
   const size_t nrm_bytes = (size_t)np * sizeof(double) + (size_t)(np + 2) * sizeof(int);
@@ -586,8 +606,9 @@ cudaError_t launch_jacobi(const JacobiArgs& a, cudaStream_t st) {
   int G = 2;
   while (G < 32 && G < n) G <<= 1;
   if (G > 2 && G >= n) G >>= 1;                 // about two elements per lane
-  int threads = n <= 16 ? 32 : (n <= 64 ? 256 : 512);
-  if (threads < G) threads = G;
+  // one lane group per pair of a step: a second pass of the groups would double
+  // the chain of a step (n = 16: 64 matrices JAC16A -> JAC16B us, 4096 JAC16C -> JAC16D ms)
+  const int threads = std::max(32, (np / 2 * G + 31) / 32 * 32);
   static std::atomic<uint64_t> attr{0};
   cudaError_t e = raise_smem_limit(k_jacobi, 200 * 1024 + 64, attr);
   if (e != cudaSuccess) return e;
