@@ -128,14 +128,14 @@ typedef struct {
  *           (8/3) n^3 + O(n^2) flops whatever the rank.
  *   AUTO    where the matrices can have full rank (n >= 64 and the
  *           plaquette's inner dimension d^2 >= n / 2): BAND's two-stage route
- *           for n a multiple of 8 from 200 to 256, BIDIAG for the other n;
+ *           for n a multiple of 8 from 200 to 1024, BIDIAG for the other n;
  *           JACOBI elsewhere; a
  *           level with d^2 < n (the first one that trajectories split on
  *           their own) through the d^2 x d^2 core of the QR factors of the
  *           plaquette's two operands, whose singular values are the nonzero
  *           ones of its matrices, by the same rule at side d^2.
  *   BAND    AUTO's choice, with the two-stage route where n is a multiple of
- *           8 from 64 to 256: the reduction's (8/3) n^3 flops as exact integer products of 8-bit digit slices on the
+ *           8 from 64 to 1024: the reduction's (8/3) n^3 flops as exact integer products of 8-bit digit slices on the
  *           tensor cores, O(n^2) FP64 work per matrix beside them
  *           (mctrg_svd_band_batched).  As an option not taken by
  *           mctrg_batch_run (EINVAL; AUTO chooses the route there too).

@@ -21,7 +21,7 @@
 //     memory, one FP32 accumulator per digit group g = i + j (Ozaki, Ogita,
 //     Oishi and Rump 2012; sums of up to 256 products of 8-bit digits are
 //     integers below 2^24 for the leading groups, so FP32 holds them
-//     exactly).  The update is applied in integer arithmetic, so apart from
+//     exactly; longer sums are read out and added in integers every 256).  The update is applied in integer arithmetic, so apart from
 //     the panel factorizations stage 1 issues no FP64 instruction per
 //     trailing element.
 //  2. band -> bidiagonal by bulge chasing (k_band_chase, one warp per matrix,
@@ -336,15 +336,12 @@ __device__ __forceinline__ int exp_of(double x) {
 }
 }  // namespace
 
-bool band_supported(int n) { return n >= 64 && n <= 256 && n % B == 0; }
+bool band_supported(int n) { return n >= 64 && n <= kBandMaxN && n % B == 0; }
 
+// sum over the sweeps i of ceil((n - 2 - i) / b)
 int band_nref(int n) {
-  int c = 0;
-  for (int i = 0; i + 1 < n; ++i) {
-    int c0 = i + 1, c1 = std::min(i + B, n - 1);
-    while (c1 > c0) { ++c; c0 += B; c1 = std::min(c1 + B, n - 1); }
-  }
-  return c;
+  const int m = n - 2, q = m / B, r = m % B;
+  return B * q * (q + 1) / 2 + r * (q + 1);
 }
 
 size_t band_work_doubles(int n) { return work_stride(n); }
@@ -448,15 +445,16 @@ __device__ __forceinline__ uint32_t prod_begin(ProdShared& ps, uint8_t* Bs, uint
   return ps.tmem_slot;
 }
 
-// The stage loop: split(st, dst) writes stage st of A (and fetches the next
-// one's data), refl(r, j) is the FP64 value of reflector j at K index r.
-// Returns false when a wait expired.
+// Stages s0 .. s1-1 of the product (at most 16, so that the sums over K stay
+// exact): split(st, dst) writes stage st of A (and fetches the next one's
+// data), refl(r, j) is the FP64 value of reflector j at K index r.  Returns
+// false when a wait expired.
 template <class Split, class Refl>
-__device__ __forceinline__ bool prod_stages(ProdShared& ps, uint32_t tmem, uint8_t* As, uint8_t* Bs, int klen,
-                                            Split split, Refl refl) {
-  const int t = threadIdx.x, nst = (klen + 15) >> 4;
-  int committed = 0;
-  for (int st = 0; st < nst; ++st) {
+__device__ __forceinline__ bool prod_stages(ProdShared& ps, uint32_t tmem, uint8_t* As, uint8_t* Bs, int klen, int s0,
+                                            int s1, Split split, Refl refl) {
+  const int t = threadIdx.x;
+  int committed = s0;
+  for (int st = s0; st < s1; ++st) {
     const int buf = st & 1;
     // the MMAs of stage st - 2 (and all before them) are done with this buffer
     if (st >= 2 && !mbar_wait(&ps.bar[buf], ((st >> 1) - 1) & 1)) atomicOr(&ps.fail, 1);
@@ -476,13 +474,13 @@ __device__ __forceinline__ bool prod_stages(ProdShared& ps, uint32_t tmem, uint8
     if (ps.fail) break;
     if (t == 0) {
       tc_fence_after();
-      issue_products(tmem, As + (size_t)buf * kStageBytes, Bb, st & 3, st == 0);
+      issue_products(tmem, As + (size_t)buf * kStageBytes, Bb, st & 3, st == s0);
       umma_commit(&ps.bar[buf]);
     }
     ++committed;
   }
   const int last = committed - 1;
-  if (last >= 0 && !mbar_wait(&ps.bar[last & 1], (last >> 1) & 1)) atomicOr(&ps.fail, 1);
+  if (last >= s0 && !mbar_wait(&ps.bar[last & 1], (last >> 1) & 1)) atomicOr(&ps.fail, 1);
   tc_fence_after();
   __syncthreads();
   return ps.fail == 0;
@@ -499,7 +497,7 @@ __device__ __forceinline__ void prod_end(ProdShared& ps, uint32_t tmem, bool ok,
   if (threadIdx.x < 32) tmem_free(tmem, 128);
 }
 
-// Columns 0 .. NJ-1 from `col` of this thread's row: the group sums g back as
+// Columns 0 .. NJ-1 from `col` of this thread's row: the group sums g, added to
 // hi 2^32 + lo.
 template <int NJ>
 __device__ __forceinline__ void prod_read(uint32_t taddr, long long (&hi)[NJ], long long (&lo)[NJ]) {
@@ -512,14 +510,34 @@ __device__ __forceinline__ void prod_read(uint32_t taddr, long long (&hi)[NJ], l
   tmem_wait_ld();
 #pragma unroll
   for (int j = 0; j < NJ; ++j) {
-    hi[j] = __float2int_rn(__uint_as_float(v[0][j]));
-    lo[j] = __float2int_rn(__uint_as_float(v[4][j]));
+    long long h = __float2int_rn(__uint_as_float(v[0][j])), l = __float2int_rn(__uint_as_float(v[4][j]));
 #pragma unroll
     for (int g = 1; g < 4; ++g) {
-      hi[j] = (hi[j] << 8) + __float2int_rn(__uint_as_float(v[g][j]));
-      lo[j] = (lo[j] << 8) + __float2int_rn(__uint_as_float(v[4 + g][j]));
+      h = (h << 8) + __float2int_rn(__uint_as_float(v[g][j]));
+      l = (l << 8) + __float2int_rn(__uint_as_float(v[4 + g][j]));
+    }
+    hi[j] += h;
+    lo[j] += l;
+  }
+}
+
+// The whole product over K = klen: the accumulators hold the sums of at most
+// 256 products (exact in FP32 for the leading groups) and are read out and
+// added in integers after every 16 stages.  read() adds them up.
+template <class Split, class Refl, class Read>
+__device__ __forceinline__ bool prod_all(ProdShared& ps, uint32_t tmem, uint8_t* As, uint8_t* Bs, int klen, Split split,
+                                         Refl refl, Read read) {
+  const int nst = (klen + 15) >> 4;
+  for (int s0 = 0; s0 < nst; s0 += 16) {
+    if (!prod_stages(ps, tmem, As, Bs, klen, s0, min(s0 + 16, nst), split, refl)) return false;
+    read();
+    if (s0 + 16 < nst) {                             // before the next stages overwrite the accumulators
+      tc_fence_before();
+      __syncthreads();
+      tc_fence_after();
     }
   }
+  return true;
 }
 constexpr size_t kProdSmem = 2 * kStageBytes + 2 * kBBytes + 1024;
 }  // namespace
@@ -548,7 +566,10 @@ __global__ void __launch_bounds__(256, 2) k_band_gemm_w(BandArgs a, int k) {
     for (int e = 0; e < 8; ++e) x[e] = in ? p[(size_t)e * n] : 0ll;
   };
   load(0);
-  const bool ok = prod_stages(
+  // row c of W^T: value = (hi 2^32 + lo) 2^(eA - 67); the two warp groups take four columns each
+  const int jh = kh * 4;
+  long long hi[4] = {}, lo[4] = {};
+  const bool ok = prod_all(
       ps, tmem, As, Bs, m,
       [&](int st, uint8_t* dst) {
         uint4 d[kSl];
@@ -557,12 +578,9 @@ __global__ void __launch_bounds__(256, 2) k_band_gemm_w(BandArgs a, int k) {
         for (int sl = 0; sl < kSl; ++sl) *(uint4*)(dst + a_piece(sl, rho, kh)) = d[sl];
         load(st + 1);                                // past the end: zeros
       },
-      [&](int r, int j) { return w.V[(size_t)r * 8 + j]; });
+      [&](int r, int j) { return w.V[(size_t)r * 8 + j]; },
+      [&]() { prod_read<4>(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)jh, hi, lo); });
   if (ok) {
-    // row c of W^T: value = (hi 2^32 + lo) 2^(eA - 67); the two warp groups take four columns each
-    const int jh = kh * 4;
-    long long hi[4], lo[4];
-    prod_read<4>(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)jh, hi, lo);
     if (c < n) {
       const double sc = p2(a.eA[s] - kFixBits - 5);
 #pragma unroll
@@ -674,7 +692,8 @@ __global__ void __launch_bounds__(256, 2) k_band_gemm_x(BandArgs a, int k) {
     }
   };
   load(0);
-  const bool ok = prod_stages(
+  long long hi[8] = {}, lo[8] = {};                  // (warps 0 .. 3)
+  const bool ok = prod_all(
       ps, tmem, As, Bs, mp,
       [&](int st, uint8_t* dst) {
 #pragma unroll
@@ -686,11 +705,10 @@ __global__ void __launch_bounds__(256, 2) k_band_gemm_x(BandArgs a, int k) {
         }
         load(st + 1);
       },
-      [&](int r, int j) { return Ad[(size_t)(k + j) * n + k + B + r]; });
+      [&](int r, int j) { return Ad[(size_t)(k + j) * n + k + B + r]; },
+      [&]() { if (warp < 4) prod_read<8>(tmem + ((uint32_t)(warp * 32) << 16), hi, lo); });
   if (ok && warp < 4) {
     const int r = r0 + t;
-    long long hi[8], lo[8];
-    prod_read<8>(tmem + ((uint32_t)(warp * 32) << 16), hi, lo);
     if (r < n) {
       const int eA = a.eA[s];
       const double sc = p2(eA - kFixBits - 5);
@@ -726,8 +744,8 @@ __global__ void __launch_bounds__(256, 2) k_band_gemm_x(BandArgs a, int k) {
 }
 
 // ---------------------------------------------------------------------------
-// Trailing update A[k+b:][k+b:] -= [V | Y] [Z ; U] for one 128-row tile, its
-// 16-column tiles in turn: K = 2b = 16 (one k-step), applied in fixed point.
+// Trailing update A[k+b:][k+b:] -= [V | Y] [Z ; U] for one 128-row tile and up
+// to 256 columns (grid z), the 16-column tiles in turn: K = 2b = 16 (one k-step), applied in fixed point.
 // The operands are [V 2^eA | Y] and [Z 2^-eA ; U] (the same product): V and U
 // are of order 1, Y and Z of order |A|.  The row operand shares one exponent
 // over the tile's rows, the column operand one over each block of 64 columns
@@ -756,7 +774,8 @@ __global__ void __launch_bounds__(256, 2) k_band_update(BandArgs a, int k) {
   uint8_t* Bs = As + kStageBytes;                    // blocks of 64 columns: 128 rows x 128 bytes
   const int s = blockIdx.x, n = a.n, t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int r0 = k + B + blockIdx.y * kTileM;       // first row of the tile
-  const int mp = n - k - B;
+  const int z0 = blockIdx.z * 256;                   // first trailing column of this CTA's (at most 256)
+  const int mp = min(256, n - k - B - z0);
   long long* A = (long long*)a.Wk + (size_t)s * n * n;
   const double* Ad = (const double*)A;
   Work w = work_of(a.work + (size_t)s * work_stride(n), n);
@@ -772,7 +791,7 @@ __global__ void __launch_bounds__(256, 2) k_band_update(BandArgs a, int k) {
   __syncthreads();
   {
     // the largest row exponent of the tile and the column exponents of the blocks
-    int e = (t < 128 && r0 + t < n) ? w.el[r0 + t - k - B] : kZeroExp, f = t < mp ? w.er[t] : kZeroExp;
+    int e = (t < 128 && r0 + t < n) ? w.el[r0 + t - k - B] : kZeroExp, f = t < mp ? w.er[z0 + t] : kZeroExp;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
@@ -809,8 +828,8 @@ __global__ void __launch_bounds__(256, 2) k_band_update(BandArgs a, int k) {
 #pragma unroll
     for (int e = 0; e < 8; ++e)
       x[e] = !in ? 0ll
-                 : part == 0 ? fix_of(w.Z[(size_t)e * n + c], kFloatP - er - eA)
-                             : fix_of(Ad[(size_t)(k + e) * n + k + B + c], kFloatP - er);
+                 : part == 0 ? fix_of(w.Z[(size_t)e * n + z0 + c], kFloatP - er - eA)
+                             : fix_of(Ad[(size_t)(k + e) * n + k + B + z0 + c], kFloatP - er);
     uint4 d[kSl];
     digits8(x, d);
     uint8_t* Bb = Bs + (size_t)(c >> 6) * kBBytes;
@@ -832,7 +851,7 @@ __global__ void __launch_bounds__(256, 2) k_band_update(BandArgs a, int k) {
   const int rw = (warp & 3) * 32 + (warp >> 2) * 16 + (lane >> 2), cl = 2 * (lane & 3);
   const uint32_t tlane = (uint32_t)((warp & 3) * 32 + (warp >> 2) * 16) << 16;
   const int ra = r0 + rw, rb = ra + 8;
-  long long* pa = A + (size_t)ra * n + k + B + cl;
+  long long* pa = A + (size_t)ra * n + k + B + z0 + cl;
   long long* pb = pa + (size_t)8 * n;
   const bool oka = ra < n && el != kZeroExp, okb = rb < n && el != kZeroExp;
   longlong2 nx[4];                                   // the next tile's elements: (row a, row b) x (columns, columns + 8)
@@ -1199,10 +1218,12 @@ constexpr size_t kUpdSmem = kStageBytes + 4 * kBBytes + 1024;
 cudaError_t launch_band_reduce(const BandArgs& a, bool chase, cudaStream_t st) {
   if (a.S <= 0) return cudaSuccess;
   if (!band_supported(a.n)) return cudaErrorInvalidValue;
-  static std::atomic<uint64_t> at_w{0}, at_x{0}, at_u{0};
+  static std::atomic<uint64_t> at_w{0}, at_x{0}, at_u{0}, at_q{0}, at_l{0};
   cudaError_t e = raise_smem_limit(k_band_gemm_w, (int)kProdSmem, at_w);
   if (e == cudaSuccess) e = raise_smem_limit(k_band_gemm_x, (int)kProdSmem, at_x);
   if (e == cudaSuccess) e = raise_smem_limit(k_band_update, (int)kUpdSmem, at_u);
+  if (e == cudaSuccess) e = raise_smem_limit(k_band_qr, (int)(B * kBandMaxN * sizeof(double)), at_q);
+  if (e == cudaSuccess) e = raise_smem_limit(k_band_lq, (int)(2 * B * kBandMaxN * sizeof(double)), at_l);
   if (e != cudaSuccess) return e;
   const int n = a.n, S = a.S;
   k_band_init<<<S, 256, 0, st>>>(a);
@@ -1219,7 +1240,7 @@ cudaError_t launch_band_reduce(const BandArgs& a, bool chase, cudaStream_t st) {
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_band_gemm_x<<<dim3(S, tiles), 256, kProdSmem, st>>>(a, k);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_band_update<<<dim3(S, tiles), 256, kUpdSmem, st>>>(a, k);
+    k_band_update<<<dim3(S, tiles, (mp + 255) / 256), 256, kUpdSmem, st>>>(a, k);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return chase ? launch_band_chase(a, st) : cudaSuccess;
@@ -1253,7 +1274,7 @@ cudaError_t launch_band_backtr(const BandVecArgs& va, cudaStream_t st) {
   static std::atomic<uint64_t> at{0};
   auto bytes = [](int n) { return (size_t)(24 * n + 16) * sizeof(double); };
   const size_t smem = bytes(a.n);
-  cudaError_t e = raise_smem_limit(k_band_backtr, (int)bytes(256), at);
+  cudaError_t e = raise_smem_limit(k_band_backtr, (int)bytes(kBandMaxN), at);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)a.S, (unsigned)((std::max(1, va.kmax) + 15) / 16));
   k_band_backtr<<<grid, kBtThreads, smem, st>>>(a, va, band_nref(a.n));

@@ -10,9 +10,9 @@ namespace mctrg {
 
 constexpr int kBandW = 8;   // band width b: stage-1 panels of b columns, b superdiagonals
 
-// Sides the band route takes: multiples of b from 64 to 256 (the inner
-// dimension of the tensor-core products stays <= 256, where their FP32 group
-// sums are exact).
+// Sides the band route takes: multiples of b from 64 to 1024 (the limit of the
+// chase's band and of the panels in shared memory).
+constexpr int kBandMaxN = 1024;
 bool band_supported(int n);
 
 // Right reflectors of the bulge chase of one n x n band.

@@ -319,7 +319,9 @@ bool route_bidiag(const mctrg_options& o, int n, int K) {
 // of n = 256 12.0 ms against 12.8, 256 of them 16.1 against 23.5, 1920 84
 // against 139; below, its panels' launches cost small batches more than large
 // ones gain: n = 144, 64 matrices 6.0 against 4.7, 256 7.0 against 7.8; n = 192,
-// one 8.2 against 7.4).  The choice looks at the side alone, so a trajectory's
+// one 8.2 against 7.4; above 256, whole L = 16 runs: chi = 20, one trajectory 48
+// ms against 77, 128 173 against 294; chi = 24, 8 trajectories 83 against 206;
+// chi = 32, one 175 against 930).  The choice looks at the side alone, so a trajectory's
 // result does not depend on the batch.  Both are as accurate: singular values
 // against a quadruple-precision Jacobi, rms error over s_1 at n = 64, 1.5e-16 on
 // a flat spectrum and 4e-17 over 14 decades (the one-stage route 1.4e-16 and

@@ -126,9 +126,13 @@ static void band_all(void* buf, int n, int64_t chunk, BandArgs& a) {
   a.err = (uint32_t*)(refl + (size_t)chunk * band_refl_doubles(n));
 }
 
+// The sides that the entry points below take (contexts use the route up to
+// kBandMaxN).
+static bool band_entry_side(int n) { return n <= 256 && band_supported(n); }
+
 extern "C" int mctrg_band_reduce_batched(const double* M, int n, int64_t batch, double* band, double* bd,
                                          void* stream) {
-  if (!M || !band || !band_supported(n) || batch < 1 || batch > (1 << 30)) return MCTRG_EINVAL;
+  if (!M || !band || !band_entry_side(n) || batch < 1 || batch > (1 << 30)) return MCTRG_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   size_t fr = 0, tot = 0;
   if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return MCTRG_ECUDA;
@@ -159,7 +163,7 @@ extern "C" int mctrg_band_reduce_batched(const double* M, int n, int64_t batch, 
 
 extern "C" int mctrg_svd_band_batched(const double* M, int n, int64_t batch, double* sigma, int n_vec,
                                       double* vt, void* stream) {
-  if (!M || !sigma || !band_supported(n) || batch < 1 || batch > (1 << 30)) return MCTRG_EINVAL;
+  if (!M || !sigma || !band_entry_side(n) || batch < 1 || batch > (1 << 30)) return MCTRG_EINVAL;
   if (n_vec < 0 || n_vec > 16 || n_vec > n || (n_vec > 0 && !vt)) return MCTRG_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   const int np = n + (n & 1);

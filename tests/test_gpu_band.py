@@ -193,3 +193,23 @@ def test_band_route_at_L1024(torch):
 def test_batch_rejects_the_band_route(torch):
     assert mctrg.mctrg_batch_run([(0.4, 0.0, 8, 4, 10, 1, 0)],
                                  mctrg.make_options(svd=mctrg.SVD_BAND))[0] == mctrg.MCTRG_EINVAL
+
+
+@pytest.mark.parametrize("chi,L,n", [(20, 16, 3), (24, 16, 3), (28, 16, 2), (32, 16, 2)])
+def test_sides_above_256_against_the_one_stage_route(torch, chi, L, n):
+    """Sides 400, 576, 784 and 1024 (several accumulations over K, column blocks of the update, one or two matrices
+    per chase CTA, groups of 16 kept vectors): the trajectories of AUTO, which takes the two-stage route there, and of
+    BIDIAG agree to 1e-10 (the per-trajectory bar; both are backward stable)."""
+    out = []
+    for svd in (mctrg.SVD_AUTO, mctrg.SVD_BIDIAG):
+        ctx = mctrg.mctrg_create(mctrg.make_options(svd=svd))
+        assert mctrg.mctrg_init_lattice(ctx, 0.42, 0.02, L, chi) == 0
+        ln, sg, fl = np.zeros(n), np.zeros(n, np.int8), np.zeros(n, np.uint8)
+        st, _ = mctrg.mctrg_run(ctx, n, 17, 0, ln, sg, fl)
+        mctrg.mctrg_destroy(ctx)
+        assert st in (mctrg.MCTRG_OK, mctrg.MCTRG_EDOMAIN)
+        out.append((ln, sg, fl))
+    (la, sa, fa), (lb, sb, fb) = out
+    ok = (fa == 0) & (fb == 0)
+    assert ok.any() and np.array_equal(fa, fb) and np.array_equal(sa[ok], sb[ok])
+    assert (np.abs(la - lb)[ok] <= 1e-10 * np.abs(lb[ok])).all()
