@@ -27,6 +27,9 @@ struct JacobiArgs {
   double zero_rel, noise_u;
 };
 cudaError_t launch_jacobi(const JacobiArgs& a, cudaStream_t st);
+// The same for a launch of a few matrices (the shared prefix): from n = 64 on,
+// eight SMs per matrix.  a.W holds the rows throughout.
+cudaError_t launch_jacobi_few(const JacobiArgs& a, cudaStream_t st);
 
 // ---- K3 + K4: stochastic truncation and split into halves -------------------
 // Per item (trajectory b, tensor t of one level): choose the kept singular

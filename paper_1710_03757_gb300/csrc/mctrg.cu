@@ -222,7 +222,7 @@ int mctrg_ctx::init_from_device_tensor(int D0, int L_, int chi_) {
     ja.perm = shPerm.as<int>(); ja.lns1 = shLns1.as<double>(); ja.nnz = shNnz.as<int>();
     ja.mflags = nullptr; ja.n = n; ja.n_pad = np; ja.S = 2; ja.max_sweeps = opt.max_sweeps;
     ja.zero_rel = opt.zero_tol_scale * (double)n * 0x1.0p-52;
-    CK(launch_jacobi(ja, st));
+    CK(launch_jacobi_few(ja, st));
     int hn[2];
     double hl[2];
     CK(cudaMemcpyAsync(hn, shNnz.p, sizeof(hn), cudaMemcpyDeviceToHost, st));

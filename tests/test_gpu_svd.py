@@ -65,3 +65,18 @@ def test_rejects_bad_sizes(torch):
     assert mctrg.lib().mctrg_svd_batched(M.data_ptr(), 0, 1, sig.data_ptr(), None, 0, None) == mctrg.MCTRG_EINVAL
     assert mctrg.lib().mctrg_svd_batched(M.data_ptr(), 2048, 1, sig.data_ptr(), None, 0, None) == mctrg.MCTRG_EINVAL
     assert mctrg.lib().mctrg_svd_batched(None, 4, 1, sig.data_ptr(), None, 0, None) == mctrg.MCTRG_EINVAL
+
+
+@pytest.mark.parametrize("D,L,chi,n", [(3, 4, 40, 12), (8, 2, 20, 40), (8, 4, 6, 20)])
+def test_shared_prefix_matrices_in_clusters(torch, D, L, chi, n):
+    """The shared level's SVD of a context (all vectors, eight CTAs per matrix from n = 64 on): an odd side with a
+    padded row (D = 3: an exact level 0, then n = 81) and the smallest side (D = 8: n = 64), per trajectory against
+    the oracle (tests/parity.py, 1e-10).  Sides of 256 with rank 16 and full rank: the chi = 16 parity tests."""
+    from oracle.trg import Problem, run_many
+    from paper_1710_03757_gb300.workloads import generic_tensor
+    from parity import compare
+    from test_gpu_parity import gpu_run
+    T0 = generic_tensor(D, seed=900 + D)
+    gpu = gpu_run(L, chi, n, 41, T0=T0)
+    orc = run_many(Problem(T0, L, chi), 41, 0, n, workers=4)
+    compare(gpu, orc, min_ok=0.8, label="cluster prefix D%d chi%d" % (D, chi))
