@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kThreads) k_sample_split(SampleArgs a) {
   double* vbuf = wn + np;                           // [KV][n]
   unsigned char* inset = (unsigned char*)(vbuf + (size_t)KV * n);   // [np]
   __shared__ int s_kept[kKeptMax];
-  __shared__ double s_sigt[kKeptMax];
+  __shared__ double s_sigt[kKeptMax], s_rootv[kKeptMax], s_rootr[kKeptMax], s_rootl[kKeptMax];
   __shared__ int s_nk;
   __shared__ uint32_t s_flags;
 
@@ -123,10 +123,15 @@ __global__ void __launch_bounds__(kThreads) k_sample_split(SampleArgs a) {
 
     if (sample) {
       const bool two = chi > 32;             // a second column per lane (32 + lane + 1)
+      // quotients of weights as products with reciprocals (a division issues some
+      // twenty FP64 instructions, and one per row was most of the recurrences'
+      // chains), unless the smallest weight's reciprocal could overflow
+      const bool tiny = w[nz - 1] < 0x1.0p-1000;
+      auto over = [&](double num, double den) { return tiny ? num / den : num * inv(den); };
       if (warp == 0) {                       // forward table E, lane l <-> columns l+1, l+33
         const int j = lane + 1, j2 = lane + 33;
-        const double wj = (j <= chi) ? w[j - 1] : 1.0;
-        const double wj2 = (j2 <= chi) ? w[j2 - 1] : 1.0;
+        const double wj = (j <= chi) ? w[j - 1] : 1.0, rj = inv(wj);
+        const double wj2 = (j2 <= chi) ? w[j2 - 1] : 1.0, rj2 = inv(wj2);
         double Ej = 0.0, Ej2 = 0.0;
         if (lane == 0) tabE[0] = 1.0;
         if (j <= chi) tabE[j] = 0.0;
@@ -140,10 +145,10 @@ __global__ void __launch_bounds__(kThreads) k_sample_split(SampleArgs a) {
             const double top = __shfl_sync(0xffffffffu, Ej, 31);
             double prev2 = __shfl_up_sync(0xffffffffu, Ej2, 1);
             if (lane == 0) prev2 = top;
-            Ej2 = Ej2 + (wi / wj2) * prev2;
+            Ej2 = fma(tiny ? wi / wj2 : wi * rj2, prev2, Ej2);
             if (j2 <= chi) row[j2] = Ej2;
           }
-          Ej = Ej + (wi / wj) * prev;
+          Ej = fma(tiny ? wi / wj : wi * rj, prev, Ej);
           if (lane == 0) row[0] = 1.0;
           if (j <= chi) row[j] = Ej;
         }
@@ -157,12 +162,14 @@ __global__ void __launch_bounds__(kThreads) k_sample_split(SampleArgs a) {
           double prev = __shfl_up_sync(0xffffffffu, Gb, 1);
           if (lane == 0) prev = 1.0;
           double* row = tabG + (size_t)i * chi;
+          const double ri = inv(w[i]);
+          auto ratio = [&](double num) { return tiny ? num / w[i] : num * ri; };
           if (two) {
             const double top = __shfl_sync(0xffffffffu, Gb, 31);
             double prev2 = __shfl_up_sync(0xffffffffu, Gb2, 1);
             if (lane == 0) prev2 = top;
             if (bb2 <= nz - i) {
-              const double first = (i + bb2 + 1 <= nz) ? Gb2 * (w[i + bb2] / w[i]) : 0.0;
+              const double first = (i + bb2 + 1 <= nz) ? Gb2 * ratio(w[i + bb2]) : 0.0;
               Gb2 = first + prev2;
             } else {
               Gb2 = 0.0;
@@ -170,7 +177,7 @@ __global__ void __launch_bounds__(kThreads) k_sample_split(SampleArgs a) {
             if (bb2 < chi) row[bb2] = Gb2;
           }
           if (bb <= nz - i) {
-            const double first = (i + bb + 1 <= nz) ? Gb * (w[i + bb] / w[i]) : 0.0;
+            const double first = (i + bb + 1 <= nz) ? Gb * ratio(w[i + bb]) : 0.0;
             Gb = first + prev;
           } else {
             Gb = 0.0;
@@ -209,11 +216,11 @@ __global__ void __launch_bounds__(kThreads) k_sample_split(SampleArgs a) {
           const int I = s_kept[pk] + 1;                         // 1-based
           const int alo = max(0, chi - 1 - (nz - I)), ahi = min(chi - 1, I - 1);
           double R = 1.0;
-          for (int q = 0; q < chi - ahi; ++q) R *= w[I - 1 + q] / w[ahi + q];
+          for (int q = 0; q < chi - ahi; ++q) R *= over(w[I - 1 + q], w[ahi + q]);
           double acc = 0.0;
           for (int aa = ahi; aa >= alo; --aa) {
             acc += tabE[(size_t)(I - 1) * (chi + 1) + aa] * tabG[(size_t)I * chi + (chi - 1 - aa)] * R;
-            if (aa > alo) R *= w[I + chi - aa - 1] / w[aa - 1];
+            if (aa > alo) R *= over(w[I + chi - aa - 1], w[aa - 1]);
           }
           const double r = acc / tabE[(size_t)nz * (chi + 1) + chi];
           s_sigt[pk] = wn[I - 1] / r;
@@ -269,13 +276,22 @@ __global__ void __launch_bounds__(kThreads) k_sample_split(SampleArgs a) {
     double* Hr = Hl + (size_t)n * kc;
     const double* Wm = a.W + (size_t)slot * np * n;
     const int* pm = a.perm + (size_t)slot * np;
+    // the kept values' factors once (a root and two divisions, some sixty FP64
+    // instructions, per entry of the halves cost as much as a fifth of M v)
+    if (tid < nk) {
+      const double root = sqrt(s_sigt[tid]), sr = sg[s_kept[tid]];
+      s_rootv[tid] = root;
+      s_rootr[tid] = root / sr;
+      s_rootl[tid] = root / sr / sr;
+    }
+    __syncthreads();
     for (int idx = tid; idx < kc * n; idx += kThreads) {
       const int al = idx / n, col = idx - al * n;
       double v = 0.0;
       if (al < nk) {
         const int r = s_kept[al];
         const double* brow = a.mode == 2 ? a.vrows + ((size_t)it * ks + al) * n : Wm + (size_t)pm[r] * n;
-        v = sqrt(s_sigt[al]) * brow[col] / sg[r];
+        v = s_rootr[al] * brow[col];
       }
       Hr[idx] = v;
     }
@@ -284,7 +300,7 @@ __global__ void __launch_bounds__(kThreads) k_sample_split(SampleArgs a) {
       for (int idx = tid; idx < n * kc; idx += kThreads) {
         const int row = idx / kc, al = idx - row * kc;
         double v = 0.0;
-        if (al < nk) v = sqrt(s_sigt[al]) * Ur[(size_t)s_kept[al] * n + row];
+        if (al < nk) v = s_rootv[al] * Ur[(size_t)s_kept[al] * n + row];
         Hl[idx] = v;
       }
     } else {
@@ -315,11 +331,7 @@ __global__ void __launch_bounds__(kThreads) k_sample_split(SampleArgs a) {
           }
           const double sum = warp_sum_k<KV>(acc, lane);
           const int q = lane / (32 / KV);
-          if (lane % (32 / KV) == 0 && q < nv) {
-            const int r = s_kept[a0 + q];
-            const double sr = sg[r];
-            Hl[(size_t)row * kc + a0 + q] = sqrt(s_sigt[a0 + q]) * sum / (sr * sr);
-          }
+          if (lane % (32 / KV) == 0 && q < nv) Hl[(size_t)row * kc + a0 + q] = s_rootl[a0 + q] * sum;
         }
       }
     }
