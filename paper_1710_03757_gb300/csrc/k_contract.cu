@@ -107,12 +107,18 @@ cudaError_t launch_form_xy(const XYArgs& a, cudaStream_t st) {
 }
 
 // ---- FP64 GEMM with the matricization epilogue -------------------------------
-// 64 x 64 output tile per CTA, K step 16, 256 threads with 4 x 4 outputs each.
+// A T x T output tile per CTA, T = 16 Q, K step 16, 256 threads with Q x Q
+// outputs each.  Bound by the FP64 pipe (1.24 of the measured 1.257 TFLOP/s on
+// full 64-tiles), so padding is what is left to save: T = 48 where 64 would
+// cover more than it (n = 144: 9 tiles of 48 instead of 9 of 64, 384
+// products 3.30 -> 1.87 ms, 1.23 TFLOP/s of algorithmic work).
 namespace {
-constexpr int TM = 64, TK = 16;
+constexpr int TK = 16;
 }
 
+template <int Q>
 __global__ void __launch_bounds__(256) k_gemm_f64(GemmArgs a) {
+  constexpr int TM = 16 * Q;
   __shared__ double sX[TK][TM + 1];
   __shared__ double sY[TK][TM + 1];
   const int D = a.D, n = D * D, K = a.K;
@@ -124,7 +130,7 @@ __global__ void __launch_bounds__(256) k_gemm_f64(GemmArgs a) {
   const double* Y = a.Yt + it * stride;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int r0 = tr * TM, c0 = tcol * TM;
-  double acc[4][4] = {};
+  double acc[Q][Q] = {};
   for (int k0 = a.upper ? max(r0, c0) : 0; k0 < K; k0 += TK) {
     for (int e = threadIdx.x; e < TM * TK; e += 256) {
       const int rr = e / TK, kk = e - rr * TK;
@@ -135,13 +141,13 @@ __global__ void __launch_bounds__(256) k_gemm_f64(GemmArgs a) {
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < TK; ++kk) {
-      double xr[4], yc[4];
+      double xr[Q], yc[Q];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) { xr[q] = sX[kk][ty + 16 * q]; yc[q] = sY[kk][tx + 16 * q]; }
+      for (int q = 0; q < Q; ++q) { xr[q] = sX[kk][ty + 16 * q]; yc[q] = sY[kk][tx + 16 * q]; }
 #pragma unroll
-      for (int p = 0; p < 4; ++p)
+      for (int p = 0; p < Q; ++p)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] = fma(xr[p], yc[q], acc[p][q]);
+        for (int q = 0; q < Q; ++q) acc[p][q] = fma(xr[p], yc[q], acc[p][q]);
     }
     __syncthreads();
   }
@@ -150,12 +156,12 @@ __global__ void __launch_bounds__(256) k_gemm_f64(GemmArgs a) {
   if (par < 0) par = tensor_parity(a.L, a.level_new, item % a.Nnew);
   double* Mo = a.M + (int64_t)it * n * n;
 #pragma unroll
-  for (int p = 0; p < 4; ++p) {
+  for (int p = 0; p < Q; ++p) {
     const int r = r0 + ty + 16 * p;
     if (r >= n) continue;
     const int al = r / D, be = r - al * D;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < Q; ++q) {
       const int cc = c0 + tx + 16 * q;
       if (cc >= n) continue;
       const int de = cc / D, ga = cc - de * D;
@@ -170,9 +176,18 @@ __global__ void __launch_bounds__(256) k_gemm_f64(GemmArgs a) {
 cudaError_t launch_gemm_f64(const GemmArgs& a, cudaStream_t st) {
   if (a.n_items <= 0) return cudaSuccess;
   const int n = a.D * a.D;
-  const int tiles = (n + TM - 1) / TM;
-  dim3 grid((unsigned)a.n_items, tiles * tiles);
-  k_gemm_f64<<<grid, 256, 0, st>>>(a);
+  // the tile that pads least (each product is summed in the same order whatever the tile, except that an upper
+  // triangular one starts at its tile's corner, where the skipped terms are zeros)
+  const int t64 = (n + 63) / 64, t48 = (n + 47) / 48, t32 = (n + 31) / 32;
+  const int64_t p64 = (int64_t)t64 * t64 * 64 * 64, p48 = (int64_t)t48 * t48 * 48 * 48, p32 = (int64_t)t32 * t32 * 32 * 32;
+  // smaller tiles read shared memory and the operands more often: they have to save a tenth and a quarter
+  if (10 * p32 < 7 * std::min(p48, p64)) {
+    k_gemm_f64<2><<<dim3((unsigned)a.n_items, t32 * t32), 256, 0, st>>>(a);
+  } else if (10 * p48 < 9 * p64) {
+    k_gemm_f64<3><<<dim3((unsigned)a.n_items, t48 * t48), 256, 0, st>>>(a);
+  } else {
+    k_gemm_f64<4><<<dim3((unsigned)a.n_items, t64 * t64), 256, 0, st>>>(a);
+  }
   return cudaGetLastError();
 }
 
