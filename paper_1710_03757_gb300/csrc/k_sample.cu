@@ -285,7 +285,9 @@ __global__ void __launch_bounds__(kThreads) k_sample_split(SampleArgs a) {
       s_rootl[tid] = root / sr / sr;
     }
     __syncthreads();
-    for (int idx = tid; idx < kc * n; idx += kThreads) {
+    // the halves of a few items are shared by the CTAs of grid y, rows and entries in turn (mode 2)
+    const int part = blockIdx.y, parts = gridDim.y;
+    for (int idx = part * kThreads + tid; idx < kc * n; idx += parts * kThreads) {
       const int al = idx / n, col = idx - al * n;
       double v = 0.0;
       if (al < nk) {
@@ -305,7 +307,7 @@ __global__ void __launch_bounds__(kThreads) k_sample_split(SampleArgs a) {
       }
     } else {
       const double* Mm = a.M + (size_t)slot * n * n;
-      for (int idx = tid; idx < n * kc; idx += kThreads) {
+      for (int idx = part * kThreads + tid; idx < n * kc; idx += parts * kThreads) {
         const int al = idx - (idx / kc) * kc;
         if (al >= nk) Hl[idx] = 0.0;
       }
@@ -318,7 +320,7 @@ __global__ void __launch_bounds__(kThreads) k_sample_split(SampleArgs a) {
                                   : Wm[(size_t)pm[s_kept[a0 + q]] * n + col];
         }
         __syncthreads();
-        for (int row = warp; row < n; row += kThreads / 32) {
+        for (int row = part * (kThreads / 32) + warp; row < n; row += parts * (kThreads / 32)) {
           double acc[KV];
 #pragma unroll
           for (int q = 0; q < KV; ++q) acc[q] = 0.0;
@@ -349,18 +351,21 @@ cudaError_t launch_sample_split(const SampleArgs& a, cudaStream_t st, int grid) 
     return (size_t)a.n_pad * 2 * sizeof(double) + (size_t)kv * a.n * sizeof(double) + (size_t)a.n_pad + 16;
   };
   if (grid > a.n_items) grid = (int)a.n_items;
+  // the second pass over fewer items than two per SM: several CTAs per item, each
+  // with at least 16 rows of M v (16 items of n = 576 6.65 -> 0.43 ms)
+  const int parts = a.mode == 2 ? (int)std::max<int64_t>(1, std::min<int64_t>(2 * 152 / a.n_items, a.n / 16)) : 1;
   constexpr size_t kSmemCap = 227 * 1024;
   if (smem_for(16) <= 160 * 1024) {
     static std::atomic<uint64_t> attr{0};
     cudaError_t e = raise_smem_limit(k_sample_split<16>, kSmemCap, attr);
     if (e != cudaSuccess) return e;
-    k_sample_split<16><<<grid, kThreads, smem_for(16), st>>>(a);
+    k_sample_split<16><<<dim3(grid, parts), kThreads, smem_for(16), st>>>(a);
   } else {
     if (smem_for(8) > kSmemCap) return cudaErrorInvalidValue;
     static std::atomic<uint64_t> attr{0};
     cudaError_t e = raise_smem_limit(k_sample_split<8>, kSmemCap, attr);
     if (e != cudaSuccess) return e;
-    k_sample_split<8><<<grid, kThreads, smem_for(8), st>>>(a);
+    k_sample_split<8><<<dim3(grid, parts), kThreads, smem_for(8), st>>>(a);
   }
   return cudaGetLastError();
 }
