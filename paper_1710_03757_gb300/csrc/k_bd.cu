@@ -570,6 +570,19 @@ __device__ __forceinline__ int sturm_eval_ff(const float2* __restrict__ oo, int 
   return neg - n;
 }
 
+// #{s_i > zr s_1} and ln s_1 of a spectrum, by a block.
+__device__ __forceinline__ void bd_rank(const double* sg, int n, double zr, int& s_nnz, int* nnz, double* lns1) {
+  const double s1 = sg[0], tau = zr * s1;
+  int c = 0;
+  for (int r = threadIdx.x; r < n; r += blockDim.x) c += sg[r] > tau;
+  if (c) atomicAdd(&s_nnz, c);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    *nnz = s1 > 0.0 ? s_nnz : 0;
+    if (lns1) *lns1 = s1 > 0.0 ? log(s1) : -INFINITY;
+  }
+}
+
 // Each thread finds the values of its ranks in three precisions, each
 // narrowing what the next verifies: the bracket from a coarse grid of FP32
 // counts (the lowest bin starting at the zero bound), narrowed by FP32
@@ -599,7 +612,8 @@ __global__ void __launch_bounds__(kBisThreads) k_bd_bisect(const double* bd, int
     zero_rel = t.zero_rel;
     mat = 0;
   }
-  const int nt = blockDim.x;
+  // the ranks are shared by the CTAs of grid y (each value is found by itself)
+  const int nt = blockDim.x, part = blockIdx.y, parts = gridDim.y;
   double* oo = sm;                                   // [2n]
   float2* oof = (float2*)(oo + 2 * n);               // [2n] oo as two FP32
   int* cnt = (int*)(oof + 2 * n);                    // [kBisGrid] FP32 grid counts
@@ -620,6 +634,7 @@ __global__ void __launch_bounds__(kBisThreads) k_bd_bisect(const double* bd, int
   const double G = block_max(g, red);
   const double omax = block_max(om, red);
   if (!(G > 0.0)) {                                  // the zero matrix
+    if (part > 0) return;
     for (int r = tid; r < n_pad; r += nt) { sg[r] = 0.0; perm[(size_t)mat * n_pad + r] = r; }
     if (tid == 0) { nnz[mat] = 0; if (lns1) lns1[mat] = -INFINITY; }
     return;
@@ -650,7 +665,7 @@ __global__ void __launch_bounds__(kBisThreads) k_bd_bisect(const double* bd, int
   const int zlo = s_zlo;
   const double tol = 0x1.0p-51;
   const double mff = (double)n * 0x1.0p-43;          // relative error allowed to a two-FP32 count
-  for (int r = tid; r < n; r += nt) {
+  for (int r = part * nt + tid; r < n; r += parts * nt) {
     const int j = n - 1 - r;                         // ascending index of the r-th largest
     if (j < zlo) { sg[r] = 0.0; continue; }          // below tlo: a zero
     // FP32: the grid bin, then bisection (geometric across decades) to a
@@ -767,20 +782,24 @@ __global__ void __launch_bounds__(kBisThreads) k_bd_bisect(const double* bd, int
     }
     sg[r] = G * (0.5 * (lo + hi));
   }
+  if (part > 0) return;
   for (int r = n + tid; r < n_pad; r += nt) sg[r] = 0.0;
   for (int r = tid; r < n_pad; r += nt) perm[(size_t)mat * n_pad + r] = r;
+  if (parts > 1) return;                             // k_bd_rank counts
   if (tid == 0) s_nnz = 0;
   __syncthreads();
-  const double s1 = sg[0];
-  const double tau = zr * s1;
-  int c = 0;
-  for (int r = tid; r < n; r += nt) c += sg[r] > tau;
-  if (c) atomicAdd(&s_nnz, c);
+  bd_rank(sg, n, zr, s_nnz, nnz + mat, lns1 ? lns1 + mat : nullptr);
+}
+
+// Nonzero count and ln s_1 of matrices whose ranks several CTAs have found.
+__global__ void __launch_bounds__(128) k_bd_rank(const double* sig, int n, int n_pad, int* nnz, double* lns1,
+                                                 double zero_rel) {
+  __shared__ int s_nnz;
+  const int mat = blockIdx.x;
+  if (threadIdx.x == 0) s_nnz = 0;
   __syncthreads();
-  if (tid == 0) {
-    nnz[mat] = s1 > 0.0 ? s_nnz : 0;
-    if (lns1) lns1[mat] = s1 > 0.0 ? log(s1) : -INFINITY;
-  }
+  bd_rank(sig + (size_t)mat * n_pad, n, zero_rel > 0.0 ? zero_rel : (double)n * kEps, s_nnz, nnz + mat,
+          lns1 ? lns1 + mat : nullptr);
 }
 
 // ---------------------------------------------------------------------------
@@ -796,6 +815,18 @@ __device__ void block_cgs2(At at, int p0, int c, int len, double* s_dot, double*
     if (t >= p0 && t < c) {
       double d0 = 0.0, d1 = 0.0, d2 = 0.0, d3 = 0.0;
       int i = 0;
+      for (; i + 16 <= len; i += 16) {                // sixteen pairs of loads in flight
+        double x[16], y[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) { x[q] = at(t, i + q); y[q] = at(c, i + q); }
+#pragma unroll
+        for (int q = 0; q < 16; q += 4) {
+          d0 = fma(x[q], y[q], d0);
+          d1 = fma(x[q + 1], y[q + 1], d1);
+          d2 = fma(x[q + 2], y[q + 2], d2);
+          d3 = fma(x[q + 3], y[q + 3], d3);
+        }
+      }
       for (; i + 4 <= len; i += 4) {
         d0 = fma(at(t, i), at(c, i), d0);
         d1 = fma(at(t, i + 1), at(c, i + 1), d1);
@@ -1133,7 +1164,14 @@ cudaError_t launch_bd_bisect(const double* bd, int n, int n_pad, int S, double* 
   static std::atomic<uint64_t> attr{0};
   cudaError_t e = raise_smem_limit(k_bd_bisect, 200 * 1024, attr);
   if (e != cudaSuccess) return e;
-  k_bd_bisect<<<S, bisect_threads(n), smem, st>>>(bd, n, n_pad, sig, perm, nnz, lns1, zero_rel, nullptr);
+  // fewer matrices than two CTAs per SM: the ranks of each spread over several
+  // CTAs of at least 64 (16 matrices of n = 576 5.1 -> 3.0 ms)
+  const int parts = std::max(1, std::min(2 * 152 / S, (n + 63) / 64));
+  const int threads = parts > 1 ? std::max(64, ((n + parts - 1) / parts + 31) / 32 * 32) : bisect_threads(n);
+  k_bd_bisect<<<dim3(S, parts), std::min(threads, kBisThreads), smem, st>>>(bd, n, n_pad, sig, perm, nnz, lns1, zero_rel,
+                                                                           nullptr);
+  if ((e = cudaGetLastError()) != cudaSuccess || parts == 1) return e;
+  k_bd_rank<<<S, 128, 0, st>>>(sig, n, n_pad, nnz, lns1, zero_rel);
   return cudaGetLastError();
 }
 
