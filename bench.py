@@ -580,7 +580,7 @@ def main():
     mctrg.mctrg_destroy(c2)
     e2e_s = time.perf_counter() - t0
     # the same trajectories with the contraction on the tensor cores: error-compensated
-    # TF32 (TF32X3), and BF16 slices at FP64 accuracy (FP64TC, Ozaki scheme)
+    # TF32 (TF32X3), and FP16 slices at FP64 accuracy (FP64TC, Ozaki scheme)
     mixed = None
     if wl["precision"] == 0 and not args.no_mixed:
         mixed = {}
@@ -590,7 +590,7 @@ def main():
         peaks_m, _ = measured_peaks()
         for name, prec, note, ratio in (
                 ("tf32x3", mctrg.MCTRG_TF32X3, "TF32 hi/lo split, three tcgen05 passes, FP32 accumulation", 0.5),
-                ("fp64tc", mctrg.MCTRG_FP64TC, "BF16 slices multiplied exactly on tcgen05, summed in FP64 "
+                ("fp64tc", mctrg.MCTRG_FP64TC, "FP16 slices multiplied exactly on tcgen05, summed in integers "
                                                "(Ozaki scheme), in the contraction and in the SVD's dense -> "
                                                "band reduction (8-bit digits of a fixed-point trailing matrix)",
                  1.0)):
@@ -699,7 +699,7 @@ def main():
     line = {"metric": "trajectories/s", "value": value, "unit": "trajectories/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_max / args.steps,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": ["f64", "f64+tf32", "f64+bf16", "f64+tf32x3", "f64+bf16x3", "f64 (bf16 slices)"][wl["precision"]],
+            "dtype": ["f64", "f64+tf32", "f64+bf16", "f64+tf32x3", "f64+bf16x3", "f64 (fp16 slices)"][wl["precision"]],
             "data": "synthetic",
             "config": {"workload": args.workload, "L": wl["L"], "chi": wl["chi"], "beta": wl["beta"],
                        "h": wl["h"], "trajectories_per_step_per_gpu": B, "parallelism": "replicas%d" % world,

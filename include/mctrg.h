@@ -72,11 +72,11 @@ extern "C" {
  * (matrix side not a multiple of 256, or above 1024) use the FP64 GEMM and
  * the FP64 threshold. */
 /* FP64TC: the plaquette GEMM at FP64 accuracy on the tensor cores: each row
- * of X and Yt is scaled by a power of two and split exactly into s BF16
+ * of X and Yt is scaled by a power of two and split exactly into s FP16
  * slices of b bits (b = 8, s = 7 for inner dimension K <= 256; b = 7, s = 8
  * up to 1024), the s(s+1)/2 leading slice products are formed exactly by
  * tcgen05 (one FP32 accumulator per slice-sum group, exact below 2^24) and
- * summed in FP64 (Ozaki, Ogita, Oishi and Rump 2012).  The result carries an
+ * summed in integers and rounded once to FP64 (Ozaki, Ogita, Oishi and Rump 2012).  The result carries an
  * error below 2^-43 K |row max| |column max|, the order of an FP64 dot
  * product's, so the FP64 zero threshold applies.  Levels whose inner
  * dimension is not a multiple of 64 up to 1024 use the FP64 GEMM. */
@@ -383,10 +383,10 @@ int mctrg_svd_batched_noalloc(const double* M, int n, int64_t batch, double* sig
  * ends in one matrix product per new tensor, M = X Yt^T; this runs it for a
  * batch: X, Yt (device, batch x n x K, row-major, n = D^2) and M (device,
  * batch x n x n, row-major; written, not accumulated).  precision:
- * MCTRG_FP64 (FP64 on the CUDA cores) or MCTRG_FP64TC (BF16 slices on the
+ * MCTRG_FP64 (FP64 on the CUDA cores) or MCTRG_FP64TC (FP16 slices on the
  * tensor cores, FP64-accurate; K a multiple of 64, at most 1024).  1 <= D,
  * n <= 1024, K >= 1, batch >= 1.  Allocates its working memory (FP64TC: the
- * slice planes and row exponents) for the call and frees it; runs on
+ * row exponents) for the call and frees it; runs on
  * `stream` and returns once the stream has completed.  Errors: EINVAL,
  * ENOMEM, ECUDA. */
 int mctrg_contract_batched(const double* X, const double* Yt, int D, int K, int64_t batch, double* M,

@@ -130,7 +130,7 @@ __global__ void k_fill_random(double* x, int64_t n, uint64_t seed) {
 
 // Workspace bytes of one item of level k of a job (packed per segment).
 struct ItemLayout {
-  size_t x, m, w, bd, sig, perm, nnz, kept, sigt, nk, vrows, oz, ozexp, lr_vt, lr_tau, lr_h;
+  size_t x, m, w, bd, sig, perm, nnz, kept, sigt, nk, vrows, ozexp, lr_vt, lr_tau, lr_h;
 };
 
 ItemLayout layout(const mctrg_ctx* c, int k, int prec) {
@@ -157,8 +157,7 @@ ItemLayout layout(const mctrg_ctx* c, int k, int prec) {
   L.sigt = ks * sizeof(double);
   L.nk = sizeof(int);
   L.vrows = ks * n * sizeof(double);
-  L.oz = (prec == MCTRG_FP64TC && !v.lowrank && gemm_ozaki_supported((int)n, (int)d2)) ? 8 * n * d2 * 2 : 0;
-  L.ozexp = L.oz ? n * sizeof(int) : 0;
+  L.ozexp = (prec == MCTRG_FP64TC && !v.lowrank && gemm_ozaki_supported((int)n, (int)d2)) ? 2 * n * sizeof(int) : 0;
   return L;
 }
 
@@ -166,8 +165,7 @@ ItemLayout layout(const mctrg_ctx* c, int k, int prec) {
 // segment's cnt items contiguously).
 struct SegPtrs {
   double *X, *Y, *M, *W, *bd, *sig, *sigt, *vrows, *lr_vt, *lr_tau, *lr_h;
-  int *perm, *nnz, *kept, *nk, *ezX, *ezY;
-  void *ozX, *ozY;
+  int *perm, *nnz, *kept, *nk, *ez;
 };
 
 SegPtrs carve(char* base, size_t off, const ItemLayout& L, int64_t cnt) {
@@ -186,12 +184,7 @@ SegPtrs carve(char* base, size_t off, const ItemLayout& L, int64_t cnt) {
   p.sigt = (double*)take(L.sigt);
   p.nk = (int*)take(L.nk);
   p.vrows = (double*)take(L.vrows);
-  if (L.oz) {
-    p.ozX = take(L.oz);
-    p.ozY = take(L.oz);
-    p.ezX = (int*)take(L.ozexp);
-    p.ezY = (int*)take(L.ozexp);
-  }
+  if (L.ozexp) p.ez = (int*)take(L.ozexp);
   if (L.lr_vt) {
     p.lr_vt = (double*)take(L.lr_vt);
     p.lr_tau = (double*)take(L.lr_tau);
@@ -205,7 +198,7 @@ size_t segment_bytes(const ItemLayout& L, int64_t cnt) {
   const size_t per[] = {L.x,    L.x,    L.m,     L.w,      L.bd,    L.sig, L.perm, L.nnz,
                         L.kept, L.sigt, L.nk, L.vrows, L.lr_vt, L.lr_tau, L.lr_h};
   for (size_t s : per) b += align_up(s * (size_t)cnt);
-  if (L.oz) b += 2 * align_up(L.oz * (size_t)cnt) + 2 * align_up(L.ozexp * (size_t)cnt);
+  if (L.ozexp) b += align_up(L.ozexp * (size_t)cnt);
   return b;
 }
 
@@ -391,16 +384,11 @@ struct BatchRunner {
         BCK(launch_gemm_f64(gm, ss));
         launches += 2;
       } else if (oz_mode && gemm_ozaki_supported(a.n, Kd)) {
-        int bits, slices;
-        ozaki_params(Kd, &bits, &slices);
-        BCK(launch_ozaki_split(q.X, g.cnt * a.n, Kd, q.ozX, q.ezX, ss));
-        BCK(launch_ozaki_split(q.Y, g.cnt * a.n, Kd, q.ozY, q.ezY, ss));
         GemmOzArgs ga{};
-        ga.M = q.M; ga.D = a.D; ga.n = a.n; ga.K = Kd; ga.c0 = g.i0; ga.n_items = g.cnt; ga.Nnew = a.N;
-        ga.L = c->L; ga.level_new = g.k; ga.fixed_parity = -1; ga.expX = q.ezX; ga.expY = q.ezY;
-        ga.slices = slices; ga.bits = bits; ga.err = err.as<uint32_t>();
-        BCK(launch_gemm_ozaki(ga, q.ozX, q.ozY, ss));
-        launches += 3;
+        ga.X = q.X; ga.Y = q.Y; ga.expX = q.ez; ga.M = q.M; ga.D = a.D; ga.n = a.n; ga.K = Kd; ga.c0 = g.i0; ga.n_items = g.cnt; ga.Nnew = a.N;
+        ga.L = c->L; ga.level_new = g.k; ga.fixed_parity = -1; ga.err = err.as<uint32_t>();
+        BCK(launch_gemm_ozaki(ga, ss));
+        launches += 2;
       } else if (tc_mode && gemm_tc_supported(a.n, Kd, tc_kind)) {
         return MCTRG_EINVAL;   // the TF32/BF16 modes run through mctrg_run, not batches
       } else {

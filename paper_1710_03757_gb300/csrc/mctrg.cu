@@ -433,8 +433,8 @@ extern "C" int mctrg_init_tensor(mctrg_ctx_t c, const double* T0, int D, int L, 
 
 // ---------------------------------------------------------------------------
 // Device bytes of one item's tensor-core operands (X and Yt, n x d2 each):
-// the rounded operands (and residuals) of the mixed modes, or the BF16 slice
-// planes and row exponents of the FP64-accurate mode.
+// the rounded operands (and residuals) of the mixed modes, or the row exponents
+// of the FP64-accurate mode.
 static size_t tc_operand_bytes(int prec, int n, int d2) {
   const size_t e = (size_t)n * d2;
   switch (prec) {
@@ -442,7 +442,7 @@ static size_t tc_operand_bytes(int prec, int n, int d2) {
     case MCTRG_BF16: return 2 * 2 * e;
     case MCTRG_TF32X3: return 2 * 2 * 4 * e;
     case MCTRG_BF16X3: return 2 * 2 * 2 * e;
-    case MCTRG_FP64TC: return gemm_ozaki_supported(n, d2) ? 2 * 8 * 2 * e + 2 * (size_t)n * sizeof(int) : 0;
+    case MCTRG_FP64TC: return gemm_ozaki_supported(n, d2) ? 2 * (size_t)n * sizeof(int) : 0;
     default: return 0;
   }
 }
@@ -688,7 +688,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
     }
     // tensor-core operands (mixed precision): per item X and Yt rounded, with scales
     const int prec = opt.precision;
-    const bool oz_mode = prec == MCTRG_FP64TC;    // FP64-accurate tensor-core GEMM (BF16 slices)
+    const bool oz_mode = prec == MCTRG_FP64TC;    // FP64-accurate tensor-core GEMM (FP16 slices)
     const bool tc_mode = prec != MCTRG_FP64 && !oz_mode;
     const int tc_kind = (prec == MCTRG_TF32 || prec == MCTRG_TF32X3) ? 0 : 1;
     const int tc_passes = (prec == MCTRG_TF32X3 || prec == MCTRG_BF16X3) ? 3 : 1;
@@ -703,19 +703,14 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
       }
       CK(tcScale.ensure(sizeof(double) * 2 * std::max<int64_t>(S, 1)));
     }
-    if (oz_mode) {   // slice planes (at most 8 per operand) and row exponents
-      size_t oz_elems = 0, oz_rows = 0;
+    if (oz_mode) {   // row exponents
+      size_t oz_rows = 0;
       for (int k = s0 + 1; k < nlev; ++k) {
         const int Kd = lv[k - 1].D * lv[k - 1].D;
         if (route_lowrank(opt, lv[k].n, Kd) || !gemm_ozaki_supported(lv[k].n, Kd)) continue;
-        oz_elems = std::max(oz_elems, (size_t)S * lv[k].n * Kd);
         oz_rows = std::max(oz_rows, (size_t)S * lv[k].n);
       }
-      if (oz_elems) {
-        CK(tcXh.ensure(2 * 8 * oz_elems));
-        CK(tcYh.ensure(2 * 8 * oz_elems));
-        CK(ozExp.ensure(sizeof(int) * 2 * oz_rows));
-      }
+      if (oz_rows) CK(ozExp.ensure(sizeof(int) * 2 * oz_rows));
     }
     if (prec != MCTRG_FP64 || any_band) {
       CK(tcErr.ensure(sizeof(uint32_t)));
@@ -814,23 +809,14 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
             CK(timed(MCTRG_K_GEMM, Si, Si * 2.0 / 3.0 * kd * kd * kd, 8.0 * Si * 2.0 * kd * kd,
                      [&] { return launch_gemm_f64(gm, st); }));
           } else if (used_oz) {
-            // FP64-accurate on the tensor cores: BF16 slices of X and Yt, exact slice products
-            int oz_bits, oz_slices;
-            ozaki_params(Kd, &oz_bits, &oz_slices);
-            int* eX = ozExp.as<int>();
-            int* eY = eX + Si * a.n;
-            const int64_t rows = Si * a.n;
-            CK(timed(MCTRG_K_FORM_XY, Si, 0.0, Si * 2.0 * a.n * Kd * (8.0 + 2.0 * oz_slices), [&] {
-              cudaError_t e = launch_ozaki_split(Xb.as<double>(), rows, Kd, tcXh.p, eX, st);
-              if (e != cudaSuccess) return e;
-              return launch_ozaki_split(Yb.as<double>(), rows, Kd, tcYh.p, eY, st); }));
+            // FP64-accurate on the tensor cores: FP16 digits of X and Yt, exact digit products
             GemmOzArgs ga{};
+            ga.X = Xb.as<double>(); ga.Y = Yb.as<double>(); ga.expX = ozExp.as<int>();
             ga.M = Mb.as<double>(); ga.D = a.D; ga.n = a.n; ga.K = Kd; ga.c0 = i0; ga.n_items = Si;
-            ga.Nnew = a.N; ga.L = L; ga.level_new = k; ga.fixed_parity = -1; ga.expX = eX; ga.expY = eY;
-            ga.slices = oz_slices; ga.bits = oz_bits; ga.err = tcErr.as<uint32_t>();
-            CK(timed(MCTRG_K_GEMM, Si, Si * 2.0 * a.n * a.n * Kd,
-                     Si * (2.0 * 2.0 * oz_slices * a.n * Kd + 8.0 * a.n * a.n), [&] {
-              return launch_gemm_ozaki(ga, tcXh.p, tcYh.p, st); }));
+            ga.Nnew = a.N; ga.L = L; ga.level_new = k; ga.fixed_parity = -1;
+            ga.err = tcErr.as<uint32_t>();
+            CK(timed(MCTRG_K_GEMM, Si, Si * 2.0 * a.n * a.n * Kd, 8.0 * Si * (2.0 * a.n * Kd + 1.0 * a.n * a.n),
+                     [&] { return launch_gemm_ozaki(ga, st); }));
           } else if (used_tc) {
             // tensor cores: scale and round the operands, then tcgen05 GEMM
             double* sX = tcScale.as<double>();

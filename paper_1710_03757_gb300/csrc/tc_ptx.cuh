@@ -120,17 +120,6 @@ static __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[3
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-
-// 4-D tiled load (coordinates innermost first) into shared memory, completing
-// on `bar` (transaction bytes).
-static __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, int x, int y, int z, int w,
-                                                   uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
-      ::"r"(smem_u32(dst)), "l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar))
-      : "memory");
-}
-
 // cuTensorMapEncodeTiled from the driver, looked up once (thread-safe static).
 static inline PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
   static const PFN_cuTensorMapEncodeTiled_v12000 fn = [] {

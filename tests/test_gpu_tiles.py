@@ -32,6 +32,36 @@ def test_fp64_products_of_integers(torch, D):
     np.testing.assert_array_equal(M.cpu().numpy(), np.einsum('bik,bjk->bij', X, Y))
 
 
+@pytest.mark.parametrize("K", [64, 320])
+def test_tensor_core_products_at_the_edges(torch, K):
+    # rows at the ends of the exponent range, values that round up to the row's power of two, zeros, and inputs
+    # off a 16-byte boundary.  With one nonzero per row and column each product is exact up to the 55 bits kept
+    # of either factor: within 2^-54 of it relative to |row max| |column max|, rounded once (2^-53)
+    n, batch = 49, 2
+    rng = np.random.default_rng(K)
+    X, Y = np.zeros((batch, n, K)), np.zeros((batch, n, K))
+    k = rng.integers(0, K, size=(batch, n))
+    for b in range(batch):
+        for r in range(n):
+            X[b, r, k[b, r]] = rng.choice([-1.0, 1.0]) * 2.0 ** rng.integers(-500, 500) * rng.uniform(1, 2)
+            Y[b, r, k[b, r]] = rng.choice([-1.0, 1.0]) * 2.0 ** rng.integers(-500, 500) * rng.uniform(1, 2)
+    X[0, 0] = 0.0
+    X[0, 1, k[0, 1]], Y[0, 1, k[0, 1]] = 1.0 - 2.0 ** -53, -(1.0 - 2.0 ** -53)
+    X[0, 2, k[0, 2]], Y[0, 2, k[0, 2]] = 5e-324 * 12345, 2.0 ** 1000      # a row of subnormal numbers
+    X[0, 3, k[0, 3]], Y[0, 3, k[0, 3]] = 2.0 ** -1000, 2.0 ** -60         # a subnormal product
+    ref = np.einsum('bik,bjk->bij', X, Y)
+    pad = torch.zeros(2 * batch * n * K + 3, dtype=torch.float64, device="cuda")
+    Xd = pad[1:1 + batch * n * K].view(batch, n, K)
+    Yd = pad[2 + batch * n * K:2 + 2 * batch * n * K].view(batch, n, K)
+    Xd.copy_(torch.tensor(X))
+    Yd.copy_(torch.tensor(Y))
+    M = torch.full((batch, n, n), float("nan"), dtype=torch.float64, device="cuda")
+    assert mctrg.mctrg_contract_batched(Xd, Yd, M, precision=mctrg.MCTRG_FP64TC) == mctrg.MCTRG_OK
+    scale = np.abs(X).max(2)[:, :, None] * np.abs(Y).max(2)[:, None, :]
+    assert (np.abs(M.cpu().numpy() - ref) <= 2.0 ** -51 * scale + 5e-324).all()
+    assert (M.cpu().numpy()[ref == 0] == 0).all()
+
+
 @pytest.mark.parametrize("chi,svd", [(8, mctrg.SVD_BIDIAG), (9, mctrg.SVD_AUTO), (12, mctrg.SVD_AUTO),
                                      (16, mctrg.SVD_AUTO)])
 def test_few_trajectories_equal_the_same_of_many(torch, chi, svd):
