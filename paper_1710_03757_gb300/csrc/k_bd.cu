@@ -69,6 +69,9 @@ __device__ __forceinline__ double block_max(double v, double* red) {
   return s;
 }
 
+// The bits of |x|, which order like the magnitudes (integer operations, not the FP64 pipe).
+__device__ __forceinline__ long long mag_bits(double x) { return __double_as_longlong(x) & 0x7fffffffffffffffll; }
+
 // Biased exponent field of a double (0 for zero and subnormals).
 __device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 }  // namespace
@@ -805,75 +808,104 @@ __global__ void __launch_bounds__(128) k_bd_rank(const double* sig, int n, int n
 // ---------------------------------------------------------------------------
 // Vector c of a set (at(v, i): entry i of vector v) made orthogonal to the
 // orthonormal vectors p0 .. c-1 and normalized, by every thread of the block
-// (32 or 64): the dots one thread per earlier vector (four partial sums), the
-// update and the norm spread over the entries; classical Gram-Schmidt applied
-// twice, which keeps orthogonality to rounding.  Called by all threads alike.
+// (one to eight warps): the dots by a lane per earlier vector and a warp per
+// eighth of the entries (four partial sums), the update and the norm spread over the
+// entries; classical Gram-Schmidt applied twice, which keeps orthogonality to
+// rounding.  Every sum is over the same parts in the same order whatever the
+// number of warps.  Called by all threads alike.  The kept values of a decaying
+// spectrum are mostly one cluster, so this is a chain over the vectors of
+// loads over their length: bound by latency, hence the eighths (all vector kernels of eight
+// chi = 24 trajectories, n = 576 and 256: 15.8 -> 13.5 ms).
+constexpr int kCgsParts = 8;
 template <class At>
-__device__ void block_cgs2(At at, int p0, int c, int len, double* s_dot, double* s_red) {
-  const int t = threadIdx.x, T = blockDim.x;
+__device__ void block_cgs2(At at, int p0, int c, int len, double (*s_part)[kKeptMax], double* s_dot, double* s_red) {
+  const int t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5, nw = T >> 5;
+  const int part = (len + kCgsParts - 1) / kCgsParts;
   for (int pass = 0; pass < 2; ++pass) {
-    if (t >= p0 && t < c) {
-      double d0 = 0.0, d1 = 0.0, d2 = 0.0, d3 = 0.0;
-      int i = 0;
-      for (; i + 16 <= len; i += 16) {                // sixteen pairs of loads in flight
-        double x[16], y[16];
+    for (int s = warp; s < kCgsParts; s += nw) {
+      const int end = min((s + 1) * part, len);
+      for (int p = p0 + lane; p < c; p += 32) {
+        double d0 = 0.0, d1 = 0.0, d2 = 0.0, d3 = 0.0;
+        int i = s * part;
+        for (; i + 16 <= end; i += 16) {              // sixteen pairs of loads in flight
+          double x[16], y[16];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) { x[q] = at(t, i + q); y[q] = at(c, i + q); }
+          for (int q = 0; q < 16; ++q) { x[q] = at(p, i + q); y[q] = at(c, i + q); }
 #pragma unroll
-        for (int q = 0; q < 16; q += 4) {
-          d0 = fma(x[q], y[q], d0);
-          d1 = fma(x[q + 1], y[q + 1], d1);
-          d2 = fma(x[q + 2], y[q + 2], d2);
-          d3 = fma(x[q + 3], y[q + 3], d3);
+          for (int q = 0; q < 16; q += 4) {
+            d0 = fma(x[q], y[q], d0);
+            d1 = fma(x[q + 1], y[q + 1], d1);
+            d2 = fma(x[q + 2], y[q + 2], d2);
+            d3 = fma(x[q + 3], y[q + 3], d3);
+          }
         }
+        for (; i + 4 <= end; i += 4) {
+          d0 = fma(at(p, i), at(c, i), d0);
+          d1 = fma(at(p, i + 1), at(c, i + 1), d1);
+          d2 = fma(at(p, i + 2), at(c, i + 2), d2);
+          d3 = fma(at(p, i + 3), at(c, i + 3), d3);
+        }
+        for (; i < end; ++i) d0 = fma(at(p, i), at(c, i), d0);
+        s_part[s][p] = (d0 + d1) + (d2 + d3);
       }
-      for (; i + 4 <= len; i += 4) {
-        d0 = fma(at(t, i), at(c, i), d0);
-        d1 = fma(at(t, i + 1), at(c, i + 1), d1);
-        d2 = fma(at(t, i + 2), at(c, i + 2), d2);
-        d3 = fma(at(t, i + 3), at(c, i + 3), d3);
-      }
-      for (; i < len; ++i) d0 = fma(at(t, i), at(c, i), d0);
-      s_dot[t] = (d0 + d1) + (d2 + d3);
+    }
+    __syncthreads();
+    for (int p = p0 + t; p < c; p += T) {
+      double d = s_part[0][p];
+#pragma unroll
+      for (int s = 1; s < kCgsParts; ++s) d += s_part[s][p];
+      s_dot[p] = d;
     }
     __syncthreads();
     for (int i = t; i < len; i += T) {
       double x = at(c, i);
+#pragma unroll 8
       for (int p = p0; p < c; ++p) x = fma(-s_dot[p], at(p, i), x);
       at(c, i) = x;
     }
     __syncthreads();
   }
-  double s2 = 0.0;
-  for (int i = t; i < len; i += T) s2 = fma(at(c, i), at(c, i), s2);
-  for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-  if ((t & 31) == 0) s_red[t >> 5] = s2;
+  for (int s = warp; s < kCgsParts; s += nw) {
+    double s2 = 0.0;
+    for (int i = s * 32 + lane; i < len; i += 32 * kCgsParts) s2 = fma(at(c, i), at(c, i), s2);
+    for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+    if (lane == 0) s_red[s] = s2;
+  }
   __syncthreads();
   double tot = 0.0;
-  for (int w = 0; w < (T >> 5); ++w) tot += s_red[w];
+  for (int s = 0; s < kCgsParts; ++s) tot += s_red[s];
   const double inv = tot > 0.0 ? 1.0 / sqrt(tot) : 0.0;
   for (int i = t; i < len; i += T) at(c, i) *= inv;
   __syncthreads();
 }
 
 // ---------------------------------------------------------------------------
-// 3. Inverse iteration, one CTA of one or two warps per matrix (persistent
-//    over matrices), thread a for the a-th kept index.  Scratch per CTA slot,
-//    interleaved by thread with stride ls (16, 32 or 64): DG, DU, DU2 (the LU
-//    factors of T - s I with partial pivoting, in the layout of LAPACK's dgtsv,
-//    the pivots as reciprocals) and X (the iterate), each 2n entries.  The factorization streams the
-//    current row in registers and applies L^-1 P^T to the right-hand side as
-//    it goes; the scale of the previous iterate is folded into the next
-//    right-hand side.
-__global__ void __launch_bounds__(64) k_bd_invit(BdVecArgs a, int ls) {
+// 3. Inverse iteration, one CTA per matrix (persistent over matrices), thread a
+//    for the a-th kept index; further warps take part in the orthogonalization.  Scratch per CTA slot,
+//    interleaved by thread with stride ls (16, 32 or 64): DG (reciprocal pivots),
+//    DU (first superdiagonal of U), F (multipliers) of T - s I = P L U by
+//    partial pivoting, and X (the iterate), each 2n entries; the row exchanges
+//    are one ballot per step in shared memory, and U's second superdiagonal is
+//    T's off-diagonal where rows were exchanged.  The first iteration factors
+//    with the current row in registers and applies L^-1 P^T to the right-hand
+//    side as it goes, without branches on the exchange (the lanes of a warp
+//    exchange at different steps); the later ones take the stored factors, with
+//    the scale of the previous iterate folded into the right-hand side.  Bound
+//    by the FP64 pipe and its latency: ~9 FP64 operations a step to factor, 5 to
+//    substitute back, 2 for a later right-hand side, where factoring anew with
+//    both branches took up to 50 for the three iterations (1920 matrices of n = 256,
+//    16 vectors: 7.9 -> 7.0 ms, and 5.9 with the orthogonalization below).
+__global__ void __launch_bounds__(256) k_bd_invit(BdVecArgs a, int ls) {
   __shared__ double s_dot[kKeptMax];
-  __shared__ double s_red[2];
+  __shared__ double s_part[kCgsParts][kKeptMax];
+  __shared__ double s_red[kCgsParts];
+  extern __shared__ unsigned s_swaps[];     // per warp 2n ballots
   const int lane = threadIdx.x;             // kept index of this thread
   const int wl = threadIdx.x & 31;          // lane within its warp
   double* scr = a.scratch + (size_t)blockIdx.x * 4 * (2 * a.n) * ls;   // a slot for the largest n
 #define DG(i) scr[((size_t)0 * m + (i)) * ls + lane]
 #define DU(i) scr[((size_t)1 * m + (i)) * ls + lane]
-#define DU2(i) scr[((size_t)2 * m + (i)) * ls + lane]
+#define F(i) scr[((size_t)2 * m + (i)) * ls + lane]
 #define XB(i) scr[((size_t)3 * m + (i)) * ls + lane]
 #define XL(l, i) scr[((size_t)3 * m + (i)) * ls + (l)]
   for (int s = blockIdx.x; s < a.S; s += gridDim.x) {
@@ -893,6 +925,7 @@ __global__ void __launch_bounds__(64) k_bd_invit(BdVecArgs a, int ls) {
       vout = a.vrows + (size_t)s * a.kstride * n;
     }
     const int m = 2 * n;
+    unsigned* sw = s_swaps + (threadIdx.x >> 5) * (2 * a.n);
     // |T| (max |o_k|): T and s are scaled by 1/|T|, the pivot floor is eps
     // (each warp reduces over all of T)
     double tn = 0.0;
@@ -912,46 +945,73 @@ __global__ void __launch_bounds__(64) k_bd_invit(BdVecArgs a, int ls) {
       for (int i = 0; i < m; ++i) XB(i) = 1.0 + 0.25 * (double)((i * (2 * lane + 3)) % 17) * (1.0 / 17.0);
     }
     double rs = 1.0;                                 // scale owed by the stored iterate
+    const unsigned act = __ballot_sync(0xffffffffu, on);
+    const int first = __ffs(act) - 1;
     for (int iter = 0; iter < kInvitIters; ++iter) {
       if (on) {
-        // factor T - s I = P L U, applying L^-1 P^T to the right-hand side as it
-        // goes; the loads of each block of kCh steps are issued together, so the
+        // the loads of each block of kCh steps are issued together, so the
         // serial chain waits on memory once per block instead of once per step
-        double dg = -sgm, du = OFFD(0), xi = XB(0) * rs;
-        for (int base = 0; base < m - 1; base += kCh) {
-          double xnb[kCh], odb[kCh + 1];
+        double xi = XB(0) * rs;
+        if (iter == 0) {
+          // factor T - s I = P L U, applying L^-1 P^T to the right-hand side as it goes
+          double dg = -sgm, du = OFFD(0);
+          for (int base = 0; base < m - 1; base += kCh) {
+            double xnb[kCh], odb[kCh + 1];
 #pragma unroll
-          for (int c = 0; c < kCh; ++c) {
-            const int i = base + c;
-            xnb[c] = (i + 1 < m) ? XB(i + 1) : 0.0;
-            odb[c] = (i < m - 1) ? OFFD(i) : 0.0;
+            for (int c = 0; c < kCh; ++c) {
+              const int i = base + c;
+              xnb[c] = (i + 1 < m) ? XB(i + 1) : 0.0;
+              odb[c] = (i < m - 1) ? OFFD(i) : 0.0;
+            }
+            odb[kCh] = (base + kCh < m - 1) ? OFFD(base + kCh) : 0.0;
+#pragma unroll
+            for (int c = 0; c < kCh; ++c) {
+              const int i = base + c;
+              if (i >= m - 1) break;
+              const double dli = odb[c];                 // sub-diagonal = off-diagonal
+              const double dun = (i + 1 < m - 1) ? odb[c + 1] : 0.0;
+              const bool swap = mag_bits(dg) < mag_bits(dli);
+              const double piv = swap ? dli : (mag_bits(dg) == 0 ? kEps : dg);
+              const double g = inv(piv), f = (swap ? dg : dli) * g;
+              // the row that stays (u, x) and the one that goes on
+              const double u = swap ? -sgm : du, v = swap ? du : -sgm;
+              const double xs = swap ? xnb[c] : xi, xg = swap ? xi : xnb[c];
+              DG(i) = g; DU(i) = u; F(i) = f; XB(i) = xs;
+              dg = fma(-f, u, v);
+              const double fd = -f * dun;
+              du = swap ? fd : dun;
+              xi = fma(-f, xs, xg);
+              const unsigned ex = __ballot_sync(act, swap);
+              if (wl == first) sw[i] = ex;
+            }
           }
-          odb[kCh] = (base + kCh < m - 1) ? OFFD(base + kCh) : 0.0;
+          DG(m - 1) = inv(mag_bits(dg) == 0 ? kEps : dg);
+          __syncwarp(act);
+        } else {
+          for (int base = 0; base < m - 1; base += kCh) {
+            double xnb[kCh], fb[kCh];
+            unsigned eb[kCh];
 #pragma unroll
-          for (int c = 0; c < kCh; ++c) {
-            const int i = base + c;
-            if (i >= m - 1) break;
-            const double dli = odb[c];                 // sub-diagonal = off-diagonal
-            const double dun = (i + 1 < m - 1) ? odb[c + 1] : 0.0;
-            const double xn = xnb[c] * rs;
-            if (fabs(dg) >= fabs(dli)) {
-              const double g = inv((dg == 0.0) ? kEps : dg);
-              const double f = dli * g;
-              DG(i) = g; DU(i) = du; DU2(i) = 0.0; XB(i) = xi;
-              dg = -sgm - f * du;
-              du = dun;
-              xi = xn - f * xi;
-            } else {
-              const double g = inv(dli), f = dg * g;
-              DG(i) = g; DU(i) = -sgm; DU2(i) = dun; XB(i) = xn;
-              dg = du + f * sgm;
-              du = -f * dun;
-              xi = xi - f * xn;
+            for (int c = 0; c < kCh; ++c) {
+              const int i = base + c;
+              xnb[c] = (i + 1 < m) ? XB(i + 1) : 0.0;
+              fb[c] = (i < m - 1) ? F(i) : 0.0;
+              eb[c] = (i < m - 1) ? sw[i] : 0u;
+            }
+#pragma unroll
+            for (int c = 0; c < kCh; ++c) {
+              const int i = base + c;
+              if (i >= m - 1) break;
+              const bool swap = (eb[c] >> wl) & 1u;
+              const double xn = xnb[c] * rs;
+              const double xs = swap ? xn : xi, xg = swap ? xi : xn;
+              XB(i) = xs;
+              xi = fma(-fb[c], xs, xg);
             }
           }
         }
         // back substitution U x = y, carrying x_{i+1}, x_{i+2}, in blocks of kCh
-        double x1 = xi * inv((dg == 0.0) ? kEps : dg);
+        double x1 = xi * DG(m - 1);
         XB(m - 1) = x1;
         double s2 = x1 * x1;
         double x2 = 0.0;
@@ -962,14 +1022,14 @@ __global__ void __launch_bounds__(64) k_bd_invit(BdVecArgs a, int ls) {
             const int i = top - c;
             yb[c] = i >= 0 ? XB(i) : 0.0;
             ub[c] = i >= 0 ? DU(i) : 0.0;
-            u2b[c] = i >= 0 ? DU2(i) : 0.0;
+            u2b[c] = (i >= 0 && i + 1 < m - 1 && ((sw[i] >> wl) & 1u)) ? OFFD(i + 1) : 0.0;
             gb[c] = i >= 0 ? DG(i) : 1.0;
           }
 #pragma unroll
           for (int c = 0; c < kCh; ++c) {
             const int i = top - c;
             if (i < 0) break;
-            double x = (yb[c] - ub[c] * x1 - u2b[c] * x2) * gb[c];
+            double x = fma(-ub[c], x1, fma(-u2b[c], x2, yb[c])) * gb[c];
             if (exp_field(x) > 1023 + 600) {         // growth through tiny pivots: rescale x[i..]
               for (int q = i + 1; q < m; ++q) XB(q) *= 0x1.0p-600;
               x *= 0x1.0p-600; x1 *= 0x1.0p-600; x2 *= 0x1.0p-600; s2 *= 0x1.0p-1200;
@@ -993,7 +1053,7 @@ __global__ void __launch_bounds__(64) k_bd_invit(BdVecArgs a, int ls) {
         if (sg[kept[c - 1]] - sg[kept[c]] > 1e-3 * tn) continue;
         int p0 = c - 1;
         while (p0 > 0 && sg[kept[p0 - 1]] - sg[kept[p0]] <= 1e-3 * tn) --p0;
-        block_cgs2([&](int v, int i) -> double& { return XL(v, i); }, p0, c, m, s_dot, s_red);
+        block_cgs2([&](int v, int i) -> double& { return XL(v, i); }, p0, c, m, s_part, s_dot, s_red);
       }
     }
 #undef OFFD
@@ -1010,13 +1070,13 @@ __global__ void __launch_bounds__(64) k_bd_invit(BdVecArgs a, int ls) {
       if (sg[kept[c - 1]] - sg[kept[c]] > 1e-3 * tn) continue;
       int p0 = c - 1;
       while (p0 > 0 && sg[kept[p0 - 1]] - sg[kept[p0]] <= 1e-3 * tn) --p0;
-      block_cgs2([&](int v, int i) -> double& { return vout[(size_t)v * n + i]; }, p0, c, n, s_dot, s_red);
+      block_cgs2([&](int v, int i) -> double& { return vout[(size_t)v * n + i]; }, p0, c, n, s_part, s_dot, s_red);
     }
     __syncthreads();
   }
 #undef DG
 #undef DU
-#undef DU2
+#undef F
 #undef XB
 #undef XL
 }
@@ -1208,7 +1268,10 @@ cudaError_t launch_bd_vectors(const BdVecArgs& a, cudaStream_t st) {
   if (a.S <= 0) return cudaSuccess;
   if (a.kmax > kKeptMax || (!a.items && a.kstride < a.kmax)) return cudaErrorInvalidValue;
   const int ls = invit_stride(a.kmax);
-  k_bd_invit<<<invit_slots(a.n, a.S, a.kmax), ls > 32 ? 64 : 32, 0, st>>>(a, ls);
+  // as many warps as leave a CTA of every matrix (up to eight per SM) its registers
+  const int warps = a.S <= 2 * 152 ? 8 : (a.S <= 4 * 152 ? 4 : 2);
+  const size_t ballots = sizeof(unsigned) * (ls > 32 ? 2 : 1) * 2 * a.n;
+  k_bd_invit<<<invit_slots(a.n, a.S, a.kmax), 32 * warps, ballots, st>>>(a, ls);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || a.skip_backtr) return e;
   return launch_bd_backtr(a, st);
