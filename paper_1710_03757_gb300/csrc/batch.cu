@@ -248,7 +248,7 @@ struct BatchRunner {
     BCK(cudaMemsetAsync(c->iflags.p, 0, sizeof(uint32_t) * items, st));
     SampleArgs sa{};
     sa.M = c->shM.as<double>(); sa.W = c->shW.as<double>(); sa.sig = c->shSig.as<double>();
-    sa.perm = c->shPerm.as<int>(); sa.nnz = c->shNnz.as<int>(); sa.Urows = c->shU.as<double>();
+    sa.perm = c->shPerm.as<int>(); sa.nnz = c->sh_nnz(); sa.Urows = c->shU.as<double>();
     sa.n = a.n; sa.n_pad = a.n_pad; sa.chi = c->chi; sa.kc = a.kc; sa.stochastic = 1; sa.shared_svd = 1;
     sa.item0 = 0; sa.n_items = items; sa.N = a.N; sa.L = c->L; sa.level = c->s0; sa.seed = r.job.seed;
     sa.traj0 = r.job.first_traj; sa.H = c->Hbuf[0].as<double>(); sa.h_item0 = 0;
@@ -780,7 +780,7 @@ extern "C" int mctrg_batch_run(const mctrg_options* opt, const mctrg_job* jobs, 
         break;
       }
     }
-    double hs[6];
+    double hs[7];
     if (launch_estimate(c->o_lnabs.as<double>(), c->o_sign.as<int8_t>(), c->o_flags.as<uint8_t>(), B,
                         c->stats.as<double>(), R.st) != cudaSuccess ||
         cudaMemcpyAsync(hs, c->stats.p, sizeof(hs), cudaMemcpyDeviceToHost, R.st) != cudaSuccess ||
@@ -796,7 +796,7 @@ extern "C" int mctrg_batch_run(const mctrg_options* opt, const mctrg_job* jobs, 
     e.n = B; e.ln_scale = hs[0]; e.sum_x = hs[1]; e.m2_x = hs[2]; e.n_negative = (int64_t)hs[3];
     e.n_flagged = (int64_t)hs[4];
     finish_estimate(&e);
-    if (e.status == MCTRG_OK && c->any_noconv(B)) e.status = MCTRG_ENOCONV;
+    if (e.status == MCTRG_OK && hs[6] > 0.0) e.status = MCTRG_ENOCONV;
     off += B;
   }
   cudaStreamSynchronize(R.st);

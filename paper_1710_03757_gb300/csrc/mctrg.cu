@@ -166,7 +166,7 @@ extern "C" int mctrg_reset_kernel_stats(mctrg_ctx_t c) {
 }
 
 size_t mctrg_ctx::held_bytes() const {
-  const DevBuf* all[] = {&T0, &shM, &shW, &shSig, &shPerm, &shNnz, &shLns1, &shU, &shH, &Hbuf[0], &Hbuf[1],
+  const DevBuf* all[] = {&T0, &shM, &shW, &shSig, &shPerm, &shLns1, &shU, &shH, &Hbuf[0], &Hbuf[1],
                          &Mb, &Wb, &Xb, &Yb, &sigb, &permb, &nnzb, &ilns1, &iflags, &lnacc, &tflags,
                          &scratch, &o_lnabs, &o_sign, &o_flags, &o_tflags, &stats, &tcXh, &tcYh, &tcXl,
                          &tcYl, &tcScale, &tcErr, &ozExp, &Timp, &bdb, &keptb, &sigtb, &nkb, &vrowsb, &bdscr,
@@ -180,7 +180,7 @@ void mctrg_ctx::release_all() {
   resolve_events();
   for (cudaEvent_t e : event_pool) cudaEventDestroy(e);
   event_pool.clear();
-  DevBuf* all[] = {&T0, &shM, &shW, &shSig, &shPerm, &shNnz, &shLns1, &shU, &shH, &Hbuf[0], &Hbuf[1],
+  DevBuf* all[] = {&T0, &shM, &shW, &shSig, &shPerm, &shLns1, &shU, &shH, &Hbuf[0], &Hbuf[1],
                    &Mb, &Wb, &Xb, &Yb, &sigb, &permb, &nnzb, &ilns1, &iflags, &lnacc, &tflags,
                    &scratch, &o_lnabs, &o_sign, &o_flags, &o_tflags, &stats, &tcXh, &tcYh, &tcXl,
                    &tcYl, &tcScale, &tcErr, &ozExp, &Timp, &bdb, &keptb, &sigtb, &nkb, &vrowsb, &bdscr,
@@ -206,7 +206,7 @@ int mctrg_ctx::init_from_device_tensor(int D0, int L_, int chi_) {
   level0_distinct = false;
   imp0 = imp1 = -1;
   int D = D0;
-  // cur raw tensor lives in T0 (D^4); the plaquette result goes to shM scratch then back
+  // the current raw tensor lives in T0 (D^4)
   for (int k = 0; k < nlev; ++k) {
     const int n = D * D, np = n + (n & 1);
     const int64_t N = level_count(L, k);
@@ -214,20 +214,20 @@ int mctrg_ctx::init_from_device_tensor(int D0, int L_, int chi_) {
     CK(shW.ensure(sizeof(double) * 2 * np * n));
     CK(shSig.ensure(sizeof(double) * 2 * np));
     CK(shPerm.ensure(sizeof(int) * 2 * np));
-    CK(shNnz.ensure(sizeof(int) * 2));
-    CK(shLns1.ensure(sizeof(double) * 2));
+    CK(shLns1.ensure(2 * (sizeof(double) + sizeof(int))));   // ln s_1 of both, then their nonzero counts
+    int* const nnz = sh_nnz();
     CK(launch_matricize2(T0.as<double>(), D, shM.as<double>(), st));
     JacobiArgs ja{};
     ja.M = shM.as<double>(); ja.W = shW.as<double>(); ja.sig = shSig.as<double>();
-    ja.perm = shPerm.as<int>(); ja.lns1 = shLns1.as<double>(); ja.nnz = shNnz.as<int>();
+    ja.perm = shPerm.as<int>(); ja.lns1 = shLns1.as<double>(); ja.nnz = nnz;
     ja.mflags = nullptr; ja.n = n; ja.n_pad = np; ja.S = 2; ja.max_sweeps = opt.max_sweeps;
     ja.zero_rel = opt.zero_tol_scale * (double)n * 0x1.0p-52;
     CK(launch_jacobi_few(ja, st));
-    int hn[2];
-    double hl[2];
-    CK(cudaMemcpyAsync(hn, shNnz.p, sizeof(hn), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(hl, shLns1.p, sizeof(hl), cudaMemcpyDeviceToHost, st));
+    struct { double lns1[2]; int nnz[2]; } host;
+    CK(cudaMemcpyAsync(&host, shLns1.p, sizeof(host), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    const double* hl = host.lns1;
+    const int* hn = host.nnz;
     lnacc0 += (double)(N / 2) * (hl[0] + hl[1]);
     const int nu = std::max(hn[0], hn[1]);
     const int kc = std::max(1, std::min(chi, nu));
@@ -251,7 +251,7 @@ int mctrg_ctx::init_from_device_tensor(int D0, int L_, int chi_) {
       CK(scratch.ensure(sizeof(double) * sample_scratch_doubles(n, chi, 2)));
       SampleArgs sa{};
       sa.M = shM.as<double>(); sa.W = shW.as<double>(); sa.sig = shSig.as<double>();
-      sa.perm = shPerm.as<int>(); sa.nnz = shNnz.as<int>(); sa.Urows = nullptr;
+      sa.perm = shPerm.as<int>(); sa.nnz = nnz; sa.Urows = nullptr;
       sa.n = n; sa.n_pad = np; sa.chi = chi; sa.kc = kc; sa.stochastic = 0; sa.shared_svd = 0;
       sa.item0 = 0; sa.n_items = 2; sa.N = 2; sa.L = L; sa.level = k; sa.seed = 0; sa.traj0 = 0;
       sa.H = shH.as<double>(); sa.h_item0 = 0; sa.iflags = nullptr; sa.scratch = scratch.as<double>();
@@ -277,13 +277,11 @@ int mctrg_ctx::init_from_device_tensor(int D0, int L_, int chi_) {
         break;
       }
       const size_t tbytes = sizeof(double) * (size_t)kc * kc * kc * kc;
-      CK(Mb.ensure(tbytes));
+      CK(T0.ensure(tbytes));                         // the old tensor is spent
       GemmArgs gm{};
-      gm.X = Xb.as<double>(); gm.Yt = Yb.as<double>(); gm.M = Mb.as<double>(); gm.D = kc; gm.K = n;
+      gm.X = Xb.as<double>(); gm.Yt = Yb.as<double>(); gm.M = T0.as<double>(); gm.D = kc; gm.K = n;
       gm.c0 = 0; gm.n_items = 1; gm.Nnew = 1; gm.L = L; gm.level_new = k + 1; gm.fixed_parity = 0;
       CK(launch_gemm_f64(gm, st));
-      CK(T0.ensure(tbytes));
-      CK(cudaMemcpyAsync(T0.p, Mb.p, tbytes, cudaMemcpyDeviceToDevice, st));
       D = kc;
       continue;
     }
@@ -291,7 +289,7 @@ int mctrg_ctx::init_from_device_tensor(int D0, int L_, int chi_) {
     s0 = k;
     CK(shU.ensure(sizeof(double) * 2 * (size_t)np * n));
     CK(launch_u_rows(shM.as<double>(), shW.as<double>(), shSig.as<double>(), shPerm.as<int>(),
-                     shNnz.as<int>(), shU.as<double>(), n, np, 2, st));
+                     nnz, shU.as<double>(), n, np, 2, st));
     break;
   }
   if (!all_exact) {
@@ -759,7 +757,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
         CK(cudaMemsetAsync(iflags.p, 0, sizeof(uint32_t) * items, st));
         SampleArgs sa{};
         sa.M = shM.as<double>(); sa.W = shW.as<double>(); sa.sig = shSig.as<double>();
-        sa.perm = shPerm.as<int>(); sa.nnz = shNnz.as<int>(); sa.Urows = shU.as<double>();
+        sa.perm = shPerm.as<int>(); sa.nnz = sh_nnz(); sa.Urows = shU.as<double>();
         sa.n = a.n; sa.n_pad = a.n_pad; sa.chi = chi; sa.kc = a.kc; sa.stochastic = 1; sa.shared_svd = 1;
         sa.item0 = 0; sa.n_items = items; sa.N = a.N; sa.L = L; sa.level = s0; sa.seed = seed;
         sa.traj0 = traj0; sa.H = Hbuf[cur].as<double>(); sa.h_item0 = 0; sa.iflags = iflags.as<uint32_t>();
@@ -945,7 +943,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
   CK(timed(MCTRG_K_OTHER, n, 0.0, 10.0 * n, [&] {
     return launch_estimate(o_lnabs.as<double>(), o_sign.as<int8_t>(), o_flags.as<uint8_t>(), n,
                            stats.as<double>(), st); }));
-  double hs[6];
+  double hs[7];
   CK(cudaMemcpyAsync(hs, stats.p, sizeof(hs), cudaMemcpyDeviceToHost, st));
   if (lnabs_out) CK(cudaMemcpyAsync(lnabs_out, o_lnabs.p, sizeof(double) * n, cudaMemcpyDefault, st));
   if (sign_out) CK(cudaMemcpyAsync(sign_out, o_sign.p, (size_t)n, cudaMemcpyDefault, st));
@@ -958,18 +956,8 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
   if (tc_err) return MCTRG_ECUDA;   // a tensor-core pipeline wait expired
   finalize_estimate(hs, n, est);
   // any trajectory whose SVD hit the sweep cap
-  if (est->status == MCTRG_OK && any_noconv(n)) est->status = MCTRG_ENOCONV;
+  if (est->status == MCTRG_OK && hs[6] > 0.0) est->status = MCTRG_ENOCONV;
   return est->status == MCTRG_EDOMAIN ? MCTRG_EDOMAIN : est->status;
-}
-
-bool mctrg_ctx::any_noconv(int64_t n) {
-  std::vector<uint8_t> f((size_t)n);
-  if (cudaMemcpyAsync(f.data(), o_flags.p, (size_t)n, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-      cudaStreamSynchronize(st) != cudaSuccess)
-    return false;
-  for (uint8_t v : f)
-    if (v & FLAG_NOCONV) return true;
-  return false;
 }
 
 extern "C" int mctrg_run(mctrg_ctx_t c, int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs,

@@ -69,7 +69,7 @@ struct mctrg_ctx {
   int imp0 = -1, imp1 = -1;
   double const_lnabs = 0.0;
   int const_sign = 0;
-  mctrg::DevBuf T0, shM, shW, shSig, shPerm, shNnz, shLns1, shU, shH;
+  mctrg::DevBuf T0, shM, shW, shSig, shPerm, shLns1, shU, shH;
   mctrg::DevBuf Hbuf[2], Mb, Wb, Xb, Yb, sigb, permb, nnzb, ilns1, iflags, lnacc, tflags, scratch;
   mctrg::DevBuf o_lnabs, o_sign, o_flags, o_tflags, stats;
   mctrg::DevBuf tcXh, tcYh, tcXl, tcYl, tcScale, tcErr;   // tensor-core operands
@@ -114,7 +114,7 @@ struct mctrg_ctx {
   void plan_chunks(int64_t n_samples, int64_t& B, int64_t& S, size_t& total) const;
   int run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs, int8_t* sign, uint8_t* flags,
           mctrg_estimate* est);
-  bool any_noconv(int64_t n);
+  int* sh_nnz() const { return (int*)(shLns1.as<double>() + 2); }   // nonzero counts of the shared matrices
   void release_all();
   size_t held_bytes() const;   // device bytes the context's buffers hold now
 };
