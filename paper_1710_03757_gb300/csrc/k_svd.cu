@@ -59,14 +59,22 @@ __device__ __forceinline__ void rotation(double al, double be, double g, double&
   cs = inv_sqrt(fma(t, t, 1.0));
 }
 
-__global__ void k_jacobi(JacobiArgs a, int use_smem, int G) {
+// n <= 32, one CTA per matrix, the rows in shared memory, G lanes per pair with
+// at most two entries of a row each; every pair of a step has its lanes, so a
+// step is one chain: dot product, rotation, update, barrier.  Bound by the
+// latency of that chain (some thirty dependent FP64 operations): the rows'
+// entries stay in registers from the dot product to the update, the next step's
+// pair is fetched a step ahead (its place in the round-robin order moves by one),
+// and the rotations are counted once a sweep (64 matrices of n = 16 in one launch
+// 0.238 -> 0.213 ms).
+template <int G>
+__global__ void __launch_bounds__(256) k_jacobi(JacobiArgs a) {
   extern __shared__ double smem[];
   const double nu = a.noise_u > 0.0 ? a.noise_u : 0x1.0p-52;
-  __shared__ int s_rot;
   const int mat = blockIdx.x;
   const int n = a.n, np = a.n_pad;
-  double* A = use_smem ? smem : a.W + (size_t)mat * np * n;
-  double* nrm = use_smem ? smem + (size_t)np * n : smem;
+  double* A = smem;
+  double* nrm = smem + (size_t)np * n;
   int* act = (int*)(nrm + np);                      // [np + 1] active rows of a sweep
   const double* Mm = a.M + (size_t)mat * n * n;
   for (int idx = threadIdx.x; idx < np * n; idx += blockDim.x)
@@ -76,6 +84,7 @@ __global__ void k_jacobi(JacobiArgs a, int use_smem, int G) {
   const int gl = threadIdx.x & (G - 1);
   const int grp = threadIdx.x / G;
   const int ngrp = blockDim.x / G;
+  const bool c0 = gl < n, c1 = gl + G < n;          // this lane's columns
   const double tol = (double)np * 0x1.0p-53;
   bool converged = false;
   __shared__ int s_na;
@@ -105,62 +114,55 @@ __global__ void k_jacobi(JacobiArgs a, int use_smem, int G) {
       if (r == 0) {
         if (na & 1) act[na] = -1;
         s_na = na;
-        s_rot = 0;
       }
     }
     __syncthreads();
     const int na = s_na, nap = na + (na & 1), npairs = nap >> 1;
+    const bool mine = grp < npairs;
+    // places of the pair in the order of the rows 1 .. nap-1, which turns by one a step
+    int i1 = grp - 1, i2 = nap - 2 - grp, myrot = 0;
+    int P = mine ? act[grp == 0 ? 0 : 1 + i1] : -1, Q = mine ? act[1 + i2] : -1;
     for (int step = 0; step + 1 < nap; ++step) {
-      int myrot = 0;
-      for (int base = 0; base < npairs; base += ngrp) {
-        const int pk = base + grp;
-        int P = -1, Q = -1;
-        if (pk < npairs) {
-          P = act[pk == 0 ? 0 : 1 + (pk - 1 + step) % (nap - 1)];
-          Q = act[1 + (nap - 2 - pk + step) % (nap - 1)];
-        }
-        const bool act_pair = P >= 0 && Q >= 0;
-        if (!act_pair) { P = 0; Q = 0; }
-        double* ap = A + (size_t)P * n;
-        double* aq = A + (size_t)Q * n;
-        double g = 0.0;
-        if (act_pair)
-          for (int c = gl; c < n; c += G) g = fma(ap[c], aq[c], g);
-        g = group_sum(g, G);                       // every lane of the warp takes part
-        const double al = act_pair ? nrm[P] : 0.0, be = act_pair ? nrm[Q] : 0.0;
-        const bool rot = act_pair && rotate_pair(al, be, g, tol);
-        double nal = al, nbe = be;
-        if (rot) {                                 // uniform within the lane group
-          double t, cs;
-          rotation(al, be, g, t, cs);
-          const double sn = cs * t;
-          for (int c = gl; c < n; c += G) {
-            const double x = ap[c], y = aq[c];
-            ap[c] = fma(-sn, y, cs * x);
-            aq[c] = fma(sn, x, cs * y);
-          }
-          nal = fma(-t, g, al);
-          nbe = fma(t, g, be);
-          ++myrot;
-        }
-        // heavy cancellation in the norm update: recompute from the rotated rows
-        const bool fixP = rot && nal < 0.01 * al, fixQ = rot && nbe < 0.01 * be;
-        if (__any_sync(0xffffffffu, fixP || fixQ)) {
-          double sp = 0.0, sq = 0.0;
-          if (fixP) for (int c = gl; c < n; c += G) sp = fma(ap[c], ap[c], sp);
-          if (fixQ) for (int c = gl; c < n; c += G) sq = fma(aq[c], aq[c], sq);
-          sp = group_sum(sp, G);
-          sq = group_sum(sq, G);
-          if (fixP) nal = sp;
-          if (fixQ) nbe = sq;
-        }
-        if (rot && gl == 0) { nrm[P] = nal; nrm[Q] = nbe; }
+      const bool act_pair = P >= 0 && Q >= 0;
+      const int p = act_pair ? P : 0, q = act_pair ? Q : 0;
+      double* ap = A + (size_t)p * n + gl;
+      double* aq = A + (size_t)q * n + gl;
+      const double x0 = c0 ? ap[0] : 0.0, y0 = c0 ? aq[0] : 0.0, x1 = c1 ? ap[G] : 0.0, y1 = c1 ? aq[G] : 0.0;
+      const double al = act_pair ? nrm[p] : 0.0, be = act_pair ? nrm[q] : 0.0;
+      if (mine) {                                  // the next step's pair
+        if (++i1 == nap - 1) i1 = 0;
+        if (++i2 == nap - 1) i2 = 0;
+        if (grp > 0) P = act[1 + i1];
+        Q = act[1 + i2];
       }
-      if (myrot && gl == 0) atomicAdd(&s_rot, myrot);
+      const double g = group_sum(act_pair ? fma(x1, y1, x0 * y0) : 0.0, G);   // every lane of the warp takes part
+      const bool rot = act_pair && rotate_pair(al, be, g, tol);
+      double nal = al, nbe = be, u0 = 0.0, u1 = 0.0, v0 = 0.0, v1 = 0.0;
+      if (rot) {                                   // uniform within the lane group
+        double t, cs;
+        rotation(al, be, g, t, cs);
+        const double sn = cs * t;
+        u0 = fma(-sn, y0, cs * x0);
+        u1 = fma(-sn, y1, cs * x1);
+        v0 = fma(sn, x0, cs * y0);
+        v1 = fma(sn, x1, cs * y1);
+        if (c0) { ap[0] = u0; aq[0] = v0; }
+        if (c1) { ap[G] = u1; aq[G] = v1; }
+        nal = fma(-t, g, al);
+        nbe = fma(t, g, be);
+        ++myrot;
+      }
+      // heavy cancellation in the norm update: recompute from the rotated rows
+      const bool fixP = rot && nal < 0.01 * al, fixQ = rot && nbe < 0.01 * be;
+      if (__any_sync(0xffffffffu, fixP || fixQ)) {
+        const double sp = group_sum(fma(u1, u1, u0 * u0), G), sq = group_sum(fma(v1, v1, v0 * v0), G);
+        if (fixP) nal = sp;
+        if (fixQ) nbe = sq;
+      }
+      if (rot && gl == 0) { nrm[p] = nal; nrm[q] = nbe; }
       __syncthreads();
     }
-    converged = (s_rot == 0);
-    __syncthreads();
+    converged = !__syncthreads_or(myrot);
   }
 
   // exact final norms
@@ -186,10 +188,8 @@ __global__ void k_jacobi(JacobiArgs a, int use_smem, int G) {
     sg[rank] = v;
     pm[rank] = r;
   }
-  if (use_smem) {
-    double* Wm = a.W + (size_t)mat * np * n;
-    for (int idx = threadIdx.x; idx < np * n; idx += blockDim.x) Wm[idx] = A[idx];
-  }
+  double* Wm = a.W + (size_t)mat * np * n;
+  for (int idx = threadIdx.x; idx < np * n; idx += blockDim.x) Wm[idx] = A[idx];
   __syncthreads();
   if (threadIdx.x == 0) {
     double s1 = sg[0];
@@ -1048,6 +1048,14 @@ static cudaError_t launch_warp_variant(const JacobiArgs& a, int threads, cudaStr
   return cudaGetLastError();
 }
 
+template <int G>
+static cudaError_t launch_small(const JacobiArgs& a, cudaStream_t st) {
+  const int np = a.n_pad;
+  const size_t smem = (size_t)np * a.n * sizeof(double) + (size_t)np * sizeof(double) + (size_t)(np + 2) * sizeof(int);
+  k_jacobi<G><<<a.S, std::max(32, (np / 2 * G + 31) / 32 * 32), smem, st>>>(a);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_jacobi(const JacobiArgs& a, cudaStream_t st) {
   if (a.S <= 0) return cudaSuccess;
   if (a.n > 32) {
@@ -1067,27 +1075,15 @@ cudaError_t launch_jacobi(const JacobiArgs& a, cudaStream_t st) {
     }
   }
 
-  // n <= 32: lane groups of G < 32 lanes per pair
-  const int n = a.n, np = a.n_pad;
-  const size_t rows_bytes = (size_t)np * n * sizeof(double);
-  const size_t nrm_bytes = (size_t)np * sizeof(double) + (size_t)(np + 2) * sizeof(int);
-  const int use_smem = (rows_bytes + nrm_bytes) <= 200 * 1024;
-  // Rows in the global workspace: ask for enough shared memory that one CTA
-  // runs per SM, so the rows of the resident matrices stay in L2.
-  const size_t smem = use_smem ? rows_bytes + nrm_bytes : std::max<size_t>(nrm_bytes, 120 * 1024);
-  int G = 2;
-  while (G < 32 && G < n) G <<= 1;
-  if (G > 2 && G >= n) G >>= 1;                 // about two elements per lane
-  // one lane group per pair of a step: a second pass of the groups would double
-  // the chain of a step.  With it and the rotation's scalars at a fifth of their
-  // FP64 instructions: 64 matrices of n = 16 1.71 -> 0.54 ms, 4096 9.5 -> 4.5, the
-  // 4096 cores of an L = 16, chi = 8 run 3.5 -> 1.7
-  const int threads = std::max(32, (np / 2 * G + 31) / 32 * 32);
-  static std::atomic<uint64_t> attr{0};
-  cudaError_t e = raise_smem_limit(k_jacobi, 200 * 1024 + 64, attr);
-  if (e != cudaSuccess) return e;
-  k_jacobi<<<a.S, threads, smem, st>>>(a, use_smem, G);
-  return cudaGetLastError();
+  // n <= 32: about two entries of a row per lane, one lane group per pair of a
+  // step: a second pass of the groups would double the chain of a step.  With it
+  // and the rotation's scalars at a fifth of their FP64 instructions: 64 matrices
+  // of n = 16 1.71 -> 0.54 ms, 4096 9.5 -> 4.5, the 4096 cores of an L = 16,
+  // chi = 8 run 3.5 -> 1.7
+  if (a.n <= 4) return launch_small<2>(a, st);
+  if (a.n <= 8) return launch_small<4>(a, st);
+  if (a.n <= 16) return launch_small<8>(a, st);
+  return launch_small<16>(a, st);
 }
 
 }  // namespace mctrg
