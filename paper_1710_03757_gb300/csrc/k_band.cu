@@ -1116,24 +1116,26 @@ __global__ void __launch_bounds__(kChaseWarps * 32) k_band_chase(BandArgs a, int
 }
 
 // ---------------------------------------------------------------------------
-// v = P1 P2 v_B for a group of up to 16 kept vectors of one matrix, one CTA of 128
-// threads; the vectors in shared memory (row stride n + 1: the 16 vectors in
-// different banks).  P2: the chase's sweeps in reverse order; the right
+// v = P1 P2 v_B for a group of up to GV kept vectors of one matrix, one CTA of 128
+// threads; the vectors in shared memory (row stride n + 1: the vectors in
+// different banks).  GV is 16, or 4 where groups of 16 are fewer than the SMs (the
+// same sums either way; 16 matrices of n = 576, 24 vectors: 5.0 -> 2.6 ms).  P2: the chase's sweeps in reverse order; the right
 // reflectors of one sweep act on disjoint column blocks c0 = i + 1 + 8q, so
 // they commute and are applied at once, one (reflector, vector) pair per
 // thread.  P1: the panels' compact reflectors in reverse order,
 // v <- v - U^T T_U U v: U staged in shared memory, thread (a, j) forms
-// (U v_a)_j, then (T_U U v_a)_j, then thread (a, part) updates every eighth
-// entry of v_a.
+// (U v_a)_j, then (T_U U v_a)_j, then the threads (a, part) update
+// v_a.
 constexpr int kBtThreads = 128;
+template <int GV>
 __global__ void __launch_bounds__(kBtThreads) k_band_backtr(BandArgs a, BandVecArgs va, int nref) {
-  extern __shared__ double Vs[];                     // [16][n+1], then U [8][n]
-  __shared__ double tv[16][B + 1], tp[16][B + 1];
+  extern __shared__ double Vs[];                     // [GV][n+1], then U [8][n]
+  __shared__ double tv[GV][B + 1], tp[GV][B + 1];
   const int s = blockIdx.x, n = a.n, t = threadIdx.x;
   const int ld = n + 1;
-  double* Us = Vs + (size_t)16 * ld;
-  const int g0 = 16 * blockIdx.y;                     // first kept vector of this group
-  const int nk = min(va.nk[s] - g0, 16);
+  double* Us = Vs + (size_t)GV * ld;
+  const int g0 = GV * blockIdx.y;                     // first kept vector of this group
+  const int nk = min(va.nk[s] - g0, GV);
   if (nk <= 0) return;
   double* vrow = va.vrows + ((size_t)s * va.kstride + g0) * n;
   for (int e = t; e < nk * n; e += kBtThreads) Vs[(e / n) * ld + e % n] = vrow[e];
@@ -1166,7 +1168,7 @@ __global__ void __launch_bounds__(kBtThreads) k_band_backtr(BandArgs a, BandVecA
     __syncthreads();
   }
   const double* Ad = (const double*)(a.Wk + (size_t)s * n * n);
-  const int av = t & 15, hj = t >> 4;                 // vector, and j (or the part of the columns)
+  const int av = t & (GV - 1), hj = t / GV;           // vector, and j (or the part of the columns)
   for (int k = n - 2 * B; k >= 0 && nk > 0; k -= B) {
     const int cb = k + B, mp = n - cb;
     for (int e = t; e < B * mp; e += kBtThreads) {
@@ -1174,7 +1176,7 @@ __global__ void __launch_bounds__(kBtThreads) k_band_backtr(BandArgs a, BandVecA
       Us[j * n + c] = Ad[(size_t)(k + j) * n + cb + c];
     }
     __syncthreads();
-    if (av < nk) {                                    // (U v_a)_j
+    if (av < nk && hj < B) {                          // (U v_a)_j
       const double* x = Vs + (size_t)av * ld + cb;
       const double* u = Us + (size_t)hj * n;
       double acc = 0.0;
@@ -1182,7 +1184,7 @@ __global__ void __launch_bounds__(kBtThreads) k_band_backtr(BandArgs a, BandVecA
       tv[av][hj] = acc;
     }
     __syncthreads();
-    if (av < nk) {                                    // (T_U U v_a)_i, T_U upper triangular
+    if (av < nk && hj < B) {                          // (T_U U v_a)_i, T_U upper triangular
       double acc = 0.0;
       for (int j = hj; j < B; ++j) acc = fma(Ad[(size_t)(k + hj) * n + k + j], tv[av][j], acc);
       tp[av][hj] = acc;
@@ -1193,7 +1195,7 @@ __global__ void __launch_bounds__(kBtThreads) k_band_backtr(BandArgs a, BandVecA
       double tq[B];
 #pragma unroll
       for (int j = 0; j < B; ++j) tq[j] = tp[av][j];
-      for (int c = hj; c < mp; c += B) {
+      for (int c = hj; c < mp; c += kBtThreads / GV) {
         double y = x[c];
 #pragma unroll
         for (int j = 0; j < B; ++j) y = fma(-Us[j * n + c], tq[j], y);
@@ -1268,17 +1270,22 @@ cudaError_t launch_band_chase(const BandArgs& a, cudaStream_t st) {
   return launch_chase<16>(a, 2 * per <= kCap ? 2 : 1, st);
 }
 
-cudaError_t launch_band_backtr(const BandVecArgs& va, cudaStream_t st) {
+template <int GV>
+static cudaError_t launch_backtr(const BandVecArgs& va, cudaStream_t st) {
   const BandArgs& a = *va.band;
-  if (a.S <= 0) return cudaSuccess;
   static std::atomic<uint64_t> at{0};
-  auto bytes = [](int n) { return (size_t)(24 * n + 16) * sizeof(double); };
-  const size_t smem = bytes(a.n);
-  cudaError_t e = raise_smem_limit(k_band_backtr, (int)bytes(kBandMaxN), at);
+  auto bytes = [](int n) { return (size_t)((GV + B) * n + GV) * sizeof(double); };
+  cudaError_t e = raise_smem_limit(k_band_backtr<GV>, (int)bytes(kBandMaxN), at);
   if (e != cudaSuccess) return e;
-  const dim3 grid((unsigned)a.S, (unsigned)((std::max(1, va.kmax) + 15) / 16));
-  k_band_backtr<<<grid, kBtThreads, smem, st>>>(a, va, band_nref(a.n));
+  const dim3 grid((unsigned)a.S, (unsigned)((std::max(1, va.kmax) + GV - 1) / GV));
+  k_band_backtr<GV><<<grid, kBtThreads, bytes(a.n), st>>>(a, va, band_nref(a.n));
   return cudaGetLastError();
+}
+
+cudaError_t launch_band_backtr(const BandVecArgs& va, cudaStream_t st) {
+  const int64_t S = va.band->S;
+  if (S <= 0) return cudaSuccess;
+  return S * ((std::max(1, va.kmax) + 15) / 16) < 152 ? launch_backtr<4>(va, st) : launch_backtr<16>(va, st);
 }
 
 }  // namespace mctrg

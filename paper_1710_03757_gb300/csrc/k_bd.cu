@@ -1122,24 +1122,40 @@ __global__ void __launch_bounds__(128) k_bd_backtr(BdVecArgs a, int gs) {
       if (taur == 0.0) continue;
       const double* u = R + (size_t)k * n;           // u[k+1] = 1, u[k+2..n-1] stored
       double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0;
-      for (int j = k + 1 + lane; j < n; j += 32) {
-        const double uj = (j == k + 1) ? 1.0 : u[j];
-        p0 = fma(uj, V0[j], p0);
-        if (na > 1) p1 = fma(uj, V0[n + j], p1);
-        if (na > 2) p2 = fma(uj, V0[2 * n + j], p2);
-        if (na > 3) p3 = fma(uj, V0[3 * n + j], p3);
+      for (int j0 = k + 1 + lane; j0 < n; j0 += 256) {   // eight loads of the reflector in flight
+        double uu[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) uu[c] = j0 + 32 * c < n ? u[j0 + 32 * c] : 0.0;
+        if (j0 == k + 1) uu[0] = 1.0;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const int j = j0 + 32 * c;
+          if (j >= n) break;
+          p0 = fma(uu[c], V0[j], p0);
+          if (na > 1) p1 = fma(uu[c], V0[n + j], p1);
+          if (na > 2) p2 = fma(uu[c], V0[2 * n + j], p2);
+          if (na > 3) p3 = fma(uu[c], V0[3 * n + j], p3);
+        }
       }
       const double t = reduce4(p0, p1, p2, p3, lane);
       const double w0 = taur * __shfl_sync(0xffffffffu, t, 0);
       const double w1 = taur * __shfl_sync(0xffffffffu, t, 8);
       const double w2 = taur * __shfl_sync(0xffffffffu, t, 16);
       const double w3 = taur * __shfl_sync(0xffffffffu, t, 24);
-      for (int j = k + 1 + lane; j < n; j += 32) {
-        const double uj = (j == k + 1) ? 1.0 : u[j];
-        V0[j] = fma(-w0, uj, V0[j]);
-        if (na > 1) V0[n + j] = fma(-w1, uj, V0[n + j]);
-        if (na > 2) V0[2 * n + j] = fma(-w2, uj, V0[2 * n + j]);
-        if (na > 3) V0[3 * n + j] = fma(-w3, uj, V0[3 * n + j]);
+      for (int j0 = k + 1 + lane; j0 < n; j0 += 256) {
+        double uu[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) uu[c] = j0 + 32 * c < n ? u[j0 + 32 * c] : 0.0;
+        if (j0 == k + 1) uu[0] = 1.0;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const int j = j0 + 32 * c;
+          if (j >= n) break;
+          V0[j] = fma(-w0, uu[c], V0[j]);
+          if (na > 1) V0[n + j] = fma(-w1, uu[c], V0[n + j]);
+          if (na > 2) V0[2 * n + j] = fma(-w2, uu[c], V0[2 * n + j]);
+          if (na > 3) V0[3 * n + j] = fma(-w3, uu[c], V0[3 * n + j]);
+        }
       }
       __syncwarp();
     }
@@ -1280,7 +1296,9 @@ cudaError_t launch_bd_vectors(const BdVecArgs& a, cudaStream_t st) {
 cudaError_t launch_bd_backtr(const BdVecArgs& a, cudaStream_t st) {
   if (a.S <= 0) return cudaSuccess;
   constexpr size_t kSmemCap = 227 * 1024;
-  const int gs = (size_t)16 * a.n * sizeof(double) <= kSmemCap ? 16 : 8;
+  int gs = (size_t)16 * a.n * sizeof(double) <= kSmemCap ? 16 : 8;
+  // groups of four, a warp each, where the larger ones are fewer than the SMs (the same quads of vectors)
+  if ((int64_t)a.S * ((std::max(1, a.kmax) + gs - 1) / gs) < 152) gs = 4;
   const size_t smem = (size_t)gs * a.n * sizeof(double);
   if (smem > kSmemCap) return cudaErrorInvalidValue;
   static std::atomic<uint64_t> attr{0};

@@ -222,22 +222,36 @@ __global__ void __launch_bounds__(128) k_lowrank_expand(LowRankExpandArgs a, int
       if (tau == 0.0) continue;
       const double* u = Vt + (size_t)k * n;
       double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0;
-      for (int j = k + lane; j < n; j += 32) {
-        const double uj = u[j];
-        p0 = fma(uj, V0[j], p0);
-        if (na > 1) p1 = fma(uj, V0[n + j], p1);
-        if (na > 2) p2 = fma(uj, V0[2 * n + j], p2);
-        if (na > 3) p3 = fma(uj, V0[3 * n + j], p3);
+      for (int j0 = k + lane; j0 < n; j0 += 256) {     // eight loads of the reflector in flight
+        double uu[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) uu[c] = j0 + 32 * c < n ? u[j0 + 32 * c] : 0.0;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const int j = j0 + 32 * c;
+          if (j >= n) break;
+          p0 = fma(uu[c], V0[j], p0);
+          if (na > 1) p1 = fma(uu[c], V0[n + j], p1);
+          if (na > 2) p2 = fma(uu[c], V0[2 * n + j], p2);
+          if (na > 3) p3 = fma(uu[c], V0[3 * n + j], p3);
+        }
       }
       const double t = tau * reduce4(p0, p1, p2, p3, lane);
       const double w0 = __shfl_sync(0xffffffffu, t, 0), w1 = __shfl_sync(0xffffffffu, t, 8);
       const double w2 = __shfl_sync(0xffffffffu, t, 16), w3 = __shfl_sync(0xffffffffu, t, 24);
-      for (int j = k + lane; j < n; j += 32) {
-        const double uj = u[j];
-        V0[j] = fma(-w0, uj, V0[j]);
-        if (na > 1) V0[n + j] = fma(-w1, uj, V0[n + j]);
-        if (na > 2) V0[2 * n + j] = fma(-w2, uj, V0[2 * n + j]);
-        if (na > 3) V0[3 * n + j] = fma(-w3, uj, V0[3 * n + j]);
+      for (int j0 = k + lane; j0 < n; j0 += 256) {
+        double uu[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) uu[c] = j0 + 32 * c < n ? u[j0 + 32 * c] : 0.0;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const int j = j0 + 32 * c;
+          if (j >= n) break;
+          V0[j] = fma(-w0, uu[c], V0[j]);
+          if (na > 1) V0[n + j] = fma(-w1, uu[c], V0[n + j]);
+          if (na > 2) V0[2 * n + j] = fma(-w2, uu[c], V0[2 * n + j]);
+          if (na > 3) V0[3 * n + j] = fma(-w3, uu[c], V0[3 * n + j]);
+        }
       }
       __syncwarp();
     }
@@ -280,7 +294,10 @@ cudaError_t launch_lowrank_expand(const LowRankExpandArgs& a, cudaStream_t st) {
   if (a.S <= 0) return cudaSuccess;
   if (!lowrank_supported(a.n, a.K)) return cudaErrorInvalidValue;
   constexpr size_t kCap = 200 * 1024;
-  const int gs = (size_t)16 * a.n * sizeof(double) <= kCap ? 16 : 8;   // n <= 2304: 8 vectors take 147 KB
+  int gs = (size_t)16 * a.n * sizeof(double) <= kCap ? 16 : 8;   // n <= 2304: 8 vectors take 147 KB
+  // groups of four, a warp each, where the larger ones are fewer than the SMs (the same quads of vectors; 32
+  // matrices of n = 576, 24 vectors: 3.2 -> 3.0 ms, and 1.7 with eight loads of a reflector in flight)
+  if ((int64_t)a.S * 2 * ((a.kc + gs - 1) / gs) < 152) gs = 4;
   const size_t smem = (size_t)std::min(gs, a.kc) * a.n * sizeof(double);
   static std::atomic<uint64_t> attr{0};
   cudaError_t e = raise_smem_limit(k_lowrank_expand, (int)kCap, attr);
