@@ -11,12 +11,12 @@
 // The one-sided Jacobi that these levels took before works on all of M: 18.6 ms
 // for 4096 matrices of n = 64, 23.3 ms for 768 of n = 144 (both K = 16), 424 ms
 // for 32 of n = 576 (K = 256; one matrix per CTA).  Now, for the same levels:
-// the QR of both factors 1.0, 0.5 and 11 ms, the cores' SVD 3.5 ms and 0.9 ms
-// (K = 16, Jacobi) and 13 ms (K = 256, bidiagonalization and bisection), the
-// expansion 0.4, 0.25 and 7 ms; and the n x n product goes, since only the
-// core is needed.  Whole runs: L = 16, chi = 8, 256 trajectories 50.6 -> 35.6
-// ms; chi = 12, 48 trajectories 60.3 -> 36.7; chi = 24, 8 trajectories 556 ->
-// 149.
+// the QR of both factors 1.0, 0.42 and 11 ms, the cores' SVD 1.7 ms and 0.45 ms
+// (K = 16, Jacobi) and 13 ms (K = 256, two-stage reduction and bisection), the
+// expansion 0.4, 0.24 and 1.7 ms; and the n x n product goes, since only the
+// core is needed.  Whole runs when this came: L = 16, chi = 8, 256 trajectories
+// 50.6 -> 35.6 ms; chi = 12, 48 trajectories 60.3 -> 36.7; chi = 24, 8
+// trajectories 556 -> 149.
 #include <algorithm>
 
 #include "common.cuh"
