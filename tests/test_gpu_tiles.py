@@ -62,6 +62,18 @@ def test_tensor_core_products_at_the_edges(torch, K):
     assert (M.cpu().numpy()[ref == 0] == 0).all()
 
 
+@pytest.mark.parametrize("over", ["X", "Yt"])
+def test_tensor_core_product_over_an_operand(torch, over):
+    # D = 16, K = 256: the result has the operands' shape and may be written over one of them
+    rng = np.random.default_rng(3)
+    X, Y = (torch.tensor(rng.standard_normal((40, 256, 256)), device="cuda") for _ in range(2))
+    ref = torch.empty_like(X)
+    assert mctrg.mctrg_contract_batched(X, Y, ref, precision=mctrg.MCTRG_FP64TC) == mctrg.MCTRG_OK
+    out = X if over == "X" else Y
+    assert mctrg.mctrg_contract_batched(X, Y, out, precision=mctrg.MCTRG_FP64TC) == mctrg.MCTRG_OK
+    assert torch.equal(out, ref)
+
+
 @pytest.mark.parametrize("chi,svd", [(8, mctrg.SVD_BIDIAG), (9, mctrg.SVD_AUTO), (12, mctrg.SVD_AUTO),
                                      (16, mctrg.SVD_AUTO)])
 def test_few_trajectories_equal_the_same_of_many(torch, chi, svd):
