@@ -167,10 +167,9 @@ extern "C" int mctrg_reset_kernel_stats(mctrg_ctx_t c) {
 
 size_t mctrg_ctx::held_bytes() const {
   const DevBuf* all[] = {&T0, &shM, &shW, &shSig, &shPerm, &shLns1, &shU, &shH, &Hbuf[0], &Hbuf[1],
-                         &Mb, &Wb, &Xb, &Yb, &sigb, &permb, &nnzb, &ilns1, &iflags, &lnacc, &tflags,
+                         &workb, &Xb, &Yb, &sigb, &permb, &nnzb, &ilns1, &iflags, &lnacc, &tflags,
                          &scratch, &o_lnabs, &o_sign, &o_flags, &o_tflags, &stats, &tcXh, &tcYh, &tcXl,
-                         &tcYl, &tcScale, &tcErr, &ozExp, &Timp, &bdb, &keptb, &sigtb, &nkb, &vrowsb, &bdscr,
-                         &lrb};
+                         &tcYl, &tcScale, &tcErr, &ozExp, &Timp, &bdb, &keptb, &sigtb, &nkb, &vrowsb, &bdscr};
   size_t b = 0;
   for (const DevBuf* d : all) b += d->bytes;
   return b;
@@ -181,10 +180,9 @@ void mctrg_ctx::release_all() {
   for (cudaEvent_t e : event_pool) cudaEventDestroy(e);
   event_pool.clear();
   DevBuf* all[] = {&T0, &shM, &shW, &shSig, &shPerm, &shLns1, &shU, &shH, &Hbuf[0], &Hbuf[1],
-                   &Mb, &Wb, &Xb, &Yb, &sigb, &permb, &nnzb, &ilns1, &iflags, &lnacc, &tflags,
+                   &workb, &Xb, &Yb, &sigb, &permb, &nnzb, &ilns1, &iflags, &lnacc, &tflags,
                    &scratch, &o_lnabs, &o_sign, &o_flags, &o_tflags, &stats, &tcXh, &tcYh, &tcXl,
-                   &tcYl, &tcScale, &tcErr, &ozExp, &Timp, &bdb, &keptb, &sigtb, &nkb, &vrowsb, &bdscr,
-                   &lrb};
+                   &tcYl, &tcScale, &tcErr, &ozExp, &Timp, &bdb, &keptb, &sigtb, &nkb, &vrowsb, &bdscr};
   for (DevBuf* b : all) b->release();
 }
 
@@ -430,21 +428,6 @@ extern "C" int mctrg_init_tensor(mctrg_ctx_t c, const double* T0, int D, int L, 
 }
 
 // ---------------------------------------------------------------------------
-// Device bytes of one item's tensor-core operands (X and Yt, n x d2 each):
-// the rounded operands (and residuals) of the mixed modes, or the row exponents
-// of the FP64-accurate mode.
-static size_t tc_operand_bytes(int prec, int n, int d2) {
-  const size_t e = (size_t)n * d2;
-  switch (prec) {
-    case MCTRG_TF32: return 2 * 4 * e;
-    case MCTRG_BF16: return 2 * 2 * e;
-    case MCTRG_TF32X3: return 2 * 2 * 4 * e;
-    case MCTRG_BF16X3: return 2 * 2 * 2 * e;
-    case MCTRG_FP64TC: return gemm_ozaki_supported(n, d2) ? 2 * (size_t)n * sizeof(int) : 0;
-    default: return 0;
-  }
-}
-
 namespace mctrg {
 SvdDims svd_dims(const mctrg_options& o, const LevelInfo& a, int K) {
   if (route_lowrank(o, a.n, K)) return SvdDims{true, K, K + (K & 1)};
@@ -465,6 +448,76 @@ size_t run_sample_scratch(const std::vector<LevelInfo>& lv, int s0, int nlev, in
   return m;
 }
 
+// What a run holds for one item of a sub-batch and for one trajectory of a
+// chunk, from which plan_run plans and mctrg_ctx::run allocates.  At each level
+// the operands X and Yt, the split's matrices, their working copies and a
+// low-rank level's reflectors and core halves (each doubles per item) share one
+// array (RunWork below); every other array is held at its largest over the levels.
+struct RunSizes {
+  size_t work = 0;                  // doubles of the shared array
+  size_t tc_elems = 0, oz_rows = 0; // elements of a rounded operand, row exponents
+  size_t np = 0, bd_n = 0;          // padded side; side on the bidiagonalization route
+  bool band = false;
+  size_t halves[2] = {0, 0};        // doubles per trajectory: levels s0, s0+2, ... and the others
+  size_t items = 0, final_xy = 0;   // items per trajectory; doubles of the last contraction's X (and Yt)
+};
+
+// The shared array of S items: X, Yt, M, W and the low-rank arrays in turn, each from a 256-byte boundary.
+struct RunWork {
+  size_t off[6];
+  RunWork(int64_t S, size_t xy, size_t m, size_t w, size_t lr) {
+    const size_t per[5] = {xy, xy, m, w, lr};
+    off[0] = 0;
+    for (int i = 0; i < 5; ++i) off[i + 1] = off[i] + (((size_t)S * per[i] + 31) & ~(size_t)31);
+  }
+  static constexpr size_t kSlack = 5 * 31;   // most doubles that the boundaries add
+  size_t doubles() const { return off[5]; }
+};
+static RunWork level_work(const LevelInfo& a, const SvdDims& v, size_t d2, int64_t S) {
+  return RunWork(S, (size_t)a.n * d2, (size_t)v.n * v.n, (size_t)v.n_pad * v.n,
+                 v.lowrank ? lowrank_item_doubles(a.n, v.n, a.kc) : 0);
+}
+// Level 0 of a lattice with impurities: its own matrices, no operands.
+static RunWork level0_work(const LevelInfo& a, int64_t S) {
+  return RunWork(S, 0, (size_t)a.n * a.n, (size_t)a.n_pad * a.n, 0);
+}
+
+static int tc_kind_of(int prec) { return (prec == MCTRG_TF32 || prec == MCTRG_TF32X3) ? 0 : 1; }
+static int tc_passes_of(int prec) { return (prec == MCTRG_TF32X3 || prec == MCTRG_BF16X3) ? 3 : 1; }
+static bool tc_mode_of(int prec) { return prec != MCTRG_FP64 && prec != MCTRG_FP64TC; }
+
+static RunSizes run_sizes(const std::vector<LevelInfo>& lv, int s0, int nlev, const mctrg_options& opt) {
+  RunSizes r;
+  for (int k = s0; k < nlev; ++k) {
+    const LevelInfo& a = lv[k];
+    size_t& h = r.halves[(k - s0) & 1];
+    h = std::max(h, (size_t)a.N * 2 * a.n * a.kc);
+    r.items = std::max(r.items, (size_t)a.N);
+    if (k == s0) {   // split per item in a lattice with impurities
+      r.work = (size_t)a.n * a.n + (size_t)a.n_pad * a.n;
+      r.np = a.n_pad;
+      continue;
+    }
+    const int d2 = lv[k - 1].D * lv[k - 1].D;
+    const SvdDims v = svd_dims(opt, a, d2);
+    const size_t d = 2 * (size_t)a.n * d2 + (size_t)v.n * v.n + (size_t)v.n_pad * v.n +
+                     (v.lowrank ? lowrank_item_doubles(a.n, v.n, a.kc) : 0);
+    r.work = std::max(r.work, d);
+    r.np = std::max<size_t>(r.np, v.n_pad);
+    if (!v.lowrank && tc_mode_of(opt.precision) && gemm_tc_supported(a.n, d2, tc_kind_of(opt.precision)))
+      r.tc_elems = std::max(r.tc_elems, (size_t)a.n * d2);
+    if (!v.lowrank && opt.precision == MCTRG_FP64TC && gemm_ozaki_supported(a.n, d2))
+      r.oz_rows = std::max(r.oz_rows, (size_t)a.n);
+    if (route_bidiag(opt, v.n, d2)) {
+      r.bd_n = std::max<size_t>(r.bd_n, v.n);
+      r.band = r.band || route_band(opt, v.n, d2);
+    }
+  }
+  const LevelInfo& fl = lv[nlev - 1];
+  r.final_xy = (size_t)fl.kc * fl.kc * fl.n;
+  return r;
+}
+
 // Memory plan of a run of n_samples trajectories over levels s0 .. nlev-1 of
 // lv (sampled; the shared prefix is held separately): B trajectories per
 // chunk, S items per sub-batch, and the device bytes the run holds.  At most
@@ -473,47 +526,31 @@ size_t run_sample_scratch(const std::vector<LevelInfo>& lv, int s0, int nlev, in
 // B < 1 means that not even one trajectory fits.
 void plan_run(const std::vector<LevelInfo>& lv, int s0, int nlev, int chi, const mctrg_options& opt,
               size_t budget, int64_t n_samples, int64_t& B, int64_t& S, size_t& total) {
-  size_t per_traj = 2 * sizeof(double) + sizeof(uint32_t);   // lnacc, tflags
-  size_t max_pair = 0, max_items = 0, per_item = 0, bd_scr = 0;
+  const RunSizes r = run_sizes(lv, s0, nlev, opt);
+  const size_t ks = kept_stride(chi);
+  size_t bd_scr = 0;
   int64_t maxN = 1;
-  for (int k = s0; k < nlev; ++k) {
-    const LevelInfo& a = lv[k];
-    size_t hk = (size_t)a.N * 2 * a.n * a.kc * sizeof(double);
-    size_t hp = (k > s0) ? (size_t)lv[k - 1].N * 2 * lv[k - 1].n * lv[k - 1].kc * sizeof(double) : 0;
-    max_pair = std::max(max_pair, hk + hp);
-    max_items = std::max(max_items, (size_t)a.N);
-    if (k > s0) {
-      maxN = std::max<int64_t>(maxN, a.N);
-      const size_t d2 = (size_t)lv[k - 1].D * lv[k - 1].D;
-      const SvdDims v = svd_dims(opt, a, (int)d2);      // the split's matrices: the level's, or its cores
-      size_t pi = (2 * (size_t)a.n * d2 + (size_t)v.n * v.n + (size_t)v.n_pad * v.n + v.n_pad) * sizeof(double) +
-                  (v.n_pad + 1) * sizeof(int) + sizeof(double) + sizeof(uint32_t);
-      if (v.lowrank) pi += lowrank_item_doubles(a.n, v.n, a.kc) * sizeof(double);
-      else pi += tc_operand_bytes(opt.precision, a.n, (int)d2);
-      if (route_bidiag(opt, v.n, (int)d2)) {   // d, e, tau; kept values and vectors
-        const size_t ks = kept_stride(chi);
-        pi += (3 * (size_t)v.n + ks + ks * (size_t)v.n) * sizeof(double) + (ks + 1) * sizeof(int);
-        bd_scr = std::max(bd_scr, bd_vectors_scratch_doubles(v.n, 1 << 16, a.kc) * sizeof(double));
-        // (the band route's own buffers take the place of X and Yt)
-      }
-      per_item = std::max(per_item, pi);
-    }
+  for (int k = s0 + 1; k < nlev; ++k) {
+    maxN = std::max<int64_t>(maxN, lv[k].N);
+    const int d2 = lv[k - 1].D * lv[k - 1].D, n = svd_dims(opt, lv[k], d2).n;
+    if (route_bidiag(opt, n, d2))
+      bd_scr = std::max(bd_scr, bd_vectors_scratch_doubles(n, 1 << 16, lv[k].kc) * sizeof(double));
   }
-  {  // final contraction X, Yt per trajectory
-    const LevelInfo& a = lv[nlev - 1];
-    size_t fin = 2 * (size_t)a.kc * a.kc * a.n * sizeof(double);
-    per_traj += fin;
-  }
-  per_traj += max_pair + max_items * (sizeof(double) + sizeof(uint32_t));
-  {  // level s0 split per item (a lattice with impurities): its matrices, rows and values
-    const LevelInfo& a = lv[s0];
-    per_item = std::max(per_item, ((size_t)a.n * a.n + (size_t)a.n_pad * a.n + a.n_pad) * sizeof(double) +
-                                      (a.n_pad + 1) * sizeof(int) + sizeof(double) + sizeof(uint32_t));
-  }
-  const size_t tables = run_sample_scratch(lv, s0, nlev, chi) * sizeof(double) + bd_scr;
+  size_t per_item = (r.work + r.np) * sizeof(double) + (r.np + 1) * sizeof(int);   // sigma, order, nonzero count
+  // d, e, tau; kept values and vectors (the band route's own buffers take the place of X and Yt)
+  if (r.bd_n) per_item += (3 * r.bd_n + ks + ks * r.bd_n) * sizeof(double) + (ks + 1) * sizeof(int);
+  if (tc_mode_of(opt.precision))
+    per_item += 2 * sizeof(double) + 2 * (tc_passes_of(opt.precision) == 3 ? 2 : 1) *
+                                         (tc_kind_of(opt.precision) == 0 ? 4 : 2) * r.tc_elems;
+  per_item += 2 * r.oz_rows * sizeof(int);
+  const size_t per_traj = 2 * sizeof(double) + sizeof(uint32_t) +                   // lnacc, tflags
+                          2 * r.final_xy * sizeof(double) + (r.halves[0] + r.halves[1]) * sizeof(double) +
+                          r.items * (sizeof(double) + sizeof(uint32_t));
+  const size_t tables =
+      run_sample_scratch(lv, s0, nlev, chi) * sizeof(double) + bd_scr + RunWork::kSlack * sizeof(double);
   const int64_t Bmax = opt.max_chunk > 0 ? std::min<int64_t>(opt.max_chunk, n_samples) : n_samples;
   const size_t work_budget = std::max<size_t>(budget / 4, 1);
-  S = per_item ? (int64_t)std::max<size_t>(1, std::min<size_t>(work_budget / per_item, 1 << 16)) : 1;
+  S = (int64_t)std::max<size_t>(1, std::min<size_t>(work_budget / per_item, 1 << 16));
   S = std::max<int64_t>(1, std::min<int64_t>(S, Bmax * maxN));   // no more than a level's items
   const size_t work = per_item * (size_t)S + tables;
   const size_t rest = budget > work ? budget - work : 0;
@@ -524,8 +561,10 @@ void plan_run(const std::vector<LevelInfo>& lv, int s0, int nlev, int chi, const
 
 // The same plan for a lattice not yet set up, from the largest leg dimensions
 // its levels can have (D' = min(chi, D^2) from D0, sampling from the first
-// level with D^2 > chi): an upper bound of what plan_run gives after
-// mctrg_init_*, where ranks can only be smaller and exact levels longer.
+// level with D^2 > chi).  After mctrg_init_* ranks can only be smaller and exact
+// levels longer, so plan_run needs no more, save where a smaller leg of the
+// parents makes a level low-rank (at most 1.3 times the array of an item, legs
+// 15 -> 16); a context plans anew within the budget that it is given.
 void plan_run_bound(int L, int chi, int D0, const mctrg_options& opt, size_t budget, int64_t n_samples,
                     int64_t& B, int64_t& S, size_t& total) {
   int m = 0;
@@ -622,95 +661,58 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
     CK(lnacc.ensure(sizeof(double) * (size_t)B));
     const int grid_s = run_sample_grid(lv, s0, nlev, chi);
     const int ks = kept_stride(chi);
-    size_t max_h = 0, max_items = 0, max_xy = 0, max_m = 0, max_w = 0, max_np = 0, max_scr = 0, max_lr = 0;
+    const RunSizes rs = run_sizes(lv, s0, nlev, opt);
+    size_t max_scr = 0, work = 2 * (((size_t)B * rs.final_xy + 31) & ~(size_t)31);
     for (int k = s0; k < nlev; ++k) {
-      const LevelInfo& a = lv[k];
-      max_h = std::max(max_h, (size_t)B * a.N * 2 * a.n * a.kc);
-      max_items = std::max(max_items, (size_t)B * a.N);
-      max_scr = std::max(max_scr, sample_scratch_doubles(a.n, chi, grid_s));
-      if (k > s0) {
-        const size_t d2 = (size_t)lv[k - 1].D * lv[k - 1].D;
-        const SvdDims v = svd_dims(opt, a, (int)d2);
-        max_xy = std::max(max_xy, (size_t)S * a.n * d2);
-        max_m = std::max(max_m, (size_t)S * v.n * v.n);
-        max_w = std::max(max_w, (size_t)S * v.n_pad * v.n);
-        max_np = std::max(max_np, (size_t)S * v.n_pad);
-        if (v.lowrank) max_lr = std::max(max_lr, (size_t)S * lowrank_item_doubles(a.n, v.n, a.kc));
+      max_scr = std::max(max_scr, sample_scratch_doubles(lv[k].n, chi, grid_s));
+      if (k == s0) {
+        if (level0_distinct) work = std::max(work, level0_work(lv[0], S).doubles());
+        continue;
       }
+      const int d2 = lv[k - 1].D * lv[k - 1].D;
+      work = std::max(work, level_work(lv[k], svd_dims(opt, lv[k], d2), d2, S).doubles());
     }
-    {
-      const LevelInfo& a = lv[nlev - 1];
-      max_xy = std::max(max_xy, (size_t)B * a.kc * a.kc * a.n);
-    }
-    if (level0_distinct) {   // level 0's own matrices, SVD and sampling per item
-      const LevelInfo& a = lv[0];
-      max_m = std::max(max_m, (size_t)S * a.n * a.n);
-      max_w = std::max(max_w, (size_t)S * a.n_pad * a.n);
-      max_np = std::max(max_np, (size_t)S * a.n_pad);
-      max_items = std::max(max_items, (size_t)B * a.N);
-    }
-    CK(Hbuf[0].ensure(sizeof(double) * max_h));
-    CK(Hbuf[1].ensure(sizeof(double) * max_h));
-    CK(iflags.ensure(sizeof(uint32_t) * max_items));
-    CK(ilns1.ensure(sizeof(double) * max_items));
-    CK(Xb.ensure(sizeof(double) * std::max<size_t>(max_xy, 1)));
-    CK(Yb.ensure(sizeof(double) * std::max<size_t>(max_xy, 1)));
-    CK(Mb.ensure(sizeof(double) * std::max<size_t>(max_m, 1)));
-    CK(Wb.ensure(sizeof(double) * std::max<size_t>(max_w, 1)));
-    CK(sigb.ensure(sizeof(double) * std::max<size_t>(max_np, 1)));
-    CK(permb.ensure(sizeof(int) * std::max<size_t>(max_np, 1)));
+    for (int q = 0; q < 2; ++q) CK(Hbuf[q].ensure(sizeof(double) * (size_t)B * rs.halves[q]));
+    CK(iflags.ensure(sizeof(uint32_t) * (size_t)B * rs.items));
+    CK(ilns1.ensure(sizeof(double) * (size_t)B * rs.items));
+    CK(workb.ensure(sizeof(double) * work));
+    CK(sigb.ensure(sizeof(double) * (size_t)S * rs.np));
+    CK(permb.ensure(sizeof(int) * (size_t)S * rs.np));
     CK(nnzb.ensure(sizeof(int) * std::max<int64_t>(S, 1)));
     CK(scratch.ensure(sizeof(double) * max_scr));
-    CK(lrb.ensure(sizeof(double) * max_lr));
-    bool any_band = false;
-    {  // bidiagonalization route buffers (levels that take it)
-      size_t bd_n = 0, bd_scr = 0;
+    if (rs.bd_n) {  // bidiagonalization route buffers (levels that take it)
+      size_t bd_scr = 0;
       for (int k = s0 + 1; k < nlev; ++k) {
-        const LevelInfo& a = lv[k];
-        const int Kd = lv[k - 1].D * lv[k - 1].D;
-        const SvdDims v = svd_dims(opt, a, Kd);
-        if (!use_bidiag(v.n, Kd)) continue;
-        any_band = any_band || use_band(v.n, Kd);
-        bd_n = std::max(bd_n, (size_t)v.n);
-        bd_scr = std::max(bd_scr, bd_vectors_scratch_doubles(v.n, (int)std::min<int64_t>(S, 1 << 16), a.kc));
+        const int Kd = lv[k - 1].D * lv[k - 1].D, nk = svd_dims(opt, lv[k], Kd).n;
+        if (use_bidiag(nk, Kd))
+          bd_scr = std::max(bd_scr, bd_vectors_scratch_doubles(nk, (int)std::min<int64_t>(S, 1 << 16), lv[k].kc));
       }
-      if (bd_n) {
-        const size_t Ss = (size_t)std::max<int64_t>(S, 1);
-        CK(bdb.ensure(sizeof(double) * Ss * 3 * bd_n));
-        CK(keptb.ensure(sizeof(int) * Ss * ks));
-        CK(sigtb.ensure(sizeof(double) * Ss * ks));
-        CK(nkb.ensure(sizeof(int) * Ss));
-        CK(vrowsb.ensure(sizeof(double) * Ss * ks * bd_n));
-        CK(bdscr.ensure(sizeof(double) * bd_scr));
-      }
+      const size_t Ss = (size_t)S;
+      CK(bdb.ensure(sizeof(double) * Ss * 3 * rs.bd_n));
+      CK(keptb.ensure(sizeof(int) * Ss * ks));
+      CK(sigtb.ensure(sizeof(double) * Ss * ks));
+      CK(nkb.ensure(sizeof(int) * Ss));
+      CK(vrowsb.ensure(sizeof(double) * Ss * ks * rs.bd_n));
+      CK(bdscr.ensure(sizeof(double) * bd_scr));
     }
     // tensor-core operands (mixed precision): per item X and Yt rounded, with scales
     const int prec = opt.precision;
     const bool oz_mode = prec == MCTRG_FP64TC;    // FP64-accurate tensor-core GEMM (FP16 slices)
-    const bool tc_mode = prec != MCTRG_FP64 && !oz_mode;
-    const int tc_kind = (prec == MCTRG_TF32 || prec == MCTRG_TF32X3) ? 0 : 1;
-    const int tc_passes = (prec == MCTRG_TF32X3 || prec == MCTRG_BF16X3) ? 3 : 1;
+    const bool tc_mode = tc_mode_of(prec);
+    const int tc_kind = tc_kind_of(prec), tc_passes = tc_passes_of(prec);
     const size_t tc_esize = tc_kind == 0 ? 4 : 2;
     if (tc_mode) {
-      const size_t elems = std::max<size_t>(max_xy, 1);
+      const size_t elems = (size_t)S * rs.tc_elems;
       CK(tcXh.ensure(tc_esize * elems));
       CK(tcYh.ensure(tc_esize * elems));
       if (tc_passes == 3) {
         CK(tcXl.ensure(tc_esize * elems));
         CK(tcYl.ensure(tc_esize * elems));
       }
-      CK(tcScale.ensure(sizeof(double) * 2 * std::max<int64_t>(S, 1)));
+      CK(tcScale.ensure(sizeof(double) * 2 * S));
     }
-    if (oz_mode) {   // row exponents
-      size_t oz_rows = 0;
-      for (int k = s0 + 1; k < nlev; ++k) {
-        const int Kd = lv[k - 1].D * lv[k - 1].D;
-        if (route_lowrank(opt, lv[k].n, Kd) || !gemm_ozaki_supported(lv[k].n, Kd)) continue;
-        oz_rows = std::max(oz_rows, (size_t)S * lv[k].n);
-      }
-      if (oz_rows) CK(ozExp.ensure(sizeof(int) * 2 * oz_rows));
-    }
-    if (prec != MCTRG_FP64 || any_band) {
+    if (rs.oz_rows) CK(ozExp.ensure(sizeof(int) * 2 * (size_t)S * rs.oz_rows));   // row exponents
+    if (prec != MCTRG_FP64 || rs.band) {
       CK(tcErr.ensure(sizeof(uint32_t)));
       CK(cudaMemsetAsync(tcErr.p, 0, sizeof(uint32_t), st));
     }
@@ -724,14 +726,17 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
       if (level0_distinct) {  // level 0 of a lattice with impurities: every tensor split on its own
         const LevelInfo& a = lv[0];
         const int64_t items = Bc * a.N;
+        const RunWork wk = level0_work(a, S);
+        double* const Mb = workb.as<double>() + wk.off[2];
+        double* const Wb = workb.as<double>() + wk.off[3];
         CK(cudaMemsetAsync(iflags.p, 0, sizeof(uint32_t) * items, st));
         for (int64_t i0 = 0; i0 < items; i0 += S) {
           const int64_t Si = std::min(S, items - i0);
           CK(timed(MCTRG_K_OTHER, Si, 0.0, 8.0 * Si * a.n * a.n, [&] {
             return launch_level0_matrices(T0.as<double>(), Timp.as<double>(), imp0, imp1, L, i0, Si, a.N,
-                                          Mb.as<double>(), st); }));
+                                          Mb, st); }));
           JacobiArgs ja{};
-          ja.M = Mb.as<double>(); ja.W = Wb.as<double>(); ja.sig = sigb.as<double>();
+          ja.M = Mb; ja.W = Wb; ja.sig = sigb.as<double>();
           ja.perm = permb.as<int>(); ja.lns1 = ilns1.as<double>() + i0; ja.nnz = nnzb.as<int>();
           ja.mflags = iflags.as<uint32_t>() + i0; ja.n = a.n; ja.n_pad = a.n_pad; ja.S = (int)Si;
           ja.max_sweeps = opt.max_sweeps;
@@ -740,7 +745,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
           CK(timed(MCTRG_K_JACOBI, Si, Si * ((8.0 / 3.0) * nn * nn * nn + 4.0 * nn * nn * a.kc),
                    8.0 * Si * (nn * nn + (double)a.n_pad * nn + 1.5 * a.n_pad), [&] { return launch_jacobi(ja, st); }));
           SampleArgs sa{};
-          sa.M = Mb.as<double>(); sa.W = Wb.as<double>(); sa.sig = sigb.as<double>(); sa.perm = permb.as<int>();
+          sa.M = Mb; sa.W = Wb; sa.sig = sigb.as<double>(); sa.perm = permb.as<int>();
           sa.nnz = nnzb.as<int>(); sa.Urows = nullptr; sa.n = a.n; sa.n_pad = a.n_pad; sa.chi = chi; sa.kc = a.kc;
           sa.stochastic = 1; sa.shared_svd = 0; sa.item0 = i0; sa.n_items = Si; sa.N = a.N; sa.L = L; sa.level = 0;
           sa.seed = seed; sa.traj0 = traj0; sa.H = Hbuf[cur].as<double>(); sa.h_item0 = 0;
@@ -774,34 +779,38 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
         const int prev = cur;
         cur ^= 1;
         const int64_t items = Bc * a.N;
+        const int Kd = p.D * p.D;
+        const SvdDims v = svd_dims(opt, a, Kd);
+        const RunWork wk = level_work(a, v, Kd, S);
+        double* const work0 = workb.as<double>();
+        double *const Xb = work0, *const Yb = work0 + wk.off[1], *const Mb = work0 + wk.off[2],
+               *const Wb = work0 + wk.off[3];
         CK(cudaMemsetAsync(iflags.p, 0, sizeof(uint32_t) * items, st));
         for (int64_t i0 = 0; i0 < items; i0 += S) {
           const int64_t Si = std::min(S, items - i0);
           XYArgs xa{};
           xa.H = Hbuf[prev].as<double>(); xa.h_item0 = 0; xa.d = p.D; xa.D = p.kc; xa.c0 = i0;
           xa.n_items = Si; xa.Nnew = a.N; xa.Nold = p.N; xa.L = L; xa.level_old = k - 1;
-          xa.fixed_parents = 0; xa.X = Xb.as<double>(); xa.Yt = Yb.as<double>();
-          const int Kd = p.D * p.D;
-          const SvdDims v = svd_dims(opt, a, Kd);
+          xa.fixed_parents = 0; xa.X = Xb; xa.Yt = Yb;
           xa.by_parity = v.lowrank;
           const double D2 = (double)p.kc * p.kc, dd = p.D;
           CK(timed(MCTRG_K_FORM_XY, Si, Si * 4.0 * D2 * dd * dd * dd,
                    8.0 * Si * (4.0 * p.kc * dd * dd + 2.0 * D2 * dd * dd), [&] { return launch_form_xy(xa, st); }));
           const bool used_tc = !v.lowrank && tc_mode && gemm_tc_supported(a.n, Kd, tc_kind);
           const bool used_oz = !v.lowrank && oz_mode && gemm_ozaki_supported(a.n, Kd);
-          double* const lr_vt = lrb.as<double>();       // low-rank levels: reflectors, taus, the cores' halves
+          double* const lr_vt = work0 + wk.off[4];       // low-rank levels: reflectors, taus, the cores' halves
           double* const lr_tau = lr_vt + Si * lowrank_vt_doubles(a.n, Kd);
           double* const lr_h = lr_tau + Si * lowrank_tau_doubles(Kd);
           if (v.lowrank) {
             // QR of both factors, then the K x K core in the place of M
             LowRankQrArgs qa{};
-            qa.X = Xb.as<double>(); qa.Yt = Yb.as<double>(); qa.Vt = lr_vt; qa.taus = lr_tau;
+            qa.X = Xb; qa.Yt = Yb; qa.Vt = lr_vt; qa.taus = lr_tau;
             qa.n = a.n; qa.K = Kd; qa.S = (int)Si;
             const double nd = a.n, kd = Kd;
             CK(timed(MCTRG_K_OTHER, Si, Si * 2.0 * (2.0 * nd * kd * kd - 2.0 / 3.0 * kd * kd * kd),
                      8.0 * Si * 2.0 * (2.0 * nd * kd + kd * kd), [&] { return launch_lowrank_qr(qa, st); }));
             GemmArgs gm{};
-            gm.X = Xb.as<double>(); gm.Yt = Yb.as<double>(); gm.M = Mb.as<double>(); gm.D = p.D; gm.K = Kd;
+            gm.X = Xb; gm.Yt = Yb; gm.M = Mb; gm.D = p.D; gm.K = Kd;
             gm.c0 = 0; gm.n_items = Si; gm.Nnew = 1; gm.L = L; gm.level_new = k; gm.fixed_parity = 0;
             gm.in_stride = (int64_t)a.n * Kd; gm.upper = 1;
             CK(timed(MCTRG_K_GEMM, Si, Si * 2.0 / 3.0 * kd * kd * kd, 8.0 * Si * 2.0 * kd * kd,
@@ -809,8 +818,8 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
           } else if (used_oz) {
             // FP64-accurate on the tensor cores: FP16 digits of X and Yt, exact digit products
             GemmOzArgs ga{};
-            ga.X = Xb.as<double>(); ga.Y = Yb.as<double>(); ga.expX = ozExp.as<int>();
-            ga.M = Mb.as<double>(); ga.D = a.D; ga.n = a.n; ga.K = Kd; ga.c0 = i0; ga.n_items = Si;
+            ga.X = Xb; ga.Y = Yb; ga.expX = ozExp.as<int>();
+            ga.M = Mb; ga.D = a.D; ga.n = a.n; ga.K = Kd; ga.c0 = i0; ga.n_items = Si;
             ga.Nnew = a.N; ga.L = L; ga.level_new = k; ga.fixed_parity = -1;
             ga.err = tcErr.as<uint32_t>();
             CK(timed(MCTRG_K_GEMM, Si, Si * 2.0 * a.n * a.n * Kd, 8.0 * Si * (2.0 * a.n * Kd + 1.0 * a.n * a.n),
@@ -821,13 +830,13 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
             double* sY = sX + Si;
             const int64_t per = (int64_t)a.n * Kd;
             CK(timed(MCTRG_K_FORM_XY, Si, 0.0, Si * per * (16.0 + 2.0 * tc_esize * tc_passes), [&] {
-              cudaError_t e = launch_convert_scaled(Xb.as<double>(), per, Si, tc_kind, tcXh.p,
+              cudaError_t e = launch_convert_scaled(Xb, per, Si, tc_kind, tcXh.p,
                                                     tc_passes == 3 ? tcXl.p : nullptr, sX, st);
               if (e != cudaSuccess) return e;
-              return launch_convert_scaled(Yb.as<double>(), per, Si, tc_kind, tcYh.p,
+              return launch_convert_scaled(Yb, per, Si, tc_kind, tcYh.p,
                                            tc_passes == 3 ? tcYl.p : nullptr, sY, st); }));
             GemmTcArgs ga{};
-            ga.M = Mb.as<double>(); ga.D = a.D; ga.n = a.n; ga.K = Kd; ga.c0 = i0; ga.n_items = Si;
+            ga.M = Mb; ga.D = a.D; ga.n = a.n; ga.K = Kd; ga.c0 = i0; ga.n_items = Si;
             ga.Nnew = a.N; ga.L = L; ga.level_new = k; ga.fixed_parity = -1; ga.scaleX = sX; ga.scaleY = sY;
             ga.passes = tc_passes; ga.err = tcErr.as<uint32_t>();
             CK(timed(MCTRG_K_GEMM, Si, Si * 2.0 * a.n * a.n * Kd,
@@ -835,7 +844,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
               return launch_gemm_tc(ga, tc_kind, tcXh.p, tcYh.p, tcXl.p, tcYl.p, st); }));
           } else {
             GemmArgs gm{};
-            gm.X = Xb.as<double>(); gm.Yt = Yb.as<double>(); gm.M = Mb.as<double>(); gm.D = a.D;
+            gm.X = Xb; gm.Yt = Yb; gm.M = Mb; gm.D = a.D;
             gm.K = Kd; gm.c0 = i0; gm.n_items = Si; gm.Nnew = a.N; gm.L = L; gm.level_new = k;
             gm.fixed_parity = -1;
             CK(timed(MCTRG_K_GEMM, Si, Si * 2.0 * a.n * a.n * gm.K, 8.0 * Si * (2.0 * a.n * gm.K + (double)a.n * a.n),
@@ -846,7 +855,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
                        : (double)a.n * 0x1.0p-52);
           const double nn = v.n;
           SampleArgs sa{};
-          sa.M = Mb.as<double>(); sa.sig = sigb.as<double>(); sa.nnz = nnzb.as<int>(); sa.Urows = nullptr;
+          sa.M = Mb; sa.sig = sigb.as<double>(); sa.nnz = nnzb.as<int>(); sa.Urows = nullptr;
           sa.n = v.n; sa.n_pad = v.n_pad; sa.chi = chi; sa.kc = a.kc; sa.stochastic = 1; sa.shared_svd = 0;
           sa.item0 = i0; sa.n_items = Si; sa.N = a.N; sa.L = L; sa.level = k; sa.seed = seed;
           sa.traj0 = traj0; sa.scratch = scratch.as<double>();
@@ -860,8 +869,8 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
             const bool band = use_band(v.n, Kd);
             BandArgs bda{};
             if (band) {
-              band_carve(Xb.p, Yb.p, v.n, Si, bda);
-              bda.M = Mb.as<double>(); bda.Wk = (int64_t*)Wb.p; bda.bd = bdb.as<double>(); bda.S = (int)Si;
+              band_carve(Xb, Yb, v.n, Si, bda);
+              bda.M = Mb; bda.Wk = (int64_t*)Wb; bda.bd = bdb.as<double>(); bda.S = (int)Si;
               bda.err = band_err;
               CK(timed(MCTRG_K_BAND, Si, Si * (8.0 / 3.0) * nn * nn * nn, 8.0 * Si * (nn * nn + 9.0 * nn),
                        [&] { return launch_band_reduce(bda, false, st); }));
@@ -869,7 +878,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
                        [&] { return launch_band_chase(bda, st); }));
             } else {
               BidiagArgs ba{};
-              ba.M = Mb.as<double>(); ba.W = Wb.as<double>(); ba.bd = bdb.as<double>(); ba.n = v.n; ba.S = (int)Si;
+              ba.M = Mb; ba.W = Wb; ba.bd = bdb.as<double>(); ba.n = v.n; ba.S = (int)Si;
               CK(timed(MCTRG_K_BIDIAG, Si, Si * (8.0 / 3.0) * nn * nn * nn, 8.0 * Si * (2.0 * nn * nn + 3.0 * nn),
                        [&] { return launch_bidiag(ba, st); }));
             }
@@ -882,7 +891,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
             CK(timed(MCTRG_K_SAMPLE, Si, Si * 4.0 * nn * a.kc, 8.0 * Si * (v.n_pad + 2.0 * ks),
                      [&] { return launch_sample_split(sa, st, grid_s); }));
             BdVecArgs va{};
-            va.bd = bdb.as<double>(); va.R = Wb.as<double>(); va.sig = sigb.as<double>(); va.kept = keptb.as<int>();
+            va.bd = bdb.as<double>(); va.R = Wb; va.sig = sigb.as<double>(); va.kept = keptb.as<int>();
             va.nk = nkb.as<int>(); va.vrows = vrowsb.as<double>(); va.scratch = bdscr.as<double>();
             va.n = v.n; va.n_pad = v.n_pad; va.S = (int)Si; va.kmax = a.kc; va.kstride = ks;
             va.skip_backtr = band ? 1 : 0;
@@ -899,7 +908,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
                      [&] { return launch_sample_split(sa, st, grid_s); }));
           } else {
             JacobiArgs ja{};
-            ja.M = Mb.as<double>(); ja.W = Wb.as<double>(); ja.sig = sigb.as<double>();
+            ja.M = Mb; ja.W = Wb; ja.sig = sigb.as<double>();
             ja.perm = permb.as<int>(); ja.lns1 = ilns1.as<double>() + i0; ja.nnz = nnzb.as<int>();
             ja.mflags = iflags.as<uint32_t>() + i0; ja.n = v.n; ja.n_pad = v.n_pad; ja.S = (int)Si;
             ja.max_sweeps = opt.max_sweeps;
@@ -907,7 +916,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
             if (used_tc) ja.noise_u = tc_unit_roundoff(prec);
             CK(timed(MCTRG_K_JACOBI, Si, Si * ((8.0 / 3.0) * nn * nn * nn + 4.0 * nn * nn * a.kc),
                      8.0 * Si * (nn * nn + (double)v.n_pad * nn + 1.5 * v.n_pad), [&] { return launch_jacobi(ja, st); }));
-            sa.mode = 0; sa.W = Wb.as<double>(); sa.perm = permb.as<int>();
+            sa.mode = 0; sa.W = Wb; sa.perm = permb.as<int>();
             CK(timed(MCTRG_K_SAMPLE, Si, Si * (4.0 * nn * a.kc + 2.0 * nn * nn * a.kc),
                      8.0 * Si * (2.0 * nn * nn + 2.0 * nn * a.kc), [&] { return launch_sample_split(sa, st, grid_s); }));
           }
@@ -925,15 +934,17 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
       }
       {  // final contraction and trace
         const LevelInfo& p = lv[nlev - 1];
+        double* const Xb = workb.as<double>();
+        double* const Yb = Xb + (((size_t)B * rs.final_xy + 31) & ~(size_t)31);
         XYArgs xa{};
         xa.H = Hbuf[cur].as<double>(); xa.h_item0 = 0; xa.d = p.D; xa.D = p.kc; xa.c0 = 0;
         xa.n_items = Bc; xa.Nnew = 1; xa.Nold = p.N; xa.L = L; xa.level_old = nlev - 1;
-        xa.fixed_parents = 0; xa.X = Xb.as<double>(); xa.Yt = Yb.as<double>();
+        xa.fixed_parents = 0; xa.X = Xb; xa.Yt = Yb;
         const double D2 = (double)p.kc * p.kc, dd = p.D;
         CK(timed(MCTRG_K_FORM_XY, Bc, Bc * 4.0 * D2 * dd * dd * dd,
                  8.0 * Bc * (4.0 * p.kc * dd * dd + 2.0 * D2 * dd * dd), [&] { return launch_form_xy(xa, st); }));
         CK(timed(MCTRG_K_TRACE, Bc, Bc * 2.0 * D2 * p.n, 8.0 * Bc * 2.0 * D2 * p.n, [&] {
-          return launch_trace(Xb.as<double>(), Yb.as<double>(), (int64_t)p.kc * p.kc * p.n, Bc, lnacc0,
+          return launch_trace(Xb, Yb, (int64_t)p.kc * p.kc * p.n, Bc, lnacc0,
                               lnacc.as<double>(), o_lnabs.as<double>() + c0, o_sign.as<int8_t>() + c0, st); }));
         CK(timed(MCTRG_K_OTHER, Bc, 0.0, 5.0 * Bc, [&] {
           return launch_flags_to_u8(o_tflags.as<uint32_t>(), o_flags.as<uint8_t>() + c0, Bc, prefix_flags, st); }));

@@ -70,13 +70,13 @@ struct mctrg_ctx {
   double const_lnabs = 0.0;
   int const_sign = 0;
   mctrg::DevBuf T0, shM, shW, shSig, shPerm, shLns1, shU, shH;
-  mctrg::DevBuf Hbuf[2], Mb, Wb, Xb, Yb, sigb, permb, nnzb, ilns1, iflags, lnacc, tflags, scratch;
+  mctrg::DevBuf workb;   // a run's operands, matrices, working copies and low-rank arrays, level by level
+  mctrg::DevBuf Hbuf[2], Xb, Yb, sigb, permb, nnzb, ilns1, iflags, lnacc, tflags, scratch;
   mctrg::DevBuf o_lnabs, o_sign, o_flags, o_tflags, stats;
   mctrg::DevBuf tcXh, tcYh, tcXl, tcYl, tcScale, tcErr;   // tensor-core operands
   mctrg::DevBuf ozExp;                                     // FP64TC: row exponents of X and Yt
   mctrg::DevBuf Timp;                                      // impurity tensor (level0_distinct)
   mctrg::DevBuf bdb, keptb, sigtb, nkb, vrowsb, bdscr;    // bidiagonalization route
-  mctrg::DevBuf lrb;                                       // low-rank levels: reflectors, taus, core halves
 
   // per-kernel-class statistics (MCTRG_K_*)
   mctrg_kernel_stat kstat[MCTRG_K_COUNT]{};

@@ -192,7 +192,7 @@ struct mctrg_server {
       run_job(ctx, j);
       std::lock_guard<std::mutex> lk(mu);
       const size_t actual = ctx->held_bytes();
-      if (actual > w[wi].held) {       // the plan bound is exceeded only by the shared prefix
+      if (actual > w[wi].held) {       // the shared prefix is beside the plan
         reserved += actual - w[wi].held;
         w[wi].held = actual;
       }
