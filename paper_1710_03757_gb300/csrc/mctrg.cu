@@ -645,6 +645,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
   CK(o_sign.ensure((size_t)n));
   CK(o_flags.ensure((size_t)n));
   CK(stats.ensure(8 * sizeof(double)));
+  bool has_waits = false;   // this run's kernels can set the error word (a bounded wait expired)
   if (all_exact) {
     std::vector<double> hl((size_t)n, const_lnabs);
     std::vector<int8_t> hs((size_t)n, (int8_t)const_sign);
@@ -712,7 +713,8 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
       CK(tcScale.ensure(sizeof(double) * 2 * S));
     }
     if (rs.oz_rows) CK(ozExp.ensure(sizeof(int) * 2 * (size_t)S * rs.oz_rows));   // row exponents
-    if (prec != MCTRG_FP64 || rs.band) {
+    has_waits = prec != MCTRG_FP64 || rs.band;
+    if (has_waits) {
       CK(tcErr.ensure(sizeof(uint32_t)));
       CK(cudaMemsetAsync(tcErr.p, 0, sizeof(uint32_t), st));
     }
@@ -960,7 +962,7 @@ int mctrg_ctx::run(int64_t n, uint64_t seed, uint64_t first_traj, double* lnabs_
   if (sign_out) CK(cudaMemcpyAsync(sign_out, o_sign.p, (size_t)n, cudaMemcpyDefault, st));
   if (flags_out) CK(cudaMemcpyAsync(flags_out, o_flags.p, (size_t)n, cudaMemcpyDefault, st));
   uint32_t tc_err = 0;
-  if (tcErr.p && !all_exact)   // zeroed by every run that has such kernels
+  if (has_waits)
     CK(cudaMemcpyAsync(&tc_err, tcErr.p, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   resolve_events();
