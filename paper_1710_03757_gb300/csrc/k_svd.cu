@@ -41,10 +41,13 @@ static __device__ __forceinline__ double group_sum(double v, int G) {
 // orthogonal, in 25 FP64 instructions (three roots and three divisions are 120,
 // and each holds the pipe 16 cycles per warp): with h = be - al and q = 2 g, t = sign(h) q / (|h| + sqrt(h^2 +
 // q^2)) (Rutishauser's formula multiplied through by |q|).  Products leave the
-// exponent range only for rows of extreme scale, which take the ratio form.
+// exponent range only for rows of extreme scale, which take the root or ratio
+// form.  The squared test needs tol^2 al be normal too (tol >= 2^-52): a product
+// al be of 2^-800 to 2^1000.  Below, the threshold and g^2 would underflow, which
+// left rows of norms near 2^-250 unrotated up to a relative 2^-38.
 __device__ __forceinline__ bool rotate_pair(double al, double be, double g, double tol) {
   const double ab = al * be;
-  if (mid_range(ab)) return g * g > tol * tol * ab;
+  if ((unsigned)(((__double2hiint(ab) >> 20) & 0x7ff) - 223) < 1801u) return g * g > tol * tol * ab;
   return al > 0.0 && be > 0.0 && fabs(g) > tol * sqrt(al) * sqrt(be);
 }
 __device__ __forceinline__ void rotation(double al, double be, double g, double& t, double& cs) {
