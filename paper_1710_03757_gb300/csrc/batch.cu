@@ -68,14 +68,18 @@ struct TuneVal {
 
 std::mutex g_tune_mu;
 
-// Cache file: one line per shape, "n kc svd_items sample_grid".
+// Cache file: one line per timed shape of the one-stage reduction, "n kc
+// svd_items sample_grid".  A count of kUntimed is none that the tuner picks
+// (earlier files hold it for shapes of the two-stage route): such a line is
+// left out, so the shape is timed when the one-stage route needs it.
+constexpr int kUntimed = 1 << 16;
 void read_cache(const char* path, std::map<TuneKey, TuneVal>& m) {
   if (!path || !*path) return;
   FILE* f = std::fopen(path, "r");
   if (!f) return;
   int n, kc, s, g;
   while (std::fscanf(f, "%d %d %d %d", &n, &kc, &s, &g) == 4)
-    if (n > 0 && kc > 0 && s > 0 && g > 0) m[TuneKey{n, kc}] = TuneVal{s, g};
+    if (n > 0 && kc > 0 && s > 0 && s < kUntimed && g > 0) m[TuneKey{n, kc}] = TuneVal{s, g};
   std::fclose(f);
 }
 
@@ -302,7 +306,7 @@ struct BatchRunner {
   TuneVal tuned(int n, int kc) const {
     auto it = tune.find(TuneKey{n, kc});
     if (it != tune.end()) return it->second;
-    return TuneVal{1 << 16, sample_grid(n, kc)};
+    return TuneVal{kUntimed, sample_grid(n, kc)};
   }
 
   // ---- one sub-batch ---------------------------------------------------------
@@ -675,13 +679,9 @@ extern "C" int mctrg_batch_run(const mctrg_options* opt, const mctrg_job* jobs, 
     for (int k = c->s0 + 1; k < c->nlev && status == MCTRG_OK; ++k) {
       const int Kd = c->lv[k - 1].D * c->lv[k - 1].D;
       const int n = svd_dims(c->opt, c->lv[k], Kd).n;
-      if (!c->use_bidiag(n, Kd)) continue;
+      // (the two-stage route reduces per segment: no chunk of a merged launch to time)
+      if (!c->use_bidiag(n, Kd) || c->use_band(n, Kd)) continue;
       if (R.tune.count(TuneKey{n, c->lv[k].kc})) continue;
-      if (c->use_band(n, Kd)) {     // reduced per segment: no chunk of a merged launch to time
-        R.tune[TuneKey{n, c->lv[k].kc}] = TuneVal{1 << 16, sample_grid(n, c->lv[k].kc)};
-        R.tune_dirty = true;
-        continue;
-      }
       status = R.tune_shape(n, c->lv[k].kc);
     }
   }
