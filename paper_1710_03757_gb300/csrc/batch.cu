@@ -303,6 +303,7 @@ struct BatchRunner {
     return MCTRG_OK;
   }
 
+  // Geometry of a shape: the side of the split's matrices and the kept count.
   TuneVal tuned(int n, int kc) const {
     auto it = tune.find(TuneKey{n, kc});
     if (it != tune.end()) return it->second;
@@ -356,7 +357,8 @@ struct BatchRunner {
     // matrices of the one-stage reduction (ragged launches) and of the two-stage one
     // (reduced per segment below); bisection and inverse iteration take both
     std::vector<SvdItem> items, band_items;
-    int n_max = 0, n_one = 0, kmax = 0;
+    int n_max = 0, kmax = 0;
+    int n_one = 0, k_one = 0, kmax_one = 0;   // the largest one-stage shape; the largest kept count of any of them
     size_t smem = 0;
     BCK(fork(used) == MCTRG_OK ? cudaSuccess : cudaErrorUnknown);
     for (size_t s = 0; s < segs.size(); ++s) {
@@ -410,7 +412,10 @@ struct BatchRunner {
           BCK(launch_band_reduce(ba, true, ss));
           launches += 2 + 5 * (v.n / kBandW - 1);
         } else {
+          if (v.n > n_one) k_one = 0;
           n_one = std::max(n_one, v.n);
+          if (v.n == n_one) k_one = std::max(k_one, a.kc);
+          kmax_one = std::max(kmax_one, a.kc);
           smem = std::max(smem, bidiag_smem_bytes(v.n));
         }
         for (int64_t i = 0; i < g.cnt; ++i) {
@@ -431,7 +436,7 @@ struct BatchRunner {
         ja.nnz = q.nnz; ja.mflags = c->iflags.as<uint32_t>() + g.i0; ja.n = v.n; ja.n_pad = v.n_pad;
         ja.S = (int)g.cnt; ja.max_sweeps = c->opt.max_sweeps; ja.zero_rel = zero_fp64(a.n);
         BCK(launch_jacobi(ja, ss));
-        BCK(launch_sample_split(sample_args(r, g, q, 0, s), ss, tuned(a.n, a.kc).sample_grid));
+        BCK(launch_sample_split(sample_args(r, g, q, 0, s), ss, tuned(v.n, a.kc).sample_grid));
         BCK(expand_lowrank(r, g, q, ss));
         launches += 2;
       }
@@ -446,7 +451,7 @@ struct BatchRunner {
       BCK(table.ensure(sizeof(SvdItem) * items.size()));
       BCK(cudaMemcpyAsync(table.p, items.data(), sizeof(SvdItem) * items.size(), cudaMemcpyHostToDevice, st));
       const int S = (int)items.size();
-      const int chunk = S1 > 0 ? std::max(1, tuned(n_one, kmax).svd_items) : 1 << 16;
+      const int chunk = S1 > 0 ? std::max(1, tuned(n_one, k_one).svd_items) : kUntimed;
       for (int i0 = 0; i0 < S1; i0 += chunk) {
         BCK(launch_bidiag_items(table.as<SvdItem>() + i0, std::min(chunk, S1 - i0), n_one, smem, st));
         ++launches;
@@ -459,9 +464,8 @@ struct BatchRunner {
       for (size_t s = 0; s < segs.size(); ++s)
         if (segs[s].bidiag) {
           JobRun& r = jr[segs[s].j];
-          const LevelInfo& a = r.ctx->lv[segs[s].k];
-          BCK(launch_sample_split(sample_args(r, segs[s], ptr[s], 1, s), pool[s % kStreams],
-                                  tuned(a.n, a.kc).sample_grid));
+          const SampleArgs sa = sample_args(r, segs[s], ptr[s], 1, s);
+          BCK(launch_sample_split(sa, pool[s % kStreams], tuned(sa.n, sa.kc).sample_grid));
           ++launches;
         }
       BCK(join(used) == MCTRG_OK ? cudaSuccess : cudaErrorUnknown);
@@ -477,7 +481,7 @@ struct BatchRunner {
       }
       for (int i0 = 0; i0 < S1; i0 += chunk) {
         BdVecArgs va{};
-        va.n = n_one; va.S = std::min(chunk, S1 - i0); va.kmax = kmax; va.items = table.as<SvdItem>() + i0;
+        va.n = n_one; va.S = std::min(chunk, S1 - i0); va.kmax = kmax_one; va.items = table.as<SvdItem>() + i0;
         BCK(launch_bd_backtr(va, st));
         ++launches;
       }
@@ -485,10 +489,9 @@ struct BatchRunner {
       for (size_t s = 0; s < segs.size(); ++s)
         if (segs[s].bidiag) {
           JobRun& r = jr[segs[s].j];
-          const LevelInfo& a = r.ctx->lv[segs[s].k];
           BCK(band_backtr(r, segs[s], ptr[s], pool[s % kStreams]));
-          BCK(launch_sample_split(sample_args(r, segs[s], ptr[s], 2, s), pool[s % kStreams],
-                                  tuned(a.n, a.kc).sample_grid));
+          const SampleArgs sa = sample_args(r, segs[s], ptr[s], 2, s);
+          BCK(launch_sample_split(sa, pool[s % kStreams], tuned(sa.n, sa.kc).sample_grid));
           BCK(expand_lowrank(r, segs[s], ptr[s], pool[s % kStreams]));
           ++launches;
         }
@@ -707,9 +710,11 @@ extern "C" int mctrg_batch_run(const mctrg_options* opt, const mctrg_job* jobs, 
       size_t scr = 0;
       for (JobRun& r : R.jr)
         if (!r.ctx->all_exact)
-          for (int k = r.ctx->s0 + 1; k < r.ctx->nlev; ++k)
-            scr = std::max(scr, sample_scratch_doubles(r.ctx->lv[k].n, r.ctx->chi,
-                                                       R.tuned(r.ctx->lv[k].n, r.ctx->lv[k].kc).sample_grid));
+          for (int k = r.ctx->s0 + 1; k < r.ctx->nlev; ++k) {
+            const int Kd = r.ctx->lv[k - 1].D * r.ctx->lv[k - 1].D;
+            const int n = svd_dims(r.ctx->opt, r.ctx->lv[k], Kd).n;
+            scr = std::max(scr, sample_scratch_doubles(n, r.ctx->chi, R.tuned(n, r.ctx->lv[k].kc).sample_grid));
+          }
       R.smp_region = std::max<size_t>(scr, 1);
       if (status == MCTRG_OK && R.smp_scr.ensure(sizeof(double) * R.smp_region * BatchRunner::kStreams) != cudaSuccess)
         status = MCTRG_ENOMEM;
