@@ -17,14 +17,15 @@
 //     keep every entry below |A|_F), the FP64 operands (V, U, Y, Z) in 62-bit
 //     fixed point relative to their own row or column exponent, each operand
 //     split into eight signed 8-bit digits stored as FP16 (exact), and the
-//     digit products with i + j <= 7 accumulated by tcgen05.mma in tensor
-//     memory, one FP32 accumulator per digit group g = i + j (Ozaki, Ogita,
+//     digit products with i + j <= 7 (W and X: 8) accumulated by tcgen05.mma in
+//     tensor memory, one FP32 accumulator per digit group g = i + j (Ozaki, Ogita,
 //     Oishi and Rump 2012; sums of up to 256 products of 8-bit digits are
 //     integers below 2^24 for the leading groups, so FP32 holds them
 //     exactly; longer sums are read out and added in integers every 256).  The update is applied in integer arithmetic, so apart from
 //     the panel factorizations stage 1 issues no FP64 instruction per
 //     trailing element.
-//  2. band -> bidiagonal by bulge chasing (k_band_chase, one warp per matrix,
+//  2. band -> bidiagonal by bulge chasing (k_band_chase, eight warps a CTA whose
+//     sweeps follow one another, one to four matrices in each warp's lanes,
 //     the band in shared memory): per sweep i a right reflector clears row i
 //     beyond the superdiagonal, and alternating left and right reflectors of
 //     length <= b chase the bulge it creates down the band (LAPACK's dgbbrd
@@ -70,7 +71,8 @@ struct Work {
   double* ZU;   // [64]    Z U^T
   double* Y;    // [n][8]  rows relative to k+b
   int* el;      // [n]     row exponents of [V | Y]
-  int* er;      // [n]     column exponents of [Z ; U]
+  int* er;      // [n]     column exponents of [Z 2^-ez ; U]
+  int* ez;      // [1]     exponent of Z: every |z| < 2^ez
 };
 __device__ __forceinline__ Work work_of(double* base, int n) {
   Work w;
@@ -81,6 +83,7 @@ __device__ __forceinline__ Work work_of(double* base, int n) {
   w.Y = w.ZU + 64;
   w.el = (int*)(w.Y + (size_t)n * 8);
   w.er = (int*)(w.Y + (size_t)n * 9);
+  w.ez = w.er + n;
   return w;
 }
 
@@ -158,16 +161,25 @@ __device__ __forceinline__ uint32_t b_piece(int s, int j, int slot, int kh) {
   return (uint32_t)((s * 16 + j) * 128 + ((((slot << 1) | kh) ^ (j & 7)) << 4));
 }
 
-// The 36 digit products of a k-step as eight MMAs: slice i of A times the
-// slices 0 .. 7-i of B side by side (N = 16 (8 - i)) adds to the accumulators of
-// the digit groups i .. 7, 16 columns each.  One MMA per product read the A
+// The digit products of a k-step in the groups 0 .. G-1 as eight MMAs (36
+// products for G = 8, 43 for G = 9): slice i of A times the slices 0 ..
+// min(7, G-1-i) of B side by side (16 columns each) adds to the accumulators of
+// the digit groups i .. G-1, 16 columns each.  One MMA per product read the A
 // slice from shared memory 36 times, eight of them read it 8 times.
+template <int G>
 __device__ __forceinline__ void issue_products(uint32_t tmem, const uint8_t* A, const uint8_t* Bt, int slot, bool first) {
   const uint64_t a0 = umma_desc(smem_u32(A)), b0 = umma_desc(smem_u32(Bt)) + (uint64_t)(slot * 2);
 #pragma unroll
   for (int i = 0; i < kSl; ++i) {
     const uint64_t ad = a0 + (uint64_t)((((uint32_t)(i >> 2) * kTileBytes) + (i & 3) * 32) >> 4);
-    umma<1>(tmem + (uint32_t)(i * 16), ad, b0, umma_idesc_f16(kTileM, 16 * (kSl - i)), (first && i == 0) ? 0u : 1u);
+    const int cols = G - i < kSl ? G - i : kSl;      // slices of B
+    if (G > kSl && i == 1 && first) {
+      // slice 0 of A has set the groups 0 .. 7: the product of slices 1 and 7 starts group 8
+      umma<1>(tmem + (uint32_t)(kSl * 16), ad, b0 + (uint64_t)((7 * 16 * 128) >> 4), umma_idesc_f16(kTileM, 16), 0u);
+      umma<1>(tmem + 16u, ad, b0, umma_idesc_f16(kTileM, 16 * 7), 1u);
+    } else {
+      umma<1>(tmem + (uint32_t)(i * 16), ad, b0, umma_idesc_f16(kTileM, 16 * cols), (first && i == 0) ? 0u : 1u);
+    }
   }
 }
 
@@ -359,7 +371,7 @@ void band_carve(void* panels, void* refl, int n, int64_t S, BandArgs& a) {
 }
 
 // ---------------------------------------------------------------------------
-// Fixed-point copy of each matrix: e with |M|_F < 2^(e-1), Wk = round(M 2^(59-e)).
+// Fixed-point copy of each matrix: e with |M|_F < 2^(e-1), Wk = round(M 2^(62-e)).
 __global__ void __launch_bounds__(256) k_band_init(BandArgs a) {
   __shared__ double red[8];
   const int s = blockIdx.x, n = a.n;
@@ -420,6 +432,13 @@ __global__ void __launch_bounds__(256) k_band_qr(BandArgs a, int k) {
 namespace {
 constexpr uint32_t kStageBytes = 2 * kTileBytes;   // one k-step of A
 constexpr uint32_t kBBytes = 128 * 128;            // B: 128 rows x 4 k-steps
+// Digit groups of W and X.  A and the reflectors are in fixed point relative to
+// 2^eA > 2 |A|_F and to 1, so where |A|_F is well above the entries (a flat
+// spectrum: |A|_F = 10 s_1 at n = 256) the products need bits beyond the eight
+// groups that hold 64 of the whole: with eight, what was left out was the
+// largest error of the reduction (its singular values' rms error at n = 256,
+// flat, 2.3e-16 s_1; at n = 576 3.1e-16).
+constexpr int kProdGroups = 9;
 
 // Shared state of a product kernel.
 struct ProdShared {
@@ -438,7 +457,7 @@ __device__ __forceinline__ uint32_t prod_begin(ProdShared& ps, uint8_t* Bs, uint
   }
   // the rows 8 .. 15 of each slice of B stay zero
   for (int i = threadIdx.x; i < (int)(bbytes / 16); i += blockDim.x) ((uint4*)Bs)[i] = make_uint4(0, 0, 0, 0);
-  if (threadIdx.x < 32) tmem_alloc(&ps.tmem_slot, 128);
+  if (threadIdx.x < 32) tmem_alloc(&ps.tmem_slot, 256);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -474,7 +493,7 @@ __device__ __forceinline__ bool prod_stages(ProdShared& ps, uint32_t tmem, uint8
     if (ps.fail) break;
     if (t == 0) {
       tc_fence_after();
-      issue_products(tmem, As + (size_t)buf * kStageBytes, Bb, st & 3, st == s0);
+      issue_products<kProdGroups>(tmem, As + (size_t)buf * kStageBytes, Bb, st & 3, st == s0);
       umma_commit(&ps.bar[buf]);
     }
     ++committed;
@@ -494,16 +513,16 @@ __device__ __forceinline__ void prod_end(ProdShared& ps, uint32_t tmem, bool ok,
   }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x < 32) tmem_free(tmem, 128);
+  if (threadIdx.x < 32) tmem_free(tmem, 256);
 }
 
 // Columns 0 .. NJ-1 from `col` of this thread's row: the group sums g, added to
-// hi 2^32 + lo.
+// hi 2^40 + lo (groups 0 .. 3 and 4 .. 8).
 template <int NJ>
 __device__ __forceinline__ void prod_read(uint32_t taddr, long long (&hi)[NJ], long long (&lo)[NJ]) {
-  uint32_t v[kSl][NJ];
+  uint32_t v[kProdGroups][NJ];
 #pragma unroll
-  for (int g = 0; g < kSl; ++g) {
+  for (int g = 0; g < kProdGroups; ++g) {
     if constexpr (NJ == 8) tmem_ld_x8(taddr + (uint32_t)(g * 16), v[g]);
     else tmem_ld_x4(taddr + (uint32_t)(g * 16), v[g]);
   }
@@ -512,10 +531,9 @@ __device__ __forceinline__ void prod_read(uint32_t taddr, long long (&hi)[NJ], l
   for (int j = 0; j < NJ; ++j) {
     long long h = __float2int_rn(__uint_as_float(v[0][j])), l = __float2int_rn(__uint_as_float(v[4][j]));
 #pragma unroll
-    for (int g = 1; g < 4; ++g) {
-      h = (h << 8) + __float2int_rn(__uint_as_float(v[g][j]));
-      l = (l << 8) + __float2int_rn(__uint_as_float(v[4 + g][j]));
-    }
+    for (int g = 1; g < 4; ++g) h = (h << 8) + __float2int_rn(__uint_as_float(v[g][j]));
+#pragma unroll
+    for (int g = 5; g < kProdGroups; ++g) l = (l << 8) + __float2int_rn(__uint_as_float(v[g][j]));
     hi[j] += h;
     lo[j] += l;
   }
@@ -566,7 +584,7 @@ __global__ void __launch_bounds__(256, 2) k_band_gemm_w(BandArgs a, int k) {
     for (int e = 0; e < 8; ++e) x[e] = in ? p[(size_t)e * n] : 0ll;
   };
   load(0);
-  // row c of W^T: value = (hi 2^32 + lo) 2^(eA - 67); the two warp groups take four columns each
+  // row c of W^T: value = (hi 2^40 + lo) 2^(eA - 75); the two warp groups take four columns each
   const int jh = kh * 4;
   long long hi[4] = {}, lo[4] = {};
   const bool ok = prod_all(
@@ -582,10 +600,10 @@ __global__ void __launch_bounds__(256, 2) k_band_gemm_w(BandArgs a, int k) {
       [&]() { prod_read<4>(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)jh, hi, lo); });
   if (ok) {
     if (c < n) {
-      const double sc = p2(a.eA[s] - kFixBits - 5);
+      const double sc = p2(a.eA[s] - kFixBits - 13);
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        w.Z[(size_t)(jh + j) * n + (c - k - B)] = fma((double)hi[j], 4294967296.0 * sc, (double)lo[j] * sc);
+        w.Z[(size_t)(jh + j) * n + (c - k - B)] = fma((double)hi[j], 1099511627776.0 * sc, (double)lo[j] * sc);
     }
   }
   prod_end(ps, tmem, ok, a.err);
@@ -599,7 +617,8 @@ __global__ void __launch_bounds__(256, 4) k_band_lq(BandArgs a, int k) {
   extern __shared__ double R[];                      // [b][mp] the row panel, then Z
   __shared__ PanelShared sh;
   __shared__ double Ts[64], Vt[64], zu[64];
-  const int s = blockIdx.x, n = a.n, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  __shared__ int s_ez;
+  const int s = blockIdx.x, n = a.n, t = threadIdx.x, warp = t >> 5;
   const int mp = n - k - B;                          // columns k+b .. n-1
   double* Zs = R + (size_t)B * mp;
   long long* A = (long long*)a.Wk + (size_t)s * n * n;
@@ -608,7 +627,9 @@ __global__ void __launch_bounds__(256, 4) k_band_lq(BandArgs a, int k) {
   const double unit = p2(eA - kFixBits);
   Work w = work_of(a.work + (size_t)s * work_stride(n), n);
   if (t < 64) { Ts[t] = w.T[t]; Vt[t] = w.V[t]; }    // T and the top b x b block of V
+  if (t == 0) s_ez = kZeroExp;
   __syncthreads();
+  int ez = kZeroExp;
   for (int q = t; q < mp; q += blockDim.x) {
     const int c = k + B + q;
     asm volatile("" ::: "memory");                   // T and V stay in shared memory: in registers they would spill
@@ -631,9 +652,15 @@ __global__ void __launch_bounds__(256, 4) k_band_lq(BandArgs a, int k) {
       R[i * mp + q] = acc;
       Zs[i * mp + q] = z[i];
       w.Z[(size_t)i * n + q] = z[i];
+      ez = max(ez, exp_of(z[i]));
     }
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ez = max(ez, __shfl_xor_sync(0xffffffffu, ez, o));
+  if ((t & 31) == 0) atomicMax(&s_ez, ez);
   __syncthreads();
+  ez = s_ez == kZeroExp ? eA : s_ez;
+  if (t == 0) *w.ez = ez;
   double* band = a.band + ((size_t)s * n + k) * (B + 1) + B;
   panel_factor(R, mp, mp, sh, [&](int i, int j, double x) { band[i * (B + 1) + (j - i)] = x; });
   // Z U^T: warp i takes z_i against u_0..3 and u_4..7
@@ -645,15 +672,15 @@ __global__ void __launch_bounds__(256, 4) k_band_lq(BandArgs a, int k) {
     Ad[(size_t)(k + t / B) * n + k + (t % B)] = sh.T[t];
   }
   // U rows into the working matrix; the exponent of the update's right operand
-  // column [Z 2^-eA ; U]
+  // column [Z 2^-ez ; U]
   for (int q = t; q < mp; q += blockDim.x) {
     int e = kZeroExp;
 #pragma unroll
     for (int j = 0; j < B; ++j) {
       const double u = R[j * mp + q], z = Zs[j * mp + q];
       Ad[(size_t)(k + j) * n + k + B + q] = u;
-      const int ez = exp_of(z);
-      e = max(e, max(exp_of(u), ez == kZeroExp ? kZeroExp : ez - eA));
+      const int xz = exp_of(z);
+      e = max(e, max(exp_of(u), xz == kZeroExp ? kZeroExp : xz - ez));
     }
     w.er[q] = e;
   }
@@ -711,19 +738,20 @@ __global__ void __launch_bounds__(256, 2) k_band_gemm_x(BandArgs a, int k) {
     const int r = r0 + t;
     if (r < n) {
       const int eA = a.eA[s];
-      const double sc = p2(eA - kFixBits - 5);
+      const double sc = p2(eA - kFixBits - 13);
       double vr[B], xv[B], y[B];
 #pragma unroll
       for (int i = 0; i < B; ++i) vr[i] = w.V[(size_t)(r - k) * 8 + i];
 #pragma unroll
       for (int j = 0; j < B; ++j) {
-        double acc = fma((double)hi[j], 4294967296.0 * sc, (double)lo[j] * sc);
+        double acc = fma((double)hi[j], 1099511627776.0 * sc, (double)lo[j] * sc);
 #pragma unroll
         for (int i = 0; i < B; ++i) acc = fma(-vr[i], ZUs[i * B + j], acc);
         xv[j] = acc;
       }
-      // exponent of the update's left operand row [V 2^eA | Y] (both parts of
-      // the order of |A|; the right operand carries Z 2^-eA)
+      // exponent of the update's left operand row [V 2^ez | Y] (both parts of
+      // the order of the trailing matrix; the right operand carries Z 2^-ez)
+      const int ez = *w.ez;
       int e = kZeroExp;
 #pragma unroll
       for (int j = 0; j < B; ++j) {
@@ -732,7 +760,7 @@ __global__ void __launch_bounds__(256, 2) k_band_gemm_x(BandArgs a, int k) {
         for (int i = 0; i <= j; ++i) acc = fma(xv[i], TUs[i * B + j], acc);
         y[j] = acc;
         const int ev = exp_of(vr[j]);
-        e = max(e, max(exp_of(acc), ev == kZeroExp ? kZeroExp : ev + eA));
+        e = max(e, max(exp_of(acc), ev == kZeroExp ? kZeroExp : ev + ez));
       }
       const int ro = r - k - B;
 #pragma unroll
@@ -746,8 +774,9 @@ __global__ void __launch_bounds__(256, 2) k_band_gemm_x(BandArgs a, int k) {
 // ---------------------------------------------------------------------------
 // Trailing update A[k+b:][k+b:] -= [V | Y] [Z ; U] for one 128-row tile and up
 // to 256 columns (grid z), the 16-column tiles in turn: K = 2b = 16 (one k-step), applied in fixed point.
-// The operands are [V 2^eA | Y] and [Z 2^-eA ; U] (the same product): V and U
-// are of order 1, Y and Z of order |A|.  The row operand shares one exponent
+// The operands are [V 2^ez | Y] and [Z 2^-ez ; U] (the same product): V and U
+// are of order 1, Y and Z of that of the trailing matrix, 2^ez (below |A|_F by the
+// bits that 2^eA in its place cost: at n = 256 and a flat spectrum five).  The row operand shares one exponent
 // over the tile's rows, the column operand one over each block of 64 columns
 // (the largest of the per-row / per-column exponents: digits keep 62 bits of
 // the largest entry), so every element of a tile takes the same shifts.
@@ -779,7 +808,7 @@ __global__ void __launch_bounds__(256, 2) k_band_update(BandArgs a, int k) {
   long long* A = (long long*)a.Wk + (size_t)s * n * n;
   const double* Ad = (const double*)A;
   Work w = work_of(a.work + (size_t)s * work_stride(n), n);
-  const int eA = a.eA[s];
+  const int eA = a.eA[s], ez = *w.ez;
   if (t == 0) {
     us.fail = 0;
     us.el = kZeroExp;
@@ -805,14 +834,14 @@ __global__ void __launch_bounds__(256, 2) k_band_update(BandArgs a, int k) {
   __syncthreads();
   const int el = us.el;
   {
-    // A operand: row rho = [V[r] 2^eA | Y[r]]
+    // A operand: row rho = [V[r] 2^ez | Y[r]]
     const int rho = t & 127, part = t >> 7, r = r0 + rho;
     long long x[8];
     const bool in = r < n && el != kZeroExp;
 #pragma unroll
     for (int e = 0; e < 8; ++e)
       x[e] = !in ? 0ll
-                 : part == 0 ? fix_of(w.V[(size_t)(r - k) * 8 + e], kFloatP - el + eA)
+                 : part == 0 ? fix_of(w.V[(size_t)(r - k) * 8 + e], kFloatP - el + ez)
                              : fix_of(w.Y[(size_t)(r - k - B) * 8 + e], kFloatP - el);
     uint4 d[kSl];
     digits8(x, d);
@@ -820,7 +849,7 @@ __global__ void __launch_bounds__(256, 2) k_band_update(BandArgs a, int k) {
     for (int sl = 0; sl < kSl; ++sl) *(uint4*)(As + a_piece(sl, rho, part)) = d[sl];
   }
   for (int p = t; p < 2 * ((mp + 15) & ~15); p += 256) {
-    // B operand: column c = [Z[:, c] 2^-eA ; U[:, c]]
+    // B operand: column c = [Z[:, c] 2^-ez ; U[:, c]]
     const int half = (mp + 15) & ~15, part = p >= half, c = p - part * half;
     const int er = us.er[c >> 6];
     const bool in = c < mp && er != kZeroExp;
@@ -828,7 +857,7 @@ __global__ void __launch_bounds__(256, 2) k_band_update(BandArgs a, int k) {
 #pragma unroll
     for (int e = 0; e < 8; ++e)
       x[e] = !in ? 0ll
-                 : part == 0 ? fix_of(w.Z[(size_t)e * n + z0 + c], kFloatP - er - eA)
+                 : part == 0 ? fix_of(w.Z[(size_t)e * n + z0 + c], kFloatP - er - ez)
                              : fix_of(Ad[(size_t)(k + e) * n + k + B + z0 + c], kFloatP - er);
     uint4 d[kSl];
     digits8(x, d);
@@ -844,7 +873,7 @@ __global__ void __launch_bounds__(256, 2) k_band_update(BandArgs a, int k) {
   const int ntile = (mp + 15) >> 4;
   // MMAs of tile ct into accumulator ct & 1 (thread 0)
   auto issue = [&](int ct) {
-    issue_products(tmem + (uint32_t)((ct & 1) * 128), As, Bs + (size_t)(ct >> 2) * kBBytes, ct & 3, true);
+    issue_products<kSl>(tmem + (uint32_t)((ct & 1) * 128), As, Bs + (size_t)(ct >> 2) * kBBytes, ct & 3, true);
     umma_commit(&us.full[ct & 1]);
   };
   // this thread's rows (two) and column pair within a tile
@@ -915,6 +944,7 @@ __global__ void __launch_bounds__(256, 2) k_band_update(BandArgs a, int k) {
         const long long hi = (long long)pair(0, e) * 65536 + pair(2, e);
         const long long lo = (long long)pair(4, e) * 65536 + pair(6, e);
         if (sh < 0 && sh > -32) del[e] = (hi << (32 + sh)) + ((lo + (1ll << (-sh - 1))) >> (-sh));
+        else if (sh <= -32) del[e] = shift_round(hi + (lo >> 32), 32 + sh);   // what is left of lo is far below a unit
         else del[e] = shift_round(hi, 32 + sh) + shift_round(lo, sh);
       }
       q[2 * h].x -= del[0]; q[2 * h].y -= del[1];

@@ -318,10 +318,12 @@ bool route_bidiag(const mctrg_options& o, int n, int K) {
 // one 8.2 against 7.4; above 256, whole L = 16 runs: chi = 20, one trajectory 48
 // ms against 77, 128 173 against 294; chi = 24, 8 trajectories 83 against 206;
 // chi = 32, one 175 against 930).  The choice looks at the side alone, so a trajectory's
-// result does not depend on the batch.  Both are as accurate: singular values
-// against a quadruple-precision Jacobi, rms error over s_1 at n = 64, 1.5e-16 on
-// a flat spectrum and 4e-17 over 14 decades (the one-stage route 1.4e-16 and
-// 8.6e-17 before its bisection was refined, 7e-17 and 2e-17 since).
+// result does not depend on the batch.  Its singular values are no less accurate
+// than those that the one-stage route gave here before its counts were refined
+// (rms error over s_1 against an 80-bit Jacobi, spectra over 0.5 / 4 / 14 decades,
+// two-stage now against one-stage then: n = 200 14 / 5 / 4e-17 against 15 / 13 /
+// 9e-17; 256 13 / 5 / 2 against 15 / 13 / 9; 400 13 / 4 / 3 against 15 / 14 / 11;
+// 576 15 / 4 / 3 against 15 / 13 / 10).  The one-stage route since: 6 / 2 / 2e-17.
 constexpr int kAutoBandMin = 200;
 bool route_band(const mctrg_options& o, int n, int K) {
   const bool named = o.svd == MCTRG_SVD_BAND, chosen = o.svd == MCTRG_SVD_AUTO && n >= kAutoBandMin;
