@@ -1160,7 +1160,7 @@ constexpr int kBtThreads = 128;
 template <int GV>
 __global__ void __launch_bounds__(kBtThreads) k_band_backtr(BandArgs a, BandVecArgs va, int nref) {
   extern __shared__ double Vs[];                     // [GV][n+1], then U [8][n]
-  __shared__ double tv[GV][B + 1], tp[GV][B + 1];
+  __shared__ double tv[GV][B + 1], tp[GV][B + 1], s_scale[GV];
   const int s = blockIdx.x, n = a.n, t = threadIdx.x;
   const int ld = n + 1;
   double* Us = Vs + (size_t)GV * ld;
@@ -1234,12 +1234,18 @@ __global__ void __launch_bounds__(kBtThreads) k_band_backtr(BandArgs a, BandVecA
     }
     __syncthreads();
   }
+  // the two stages' n^2 / 16 reflectors have moved the vectors' lengths by some sqrt(n) roundings: unit again
   const double* sg = va.sig + (size_t)s * va.n_pad;
   const int* kept = va.kept + (size_t)s * va.kstride + g0;
-  for (int e = t; e < nk * n; e += kBtThreads) {
-    const double x = Vs[(e / n) * ld + e % n];
-    vrow[e] = va.unit_rows ? x : sg[kept[e / n]] * x;
+  for (int q = t >> 5; q < nk; q += kBtThreads / 32) {
+    const double* x = Vs + (size_t)q * ld;
+    double p = 0.0;
+    for (int c = t & 31; c < n; c += 32) p = fma(x[c], x[c], p);
+    p = warp_sum(p);
+    if ((t & 31) == 0) s_scale[q] = p > 0.0 ? (va.unit_rows ? 1.0 : sg[kept[q]]) * inv_sqrt(p) : 0.0;
   }
+  __syncthreads();
+  for (int e = t; e < nk * n; e += kBtThreads) vrow[e] = s_scale[e / n] * Vs[(e / n) * ld + e % n];
 }
 
 // ---------------------------------------------------------------------------

@@ -55,3 +55,15 @@ def test_rms_error_on_a_flat_spectrum(torch, n):
     rms = np.sqrt((((sig - ref) / ref[:, :1]) ** 2).mean())
     print("n %d: rms error %.2e s_1" % (n, rms))
     assert rms <= 2.0e-16
+
+
+@pytest.mark.parametrize("n,n_vec,batch", [(64, 3, 5), (200, 16, 5), (256, 16, 5), (256, 16, 200)])
+def test_vectors_have_unit_length(torch, n, n_vec, batch):
+    # the squared length is summed over n / 32 terms and five steps of a tree, at most 13 roundings, its root and the
+    # scaling take three more and each entry's rounding one: |v|^2 = 1 within 2 (13 / 2 + 4) 2^-53 at worst, and within
+    # half of that as roundings average (without the scaling 1.3e-15 to 3e-15)
+    rng = np.random.default_rng(n + batch)
+    A = rng.standard_normal((batch, n, n)) * np.logspace(0, -8, n) @ rng.standard_normal((n, n))
+    _, vt = _svd(torch, A, n_vec)
+    lengths = (vt.astype(np.longdouble) ** 2).sum(2)
+    assert float(np.abs(lengths - 1).max()) <= 10.5 * 2.0 ** -53
