@@ -132,11 +132,13 @@ __device__ __forceinline__ double reduce4(double p0, double p1, double p2, doubl
 // 1 / sqrt(t) and 1 / d for normal t > 0 and normal d: the hardware's
 // approximation (relative error below 2^-19) and one third-order step of
 // Householder's iteration (y (1 + e / 2 + 3 e^2 / 8) with e = 1 - t y^2, and
-// r (1 + e + e^2) with e = 1 - d r), whose own error is e^3 <= 2^-57; five and
-// three FP64 instructions, about half of what rsqrt() and a division issue on
-// a pipe that a warp-wide FP64 instruction holds 16 cycles.  Results within an
-// ulp of the correctly rounded ones.  Magnitudes outside 2^-1000 .. 2^1000 take
-// the functions.
+// r (1 + e + e^2) with e = 1 - d r); five and three FP64 instructions, about half
+// of what rsqrt() and a division issue on a pipe that a warp-wide FP64
+// instruction holds 16 cycles.  Relative errors: the reciprocal's e^3 <= 2^-57 and
+// a rounding, 1.07 2^-53; the root's (5 / 16) e^3 <= 2^-55.6 with e <= 2^-18, the
+// rounding of t y, which enters halved, and a last one, 1.67 2^-53 (rsqrt() is
+// within an ulp, 2 2^-53).  Magnitudes outside 2^-1000 .. 2^1000 take the
+// functions.
 __device__ __forceinline__ bool mid_range(double x) {
   return (unsigned)(((__double2hiint(x) >> 20) & 0x7ff) - 23) < 2001u;
 }
