@@ -83,11 +83,6 @@ __device__ __forceinline__ uint32_t oz_b_piece(int s, int j, int slot, int kh) {
 }
 }  // namespace
 
-void ozaki_params(int K, int* bits, int* slices) {
-  *bits = K <= 256 ? 8 : 7;
-  *slices = K <= 256 ? 7 : 8;
-}
-
 bool gemm_ozaki_supported(int n, int K) { return n >= 1 && K >= 64 && K % 64 == 0 && K <= 1024; }
 
 // Row exponents, one warp per row: e with max = f 2^e, f in [0.5, 1).

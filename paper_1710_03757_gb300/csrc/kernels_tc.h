@@ -43,8 +43,6 @@ struct GemmOzArgs {
   int* expY;
   bool aligned, wide;
 };
-// Digit width b (bits) and number of digits s for inner dimension K.
-void ozaki_params(int K, int* bits, int* slices);
 bool gemm_ozaki_supported(int n, int K);
 cudaError_t launch_gemm_ozaki(const GemmOzArgs& a, cudaStream_t st);
 
