@@ -37,10 +37,10 @@ FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0}
 # library's DFMA probe measured in the same run; this is the fallback.
 FP64_NOMINAL_TFLOPS = 1.25
 # DRAM bytes (read + write) of one 256 x 256 matrix, from ncu captures of the
-# kernels on a case of 128 such matrices (Ising 32 x 32, chi = 16):
-# k_jacobi_warp 2.66 GB and k_bidiag 917.1 MB per launch of 128.
-JACOBI_DRAM_BYTES_PER_MATRIX_N256 = 2.658e9 / 128
-BIDIAG_DRAM_BYTES_PER_MATRIX_N256 = 917.06e6 / 128
+# kernels: k_jacobi_warp 27.80 GB per launch of 128, k_bidiag 4.588 GB per
+# launch of 304 (full-rank matrices, spectra over 14 decades).
+JACOBI_DRAM_BYTES_PER_MATRIX_N256 = 27.803e9 / 128
+BIDIAG_DRAM_BYTES_PER_MATRIX_N256 = 4.5882e9 / 304
 
 
 def measured_peaks():

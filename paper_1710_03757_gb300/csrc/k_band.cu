@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(256) k_band_qr(BandArgs a, int k) {
 // What bounds them: reading the trailing matrix (8 bytes an element; W at 2.8
 // TB/s of DRAM) and splitting it (about 14 instructions an element), and X's
 // FP64 epilogue; two CTAs an SM.  Third panel of 304 matrices of n = 256: W 141
-// -> 54 us, X 129 -> 82 us, against one buffer, stages of 32 and one MMA per
+// -> 54 us, X 129 -> 85 us, against one buffer, stages of 32 and one MMA per
 // digit product.
 namespace {
 constexpr uint32_t kStageBytes = 2 * kTileBytes;   // one k-step of A
@@ -789,7 +789,7 @@ __global__ void __launch_bounds__(256, 2) k_band_gemm_x(BandArgs a, int k) {
 // four lanes the eight columns of a row, so the reads and writes of the
 // trailing matrix cover whole sectors (one row per lane, the first form of
 // this kernel, touched 32 lines with every instruction and wrote half sectors:
-// 186 us for the third panel of 304 matrices of n = 256, 88 us so).  What bounds
+// 186 us for the third panel of 304 matrices of n = 256, 87 us so).  What bounds
 // it: the 16 bytes an element read and written (2.7 TB/s of DRAM at that size).
 struct UpdShared {
   uint64_t full[2], empty[2];
